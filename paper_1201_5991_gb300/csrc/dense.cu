@@ -10,6 +10,7 @@
 //    Lambda_i = R - G_i^{-1}), K_Ci = Psi_i^T K_i Psi_i = -Lambda_i = G_i^{-1} - R, where
 //    R = diag(rho c_rho) (rho on the rows that augment A_i, 0 on Stokes pressure rows).
 #include "internal.h"
+#include "reduce.cuh"
 
 namespace bddc {
 
@@ -708,11 +709,11 @@ __global__ void __launch_bounds__(256) k_rows_matvec(LevelDev L, const T* __rest
   }
   __syncthreads();
   const int rows = min(NB, m.nc - rb * NB);
-  T acc[8][NR];
+  T acc[NR][8];
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+  for (int q = 0; q < NR; ++q)
 #pragma unroll
-    for (int q = 0; q < NR; ++q) acc[r][q] = (T)0;
+    for (int r = 0; r < 8; ++r) acc[q][r] = (T)0;
   for (int j = j0; j < j1; ++j) {
     const T* t = m_tile<T, MODE>(L, m, rb, j) + 2 * lane;
     V2 xv[NR];
@@ -724,22 +725,18 @@ __global__ void __launch_bounds__(256) k_rows_matvec(LevelDev L, const T* __rest
       if (row < rows) {
         const V2 a = __ldg((const V2*)(t + row * NB));
 #pragma unroll
-        for (int q = 0; q < NR; ++q) acc[r][q] += a.x * xv[q].x + a.y * xv[q].y;
+        for (int q = 0; q < NR; ++q) acc[q][r] += a.x * xv[q].x + a.y * xv[q].y;
       }
     }
   }
+  constexpr int NV = 8 * NR, NC = NV < 32 ? 1 : NV / 32;
+  lane_sums<NV>(&acc[0][0], lane);
+  if (lane_sum_writer<NV>(lane))
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int row = warp + 8 * r;
-    if (row >= rows) continue;   // warp-uniform
-#pragma unroll
-    for (int q = 0; q < NR; ++q) {
-      T a = acc[r][q];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-      if (lane == 0) part[((int64_t)q * sum_nc + m.c_off + rb * NB + row) * zmax + z] = (double)a;
+    for (int k = 0; k < NC; ++k) {
+      const int f = lane_sum_index<NV>(lane) + k, q = f / 8, row = warp + 8 * (f % 8);
+      if (row < rows) part[((int64_t)q * sum_nc + m.c_off + rb * NB + row) * zmax + z] = (double)(&acc[0][0])[k];
     }
-  }
 }
 
 // out[q sum_nc + g] = sum_{z < zmax} part[(q sum_nc + g) zmax + z], in order
@@ -966,13 +963,8 @@ __global__ void k_coarse_apply(const float* __restrict__ W, int64_t npad, const 
       acc[q] += a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w;
     }
   }
-#pragma unroll
-  for (int q = 0; q < NR; ++q) {
-    float v = acc[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) y[(c0 + q) * n_vec + row] = v;
-  }
+  lane_sums<NR>(acc, lane);
+  if (lane_sum_writer<NR>(lane)) y[(c0 + lane_sum_index<NR>(lane)) * n_vec + row] = acc[0];
 }
 
 }  // namespace

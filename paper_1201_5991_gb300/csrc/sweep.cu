@@ -25,6 +25,7 @@
 #include <cstdint>
 
 #include "internal.h"
+#include "reduce.cuh"
 
 namespace bddc {
 
@@ -173,12 +174,12 @@ __global__ void __launch_bounds__(kThreads, 2)
       }
       issued += pre;
     }
-    T acc[8][NR];        // forward: rows warp + 8 r, this lane's two columns, every right-hand side
+    T acc[NR][8];        // forward: rows warp + 8 r, this lane's two columns, every right-hand side
     T accc[NR][2];       // backward: this lane's two columns, summed over the warp's rows
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int q = 0; q < NR; ++q)
 #pragma unroll
-      for (int q = 0; q < NR; ++q) acc[r][q] = (T)0;
+      for (int r = 0; r < 8; ++r) acc[q][r] = (T)0;
 #pragma unroll
     for (int q = 0; q < NR; ++q) accc[q][0] = accc[q][1] = (T)0;
     int staged_end = 0;   // tiles [staged_begin, staged_end) have their solution block in ybuf
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(kThreads, 2)
           for (int q = 0; q < NR; ++q) {
             const V2 yv = *(const V2*)(&ybuf[ys][q][2 * lane]);
 #pragma unroll
-            for (int r = 0; r < 8; ++r) acc[r][q] += a[r].x * yv.x + a[r].y * yv.y;
+            for (int r = 0; r < 8; ++r) acc[q][r] += a[r].x * yv.x + a[r].y * yv.y;
           }
         } else {
 #pragma unroll
@@ -268,15 +269,19 @@ __global__ void __launch_bounds__(kThreads, 2)
       } else {
         // diagonal block: right-hand side, then D_i^{-1} (forward) or D_i^{-T} (backward)
         if (!BWD) {
+          // the row sums over the lanes (N = 8 NR values per lane): value 8 q + r is row warp + 8 r of
+          // right-hand side q.  They end a link of the dependency chain; as one butterfly per value
+          // they bound the forward sweep where the factor is small or FP64 (64 subdomains of 6^3
+          // elements, FP64 interior: 166 us against 54 us for the backward sweep).  Whole calls with
+          // lane_sums instead: FP64 24^3 elasticity 84.6 -> 73.9 ms, FP32 solve of 24^3 (8 subdomains)
+          // 18.3 -> 15.5 ms, FP64 operator on 8 columns (48^3) 9.61 -> 7.94 ms, same bits
+          constexpr int NV = 8 * NR, NC = NV < 32 ? 1 : NV / 32;
+          const int f0 = lane_sum_index<NV>(lane);
+          const bool writer = lane_sum_writer<NV>(lane);
+          lane_sums<NV>(&acc[0][0], lane);
+          if (writer)
 #pragma unroll
-          for (int q = 0; q < NR; ++q)
-#pragma unroll
-            for (int r = 0; r < 8; ++r) {
-              T a = acc[r][q];
-#pragma unroll
-              for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-              if (lane == 0) rhs[q][warp + 8 * r] -= a;
-            }
+            for (int k = 0; k < NC; ++k) rhs[(f0 + k) / 8][warp + 8 * ((f0 + k) % 8)] -= (&acc[0][0])[k];
           __syncthreads();
           const bool signed_rows = L.indefinite != 0;   // forward output is S L^{-1} b
           V2 a[8];
@@ -286,17 +291,18 @@ __global__ void __launch_bounds__(kThreads, 2)
           for (int q = 0; q < NR; ++q) {
             const V2 rv = *(const V2*)(&rhs[q][2 * lane]);
 #pragma unroll
-            for (int r = 0; r < 8; ++r) {
-              T yv = a[r].x * rv.x + a[r].y * rv.y;
-#pragma unroll
-              for (int o = 16; o > 0; o >>= 1) yv += __shfl_xor_sync(0xffffffffu, yv, o);
-              if (lane == 0) {
-                const T out = signed_rows ? yv * s_sg[warp + 8 * r] : yv;
-                v[q * vstride + i * NB + warp + 8 * r] = out;
-                pub_st(pv + q * vstride + i * NB + warp + 8 * r, out);
-              }
-            }
+            for (int r = 0; r < 8; ++r) acc[q][r] = a[r].x * rv.x + a[r].y * rv.y;
           }
+          lane_sums<NV>(&acc[0][0], lane);
+          if (writer)
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+              const int q = (f0 + k) / 8, row = warp + 8 * ((f0 + k) % 8);
+              const T yv = (&acc[0][0])[k];
+              const T out = signed_rows ? yv * s_sg[row] : yv;
+              v[q * vstride + i * NB + row] = out;
+              pub_st(pv + q * vstride + i * NB + row, out);
+            }
         } else {
 #pragma unroll
           for (int q = 0; q < NR; ++q) {

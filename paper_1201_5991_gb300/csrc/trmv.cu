@@ -10,6 +10,7 @@
 // the outer iteration applies the FP64 operator.  Several right-hand sides share each pass over
 // the triangle (up to eight per launch).
 #include "internal.h"
+#include "reduce.cuh"
 
 namespace bddc {
 
@@ -86,11 +87,11 @@ __global__ void __launch_bounds__(256) k_trmv_n(LevelDev L, const float* __restr
   const float* tiles = (const float*)L.tiles + m.tile_off;
   const float* yv = y1 + c0 + m.vec_off;
   const float* sg = (const float*)L.sgn + m.vec_off;
-  float acc[8][NR];
+  float acc[NR][8];
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+  for (int q = 0; q < NR; ++q)
 #pragma unroll
-    for (int q = 0; q < NR; ++q) acc[r][q] = 0.f;
+    for (int r = 0; r < 8; ++r) acc[q][r] = 0.f;
 #pragma unroll 2
   for (int j = m.nIb; j <= i; ++j) {
     float2 sj = make_float2(1.f, 1.f);
@@ -105,17 +106,16 @@ __global__ void __launch_bounds__(256) k_trmv_n(LevelDev L, const float* __restr
       b.x *= sj.x;
       b.y *= sj.y;
 #pragma unroll
-      for (int r = 0; r < 8; ++r) acc[r][q] += a[r].x * b.x + a[r].y * b.y;
+      for (int r = 0; r < 8; ++r) acc[q][r] += a[r].x * b.x + a[r].y * b.y;
     }
   }
+  constexpr int NV = 8 * NR, NC = NV < 32 ? 1 : NV / 32;
+  lane_sums<NV>(&acc[0][0], lane);
+  if (lane_sum_writer<NV>(lane))
 #pragma unroll
-  for (int q = 0; q < NR; ++q)
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      float v = acc[r][q];
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-      if (lane == 0) y[c0 + q * L.n_vec + m.vec_off + (int64_t)i * NB + warp + 8 * r] = v;
+    for (int k = 0; k < NC; ++k) {
+      const int f = lane_sum_index<NV>(lane) + k, q = f / 8;
+      y[c0 + q * L.n_vec + m.vec_off + (int64_t)i * NB + warp + 8 * (f % 8)] = (&acc[0][0])[k];
     }
 }
 
@@ -237,11 +237,11 @@ __global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, const float
   for (int q = 0; q < NR; ++q)
 #pragma unroll
     for (int r = 0; r < 8; ++r) xi[q][r] = xv[q * L.n_vec + (int64_t)i * NB + warp + 8 * r];
-  float acc[8][NR];
+  float acc[NR][8];
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+  for (int q = 0; q < NR; ++q)
 #pragma unroll
-    for (int q = 0; q < NR; ++q) acc[r][q] = 0.f;
+    for (int r = 0; r < 8; ++r) acc[q][r] = 0.f;
   float* prow = part + (int64_t)blockIdx.z * NR * part_stride + part_off[s] + (int64_t)i * (i - 1) / 2 * NB;
   bool lost = false;
   for (int j = 0; j < ntile; ++j) {
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, const float
       for (int r = 0; r < 8; ++r)
 #pragma unroll
         for (int q = 0; q < NR; ++q) {
-          acc[r][q] += a[r].x * xj[q].x + a[r].y * xj[q].y;
+          acc[q][r] += a[r].x * xj[q].x + a[r].y * xj[q].y;
           cs[q].x += a[r].x * xi[q][r];
           cs[q].y += a[r].y * xi[q][r];
         }
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, const float
         const float bx = c < row ? a[r].x : 0.f, by = c + 1 < row ? a[r].y : 0.f;
 #pragma unroll
         for (int q = 0; q < NR; ++q) {
-          acc[r][q] += ax * xj[q].x + ay * xj[q].y;
+          acc[q][r] += ax * xj[q].x + ay * xj[q].y;
           cs[q].x += bx * xi[q][r];
           cs[q].y += by * xi[q][r];
         }
@@ -308,20 +308,17 @@ __global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, const float
         dcol[q][c] = v;
     }
   }
-  // row sums over the lanes, fixed order (xor butterfly)
-#pragma unroll
-  for (int r = 0; r < 8; ++r)
-#pragma unroll
-    for (int q = 0; q < NR; ++q)
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc[r][q] += __shfl_xor_sync(0xffffffffu, acc[r][q], o);
+  // row sums over the lanes, fixed order
+  constexpr int NV = 8 * NR, NC = NV < 32 ? 1 : NV / 32;
+  lane_sums<NV>(&acc[0][0], lane);
   __syncthreads();   // dcol is complete
-  if (lane == 0) {
+  if (lane_sum_writer<NV>(lane)) {
     float* yv = y + c0q + m.vec_off + (int64_t)m.nIb * NB + (int64_t)i * NB;
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
-#pragma unroll
-      for (int q = 0; q < NR; ++q) yv[q * L.n_vec + warp + 8 * r] = acc[r][q] + dcol[q][warp + 8 * r];
+    for (int k = 0; k < NC; ++k) {
+      const int f = lane_sum_index<NV>(lane) + k, q = f / 8, row = warp + 8 * (f % 8);
+      yv[q * L.n_vec + row] = (&acc[0][0])[k] + dcol[q][row];
+    }
   }
   // after a lost wait, copies may still be landing in this CTA's shared memory: wait (bounded)
   // for the last phase issued on every stage before the CTA exits
