@@ -226,6 +226,9 @@ template <typename T>
 void launch_gather_glob(const LevelDev& L, const double* x, int part, T* loc, cudaStream_t st, int nr = 1);
 template <typename T>
 void launch_scatter_interior(const LevelDev& L, const T* loc, double* y, cudaStream_t st, int nr = 1);
+// y[g] = a - b at the interior positions (levels' interior DOFs are held by one subdomain each)
+void launch_scatter_interior_diff(const LevelDev& L, const double* a, const double* b, double* y, cudaStream_t st,
+                                  int nr = 1);
 // rows: flat padded row indices (interior rows, interface rows or both, of every subdomain)
 void launch_spmv_rows(const LevelDev& L, const int64_t* rows, int64_t nrows, const double* x, double* y, double alpha,
                       double beta, const int32_t* row_sub, cudaStream_t st, int nr = 1);

@@ -62,6 +62,15 @@ __global__ void k_scatter_interior(LevelDev L, const T* __restrict__ loc, double
   if (g >= 0 && L.loc2iface[p] < 0) y[(int64_t)blockIdx.y * L.n_dof + g] = (double)loc[(int64_t)blockIdx.y * L.n_vec + p];
 }
 
+__global__ void k_scatter_interior_diff(LevelDev L, const double* __restrict__ a, const double* __restrict__ b,
+                                        double* __restrict__ y) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= L.n_vec) return;
+  const int32_t g = L.loc2glob[p];
+  const int64_t o = (int64_t)blockIdx.y * L.n_vec + p;
+  if (g >= 0 && L.loc2iface[p] < 0) y[(int64_t)blockIdx.y * L.n_dof + g] = a[o] - b[o];
+}
+
 // y[row] = beta*y[row] + alpha * (K_i x)[row] for the rows of a list (interior rows, interface
 // rows or all rows of every subdomain); 16 lanes per row, two rows per warp.
 __global__ void k_spmv(LevelDev L, const int64_t* __restrict__ rows, int64_t nrows, const double* __restrict__ x,
@@ -369,6 +378,10 @@ void launch_gather_glob(const LevelDev& L, const double* x, int part, T* loc, cu
 template <typename T>
 void launch_scatter_interior(const LevelDev& L, const T* loc, double* y, cudaStream_t st, int nr) {
   if (L.n_vec > 0) { note_launch(); k_scatter_interior<T><<<dim3(nblocks(L.n_vec, 256), nr), 256, 0, st>>>(L, loc, y); }
+}
+void launch_scatter_interior_diff(const LevelDev& L, const double* a, const double* b, double* y, cudaStream_t st,
+                                  int nr) {
+  if (L.n_vec > 0) { note_launch(); k_scatter_interior_diff<<<dim3(nblocks(L.n_vec, 256), nr), 256, 0, st>>>(L, a, b, y); }
 }
 void launch_spmv_rows(const LevelDev& L, const int64_t* rows, int64_t nrows, const double* x, double* y, double alpha,
                       double beta, const int32_t* row_sub, cudaStream_t st, int nr) {
