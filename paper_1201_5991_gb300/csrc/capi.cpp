@@ -25,6 +25,7 @@
 #include "../../include/bddc.h"
 #include "analysis.h"
 #include "internal.h"
+#include "tc_items.h"
 
 namespace bddc {
 
@@ -906,9 +907,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
       int64_t acc = 0;
       for (int64_t s = 0; s < ns; ++s) {
         pref[(size_t)u * (ns + 1) + s] = acc;
-        const SubMeta& m = L.meta[s];
-        const int ib = std::min(ibeg, (int)m.Bc);
-        for (int j = jbeg; j < std::min((int)m.Bc, jend); j += 2) acc += (m.R - std::max(j, ib) + 1) / 2;
+        acc += tc_items_count(tc_items_of(L.meta[s], jbeg, jend, ibeg, v >= 3));
       }
       pref[(size_t)u * (ns + 1) + ns] = acc;
       L.tc_items[u] = acc;
@@ -2843,8 +2842,7 @@ int bddc_tc_update_check(int64_t n, int rank, float* a, double* ms) {
       const int64_t* prow_off = A.upload(std::vector<int64_t>{0}, st);
       uint8_t* split = A.alloc<uint8_t>((int64_t)nb * kPanel * 2 * NB2 * 2);
       float* rscale = A.alloc<float>((int64_t)nb * NB);
-      int64_t items = 0;
-      for (int j = nt; j < nb; j += 2) items += (nb - j + 1) / 2;
+      const int64_t items = tc_items_count(tc_items_of(m, nt, nb, 0, 0));
       const int64_t* item_pref = A.upload(std::vector<int64_t>{0, items}, st);
       TensorMap128 tmap{};
       const int r = make_tile_tmap(&tmap, (float*)d.tiles, tile_elems);

@@ -39,12 +39,13 @@
 
 #include "internal.h"
 #include "split.cuh"
+#include "tc_items.h"
 
 namespace bddc {
 
 namespace {
 
-constexpr long long kSpinLimit = 1ll << 26;
+constexpr uint32_t kSpinLimit = 1u << 26;
 
 __device__ __forceinline__ int64_t tile_index(int i, int j, int Bc) {
   return i < Bc ? ((int64_t)i * (i + 1) / 2 + j) : ((int64_t)Bc * (Bc + 1) / 2 + (int64_t)(i - Bc) * Bc + j);
@@ -77,9 +78,53 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 
 constexpr uint32_t kOpnd = 2 * kTilePart;        // one part of a 128-row operand (16 KB)
 constexpr uint32_t kStage2 = 4 * kOpnd;          // A hi, A lo, B hi, B lo (64 KB)
-constexpr int kThreads2 = 320;                   // 8 epilogue warps + 1 MMA warp + 1 producer warp
+constexpr int kThreads2 = 352;                   // 8 epilogue warps + 2 MMA warps + 1 producer warp
 constexpr int kStages2 = 3;                      // shared-memory stages (copies run two steps ahead)
+constexpr int kMmaBars = 6;                      // step-completion barriers (two steps sharing one are 6 apart)
 constexpr uint32_t kEpiBox = 32 * 128;           // per epilogue warp: one 32 x 32 FP32 output box (4 KB)
+
+__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// bounded wait for the completion of a phase (its first test stands alone: the usual case)
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+  if (mbar_try_wait(bar, parity)) return true;
+  for (uint32_t spins = 0; spins < kSpinLimit; ++spins)
+    if (mbar_try_wait(bar, parity)) return true;
+  return false;
+}
+
+// position in a ring of N barriers and the parity of its current phase
+template <int N>
+struct Ring {
+  uint32_t k = 0, phase = 0;
+  __device__ __forceinline__ void next() {
+    if (++k == N) {
+      k = 0;
+      phase ^= 1u;
+    }
+  }
+};
+
+// 32 columns of this warp's TMEM lanes (lane l: row l), complete on return
+__device__ __forceinline__ void tmem_ld32(float (&v)[32], uint32_t taddr) {
+  uint32_t* u = (uint32_t*)v;
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,"
+      "%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]), "=r"(u[7]), "=r"(u[8]),
+        "=r"(u[9]), "=r"(u[10]), "=r"(u[11]), "=r"(u[12]), "=r"(u[13]), "=r"(u[14]), "=r"(u[15]), "=r"(u[16]),
+        "=r"(u[17]), "=r"(u[18]), "=r"(u[19]), "=r"(u[20]), "=r"(u[21]), "=r"(u[22]), "=r"(u[23]), "=r"(u[24]),
+        "=r"(u[25]), "=r"(u[26]), "=r"(u[27]), "=r"(u[28]), "=r"(u[29]), "=r"(u[30]), "=r"(u[31])
+      : "r"(taddr)
+      : "memory");
+}
 
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
@@ -135,23 +180,42 @@ __global__ void __launch_bounds__(256) k_split_inverse(LevelDev L, int k0, const
   split_rows<4>(src, rm, prow_off[s] + k0 + Q, split, nullptr, rscale, nullptr);
 }
 
-// Persistent: CTA c takes the work items c, c + gridDim.x, ... of the panel (items of all
-// subdomains flattened; item_pref[s] = first item of subdomain s).  One global step per (item,
-// panel column); step g uses shared-memory stage g % 3 and TMEM accumulator pair g & 1.  Three
-// roles run in their own warps: a producer thread requests the copies of each step as soon as its
-// stage is free, one thread issues the MMAs as soon as a stage is full and an accumulator pair
-// free (a single thread doing both waited, before every refill, for the MMAs of the previous step
-// to complete: 1.7 us per step, with the copies and the tensor pipe mostly idle), and the epilogue
-// warps promote the accumulators and write back each item's output block.  The write-back is a TMA reduce-add: each epilogue warp scales
-// its 32 x 64 part of the block into a swizzled shared-memory box, 32 columns at a time, and one
-// lane adds the box into the tiles in L2 (the output is never read into the SM; every element
-// receives exactly one add per launch, so the result does not depend on timing).
+// Persistent: CTA c takes the work items c, c + gridDim.x, ... of the launch (items of all
+// subdomains flattened; item_pref[s] = first item of subdomain s).  One global step g per (item, panel
+// column).  Roles, in warps of their own: a producer thread requests the copies of each step into
+// shared-memory stage g % 3 as soon as the MMAs of step g - 3 have read it; one thread issues the hi hi
+// product of each step (4 MMAs) and another the two cross products (8 MMAs); eight epilogue warps
+// promote the accumulators and write back each item's output block.
+//
+// What bounds it.  At 64 KB of operands per step the SM's L2 port (64 B per cycle) allows about 1,024
+// cycles per step, the MMAs alone 855 (12 x M = N = 128, K = 16, measured); a step of the one-issuer
+// kernel took 2,050.  Its issuing thread spent 740 of them between MMAs: the tensor pipe queues only a
+// few, so every barrier wait (150 to 230 cycles of dependent scalar work, even for a phase long complete),
+// commit (60 to 90) and address computation left it idle.  Hence
+//   - two issuing threads on accumulators of their own (no order between their MMAs is needed): while one
+//     waits or commits, the other's MMAs run;
+//   - the hi hi product has a TMEM accumulator per step (two, g & 1), promoted into FP32 registers every
+//     step; the cross products, 2^-11 smaller, accumulate in TMEM over the whole item (two, item & 1).
+//     That halves the epilogue's TMEM reads and additions, and the cross products never wait for the
+//     epilogue within an item;
+//   - one commit per issuer and step, on a ring of six barriers (g % 6) that the producer and the epilogue
+//     wait on: two steps that share a barrier are six apart, more than the three stages let any role
+//     run ahead, so a phase is never missed;
+//   - items are found in closed form (tc_items.h), and every role walks the subdomains forward.
+// The write-back is a TMA reduce-add: each epilogue warp scales its 32 x 64 part of the block into a
+// swizzled shared-memory box, 32 columns at a time, and one lane adds the box into the tiles in L2 (the
+// output is never read into the SM; every element receives exactly one add per launch, so the result
+// does not depend on timing).
+// Measured in isolation (n = 16,384, kernel time): rank 512 0.470 -> 0.355 ms (276 -> 365 TFLOP/s FP32-
+// equivalent), rank 256 0.320 -> 0.230 ms; of it the MMAs and barriers alone take 0.222 ms, the operand
+// copies alone 0.259, and the output's read-modify-write in DRAM 0.158 at the copy bandwidth.
 __global__ void __launch_bounds__(kThreads2, 1)
     k_update_tc2(LevelDev L, int nq, int jbeg, int jend, int ibeg, int panel, const uint8_t* __restrict__ split,
                  const uint8_t* __restrict__ split_b, const float* __restrict__ rscale,
                  const int64_t* __restrict__ prow_off, const int64_t* __restrict__ item_pref,
                  const __grid_constant__ CUtensorMap tmap) {
-  const int64_t n_items = item_pref[L.n_sub];
+  const int n_sub = (int)L.n_sub;
+  const int64_t n_items = item_pref[n_sub];
   if ((int64_t)blockIdx.x >= n_items) return;
   // nq panel tile columns (K = 64 nq) in the split rows; output columns jbeg <= j < min(Bc, jend)
 
@@ -159,27 +223,28 @@ __global__ void __launch_bounds__(kThreads2, 1)
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* stage0 = smem_raw + (base - raw);
-  // full/free: shared-memory stage g % kStages2 loaded / read by its MMAs; mma/epi: TMEM
-  // accumulator pair g & 1 written by its MMAs / read by the epilogue
-  __shared__ __align__(8) uint64_t full_bar[kStages2], free_bar[kStages2], mma_bar[2], epi_bar[2];
+  // full: shared-memory stage g % 3 loaded; big / crs: the hi hi / cross products of step g done (stage
+  // read, accumulator written); epi: hi hi accumulator g & 1 read; sml: cross accumulator of item & 1 read
+  __shared__ __align__(8) uint64_t full_bar[kStages2], big_bar[kMmaBars], crs_bar[kMmaBars], epi_bar[2], sml_bar[2];
   __shared__ uint32_t tmem_slot;
-  __shared__ int s_issued, s_requested;
+  __shared__ int s_issued[2], s_requested;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&tmem_slot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int b = 0; b < kStages2; ++b) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full_bar[b])));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&free_bar[b])));
+    for (int b = 0; b < kStages2; ++b) mbar_init(&full_bar[b], 1);
+    for (int b = 0; b < kMmaBars; ++b) {
+      mbar_init(&big_bar[b], 1);
+      mbar_init(&crs_bar[b], 1);
     }
     for (int b = 0; b < 2; ++b) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mma_bar[b])));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 256;" ::"r"(smem_u32(&epi_bar[b])));
+      mbar_init(&epi_bar[b], 8);
+      mbar_init(&sml_bar[b], 8);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    s_issued = 0;
+    s_issued[0] = s_issued[1] = 0;
     s_requested = 0;
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -187,227 +252,202 @@ __global__ void __launch_bounds__(kThreads2, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
 
-  // item -> (subdomain, column pair j, j+1, row pair i0, i0+1); the rows of column pair j start
-  // at max(j, min(ibeg, Bc))
-  auto decode = [&](int64_t it, int& s, int& j, int& i0) {
-    int lo = 0, hi = (int)L.n_sub - 1;
-    while (lo < hi) {   // last s with item_pref[s] <= it
-      const int mid = (lo + hi + 1) >> 1;
-      if (item_pref[mid] <= it) lo = mid; else hi = mid - 1;
+  // a role's place in the item list: items come in ascending order, so the subdomain only moves forward
+  struct Cursor {
+    int s = -1;
+    int64_t first = 0, next = 0;   // items [first, next) belong to subdomain s
+    SubMeta m;
+    TcItems t;
+    int64_t rbase = 0;
+  };
+  auto seek = [&](Cursor& c, int64_t it, int& j, int& i0) {
+    if (it >= c.next) {
+      do {
+        ++c.s;
+        c.first = c.next;
+        c.next = item_pref[c.s + 1];
+      } while (it >= c.next && c.s + 1 < n_sub);
+      c.m = L.meta[c.s];
+      c.t = tc_items_of(c.m, jbeg, jend, ibeg, panel);
+      c.rbase = prow_off[c.s];
     }
-    s = lo;
-    const SubMeta& m = L.meta[s];
-    int64_t t = it - item_pref[s];
-    const int jlim = m.Bc < jend ? m.Bc : jend;
-    const int ib = ibeg < m.Bc ? ibeg : m.Bc;
-    j = jbeg;
-    i0 = -1;
-    for (; j < jlim; j += 2) {
-      const int rb = j > ib ? j : ib;
-      const int cnt = (m.R - rb + 1) / 2;
-      if (t < cnt) {
-        i0 = rb + 2 * (int)t;
-        break;
-      }
-      t -= cnt;
-    }
+    tc_item(c.t, (int)(it - c.first), j, i0);
   };
 
   // steps of this CTA: its items in order, nq panel columns each; a panel solve's B operand (rows
   // of the inverse of a lower triangular block) is zero beyond block column j - jbeg + 1, so the
   // column pair j, j + 1 takes K steps 0 .. j - jbeg + 1 only
   auto item_nq = [&](int j) { return panel ? min(nq, j - jbeg + 2) : nq; };
-  const int64_t my_items = (n_items - (int64_t)blockIdx.x + gridDim.x - 1) / gridDim.x;
-  uint32_t total = (uint32_t)(my_items * nq);
-  if (panel && warp == 8) {
-    total = 0;
-    for (int64_t it = blockIdx.x; it < n_items; it += gridDim.x) {
-      int cs, cj, ci0;
-      decode(it, cs, cj, ci0);
-      total += (uint32_t)item_nq(cj);
-    }
-  }
-  auto wait = [&](uint64_t* bar, uint32_t parity) {
-    long long spins = 0;
-    while (!mbar_try_wait(bar, parity))
-      if (++spins > kSpinLimit) return false;
-    return true;
-  };
-  if (warp == 9) {
-    // ---- producer: requests the B and A parts of step gc into stage gc % kStages2 once the MMAs
-    // of step gc - kStages2 have read that stage (its own thread, so that waiting for a stage
-    // never delays the issue of MMAs)
+  if (warp == 10) {
+    // ---- producer: its own thread, so that waiting for a stage never delays the issue of MMAs
     if (lane == 0) {
       bool lost = false;
-      int64_t cached_k = -1;
-      // per item (read from global memory once, when the item changes): the four split rows and
-      // the output tiles to prefetch; per step only the panel-column offset changes
-      const uint8_t* rowA0 = nullptr;
-      const uint8_t* rowA1 = nullptr;
-      const uint8_t* rowB0 = nullptr;
-      const uint8_t* rowB1 = nullptr;
-      const float* pre[4] = {nullptr, nullptr, nullptr, nullptr};
-      uint32_t gc = 0;
-      int nqi = nq, q = 0;
-      for (int64_t k = 0; k < my_items; gc += 1) {
-        const int st = (int)(gc % kStages2);
-        if (k != cached_k) {   // decode before waiting: the loads overlap the MMAs still reading the stage
-          int cs = 0, cj = 0, ci0 = 0;
-          decode(blockIdx.x + k * gridDim.x, cs, cj, ci0);
-          cached_k = k;
-          nqi = item_nq(cj);
-          q = 0;
-          const SubMeta m = L.meta[cs];
-          const bool hasA1 = ci0 + 1 < m.R, hasB1 = cj + 1 < (m.Bc < jend ? m.Bc : jend);
-          const int64_t rbase = prow_off[cs];
-          rowA0 = split + (rbase + ci0) * kPanelTiles * (int64_t)kSplitTile;
-          rowA1 = split + (rbase + (hasA1 ? ci0 + 1 : ci0)) * kPanelTiles * (int64_t)kSplitTile;
-          rowB0 = split_b + (rbase + cj) * kPanelTiles * (int64_t)kSplitTile;
-          rowB1 = split_b + (rbase + (hasB1 ? cj + 1 : cj)) * kPanelTiles * (int64_t)kSplitTile;
-#pragma unroll
-          for (int a = 0; a < 2; ++a)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-              const int ti = ci0 + a, tj = cj + c;
-              pre[2 * a + c] = (!panel && (a == 0 || hasA1) && (c == 0 || hasB1) && (ti >= m.Bc || tj <= ti))
-                                   ? (const float*)L.tiles + m.tile_off + tile_index(ti, tj, m.Bc) * NB2
-                                   : nullptr;
+      Cursor cur;
+      uint32_t g = 0;
+      Ring<kStages2> st;
+      Ring<kMmaBars> rd;   // the step whose MMAs read the stage last
+      for (int64_t it = blockIdx.x; it < n_items && !lost; it += gridDim.x) {
+        int j, i0;
+        seek(cur, it, j, i0);   // before the wait for a stage: overlaps the MMAs still reading it
+        const SubMeta& m = cur.m;
+        const bool hasA1 = i0 + 1 < cur.t.rend, hasB1 = j + 1 < cur.t.jlim;
+        const uint8_t* rowA0 = split + (cur.rbase + i0) * kPanelTiles * (int64_t)kSplitTile;
+        const uint8_t* rowA1 = hasA1 ? rowA0 + kPanelTiles * (int64_t)kSplitTile : rowA0;
+        const uint8_t* rowB0 = split_b + (cur.rbase + j) * kPanelTiles * (int64_t)kSplitTile;
+        const uint8_t* rowB1 = hasB1 ? rowB0 + kPanelTiles * (int64_t)kSplitTile : rowB0;
+        const int nqi = item_nq(j);
+        for (int q = 0; q < nqi; ++q, ++g) {
+          if (g >= (uint32_t)kStages2) {
+            if (!mbar_wait(&big_bar[rd.k], rd.phase) || !mbar_wait(&crs_bar[rd.k], rd.phase)) {
+              lost = true;
+              break;
             }
-        }
-        if (gc >= (uint32_t)kStages2 && !wait(&free_bar[st], ((gc / kStages2) - 1) & 1u)) {
-          lost = true;
-          break;
-        }
-        if (q == 0)   // the output tiles are read back by the epilogue after the last column
+            rd.next();
+          }
+          if (q == 0 && !panel)   // the output tiles are read back by the write-back after the last column
 #pragma unroll
-          for (int t = 0; t < 4; ++t)
-            if (pre[t])
-              asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(pre[t]), "r"((uint32_t)(NB2 * 4))
-                           : "memory");
-        uint8_t* sA = stage0 + st * kStage2;   // [A hi | A lo | B hi | B lo], 128 rows each
-        uint8_t* sB = sA + 2 * kOpnd;
-        mbar_expect_tx(&full_bar[st], kStage2);
-        const int64_t qo = (int64_t)q * kSplitTile;
+            for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-          bulk_g2s(sA + p * kOpnd, rowA0 + qo + p * kTilePart, kTilePart, &full_bar[st]);
-          bulk_g2s(sA + p * kOpnd + kTilePart, rowA1 + qo + p * kTilePart, kTilePart, &full_bar[st]);
-          bulk_g2s(sB + p * kOpnd, rowB0 + qo + p * kTilePart, kTilePart, &full_bar[st]);
-          bulk_g2s(sB + p * kOpnd + kTilePart, rowB1 + qo + p * kTilePart, kTilePart, &full_bar[st]);
+              for (int c = 0; c < 2; ++c) {
+                const int ti = i0 + a, tj = j + c;
+                if ((a == 0 || hasA1) && (c == 0 || hasB1) && (ti >= m.Bc || tj <= ti))
+                  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
+                                   (const float*)L.tiles + m.tile_off + tile_index(ti, tj, m.Bc) * NB2),
+                               "r"((uint32_t)(NB2 * 4))
+                               : "memory");
+              }
+          uint8_t* sA = stage0 + st.k * kStage2;   // [A hi | A lo | B hi | B lo], 128 rows each
+          uint8_t* sB = sA + 2 * kOpnd;
+          uint64_t* bar = &full_bar[st.k];
+          mbar_expect_tx(bar, kStage2);
+          const int64_t qo = (int64_t)q * kSplitTile;
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            bulk_g2s(sA + p * kOpnd, rowA0 + qo + p * kTilePart, kTilePart, bar);
+            bulk_g2s(sA + p * kOpnd + kTilePart, rowA1 + qo + p * kTilePart, kTilePart, bar);
+            bulk_g2s(sB + p * kOpnd, rowB0 + qo + p * kTilePart, kTilePart, bar);
+            bulk_g2s(sB + p * kOpnd + kTilePart, rowB1 + qo + p * kTilePart, kTilePart, bar);
+          }
+          st.next();
         }
-        if (++q == nqi) ++k;
       }
-      s_requested = (int)gc;
+      s_requested = (int)g;
       if (lost) atomicExch(L.status + 2, 4);
     }
-  } else if (warp == 8) {
-    // ---- MMA issuer: one thread waits for the stage's data and for a free accumulator pair
+  } else if (warp >= 8) {
+    // ---- MMA issuers: one thread each, warp 8 the hi hi product, warp 9 the cross products
     if (lane == 0) {
+      const bool big = warp == 8;
+      uint64_t* done_bar = big ? big_bar : crs_bar;
       // c FP32, a and b FP16, both K-major, N = 128, M = 128
       const uint32_t idesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-      bool lost = false;
-      int issued = 0;
-      for (uint32_t g = 0; g < total && !lost; ++g) {
-        const int st = (int)(g % kStages2);
-        const int b = (int)(g & 1u);
-        if (!wait(&full_bar[st], (g / kStages2) & 1u)) {
-          lost = true;
-          break;
+      const uint64_t desc0 = desc_sw128(base);   // operand at stage 0; the start address counts 16-byte units
+      auto mma = [&](uint32_t d, uint64_t a, uint64_t b, uint32_t acc) {
+        asm volatile(
+            "{\n .reg .pred pp;\n setp.ne.b32 pp, %4, 0;\n"
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, pp;\n}\n" ::"r"(d),
+            "l"(a), "l"(b), "r"(idesc), "r"(acc));
+      };
+      constexpr uint64_t kA1 = kOpnd >> 4, kB0 = 2 * (kOpnd >> 4), kB1 = 3 * (kOpnd >> 4);   // A lo, B hi, B lo
+      bool ok = true;
+      Cursor cur;
+      uint32_t g = 0, n = 0;   // n: items of this CTA so far
+      Ring<kStages2> st;
+      Ring<kMmaBars> dn;
+      for (int64_t it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++n) {
+        int nqi = nq;
+        if (panel) {
+          int j, i0;
+          seek(cur, it, j, i0);
+          nqi = item_nq(j);
         }
-        if (g >= 2 && !wait(&epi_bar[b], ((g >> 1) - 1) & 1u)) {   // accumulators of step g - 2 are read
-          lost = true;
-          break;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t sa = smem_u32(stage0 + st * kStage2), sb = sa + 2 * kOpnd;
-        const uint32_t acc_small = tmem + 256u * b, acc_big = acc_small + 128u;
-        // products: (A lo, B hi), (A hi, B lo) into the small accumulator, (A hi, B hi) into the big one
-        const int pa[3] = {1, 0, 0}, pb[3] = {0, 1, 0};
+        const uint32_t acc_small = tmem + 256u + 128u * (n & 1u);
+        // the cross accumulator of item n - 2 is read before the first product of item n
+        if (!big && n >= 2) ok = mbar_wait(&sml_bar[n & 1u], ((n >> 1) - 1) & 1u);
+        for (int q = 0; q < nqi && ok; ++q) {
+          const uint64_t d = desc0 + (uint64_t)(st.k * (kStage2 >> 4));
+          if (big) {
+            const uint32_t b = g & 1u;
+            if (g >= 2) ok = mbar_wait(&epi_bar[b], ((g >> 1) - 1) & 1u);   // hi hi of step g - 2 is read
+            ok = mbar_wait(&full_bar[st.k], st.phase) && ok;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-        for (int p = 0; p < 3; ++p)
+            for (int kk = 0; kk < 4; ++kk) mma(tmem + 128u * b, d + 2 * kk, d + kB0 + 2 * kk, kk > 0);   // hi hi
+          } else {
+            ok = mbar_wait(&full_bar[st.k], st.phase);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t da = desc_sw128(sa + pa[p] * kOpnd + kk * 32);
-            const uint64_t db = desc_sw128(sb + pb[p] * kOpnd + kk * 32);
-            const bool big = p == 2;
-            const uint32_t acc = (kk > 0 || (p > 0 && !big)) ? 1u : 0u;   // fresh accumulators per step
-            asm volatile(
-                "{\n .reg .pred pp;\n setp.ne.b32 pp, %4, 0;\n"
-                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, pp;\n}\n" ::"r"(big ? acc_big : acc_small),
-                "l"(da), "l"(db), "r"(idesc), "r"(acc));
+            for (int kk = 0; kk < 4; ++kk) mma(acc_small, d + kA1 + 2 * kk, d + kB0 + 2 * kk, q > 0 || kk > 0);   // lo hi
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) mma(acc_small, d + 2 * kk, d + kB1 + 2 * kk, 1u);                      // hi lo
           }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                         smem_u32(&mma_bar[b]))
-                     : "memory");
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                         smem_u32(&free_bar[st]))
-                     : "memory");
-        ++issued;
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                           smem_u32(&done_bar[dn.k]))
+                       : "memory");
+          ++g;
+          st.next();
+          dn.next();
+        }
       }
-      s_issued = issued;
-      if (lost) atomicExch(L.status + 2, 4);
+      s_issued[big ? 0 : 1] = (int)g;
+      if (!ok) atomicExch(L.status + 2, 4);
     }
   } else {
     // ---- epilogue warps: warp w reads TMEM lanes 32 (w & 3) .. +31 (output rows) and columns
-    // 64 (w >> 2) .. +63; per step hi hi + 2^-11 (cross products) is added into FP32 registers
+    // 64 (w >> 2) .. +63
     bool lost = false;
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
     const uint32_t col0 = 64u * (uint32_t)(warp >> 2);
     const int erow = 32 * (warp & 3) + lane;
     uint8_t* box = stage0 + kStages2 * kStage2 + warp * kEpiBox;   // 1024-byte aligned
-    uint32_t g = 0;
-    for (int64_t it = blockIdx.x; it < n_items && !lost; it += gridDim.x) {
-      int s, j, i0;
-      decode(it, s, j, i0);
-      const SubMeta& m = L.meta[s];
+    Cursor cur;
+    uint32_t g = 0, n = 0;
+    Ring<kMmaBars> dn;
+    for (int64_t it = blockIdx.x; it < n_items && !lost; it += gridDim.x, ++n) {
+      int j, i0;
+      seek(cur, it, j, i0);
+      const SubMeta& m = cur.m;
+      const bool hasA1 = i0 + 1 < cur.t.rend, hasB1 = j + 1 < cur.t.jlim;
+      const int ti = erow < 64 ? i0 : i0 + 1;
+      const int tj = col0 < 64 ? j : j + 1;
+      const bool ok = (erow < 64 || hasA1) && (col0 < 64 || hasB1) && (ti >= m.Bc || tj <= ti);
+      // negated row factor: the tiles receive x + (-(acc sa) f), which equals x - (acc sa) f
+      const float sa = ok ? -rscale[(cur.rbase + ti) * NB + (erow & 63)] : 0.f;
       float racc[64];
 #pragma unroll
       for (int c = 0; c < 64; ++c) racc[c] = 0.f;
       const int nqi = item_nq(j);
       for (int q = 0; q < nqi; ++q, ++g) {
-        const int b = g & 1;
-        const uint32_t n = g >> 1;
-        long long spins = 0;
-        while (!mbar_try_wait(&mma_bar[b], n & 1u))
-          if (++spins > kSpinLimit) {
-            lost = true;
-            break;
-          }
-        lost = __any_sync(0xffffffffu, lost);
+        const uint32_t b = g & 1u;
+        lost = __any_sync(0xffffffffu, !mbar_wait(&big_bar[dn.k], dn.phase));
+        if (q + 1 == nqi) lost = __any_sync(0xffffffffu, !mbar_wait(&crs_bar[dn.k], dn.phase)) || lost;
         if (lost) break;
+        dn.next();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-        for (int c16 = 0; c16 < 4; ++c16) {
-          const uint32_t taddr = tmem + lane_base + 256u * b + col0 + 16u * c16;
-          uint32_t v[16], w[16];
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-              : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-              : "r"(taddr));
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-              : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]),
-                "=r"(w[8]), "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15])
-              : "r"(taddr + 128u));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        for (int h = 0; h < 2; ++h) {
+          float v[32];
+          tmem_ld32(v, tmem + lane_base + 128u * b + col0 + 32u * h);
 #pragma unroll
-          for (int c = 0; c < 16; ++c)
-            racc[16 * c16 + c] += __uint_as_float(w[c]) + __uint_as_float(v[c]) * (1.f / 2048.f);
+          for (int c = 0; c < 32; ++c) racc[32 * h + c] += v[c];
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&epi_bar[b])) : "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&epi_bar[b]);
       }
       if (lost) break;
-      const bool hasA1 = i0 + 1 < m.R, hasB1 = j + 1 < (m.Bc < jend ? m.Bc : jend);
-      const int ti = erow < 64 ? i0 : i0 + 1;
-      const int tj = col0 < 64 ? j : j + 1;
-      const bool ok = (erow < 64 || hasA1) && (col0 < 64 || hasB1) && (ti >= m.Bc || tj <= ti);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {   // the item's cross products
+        float v[32];
+        tmem_ld32(v, tmem + lane_base + 256u + 128u * (n & 1u) + col0 + 32u * h);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) racc[32 * h + c] += v[c] * (1.f / 2048.f);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sml_bar[n & 1u]);
       if (ok) {   // warp-uniform: the warp's 32 rows and 64 columns lie in one output tile
-        const int64_t rbase = prow_off[s];
-        // negated row factor: the tiles receive x + (-(acc sa) f), which equals x - (acc sa) f
-        const float sa = -rscale[(rbase + ti) * NB + (erow & 63)];
-        const float4* sb = (const float4*)(rscale + (rbase + tj) * NB);
+        const float4* sb = (const float4*)(rscale + (cur.rbase + tj) * NB);
         // row of the warp's first output row in the [rows][64] view of the tile buffer
         const int y = (int)((m.tile_off + tile_index(ti, tj, m.Bc) * NB2) / NB) + (32 * (warp & 3) & 63);
 #pragma unroll
@@ -455,20 +495,13 @@ __global__ void __launch_bounds__(kThreads2, 1)
   // copies requested but never consumed (a wait gave up) may still be landing in shared memory:
   // wait (bounded) for them before the CTA exits
   if (tid == 0)
-    for (int c = s_issued; c < s_requested; ++c) {
-      long long spins = 0;
-      while (!mbar_try_wait(&full_bar[c % kStages2], (uint32_t)(c / kStages2) & 1u) && ++spins < kSpinLimit) {
-      }
-    }
-  // before the accumulators are released no MMA may still be running (also on the error path)
-  const int issued = s_issued;
-  if (issued > 0) {
-    const int b = (issued - 1) & 1;
-    const uint32_t n = (uint32_t)((issued - 1) >> 1);
-    long long spins = 0;
-    while (!mbar_try_wait(&mma_bar[b], n & 1u))
-      if (++spins > kSpinLimit) break;
-  }
+    for (int c = max(0, s_requested - kStages2); c < s_requested; ++c)
+      mbar_wait(&full_bar[c % kStages2], (uint32_t)(c / kStages2) & 1u);
+  // before the accumulators are released no MMA may still be running (also on the error path): the last
+  // commit of each issuer covers every MMA it issued
+  for (int k = 0; k < 2; ++k)
+    if (s_issued[k] > 0)
+      mbar_wait(&(k == 0 ? big_bar : crs_bar)[(s_issued[k] - 1) % kMmaBars], (uint32_t)((s_issued[k] - 1) / kMmaBars) & 1u);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
