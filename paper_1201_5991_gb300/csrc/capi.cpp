@@ -173,6 +173,8 @@ struct Level {
   int64_t n_vec = 0, tile_elems = 0, dinv_elems = 0, psi_elems = 0, g_elems = 0, sum_nc = 0;
   int max_R = 0, max_Bc = 0, max_nc = 0, max_nG = 0, max_nGb = 0, max_ncb = 0;
   int64_t psiT_elems = 0;
+  bool inverse = false;   // FP32, tensor cores: explicit A_GG^{-1} of the augmented interface matrices
+  std::vector<int> split_rows;   // [kTcLaunches p + u] grid rows of the split before launch u of super-panel p
   // explicit augmented Schur complement of the interface (mixed inner operator, level 1 only)
   bool explicit_schur = false;
   int64_t schur_elems = 0;
@@ -270,7 +272,7 @@ void alloc_level_work(Level& L, DevArena& A, int blk) {
     L.locB = A.alloc<double>(nv);
   }
   L.pub = A.alloc<double>(L.n_vec * std::min(blk, 8));
-  if (L.explicit_schur) L.symv_part = A.alloc<float>(std::max<int64_t>(L.symv_stride, 1) * blk);
+  if (L.explicit_schur || L.inverse) L.symv_part = A.alloc<float>(std::max<int64_t>(L.symv_stride, 1) * blk);
   L.dl0 = A.alloc<double>(nv);
   L.dl1 = A.alloc<double>(nv);
   L.dl2 = A.alloc<double>(nv);
@@ -370,6 +372,7 @@ struct bddc_handle_s {
     cudaEvent_t a, b;
     int cls;
     double bytes, flops;
+    int launches;
   };
   std::vector<ProfRec> prof_pending;
   std::vector<ProfRec> graph_prof;     // event pairs recorded by every replay of iter_graph
@@ -433,9 +436,10 @@ struct ProfScope {
   int cls;
   double bytes, flops;
   cudaStream_t st;
+  int launches;
   cudaEvent_t a = nullptr;
-  ProfScope(bddc_handle_s* h_, int cls_, double bytes_, double flops_, cudaStream_t st_)
-      : h(h_), cls(cls_), bytes(bytes_), flops(flops_), st(st_) {
+  ProfScope(bddc_handle_s* h_, int cls_, double bytes_, double flops_, cudaStream_t st_, int launches_ = 1)
+      : h(h_), cls(cls_), bytes(bytes_), flops(flops_), st(st_), launches(launches_) {
     if (h->opts.profile) {
       a = take_event(h);
       record_event(a, st);
@@ -454,7 +458,7 @@ struct ProfScope {
     } catch (...) {
       return;
     }
-    h->prof_pending.push_back({a, b, cls, bytes, flops});
+    h->prof_pending.push_back({a, b, cls, bytes, flops, launches});
   }
 };
 
@@ -464,7 +468,7 @@ void accumulate_graph_profile(bddc_handle_s* h) {
     float ms = 0.f;
     ck(cudaEventElapsedTime(&ms, r.a, r.b), "cudaEventElapsedTime");
     h->stats.prof_ms[r.cls] += ms;
-    h->stats.prof_launches[r.cls] += 1;
+    h->stats.prof_launches[r.cls] += r.launches;
     h->stats.prof_bytes[r.cls] += r.bytes;
     h->stats.prof_flops[r.cls] += r.flops;
   }
@@ -477,7 +481,7 @@ void flush_profile(bddc_handle_s* h) {
     float ms = 0.f;
     ck(cudaEventElapsedTime(&ms, r.a, r.b), "cudaEventElapsedTime");
     h->stats.prof_ms[r.cls] += ms;
-    h->stats.prof_launches[r.cls] += 1;
+    h->stats.prof_launches[r.cls] += r.launches;
     h->stats.prof_bytes[r.cls] += r.bytes;
     h->stats.prof_flops[r.cls] += r.flops;
     h->event_pool.push_back(r.a);
@@ -569,6 +573,8 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     }
     L.explicit_schur = h->opts.inner_operator == 2 || padded <= 1.08 * base;
   }
+  // the interface inverse comes with the tensor-core factorisation (its panel solves carry the inverse rows)
+  L.inverse = L.fp32 && !L.coarsest && h->opts.tensor_cores && h->opts.tensor_cores != 2;
   for (int64_t s = 0; s < ns; ++s) {
     SubMeta& m = L.meta[s];
     m.n = (int32_t)(mp.sub_dof_ptr[s + 1] - mp.sub_dof_ptr[s]);
@@ -581,9 +587,11 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     m.ncb = (int32_t)ceil_div(m.nc, NB);
     m.Bc = m.nIb + m.nGb;
     m.R = m.Bc + m.ncb;
-    m.pad0 = 0;
+    m.nV = L.inverse ? m.nGb : 0;
     m.tile_off = tile;
     tile += ((int64_t)m.Bc * (m.Bc + 1) / 2 + (int64_t)m.ncb * m.Bc) * NB2;
+    m.inv_off = tile + (int64_t)m.nV * (m.nV + 1) / 2 * NB2;
+    tile += (int64_t)m.nV * (m.nV + 1) * NB2;
     m.dinv_off = dinv;
     dinv += (int64_t)m.Bc * NB2;
     m.vec_off = vec;
@@ -613,7 +621,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
   L.psi_elems = psi;
   L.psiT_elems = psiT;
   L.schur_elems = schur;
-  L.symv_stride = L.explicit_schur ? symv : 0;
+  L.symv_stride = L.explicit_schur || L.inverse ? symv : 0;
   L.g_elems = goff;
   L.sum_nc = coff;
   L.max_tiles.assign(L.max_Bc, 0);
@@ -625,6 +633,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
   const int n_super = (L.max_Bc + kPanel - 1) / kPanel + 1;
   L.tc_items.assign(kTcLaunches * (size_t)n_super, 0);
   L.tc_flops.assign(kTcLaunches * (size_t)n_super, 0.0);
+  L.split_rows.assign(kTcLaunches * (size_t)n_super, 0);
   L.snap_start.assign(n_super, 0);
   L.snap_mid.assign(n_super, 0);
   const double nb3 = (double)NB * NB * NB;
@@ -656,14 +665,22 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
       for (int j = kb0 + kSub; j < std::min(kb0 + kPanel, (int)m.Bc); ++j) tiles[0] += m.R - j;
       for (int j = kb0 + kPanel; j < m.Bc; ++j) tiles[1] += m.R - j;
       const int p = kb0 / kPanel;
+      const int e0 = inverse_rows(m, kb0 + kSub), e1 = inverse_rows(m, kb0 + kPanel);   // inverse rows and columns
+      tiles[0] += (int64_t)e0 * std::max(0, std::min(kb0 + kPanel, (int)m.Bc) - (kb0 + kSub));
+      tiles[1] += (int64_t)e1 * std::max(0, (int)m.Bc - (kb0 + kPanel)) + (int64_t)e1 * (e1 + 1) / 2;
       L.tc_flops[kTcLaunches * p] += 2.0 * nb3 * kSub * (double)tiles[0];
       L.tc_flops[kTcLaunches * p + 1] += 2.0 * nb3 * kPanel * (double)tiles[1];
       L.tc_flops[kTcLaunches * p + 2] += 2.0 * nb3 * kSub * (double)(tiles[0] + tiles[1]);
+      for (int u = 0; u < kTcLaunches; ++u) {
+        const int half = u == 1 || u == 4 ? 1 : 0, panel = u >= 3;
+        const int rows = split_rows_of(m, kb0 + (half + 1) * kSub, panel ? kb0 + half * kSub : kb0, panel);
+        L.split_rows[kTcLaunches * p + u] = std::max(L.split_rows[kTcLaunches * p + u], rows);
+      }
       for (int half = 0; half < 2; ++half) {   // panel solves: rows below the block by its columns
         const int k0 = kb0 + half * kSub;
         const int nd = std::min(kSub, (int)m.Bc - k0);
         if (nd <= 0) continue;
-        const double rows = (double)NB * (m.R - std::min(k0 + kSub, (int)m.Bc));
+        const double rows = (double)NB * (m.R - std::min(k0 + kSub, (int)m.Bc) + inverse_rows(m, k0 + kSub));
         L.tc_flops[kTcLaunches * p + 3 + half] += rows * (double)(NB * nd) * (NB * nd);
       }
     }
@@ -876,6 +893,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
   d.rho = A.alloc<double>(ns);
   d.Ginv = A.alloc<double>(L.g_elems);
   d.KC = A.alloc<double>(L.g_elems);
+  d.G = L.inverse ? A.alloc<double>(L.g_elems) : nullptr;
   const size_t ts = L.fp32 ? sizeof(float) : sizeof(double);
   if (L.fp32 && h->opts.tensor_cores) {
     // pre-split panel buffer: kPanel tiles of 16 KB (FP16 hi and lo parts) for every block row
@@ -883,7 +901,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     int64_t rows = 0;
     for (int64_t s = 0; s < ns; ++s) {
       po[s] = rows;
-      rows += L.meta[s].R;
+      rows += L.meta[s].R + L.meta[s].nV;
     }
     L.prow_off = A.upload(po, st);
     L.split = A.alloc<uint8_t>(rows * kPanel * 2 * NB2 * 2);
@@ -907,7 +925,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
       int64_t acc = 0;
       for (int64_t s = 0; s < ns; ++s) {
         pref[(size_t)u * (ns + 1) + s] = acc;
-        acc += tc_items_count(tc_items_of(L.meta[s], jbeg, jend, ibeg, v >= 3));
+        acc += tc_items_count(tc_items_of(L.meta[s], jbeg, jend, ibeg, v >= 3, v >= 3 ? jbeg : kb0));
       }
       pref[(size_t)u * (ns + 1) + ns] = acc;
       L.tc_items[u] = acc;
@@ -924,7 +942,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     d.psi = A.alloc<float>(L.psi_elems);
     d.psiT = A.alloc<float>(L.psiT_elems);
     d.schur = L.explicit_schur ? A.alloc<float>(L.schur_elems) : nullptr;
-    if (L.explicit_schur) {
+    if (L.explicit_schur || L.inverse) {
       std::vector<int64_t> po(ns);
       int64_t o = 0;
       for (int64_t s2 = 0; s2 < ns; ++s2) {
@@ -1047,6 +1065,7 @@ void factor_level(bddc_handle_s* h, Level& L, cudaStream_t st) {
   ck(cudaMemsetAsync(d.tiles, 0, sizeof(T) * (size_t)std::max<int64_t>(L.tile_elems, 1), st), "memset tiles");
   launch_densify_rows<T>(d, L.row_sub, st);
   launch_add_constraints<T>(d, st);
+  if (L.inverse) launch_unit_rows(d, L.max_nGb, st);
   if (sizeof(T) == 4 && h->opts.tensor_cores) {
     // 512-wide super-panels of two 256-wide sub-panels.  Per sub-panel: its 256 x 256 diagonal
     // block factored on CUDA cores and inverted (X = L_D^{-1}); the rows below it solved on the
@@ -1081,18 +1100,19 @@ void factor_level(bddc_handle_s* h, Level& L, cudaStream_t st) {
               fused = fuse;
             }
             launch_split_inverse(d, k0, L.xinv, L.split, L.rscale, L.prow_off, st);
-            launch_split_panel(d, k0, kSub, k1, L.max_R, L.split, nullptr, L.rscale, L.prow_off, st, 1);
+            launch_split_panel(d, k0, kSub, k1, k0, L.split_rows[kTcLaunches * p + 3 + half], L.split, nullptr,
+                               L.rscale, L.prow_off, st, 1);
           }
           const int up = kTcLaunches * p + 3 + half;
           if (L.tc_items[up] > 0) {
             ProfScope ps(h, BDDC_PROF_TC_PANEL, 0.0, L.tc_flops[up], st);
-            launch_update_tc2(d, kSub, k0, k1, k1, 1, (int)std::min<int64_t>(L.tc_items[up], h->grid_max / 2),
+            launch_update_tc2(d, kSub, k0, k1, k1, 1, k0, (int)std::min<int64_t>(L.tc_items[up], h->grid_max / 2),
                               L.split, L.split, L.rscale, L.prow_off, L.item_pref + (size_t)up * (d.n_sub + 1),
                               L.tile_tmap, st);
           }
           if (L.split && L.tc_items[u] > 0) {
             ProfScope ps(h, BDDC_PROF_FACTOR, 0.0, 0.0, st);
-            launch_split_panel(d, kq, nq, k1, L.max_R, L.split, L.split_signed, L.rscale, L.prow_off, st);
+            launch_split_panel(d, kq, nq, k1, kb0, L.split_rows[u], L.split, L.split_signed, L.rscale, L.prow_off, st);
           }
         } else {
           double fl = 0.0;
@@ -1105,13 +1125,13 @@ void factor_level(bddc_handle_s* h, Level& L, cudaStream_t st) {
             fused = fuse;
           }
           if (L.split && L.tc_items[u] > 0)
-            launch_split_panel(d, kq, nq, k1, L.max_R, L.split, L.split_signed, L.rscale, L.prow_off, st);
+            launch_split_panel(d, kq, nq, k1, kb0, L.split_rows[u], L.split, L.split_signed, L.rscale, L.prow_off, st);
         }
         const int64_t items = L.tc_items[u];
         if (L.split && items > 0) {   // no launch where no subdomain has columns left
           const double fl = (split_mid && half) ? 0.5 * L.tc_flops[u] : L.tc_flops[u];
           ProfScope ps(h, BDDC_PROF_TC_UPDATE, 0.0, fl, st);
-          launch_update_tc2(d, nq, k1, jend, 0, 0, (int)std::min<int64_t>(items, h->grid_max / 2), L.split,
+          launch_update_tc2(d, nq, k1, jend, 0, 0, kb0, (int)std::min<int64_t>(items, h->grid_max / 2), L.split,
                             L.split_signed ? L.split_signed : L.split, L.rscale, L.prow_off,
                             L.item_pref + (size_t)u * (d.n_sub + 1), L.tile_tmap, st);
         }
@@ -1228,7 +1248,7 @@ void schur_apply(bddc_handle_s* h, const double* x, double* y, cudaStream_t st, 
     const float* yf = (const float*)L.locA;
     if (L.explicit_schur) {   // one pass over the lower triangle of S_i + C_i^T R C_i
       ProfScope ps(h, BDDC_PROF_TRMV, column_groups(nb, 4) * 0.5 * L.trmv_bytes, 0.0, st);
-      launch_schur_symv(L.d, L.max_nGb, L.symv_part_off, L.symv_stride, (const float*)L.locA, L.symv_part,
+      launch_schur_symv(L.d, 0, L.max_nGb, L.symv_part_off, L.symv_stride, (const float*)L.locA, L.symv_part,
                         (float*)L.locB, st, nb);
       yf = (const float*)L.locB;
     } else {
@@ -1310,11 +1330,33 @@ void interface_step_t(bddc_handle_s* h, int l, const double* rhat, double* zhat,
   launch_gather_iface<T>(L.d, rhat, 1, v, st, nb);          // r_i = E_i^T r_hat
   launch_psi_t_apply<T>(L.d, v, L.psi_part, L.sum_nc, L.rc_sub, L.max_nGb, L.max_ncb, st, nb);   // Psi_i^T r_i
   launch_coarse_gather(L.d, L.rc_sub, L.sum_nc, L.rC, st, nb);   // r_C = sum R_Ci^T Psi_i^T r_i
+  const bool last = l + 2 == (int)h->lv.size();
+  if (L.inverse) {
+    // Eq. sub_cor with the explicit inverse of the augmented interface matrix: z_i = A_GG^{-1} r_i -
+    // Psi_i G_i Psi_i^T r_i, one symmetric product over the stored lower triangle instead of a sweep pair
+    // through L_GG (chains of dependent block rows) around the products with Y_i; Psi_i^T r_i is the coarse
+    // residual's, and both multiples of Psi_i are added in one product.  48^3 workload: a sweep pair of
+    // 220 us and 33 us of products per application become 97 us at 0.8 of HBM; on 8 subdomains, whose
+    // chains the sweeps could not hide, 150 us become 19.  The inverse rows add 21 % to the tiles and
+    // about 3 ms to the set-up.
+    float* z = (float*)L.locB;
+    {
+      ProfScope ps(h, BDDC_PROF_TRSV_IFACE, column_groups(nb, 4) * L.trsv_bytes[1], 0.0, st, 2);   // rows, columns
+      launch_schur_symv(L.d, 1, L.max_nGb, L.symv_part_off, L.symv_stride, (const float*)v, L.symv_part, z, st, nb);
+    }
+    if (last)
+      coarsest_solve(h, L.rC, L.zC, st, nb);
+    else
+      full_step(h, l + 1, L.rC, L.zC, st, nb);
+    launch_coarse_coef(L.d, L.crow_sub, L.sum_nc, L.zC, L.rc_sub, L.zc_sub, st, nb);
+    launch_psi_apply_add<float>(L.d, L.zc_sub, L.sum_nc, z, L.max_nGb, L.max_ncb, st, nb);
+    launch_scatter_iface<float>(L.d, z, 1, zhat, st, nb);      // z_hat = sum E_i (...)
+    return;
+  }
   trsv_one<T>(h, L, v, 1, 0, st, nb);                       // Eq. sub_cor via the trailing factor
   launch_constraint_corr<T>(L.d, v, L.crow_sub, L.sum_nc, L.cc_t, L.cc_mu, L.psi_part, L.max_nGb, L.max_ncb, st,
                             nb);
   trsv_one<T>(h, L, v, 1, 1, st, nb);
-  const bool last = l + 2 == (int)h->lv.size();
   if (last)
     coarsest_solve(h, L.rC, L.zC, st, nb);
   else
@@ -1457,7 +1499,7 @@ void tune_sweeps(bddc_handle_s* h, Level& L, cudaStream_t st) {
   ck(cudaEventCreate(&a), "cudaEventCreate");
   ck(cudaEventCreate(&b), "cudaEventCreate");
   for (int p = 0; p < 2; ++p) {
-    if (L.ntasks[p][0] == 0) continue;
+    if (L.ntasks[p][0] == 0 || (p == 1 && L.inverse)) continue;   // no interface sweeps with the inverse
     float best = 1e30f;
     int bc = 2, bd = 1, bo = 0;
     for (int order = 0; order < 2; ++order)
@@ -2842,7 +2884,7 @@ int bddc_tc_update_check(int64_t n, int rank, float* a, double* ms) {
       const int64_t* prow_off = A.upload(std::vector<int64_t>{0}, st);
       uint8_t* split = A.alloc<uint8_t>((int64_t)nb * kPanel * 2 * NB2 * 2);
       float* rscale = A.alloc<float>((int64_t)nb * NB);
-      const int64_t items = tc_items_count(tc_items_of(m, nt, nb, 0, 0));
+      const int64_t items = tc_items_count(tc_items_of(m, nt, nb, 0, 0, 0));
       const int64_t* item_pref = A.upload(std::vector<int64_t>{0, items}, st);
       TensorMap128 tmap{};
       const int r = make_tile_tmap(&tmap, (float*)d.tiles, tile_elems);
@@ -2853,9 +2895,9 @@ int bddc_tc_update_check(int64_t n, int rank, float* a, double* ms) {
       cudaEvent_t e0, e1;
       ck(cudaEventCreate(&e0), "cudaEventCreate");
       ck(cudaEventCreate(&e1), "cudaEventCreate");
-      launch_split_panel(d, 0, nt, nt, nb, split, nullptr, rscale, prow_off, st);
+      launch_split_panel(d, 0, nt, nt, 0, nb - nt, split, nullptr, rscale, prow_off, st);
       ck(cudaEventRecord(e0, st), "cudaEventRecord");
-      launch_update_tc2(d, nt, nt, nb, 0, 0, (int)std::min<int64_t>(items, std::max(1, sms)), split, split, rscale,
+      launch_update_tc2(d, nt, nt, nb, 0, 0, 0, (int)std::min<int64_t>(items, std::max(1, sms)), split, split, rscale,
                         prow_off, item_pref, tmap, st);
       ck(cudaEventRecord(e1, st), "cudaEventRecord");
       ck(cudaGetLastError(), "tensor-core update launch");

@@ -421,6 +421,11 @@ __global__ void k_gram(LevelDev L) {
     double* G = L.Ginv + m.g_off;
     G[a * nc + b] = acc;
     G[b * nc + a] = acc;
+    if (L.G) {   // kept: Ginv is inverted in place
+      double* G0 = L.G + m.g_off;
+      G0[a * nc + b] = acc;
+      G0[b * nc + a] = acc;
+    }
   }
 }
 
@@ -657,6 +662,34 @@ __global__ void k_cc_mu(LevelDev L, const int32_t* __restrict__ crow_sub, int64_
   for (int q = lane; q < m.nc; q += 32) acc += Gi[q] * t[m.c_off + q];
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) mu[g] = acc;
+}
+
+// out_p = z_C[R_Ci p] - sum_q G_pq t_q: one warp per constraint row
+__global__ void k_coarse_coef(LevelDev L, const int32_t* __restrict__ crow_sub, int64_t total_rows,
+                              const double* __restrict__ zC, const double* __restrict__ t, double* __restrict__ out) {
+  const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (g >= total_rows) return;
+  zC += (int64_t)blockIdx.y * L.n_coarse;
+  t += (int64_t)blockIdx.y * total_rows;
+  const int s = crow_sub[g];
+  const SubMeta& m = L.meta[s];
+  const int nc = m.nc;
+  const int64_t c_off = m.c_off;
+  const double* G = L.G + m.g_off + (g - c_off) * nc;
+  double acc = 0.0;
+  for (int q = lane; q < nc; q += 32) acc += G[q] * t[c_off + q];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) out[(int64_t)blockIdx.y * total_rows + g] = zC[L.sub_coarse[g]] - acc;
+}
+
+// identity tiles of the inverse rows
+__global__ void k_unit_rows(LevelDev L) {
+  const SubMeta m = L.meta[blockIdx.y];
+  const int r = blockIdx.x;
+  if (r >= m.nV) return;
+  float* t = (float*)L.tiles + m.tile_off + tile_of(m, m.R + r, m.nIb + r) * NB2;
+  if (threadIdx.x < NB) t[threadIdx.x * NB + threadIdx.x] = 1.f;
 }
 
 // ---- products with Y_G and Psi_G^T, both held as ncb x nGb tiles of NB x NB per subdomain ----
@@ -1133,6 +1166,19 @@ void launch_psi_apply_add(const LevelDev& L, const double* zc_sub, int64_t sum_n
   if (sum_nc <= 0 || max_nGb <= 0) return;
   (void)max_ncb;
   cols_matvec<T, 1>(L, vec, zc_sub, sum_nc, max_nGb, (T)1, st, nr);
+}
+
+void launch_coarse_coef(const LevelDev& L, const int32_t* crow_sub, int64_t sum_nc, const double* zC, const double* t,
+                        double* out, cudaStream_t st, int nr) {
+  if (sum_nc <= 0) return;
+  note_launch();
+  k_coarse_coef<<<dim3((unsigned)((sum_nc + 7) / 8), nr), 256, 0, st>>>(L, crow_sub, sum_nc, zC, t, out);
+}
+
+void launch_unit_rows(const LevelDev& L, int max_nGb, cudaStream_t st) {
+  if (max_nGb <= 0 || L.n_sub <= 0) return;
+  note_launch();
+  k_unit_rows<<<dim3((unsigned)max_nGb, (unsigned)L.n_sub), NB, 0, st>>>(L);
 }
 
 template <typename T>

@@ -11,6 +11,12 @@
 //     j = 0 .. min(i, Bc-1).  Block rows Bc .. Bc+ncb-1 hold the constraint rows; after the
 //     partial Cholesky they hold Y = C L^{-T} (nonzero only in interface columns).
 //   * The inverses of the Bc diagonal factor tiles are kept next to the factor.
+//   * FP32 levels factored on the tensor cores also carry nV = nGb inverse rows: block rows R .. R+nV-1
+//     start as the identity on the interface columns (row R + r in column nIb + r) and are taken through
+//     the same panel solves and updates, so they end as V = L_GG^{-T} S (upper triangle, tiles
+//     (R + r, nIb + c), c >= r); as extra columns of the trailing updates they leave, in the tiles
+//     (R + r, R + c), c <= r, the negative inverse -A_GG^{-1} of the augmented interface matrix
+//     L_GG S L_GG^T.  The preconditioner multiplies with it instead of sweeping through L_GG.
 //   * Symmetric indefinite levels (Stokes) use a signed Cholesky A = L S L^T with S = diag(+-1)
 //     and no pivoting (velocities precede pressures in both blocks); SPD levels have S = I.
 //     Then the constraint block rows hold Y S (Y = C L^{-T}), G = C A^{-1} C^T = (Y S) S (Y S)^T,
@@ -30,7 +36,7 @@ struct SubMeta {
   int32_t n, nI, nG, nc;          // local sizes
   int32_t nIb, nGb, ncb, Bc;      // block counts; Bc = nIb + nGb
   int32_t R;                      // block rows = Bc + ncb
-  int32_t pad0;
+  int32_t nV;                     // inverse rows (nGb, or 0)
   int64_t tile_off;               // element offset of the tiles in the level's tile buffer
   int64_t dinv_off;               // element offset of the Bc diagonal inverses
   int64_t vec_off;                // offset of the padded local vector
@@ -39,8 +45,24 @@ struct SubMeta {
   int64_t g_off;                  // offset of nc x nc matrices (G^{-1}, K_C)
   int64_t psi_off;                // offset of Psi_G (nGb*NB rows x nc, row-major)
   int64_t psiT_off;               // offset of Psi_G^T as ncb x nGb tiles (set-up copy for the solve phase)
+  int64_t inv_off;                // offset of the tiles of -A_GG^{-1} (row-major lower triangle) in the tile buffer
   int64_t schur_off;              // offset of the explicit augmented Schur complement (nGb (nGb+1)/2 tiles)
 };
+
+// position of tile (i, j) among a subdomain's tiles (constraint columns exist for no row, the inverse
+// rows hold the columns described above)
+__host__ __device__ inline int64_t tile_of(const SubMeta& m, int i, int j) {
+  if (i < m.Bc) return (int64_t)i * (i + 1) / 2 + j;
+  const int64_t b = (int64_t)m.Bc * (m.Bc + 1) / 2;
+  if (i < m.R) return b + (int64_t)(i - m.Bc) * m.Bc + j;
+  const int64_t v = b + (int64_t)m.ncb * m.Bc, r = i - m.R;
+  if (j < m.Bc) return v + r * m.nV - r * (r - 1) / 2 + (j - m.nIb - r);
+  return v + (int64_t)m.nV * (m.nV + 1) / 2 + r * (r + 1) / 2 + (j - m.R);
+}
+
+__host__ __device__ inline bool tile_exists(const SubMeta& m, int i, int j) {
+  return j <= i && (i < m.R || j >= m.R || j - m.nIb >= i - m.R);
+}
 
 // Raw device pointers of one level, passed by value to kernels.
 struct LevelDev {
@@ -80,6 +102,7 @@ struct LevelDev {
   double* diag;                   // [n_vec] diagonal of K_i
   double* rho;                    // [n_sub]
   double* Ginv;                   // [sum nc*nc]
+  double* G;                      // [sum nc*nc] G_i itself (levels with inverse rows), or null
   double* KC;                     // [sum nc*nc] local coarse matrices K_Ci
   void* tiles;                    // factor tiles (float or double)
   void* dinv;                     // diagonal inverses
@@ -157,8 +180,16 @@ void launch_potrf_step(const LevelDev& L, int k, int max_R, int max_tiles, int j
 // item_pref[n_sub] = number of items; split_b = split_signed on indefinite levels, else split)
 // panel_operand = 1: the rows i >= min(ib, Bc) of every subdomain with kb0 < Bc (the rows below
 // a sub-panel's diagonal block, before their panel solve), columns >= Bc as zeros.
-void launch_split_panel(const LevelDev& L, int kb0, int nt, int ib, int max_R, uint8_t* split, uint8_t* split_signed,
-                        float* rscale, const int64_t* prow_off, cudaStream_t st, int panel_operand = 0);
+// act: the launch's first panel column (subdomains with Bc <= act take no part); rows: grid rows, at least
+// split_rows_of of every subdomain.  Inverse rows reached by the columns below ib are split too.
+inline int split_rows_of(const SubMeta& m, int ib, int act, int panel_operand) {
+  if (act >= m.Bc || (!panel_operand && !m.nV && ib >= m.Bc)) return 0;
+  const int e = ib - m.nIb;
+  return m.R - (ib < m.Bc ? ib : m.Bc) + (e <= 0 ? 0 : (e < m.nV ? e : m.nV));
+}
+void launch_split_panel(const LevelDev& L, int kb0, int nt, int ib, int act, int rows, uint8_t* split,
+                        uint8_t* split_signed, float* rscale, const int64_t* prow_off, cudaStream_t st,
+                        int panel_operand = 0);
 // The B operand of a sub-panel's panel solve L(i, D) = A(i, D) X^T S_D: the rows of -S_D X (block
 // row Q of xinv and L_QQ^{-1}, pivot signs of the block's columns) split like the panel rows into
 // the split rows prow_off[s] + k0 + Q, tile columns 0 .. 3, with their unscaling factors in rscale.
@@ -176,9 +207,12 @@ int make_tile_tmap(TensorMap128* map, float* tiles, int64_t tile_elems);
 // panel = 1 (a panel solve): the output is stored instead of subtracted (the product is -A B^T
 // with B the split rows of -S_D X; the tiles' old contents are the A operand, already split), and
 // the column pair j, j + 1 takes the K steps 0 .. j - jbeg + 1 (X is block lower triangular).
-void launch_update_tc2(const LevelDev& L, int nq, int jbeg, int jend, int ibeg, int panel, int grid, const uint8_t* split,
+// act: first panel column of the launch (tc_items.h).
+void launch_update_tc2(const LevelDev& L, int nq, int jbeg, int jend, int ibeg, int panel, int act, int grid, const uint8_t* split,
                        const uint8_t* split_b, const float* rscale, const int64_t* prow_off,
                        const int64_t* item_pref, const TensorMap128& tmap, cudaStream_t st);
+// the identity tiles (R + r, nIb + r) of the inverse rows (the other tiles start as zero)
+void launch_unit_rows(const LevelDev& L, int max_nGb, cudaStream_t st);
 void launch_gram_chol(const LevelDev& L, int precision_fp32, int max_nc, cudaStream_t st);
 template <typename T>
 void launch_psi(const LevelDev& L, int max_nGb, int max_nc, cudaStream_t st);
@@ -212,6 +246,10 @@ void launch_psi_t_apply(const LevelDev& L, const T* vec, double* part, int64_t s
 template <typename T>
 void launch_psi_apply_add(const LevelDev& L, const double* zc_sub, int64_t sum_nc, T* vec, int max_nGb,
                           int max_ncb, cudaStream_t st, int nr = 1);
+// The coarse coefficients of a level with inverse rows: out_p = z_C[R_Ci p] - sum_q G_pq t_q, t = Psi^T r
+// (the constraint part of Eq. sub_cor is Psi G Psi^T r, so both terms multiply Psi).
+void launch_coarse_coef(const LevelDev& L, const int32_t* crow_sub, int64_t sum_nc, const double* zC, const double* t,
+                        double* out, cudaStream_t st, int nr = 1);
 // psiT from Psi_G (set-up, after launch_psi)
 template <typename T>
 void launch_psi_transpose(const LevelDev& L, int max_nGb, int max_ncb, cudaStream_t st);
@@ -274,8 +312,9 @@ void launch_put_indexed(double* u, int64_t ustride, const int64_t* idx, const do
 // and right-hand side), added in a fixed order by a second kernel.  part holds
 // sum_s nGb (nGb - 1) / 2 x 64 floats per right-hand side (tri_off: its per-subdomain offsets).
 void launch_schur_snapshot(const LevelDev& L, int b, int max_nGb, cudaStream_t st);
-void launch_schur_symv(const LevelDev& L, int max_nGb, const int64_t* part_off, int64_t part_stride, const float* x,
-                       float* part, float* y, cudaStream_t st, int nr = 1);
+// inverse = 1: the same product with A_GG^{-1} (the negated inverse tiles).
+void launch_schur_symv(const LevelDev& L, int inverse, int max_nGb, const int64_t* part_off, int64_t part_stride,
+                       const float* x, float* part, float* y, cudaStream_t st, int nr = 1);
 void launch_trmv_schur(const LevelDev& L, int max_nGb, const float* x, float* y1, float* y, cudaStream_t st,
                        int nr = 1);
 void launch_sub_ctrc(const LevelDev& L, const int32_t* crow_sub, int64_t total_rows, const double* x, double* y,

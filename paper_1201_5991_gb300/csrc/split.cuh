@@ -16,10 +16,6 @@ constexpr int kPanelTiles = 8;                  // tile columns of a super-panel
 constexpr uint32_t kTilePart = 64 * 128;        // one FP16 part of one 64 x 64 tile (8 KB)
 constexpr uint32_t kSplitTile = 2 * kTilePart;  // hi and lo of one tile (16 KB)
 
-__device__ __forceinline__ int64_t split_tile_index(int i, int j, int Bc) {
-  return i < Bc ? ((int64_t)i * (i + 1) / 2 + j) : ((int64_t)Bc * (Bc + 1) / 2 + (int64_t)(i - Bc) * Bc + j);
-}
-
 __device__ __forceinline__ uint32_t sw128_off(int r, int k) {
   return (uint32_t)(r * 128 + (((k >> 3) ^ (r & 7)) << 4) + (k & 7) * 2);
 }
@@ -111,8 +107,10 @@ __device__ __forceinline__ void split_row_tile(const LevelDev& L, int s, const S
                                                uint8_t* __restrict__ split, uint8_t* __restrict__ split_signed,
                                                float* __restrict__ rscale, const int64_t* __restrict__ prow_off) {
   const int c = threadIdx.x >> 6;
-  const float* src =
-      kb0 + c < m.Bc ? (const float*)L.tiles + m.tile_off + split_tile_index(i, kb0 + c, m.Bc) * NB2 : nullptr;
+  // inverse row r has no tiles left of column nIb + r (zeros)
+  const float* src = kb0 + c < m.Bc && tile_exists(m, i, kb0 + c)
+                         ? (const float*)L.tiles + m.tile_off + tile_of(m, i, kb0 + c) * NB2
+                         : nullptr;
   const float* sq = src ? (const float*)L.sgn + m.vec_off + (int64_t)(kb0 + c) * NB : nullptr;   // column signs
   split_rows<NT>(src, nullptr, prow_off[s] + i, split, split_signed, rscale, sq);
 }

@@ -148,6 +148,11 @@ __device__ __forceinline__ int64_t schur_tile(const SubMeta& m, int i, int j) {
   return m.schur_off + ((int64_t)i * (i + 1) / 2 + j) * NB2;
 }
 
+// block row i of the symmetric matrix of a product: the explicit Schur complement, or -A_GG^{-1}
+__device__ __forceinline__ const float* symv_row(const LevelDev& L, const SubMeta& m, int inverse, int i) {
+  return inverse ? (const float*)L.tiles + m.inv_off + (int64_t)i * (i + 1) / 2 * NB2 : L.schur + schur_tile(m, i, 0);
+}
+
 // block (t, s): copy interface tile t (row-major numbering of the lower triangle) of subdomain s
 // if its interior columns are all eliminated and no interface column yet (nIb == b)
 __global__ void __launch_bounds__(256) k_schur_snapshot(LevelDev L, int b) {
@@ -204,7 +209,7 @@ __device__ __forceinline__ void tile_g2s(float* dst, const float* src, uint64_t*
 }
 
 template <int NR>
-__global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, const float* __restrict__ x,
+__global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, int inverse, const float* __restrict__ x,
                                                          const int64_t* __restrict__ part_off, int64_t part_stride,
                                                          float* __restrict__ part, float* __restrict__ y) {
   const int s = blockIdx.y;
@@ -218,7 +223,8 @@ __global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, const float
   __shared__ __align__(8) uint64_t full[kSymvStages];
   __shared__ __align__(16) float cred[2][8][NR][NB];
   __shared__ float dcol[NR][NB];
-  const float* Mrow = L.schur + schur_tile(m, i, 0);
+  const float* Mrow = symv_row(L, m, inverse, i);
+  const float sign = inverse ? -1.f : 1.f;   // the inverse tiles hold -A_GG^{-1}
   const int ntile = i + 1;
   if (tid == 0) {
     for (int k = 0; k < kSymvStages; ++k)
@@ -317,7 +323,7 @@ __global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, const float
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
       const int f = lane_sum_index<NV>(lane) + k, q = f / 8, row = warp + 8 * (f % 8);
-      yv[q * L.n_vec + row] = (&acc[0][0])[k] + dcol[q][row];
+      yv[q * L.n_vec + row] = sign * ((&acc[0][0])[k] + dcol[q][row]);
     }
   }
   // after a lost wait, copies may still be landing in this CTA's shared memory: wait (bounded)
@@ -334,7 +340,7 @@ __global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, const float
 // interleaved segments (i = j + 1 + g, j + 5 + g, ...), whose partial sums are added in segment
 // order: a fixed order, the same for any number of columns per launch.
 template <int NR>
-__global__ void __launch_bounds__(256) k_schur_symv_cols(LevelDev L, const int64_t* __restrict__ part_off,
+__global__ void __launch_bounds__(256) k_schur_symv_cols(LevelDev L, float sign, const int64_t* __restrict__ part_off,
                                                          int64_t part_stride, const float* __restrict__ part,
                                                          float* __restrict__ y) {
   constexpr int G = 4;   // row segments
@@ -359,7 +365,7 @@ __global__ void __launch_bounds__(256) k_schur_symv_cols(LevelDev L, const int64
 #pragma unroll
     for (int h = 1; h < G; ++h) t += ps[h][e];
     float* yv = y + (c0q + q) * L.n_vec + m.vec_off + (int64_t)m.nIb * NB + (int64_t)j * NB + c;
-    *yv = *yv + t;
+    *yv = *yv + sign * t;
   }
 }
 
@@ -372,7 +378,7 @@ void launch_schur_snapshot(const LevelDev& L, int b, int max_nGb, cudaStream_t s
 }
 
 template <int NR>
-void launch_symv_nr(const LevelDev& L, const dim3& grid, const int64_t* part_off, int64_t part_stride, const float* x,
+void launch_symv_nr(const LevelDev& L, int inverse, const dim3& grid, const int64_t* part_off, int64_t part_stride, const float* x,
                     float* part, float* y, cudaStream_t st) {
   const size_t dyn = sizeof(float) * kSymvStages * NB2;
   static bool attr = false;
@@ -381,13 +387,13 @@ void launch_symv_nr(const LevelDev& L, const dim3& grid, const int64_t* part_off
     attr = true;
   }
   note_launch();
-  k_schur_symv_rows<NR><<<grid, 256, dyn, st>>>(L, x, part_off, part_stride, part, y);
+  k_schur_symv_rows<NR><<<grid, 256, dyn, st>>>(L, inverse, x, part_off, part_stride, part, y);
   note_launch();
-  k_schur_symv_cols<NR><<<grid, 256, 0, st>>>(L, part_off, part_stride, part, y);
+  k_schur_symv_cols<NR><<<grid, 256, 0, st>>>(L, inverse ? -1.f : 1.f, part_off, part_stride, part, y);
 }
 
-void launch_schur_symv(const LevelDev& L, int max_nGb, const int64_t* part_off, int64_t part_stride, const float* x,
-                       float* part, float* y, cudaStream_t st, int nr) {
+void launch_schur_symv(const LevelDev& L, int inverse, int max_nGb, const int64_t* part_off, int64_t part_stride,
+                       const float* x, float* part, float* y, cudaStream_t st, int nr) {
   if (max_nGb <= 0 || L.n_sub <= 0 || nr <= 0) return;
   // columns in groups of 4, 2, 1 (the row kernel keeps 4 NR row sums and 4 NR column sums per lane)
   for (int r0 = 0; r0 < nr;) {
@@ -398,11 +404,11 @@ void launch_schur_symv(const LevelDev& L, int max_nGb, const int64_t* part_off, 
     const int64_t off = (int64_t)r0 * L.n_vec;
     float* pp = part + (int64_t)r0 * part_stride;
     if (g == 4)
-      launch_symv_nr<4>(L, grid, part_off, part_stride, x + off, pp, y + off, st);
+      launch_symv_nr<4>(L, inverse, grid, part_off, part_stride, x + off, pp, y + off, st);
     else if (g == 2)
-      launch_symv_nr<2>(L, grid, part_off, part_stride, x + off, pp, y + off, st);
+      launch_symv_nr<2>(L, inverse, grid, part_off, part_stride, x + off, pp, y + off, st);
     else
-      launch_symv_nr<1>(L, grid, part_off, part_stride, x + off, pp, y + off, st);
+      launch_symv_nr<1>(L, inverse, grid, part_off, part_stride, x + off, pp, y + off, st);
     r0 += ng * g;
   }
 }

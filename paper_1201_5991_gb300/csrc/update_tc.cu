@@ -47,10 +47,6 @@ namespace {
 
 constexpr uint32_t kSpinLimit = 1u << 26;
 
-__device__ __forceinline__ int64_t tile_index(int i, int j, int Bc) {
-  return i < Bc ? ((int64_t)i * (i + 1) / 2 + j) : ((int64_t)Bc * (Bc + 1) / 2 + (int64_t)(i - Bc) * Bc + j);
-}
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // K-major operand, 128-byte swizzle: rows of 64 16-bit entries (128 B), 8-row atoms of 1024 B
@@ -138,25 +134,19 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 }
 
 
-// one block per panel row tile i (ib <= i < R) of every subdomain with output columns (ib < Bc);
-// panel_operand: the rows i >= min(ib, Bc) of every subdomain with kb0 < Bc
+// one block per panel row tile i of every subdomain: ib <= i < R where the launch has output columns
+// (ib < Bc); panel_operand: min(ib, Bc) <= i; and the inverse rows reached by the columns below ib
 template <int NT>
-__global__ void __launch_bounds__(64 * NT) k_split_panel(LevelDev L, int kb0, int ib, int panel_operand,
+__global__ void __launch_bounds__(64 * NT) k_split_panel(LevelDev L, int kb0, int ib, int act, int panel_operand,
                                                          uint8_t* __restrict__ split,
                                                          uint8_t* __restrict__ split_signed,
                                                          float* __restrict__ rscale,
                                                          const int64_t* __restrict__ prow_off) {
   const int s = blockIdx.y;
   const SubMeta m = L.meta[s];
-  int i;
-  if (panel_operand) {
-    if (kb0 >= m.Bc) return;
-    i = (ib < m.Bc ? ib : m.Bc) + (int)blockIdx.x;
-  } else {
-    if (ib >= m.Bc) return;
-    i = ib + (int)blockIdx.x;
-  }
-  if (i >= m.R) return;
+  if (act >= m.Bc || (!panel_operand && !m.nV && ib >= m.Bc)) return;
+  const int i = (ib < m.Bc ? ib : m.Bc) + (int)blockIdx.x;
+  if (i >= m.R + inverse_rows(m, ib)) return;
   split_row_tile<NT>(L, s, m, i, kb0, split, split_signed, rscale, prow_off);
 }
 
@@ -210,7 +200,7 @@ __global__ void __launch_bounds__(256) k_split_inverse(LevelDev L, int k0, const
 // equivalent), rank 256 0.320 -> 0.230 ms; of it the MMAs and barriers alone take 0.222 ms, the operand
 // copies alone 0.259, and the output's read-modify-write in DRAM 0.158 at the copy bandwidth.
 __global__ void __launch_bounds__(kThreads2, 1)
-    k_update_tc2(LevelDev L, int nq, int jbeg, int jend, int ibeg, int panel, const uint8_t* __restrict__ split,
+    k_update_tc2(LevelDev L, int nq, int jbeg, int jend, int ibeg, int panel, int act, const uint8_t* __restrict__ split,
                  const uint8_t* __restrict__ split_b, const float* __restrict__ rscale,
                  const int64_t* __restrict__ prow_off, const int64_t* __restrict__ item_pref,
                  const __grid_constant__ CUtensorMap tmap) {
@@ -260,7 +250,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
     TcItems t;
     int64_t rbase = 0;
   };
-  auto seek = [&](Cursor& c, int64_t it, int& j, int& i0) {
+  auto seek = [&](Cursor& c, int64_t it, int& j, int& i0, int& jl) {
     if (it >= c.next) {
       do {
         ++c.s;
@@ -268,10 +258,10 @@ __global__ void __launch_bounds__(kThreads2, 1)
         c.next = item_pref[c.s + 1];
       } while (it >= c.next && c.s + 1 < n_sub);
       c.m = L.meta[c.s];
-      c.t = tc_items_of(c.m, jbeg, jend, ibeg, panel);
+      c.t = tc_items_of(c.m, jbeg, jend, ibeg, panel, act);
       c.rbase = prow_off[c.s];
     }
-    tc_item(c.t, (int)(it - c.first), j, i0);
+    tc_item(c.t, (int)(it - c.first), j, i0, jl);
   };
 
   // steps of this CTA: its items in order, nq panel columns each; a panel solve's B operand (rows
@@ -287,10 +277,10 @@ __global__ void __launch_bounds__(kThreads2, 1)
       Ring<kStages2> st;
       Ring<kMmaBars> rd;   // the step whose MMAs read the stage last
       for (int64_t it = blockIdx.x; it < n_items && !lost; it += gridDim.x) {
-        int j, i0;
-        seek(cur, it, j, i0);   // before the wait for a stage: overlaps the MMAs still reading it
+        int j, i0, jl;
+        seek(cur, it, j, i0, jl);   // before the wait for a stage: overlaps the MMAs still reading it
         const SubMeta& m = cur.m;
-        const bool hasA1 = i0 + 1 < cur.t.rend, hasB1 = j + 1 < cur.t.jlim;
+        const bool hasA1 = i0 + 1 < cur.t.rend, hasB1 = j + 1 < jl;
         const uint8_t* rowA0 = split + (cur.rbase + i0) * kPanelTiles * (int64_t)kSplitTile;
         const uint8_t* rowA1 = hasA1 ? rowA0 + kPanelTiles * (int64_t)kSplitTile : rowA0;
         const uint8_t* rowB0 = split_b + (cur.rbase + j) * kPanelTiles * (int64_t)kSplitTile;
@@ -310,9 +300,9 @@ __global__ void __launch_bounds__(kThreads2, 1)
 #pragma unroll
               for (int c = 0; c < 2; ++c) {
                 const int ti = i0 + a, tj = j + c;
-                if ((a == 0 || hasA1) && (c == 0 || hasB1) && (ti >= m.Bc || tj <= ti))
+                if ((a == 0 || hasA1) && (c == 0 || hasB1) && tile_exists(m, ti, tj))
                   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
-                                   (const float*)L.tiles + m.tile_off + tile_index(ti, tj, m.Bc) * NB2),
+                                   (const float*)L.tiles + m.tile_off + tile_of(m, ti, tj) * NB2),
                                "r"((uint32_t)(NB2 * 4))
                                : "memory");
               }
@@ -357,8 +347,8 @@ __global__ void __launch_bounds__(kThreads2, 1)
       for (int64_t it = blockIdx.x; it < n_items && ok; it += gridDim.x, ++n) {
         int nqi = nq;
         if (panel) {
-          int j, i0;
-          seek(cur, it, j, i0);
+          int j, i0, jl;
+          seek(cur, it, j, i0, jl);
           nqi = item_nq(j);
         }
         const uint32_t acc_small = tmem + 256u + 128u * (n & 1u);
@@ -404,13 +394,13 @@ __global__ void __launch_bounds__(kThreads2, 1)
     uint32_t g = 0, n = 0;
     Ring<kMmaBars> dn;
     for (int64_t it = blockIdx.x; it < n_items && !lost; it += gridDim.x, ++n) {
-      int j, i0;
-      seek(cur, it, j, i0);
+      int j, i0, jl;
+      seek(cur, it, j, i0, jl);
       const SubMeta& m = cur.m;
-      const bool hasA1 = i0 + 1 < cur.t.rend, hasB1 = j + 1 < cur.t.jlim;
+      const bool hasA1 = i0 + 1 < cur.t.rend, hasB1 = j + 1 < jl;
       const int ti = erow < 64 ? i0 : i0 + 1;
       const int tj = col0 < 64 ? j : j + 1;
-      const bool ok = (erow < 64 || hasA1) && (col0 < 64 || hasB1) && (ti >= m.Bc || tj <= ti);
+      const bool ok = (erow < 64 || hasA1) && (col0 < 64 || hasB1) && tile_exists(m, ti, tj);
       // negated row factor: the tiles receive x + (-(acc sa) f), which equals x - (acc sa) f
       const float sa = ok ? -rscale[(cur.rbase + ti) * NB + (erow & 63)] : 0.f;
       float racc[64];
@@ -449,7 +439,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
       if (ok) {   // warp-uniform: the warp's 32 rows and 64 columns lie in one output tile
         const float4* sb = (const float4*)(rscale + (cur.rbase + tj) * NB);
         // row of the warp's first output row in the [rows][64] view of the tile buffer
-        const int y = (int)((m.tile_off + tile_index(ti, tj, m.Bc) * NB2) / NB) + (32 * (warp & 3) & 63);
+        const int y = (int)((m.tile_off + tile_of(m, ti, tj) * NB2) / NB) + (32 * (warp & 3) & 63);
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
           // the previous reduce-add out of this warp's box has read it
@@ -509,16 +499,16 @@ __global__ void __launch_bounds__(kThreads2, 1)
 
 }  // namespace
 
-void launch_split_panel(const LevelDev& L, int kb0, int nt, int ib, int max_R, uint8_t* split, uint8_t* split_signed,
-                        float* rscale, const int64_t* prow_off, cudaStream_t st, int panel_operand) {
-  const int first = panel_operand ? kb0 + 1 : ib;   // the rows of a panel operand start after kb0
-  if (L.n_sub <= 0 || max_R <= first) return;
+void launch_split_panel(const LevelDev& L, int kb0, int nt, int ib, int act, int rows, uint8_t* split,
+                        uint8_t* split_signed, float* rscale, const int64_t* prow_off, cudaStream_t st,
+                        int panel_operand) {
+  if (L.n_sub <= 0 || rows <= 0) return;
   note_launch();
-  const dim3 grid((unsigned)(max_R - first), (unsigned)L.n_sub);
+  const dim3 grid((unsigned)rows, (unsigned)L.n_sub);
   if (nt == 8)
-    k_split_panel<8><<<grid, 512, 0, st>>>(L, kb0, ib, panel_operand, split, split_signed, rscale, prow_off);
+    k_split_panel<8><<<grid, 512, 0, st>>>(L, kb0, ib, act, panel_operand, split, split_signed, rscale, prow_off);
   else
-    k_split_panel<4><<<grid, 256, 0, st>>>(L, kb0, ib, panel_operand, split, split_signed, rscale, prow_off);
+    k_split_panel<4><<<grid, 256, 0, st>>>(L, kb0, ib, act, panel_operand, split, split_signed, rscale, prow_off);
 }
 
 void launch_split_inverse(const LevelDev& L, int k0, const float* xinv, uint8_t* split, float* rscale,
@@ -528,7 +518,8 @@ void launch_split_inverse(const LevelDev& L, int k0, const float* xinv, uint8_t*
   k_split_inverse<<<dim3(4, (unsigned)L.n_sub), 256, 0, st>>>(L, k0, xinv, split, rscale, prow_off);
 }
 
-void launch_update_tc2(const LevelDev& L, int nq, int jbeg, int jend, int ibeg, int panel, int grid, const uint8_t* split,
+void launch_update_tc2(const LevelDev& L, int nq, int jbeg, int jend, int ibeg, int panel, int act, int grid,
+                       const uint8_t* split,
                        const uint8_t* split_b, const float* rscale, const int64_t* prow_off,
                        const int64_t* item_pref, const TensorMap128& tmap, cudaStream_t st) {
   if (grid <= 0 || L.n_sub <= 0 || nq <= 0 || nq > kPanelTiles) return;
@@ -542,7 +533,7 @@ void launch_update_tc2(const LevelDev& L, int nq, int jbeg, int jend, int ibeg, 
   CUtensorMap m;
   static_assert(sizeof(CUtensorMap) == sizeof(TensorMap128), "tensor map size");
   std::memcpy(&m, &tmap, sizeof(m));
-  k_update_tc2<<<(unsigned)grid, kThreads2, dyn, st>>>(L, nq, jbeg, jend, ibeg, panel, split, split_b, rscale, prow_off,
+  k_update_tc2<<<(unsigned)grid, kThreads2, dyn, st>>>(L, nq, jbeg, jend, ibeg, panel, act, split, split_b, rscale, prow_off,
                                                         item_pref, m);
 }
 
