@@ -396,9 +396,8 @@ __global__ void k_syrk_update(LevelDev L, int k, int jmax, int fuse_next, int rl
 }
 
 // ---- G = Y_G Y_G^T in FP64, Cholesky, inverse; K_C = G^{-1} - rho I ----------------------
-// one warp per entry (a, b), a >= b, of one subdomain's G; lanes stride over the interface
+// FP64 levels: one warp per entry (a, b), a >= b, of one subdomain's G; lanes stride over the interface
 // columns (contiguous inside a tile row), FP64 products, fixed-order warp reduction
-template <typename T>
 __global__ void k_gram(LevelDev L) {
   const int s = blockIdx.y;
   const SubMeta m = L.meta[s];
@@ -408,9 +407,9 @@ __global__ void k_gram(LevelDev L) {
   if (pair >= nc * nc) return;
   const int a = pair / nc, b = pair % nc;
   if (b > a) return;
-  const T* ya = tile_ptr<T>(m, L.tiles, m.Bc + a / NB, m.nIb) + (a % NB) * NB;
-  const T* yb = tile_ptr<T>(m, L.tiles, m.Bc + b / NB, m.nIb) + (b % NB) * NB;
-  const T* sG = (const T*)L.sgn + m.vec_off + (int64_t)m.nIb * NB;   // G = Y S Y^T
+  const double* ya = tile_ptr<double>(m, L.tiles, m.Bc + a / NB, m.nIb) + (a % NB) * NB;
+  const double* yb = tile_ptr<double>(m, L.tiles, m.Bc + b / NB, m.nIb) + (b % NB) * NB;
+  const double* sG = (const double*)L.sgn + m.vec_off + (int64_t)m.nIb * NB;   // G = Y S Y^T
   double acc = 0.0;
   for (int c = lane; c < m.nGb * NB; c += 32) {
     const int64_t o = (int64_t)(c / NB) * NB2 + (c % NB);
@@ -421,12 +420,140 @@ __global__ void k_gram(LevelDev L) {
     double* G = L.Ginv + m.g_off;
     G[a * nc + b] = acc;
     G[b * nc + a] = acc;
-    if (L.G) {   // kept: Ginv is inverted in place
-      double* G0 = L.G + m.g_off;
-      G0[a * nc + b] = acc;
-      G0[b * nc + a] = acc;
-    }
   }
+}
+
+// ---- FP32 factors: G and Z = Y^T G^{-1} with double-float sums -------------------------------
+// The FP64 units give 2 products per cycle and SM, so these two products (n_G n_c^2 each) were bound by
+// them, with one warp or thread per entry and few blocks where n_c is large: 48^3 elasticity (n_c <= 78)
+// 1.5 + 1.4 ms per set-up, 64 k-means subdomains (n_c <= 258) 15 + 22 ms.  The factor's entries are FP32, so
+// a product a b is p + e exactly (e = fma(a, b, -p)), and a sum kept as an unevaluated FP32 pair (two-sum,
+// Knuth; Dekker) has 2^-46 relative error, far below the 2^-24 of the factor's entries: 10 FP32
+// operations per product at 128 lanes per cycle.  One block per 64 x 64 tile of the result, both
+// operands k-major in shared memory, 4 x 4 entries per thread.
+struct Pair2 {
+  float hi, lo;
+};
+
+__device__ __forceinline__ void df_add(Pair2& s, float p, float e) {   // s += p + e, no contraction
+  const float t = __fadd_rn(s.hi, p);
+  const float b = __fsub_rn(t, s.hi);
+  const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, b)), __fsub_rn(p, b));
+  s.hi = t;
+  s.lo = __fadd_rn(s.lo, __fadd_rn(err, e));
+}
+
+// tile (a, b), b <= a, of G = Y_G S Y_G^T
+__global__ void __launch_bounds__(256) k_gram_f32(LevelDev L) {
+  const int s = blockIdx.y;
+  const SubMeta m = L.meta[s];
+  int ab = 0, t = blockIdx.x;
+  while (t > ab) t -= ++ab;   // row block ab, column block t
+  const int bb = t;
+  if (ab >= m.ncb) return;
+  __shared__ __align__(16) float As[NB][LDS], Bs[NB][LDS];
+  const float* sG = (const float*)L.sgn + m.vec_off + (int64_t)m.nIb * NB;
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  Pair2 acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = {0.f, 0.f};
+  for (int c = 0; c < m.nGb; ++c) {
+    const float* ya = tile_ptr<float>(m, L.tiles, m.Bc + ab, m.nIb + c);
+    const float* yb = tile_ptr<float>(m, L.tiles, m.Bc + bb, m.nIb + c);
+    for (int e = threadIdx.x; e < NB2; e += 256) {
+      const int r = e / NB, k = e % NB;
+      As[k][r] = ya[e];
+      Bs[k][r] = sG[c * NB + k] * yb[e];   // S = +-1: exact
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < NB; ++k) {
+      float a[4], b[4];
+      load4(a, &As[k][4 * ty]);
+      load4(b, &Bs[k][4 * tx]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float p = __fmul_rn(a[i], b[j]);
+          df_add(acc[i][j], p, __fmaf_rn(a[i], b[j], -p));
+        }
+    }
+    __syncthreads();
+  }
+  const int nc = m.nc;
+  double* G = L.Ginv + m.g_off;
+  double* G0 = L.G ? L.G + m.g_off : nullptr;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int r = ab * NB + 4 * ty + i, c = bb * NB + 4 * tx + j;
+      if (r >= nc || c >= nc || c > r) continue;   // the diagonal tiles' upper halves mirror the lower
+      const double v = (double)acc[i][j].hi + (double)acc[i][j].lo;
+      G[(int64_t)r * nc + c] = v;
+      G[(int64_t)c * nc + r] = v;
+      if (G0) {   // kept: Ginv is inverted in place
+        G0[(int64_t)r * nc + c] = v;
+        G0[(int64_t)c * nc + r] = v;
+      }
+    }
+}
+
+// rows 64 j .. of Z = Y_G^T G^{-1}, columns 64 qb ..: G^{-1} as an FP32 pair (gh + gl, 2^-48)
+__global__ void __launch_bounds__(256) k_psi_rhs_f32(LevelDev L) {
+  const int j = blockIdx.x, qb = blockIdx.y, s = blockIdx.z;
+  const SubMeta m = L.meta[s];
+  if (j >= m.nGb || qb >= m.ncb) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float(*Ys)[NB] = (float(*)[NB])smem_raw;
+  float(*Gh)[NB] = Ys + NB;
+  float(*Gl)[NB] = Gh + NB;
+  const int nc = m.nc, tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const double* Gi = L.Ginv + m.g_off;
+  Pair2 acc[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[a][b] = {0.f, 0.f};
+  for (int pb = 0; pb < m.ncb; ++pb) {
+    const float* y = tile_ptr<float>(m, L.tiles, m.Bc + pb, m.nIb + j);
+    for (int e = threadIdx.x; e < NB2; e += 256) {
+      const int p = e / NB, c = e % NB, gp = pb * NB + p, gq = qb * NB + c;
+      Ys[p][c] = y[e];
+      const double g = gp < nc && gq < nc ? Gi[(int64_t)gp * nc + gq] : 0.0;
+      const float h = (float)g;
+      Gh[p][c] = h;
+      Gl[p][c] = (float)(g - (double)h);
+    }
+    __syncthreads();
+    const int pn = min(NB, nc - pb * NB);
+#pragma unroll 2
+    for (int p = 0; p < pn; ++p) {
+      float a[4], h[4], l[4];
+      load4(a, &Ys[p][4 * ty]);
+      load4(h, &Gh[p][4 * tx]);
+      load4(l, &Gl[p][4 * tx]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float v = __fmul_rn(a[i], h[k]);
+          df_add(acc[i][k], v, __fmaf_rn(a[i], l[k], __fmaf_rn(a[i], h[k], -v)));
+        }
+    }
+    __syncthreads();
+  }
+  float* Z = (float*)L.psi + m.psi_off;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int q = qb * NB + 4 * tx + k;
+      if (q < nc) Z[(int64_t)(j * NB + 4 * ty + i) * nc + q] = __fadd_rn(acc[i][k].hi, acc[i][k].lo);
+    }
 }
 
 // G^{-1} by Gauss-Jordan elimination with partial pivoting (indefinite levels), FP64, one block
@@ -557,8 +684,7 @@ __global__ void k_small_chol_inv(LevelDev L) {
   }
 }
 
-// Z = Y_G^T G^{-1}, written into the Psi buffer (rows: interface padded positions)
-template <typename T>
+// FP64 levels: Z = Y_G^T G^{-1}, written into the Psi buffer (rows: interface padded positions)
 __global__ void k_psi_rhs(LevelDev L) {
   const int s = blockIdx.y;
   const SubMeta m = L.meta[s];
@@ -567,16 +693,16 @@ __global__ void k_psi_rhs(LevelDev L) {
   const int rows = m.nGb * NB;
   const int64_t total = (int64_t)rows * nc;
   const double* Gi = L.Ginv + m.g_off;
-  T* Z = (T*)L.psi + m.psi_off;
+  double* Z = (double*)L.psi + m.psi_off;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
     const int c = (int)(t / nc), q = (int)(t % nc);
     const int jb = m.nIb + c / NB, cc = c % NB;
     double acc = 0.0;
     for (int p = 0; p < nc; ++p) {
-      const T y = tile_ptr<T>(m, L.tiles, m.Bc + p / NB, jb)[(p % NB) * NB + cc];
-      acc += (double)y * Gi[p * nc + q];
+      const double y = tile_ptr<double>(m, L.tiles, m.Bc + p / NB, jb)[(p % NB) * NB + cc];
+      acc += y * Gi[p * nc + q];
     }
-    Z[t] = (T)acc;   // Z = Y^T G^{-1}
+    Z[t] = acc;   // Z = Y^T G^{-1}
   }
 }
 
@@ -1060,26 +1186,30 @@ void launch_potrf_step(const LevelDev& L, int k, int max_R, int max_tiles, int j
   }
 }
 
-template <typename T>
-void launch_gram_chol_t(const LevelDev& L, int max_nc, cudaStream_t st) {
-  const unsigned ns = (unsigned)L.n_sub;
-  const unsigned gx = (unsigned)(((int64_t)max_nc * max_nc + 7) / 8);
-  { note_launch(); k_gram<T><<<dim3(gx, ns), 256, 0, st>>>(L); }
-  { note_launch(); k_small_chol_inv<<<ns, 256, 0, st>>>(L); }
-}
-
 void launch_gram_chol(const LevelDev& L, int precision_fp32, int max_nc, cudaStream_t st) {
-  if (precision_fp32)
-    launch_gram_chol_t<float>(L, max_nc, st);
-  else
-    launch_gram_chol_t<double>(L, max_nc, st);
+  const unsigned ns = (unsigned)L.n_sub;
+  note_launch();
+  if (precision_fp32) {
+    const unsigned nb = (unsigned)((max_nc + NB - 1) / NB);
+    k_gram_f32<<<dim3(nb * (nb + 1) / 2, ns), 256, 0, st>>>(L);
+  } else {
+    const unsigned gx = (unsigned)(((int64_t)max_nc * max_nc + 7) / 8);
+    k_gram<<<dim3(gx, ns), 256, 0, st>>>(L);
+  }
+  { note_launch(); k_small_chol_inv<<<ns, 256, 0, st>>>(L); }
 }
 
 template <typename T>
 void launch_psi(const LevelDev& L, int max_nGb, int max_nc, cudaStream_t st) {
   const unsigned ns = (unsigned)L.n_sub;
   if (max_nc <= 0 || max_nGb <= 0) return;
-  { note_launch(); k_psi_rhs<T><<<dim3(16, ns), 256, 0, st>>>(L); }
+  note_launch();
+  if constexpr (sizeof(T) == 4) {
+    const size_t sm = 3 * NB2 * sizeof(float);
+    k_psi_rhs_f32<<<dim3((unsigned)max_nGb, (unsigned)((max_nc + NB - 1) / NB), ns), 256, sm, st>>>(L);
+  } else {
+    k_psi_rhs<<<dim3(16, ns), 256, 0, st>>>(L);
+  }
   const unsigned chunks = (unsigned)((max_nc + 15) / 16);
   for (int t = 0; t < max_nGb; ++t) {   // block row Bc - 1 - t of every subdomain, bottom up
     { note_launch(); k_psi_final<T><<<dim3(chunks, ns), 256, 0, st>>>(L, t); }
