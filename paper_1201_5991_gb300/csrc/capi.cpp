@@ -214,7 +214,7 @@ struct Level {
   bool solve32 = false;
   LevelDev d32{};
   float* v32 = nullptr;            // [blk][n_vec] FP32 input of the coarse solve
-  float* v32b = nullptr;           // [blk][n_vec] FP32 output of the explicit inverse
+  int32_t* v32_pos = nullptr;      // [n_dof] position of every coarse DOF in v32
   float* winv = nullptr;           // explicit inverse of the FP32 copy (n_vec x n_vec), or null
   // sweep launch configuration per part (autotuned): CTAs per SM, deep tile ring, task order
   int sweep_ctas[2] = {2, 2};
@@ -291,7 +291,7 @@ void alloc_level_work(Level& L, DevArena& A, int blk) {
   L.gv0 = A.alloc<double>(L.mesh.n_dof * blk);
   if (L.solve32) {
     L.v32 = A.alloc<float>(nv);
-    L.v32b = A.alloc<float>(nv);
+    ck(cudaMemsetAsync(L.v32, 0, sizeof(float) * (size_t)nv, A.st), "memset");   // padding positions stay zero
   }
   L.blk = blk;
 }
@@ -343,7 +343,11 @@ struct bddc_handle_s {
   int32_t* d_lift_a = nullptr;
   // PCG
   double* scal = nullptr;              // [16]
-  double* partial = nullptr;           // [kDotBlocks]
+  double* partial = nullptr;           // [kDotBlocks], and the fused sums' 2 iface_blocks(n_iface) per column
+  int* dot_cnt = nullptr;              // [blk] counters of the fused sums
+  KrylovStore kstore;                  // directions of the running refined solve (allocated by the first one)
+  double* proj_coef = nullptr;
+  int kstore_blk = 0;
   double* h_scal = nullptr;            // pinned [16]
   double *vx = nullptr, *vr = nullptr, *vz = nullptr, *vp = nullptr, *vq = nullptr, *vrold = nullptr, *vg = nullptr;
   double *vs = nullptr, *vsh = nullptr, *vt = nullptr;   // BiCGstab s, M^{-1} s, S M^{-1} s
@@ -399,6 +403,10 @@ namespace {
 constexpr int kDotBlocks = 304;   // 2 x SM count of a GB300; fixed for reproducible sums
 
 constexpr int kRestart = 50;   // flexible GMRES restart length
+
+int64_t partial_size(int64_t n_iface, int blk) {
+  return std::max<int64_t>(kDotBlocks, 2 * iface_blocks(n_iface)) * blk;
+}
 
 int krylov_kind(const bddc_handle_s* h) {
   if (h->opts.krylov != 0) return h->opts.krylov;
@@ -1033,6 +1041,14 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     }
     L.crow_sub = A.upload(cs, st);
   }
+  d.crow = nullptr;
+  d.cval = nullptr;
+  if (L.level1 && L.fp32) {   // the inner operator's C^T R C by positions
+    d.crow = A.alloc<int32_t>(L.n_vec);
+    d.cval = A.alloc<double>(L.n_vec);
+    ck(cudaMemsetAsync(d.crow, 0xFF, sizeof(int32_t) * (size_t)std::max<int64_t>(L.n_vec, 1), st), "memset");
+    launch_constraint_positions(d, L.crow_sub, L.sum_nc, st);
+  }
   ph("row lists");
   L.slot_elem = A.upload(slot_elem, st);
   L.iface_dofs = A.upload(mp.iface_dofs, st);
@@ -1239,12 +1255,12 @@ void interior_solve_l1(bddc_handle_s* h, Level& L, const double* v, double* w, c
 // y = S x on the level-1 interface (Sec. 2, discrete Dirichlet problems).  With cur_steps = 0
 // on an FP32 level: the inner operator S~ = sum R_i^T (L_GG S L_GG^T - C_i^T R C_i) R_i from the
 // stored factor (no interior solves).
-void schur_apply(bddc_handle_s* h, const double* x, double* y, cudaStream_t st, int nb = 1) {
+void schur_apply(bddc_handle_s* h, const double* x, double* y, cudaStream_t st, int nb = 1,
+                 const FusedDot& dot = FusedDot()) {
   Level& L = h->lv[0];
   const int64_t n = L.n_vec * nb;
   if (L.fp32 && h->cur_steps == 0) {
-    launch_gather_iface<double>(L.d, x, 0, L.dl0, st, nb);
-    launch_convert<double, float>(L.dl0, (float*)L.locA, n, st);
+    launch_inner_gather(L.d, x, (float*)L.locA, L.crow_sub, L.sum_nc, L.cc_t, st, nb);
     const float* yf = (const float*)L.locA;
     if (L.explicit_schur) {   // one pass over the lower triangle of S_i + C_i^T R C_i
       ProfScope ps(h, BDDC_PROF_TRMV, column_groups(nb, 4) * 0.5 * L.trmv_bytes, 0.0, st);
@@ -1255,9 +1271,7 @@ void schur_apply(bddc_handle_s* h, const double* x, double* y, cudaStream_t st, 
       ProfScope ps(h, BDDC_PROF_TRMV, column_groups(nb, 8) * L.trmv_bytes, 0.0, st);
       launch_trmv_schur(L.d, L.max_nGb, (const float*)L.locA, (float*)L.locB, (float*)L.locA, st, nb);
     }
-    launch_convert<float, double>(yf, L.dl1, n, st);
-    launch_sub_ctrc(L.d, L.crow_sub, L.sum_nc, L.dl0, L.dl1, st, nb);
-    launch_scatter_iface<double>(L.d, L.dl1, 0, y, st, nb);
+    launch_inner_scatter(L.d, yf, L.cc_t, L.sum_nc, y, st, nb, dot);
     return;
   }
   launch_gather_iface<double>(L.d, x, 0, L.dl0, st, nb);                 // x_i = R_i x
@@ -1266,7 +1280,7 @@ void schur_apply(bddc_handle_s* h, const double* x, double* y, cudaStream_t st, 
   interior_solve_l1(h, L, L.dl1, L.dl2, st, nb);                        // w = K_II^{-1} v
   launch_axpy_loc(L.dl0, L.dl2, -1.0, n, st);                           // t = [-w ; x_i]
   launch_spmv_rows(L.d, L.rows[1], L.nrows[1], L.dl0, L.dl1, 1.0, 0.0, L.row_sub, st, nb);  // y_i = K_GG x_i - K_GI w
-  launch_scatter_iface<double>(L.d, L.dl1, 0, y, st, nb);                // y = sum R_i^T y_i
+  launch_scatter_iface<double>(L.d, L.dl1, 0, y, st, nb, dot);           // y = sum R_i^T y_i
 }
 
 // g = f_G - sum R_i^T K_GI K_II^{-1} f_I   (f: nb columns of n_free)
@@ -1302,13 +1316,12 @@ void recover(bddc_handle_s* h, const double* f, const double* uG, double* u, cud
 void coarsest_solve(bddc_handle_s* h, const double* rC, double* zC, cudaStream_t st, int nb = 1) {
   Level& C = h->lv.back();
   if (C.solve32) {   // mixed form: the preconditioner's coarse solve with the FP32 copy of the factor
-    launch_gather_glob<float>(C.d32, rC, 2, C.v32, st, nb);
-    if (C.winv) {     // explicit inverse of that copy: one product
+    if (C.winv) {     // explicit inverse of that copy: one product (v32 was filled with r_C)
       ProfScope ps(h, BDDC_PROF_COARSE, 4.0 * (double)C.n_vec * C.n_vec * column_groups(nb, 8), 0.0, st);
-      launch_coarse_apply(C.winv, C.n_vec, C.v32, C.v32b, C.n_vec, nb, st);
-      launch_scatter_interior<float>(C.d32, C.v32b, zC, st, nb);
+      launch_coarse_apply(C.winv, C.n_vec, C.v32, zC, C.d32.loc2glob, C.n_vec, C.d32.n_dof, nb, st);
       return;
     }
+    launch_gather_glob<float>(C.d32, rC, 2, C.v32, st, nb);
     trsv_pair<float>(h, C, C.v32, 0, st, nb);
     launch_scatter_interior<float>(C.d32, C.v32, zC, st, nb);
     return;
@@ -1324,13 +1337,16 @@ void full_step(bddc_handle_s* h, int l, const double* r, double* z, cudaStream_t
 // One interface step of Algorithm 2 on BDDC level l: distribute, subdomain corrections,
 // coarse residual, coarse correction (coarsest solve or the next level), combine.
 template <typename T>
-void interface_step_t(bddc_handle_s* h, int l, const double* rhat, double* zhat, cudaStream_t st, int nb) {
+void interface_step_t(bddc_handle_s* h, int l, const double* rhat, double* zhat, cudaStream_t st, int nb,
+                      const FusedDot& dot) {
   Level& L = h->lv[l];
   T* v = (T*)L.locA;
   launch_gather_iface<T>(L.d, rhat, 1, v, st, nb);          // r_i = E_i^T r_hat
-  launch_psi_t_apply<T>(L.d, v, L.psi_part, L.sum_nc, L.rc_sub, L.max_nGb, L.max_ncb, st, nb);   // Psi_i^T r_i
-  launch_coarse_gather(L.d, L.rc_sub, L.sum_nc, L.rC, st, nb);   // r_C = sum R_Ci^T Psi_i^T r_i
   const bool last = l + 2 == (int)h->lv.size();
+  const Level& C = h->lv.back();
+  launch_psi_t_apply<T>(L.d, v, L.psi_part, L.sum_nc, L.max_nGb, L.max_ncb, st, nb);   // Psi_i^T r_i
+  launch_coarse_gather(L.d, L.psi_part, rows_zmax(L.max_nGb), L.rc_sub, L.sum_nc, L.rC,
+                       last && C.winv ? C.v32 : nullptr, C.v32_pos, C.n_vec, st, nb);   // r_C = sum R_Ci^T Psi_i^T r_i
   if (L.inverse) {
     // Eq. sub_cor with the explicit inverse of the augmented interface matrix: z_i = A_GG^{-1} r_i -
     // Psi_i G_i Psi_i^T r_i, one symmetric product over the stored lower triangle instead of a sweep pair
@@ -1350,7 +1366,7 @@ void interface_step_t(bddc_handle_s* h, int l, const double* rhat, double* zhat,
       full_step(h, l + 1, L.rC, L.zC, st, nb);
     launch_coarse_coef(L.d, L.crow_sub, L.sum_nc, L.zC, L.rc_sub, L.zc_sub, st, nb);
     launch_psi_apply_add<float>(L.d, L.zc_sub, L.sum_nc, z, L.max_nGb, L.max_ncb, st, nb);
-    launch_scatter_iface<float>(L.d, z, 1, zhat, st, nb);      // z_hat = sum E_i (...)
+    launch_scatter_iface<float>(L.d, z, 1, zhat, st, nb, dot); // z_hat = sum E_i (...)
     return;
   }
   trsv_one<T>(h, L, v, 1, 0, st, nb);                       // Eq. sub_cor via the trailing factor
@@ -1363,14 +1379,15 @@ void interface_step_t(bddc_handle_s* h, int l, const double* rhat, double* zhat,
     full_step(h, l + 1, L.rC, L.zC, st, nb);
   launch_coarse_scatter_n(L.d.sub_coarse, L.sum_nc, L.zC, L.d.n_coarse, L.zc_sub, st, nb);
   launch_psi_apply_add<T>(L.d, L.zc_sub, L.sum_nc, v, L.max_nGb, L.max_ncb, st, nb);   // Psi_i R_Ci z_C + z_i
-  launch_scatter_iface<T>(L.d, v, 1, zhat, st, nb);            // z_hat = sum E_i (...)
+  launch_scatter_iface<T>(L.d, v, 1, zhat, st, nb, dot);       // z_hat = sum E_i (...)
 }
 
-void interface_step(bddc_handle_s* h, int l, const double* rhat, double* zhat, cudaStream_t st, int nb) {
+void interface_step(bddc_handle_s* h, int l, const double* rhat, double* zhat, cudaStream_t st, int nb,
+                    const FusedDot& dot = FusedDot()) {
   if (h->lv[l].fp32)
-    interface_step_t<float>(h, l, rhat, zhat, st, nb);
+    interface_step_t<float>(h, l, rhat, zhat, st, nb, dot);
   else
-    interface_step_t<double>(h, l, rhat, zhat, st, nb);
+    interface_step_t<double>(h, l, rhat, zhat, st, nb, dot);
 }
 
 // Levels l > 1: interior pre-correction, interface step, interior post-correction
@@ -1403,8 +1420,9 @@ void full_step(bddc_handle_s* h, int l, const double* r, double* z, cudaStream_t
     full_step_t<double>(h, l, r, z, st, nb);
 }
 
-void precond(bddc_handle_s* h, const double* r, double* z, cudaStream_t st, int nb = 1) {
-  interface_step(h, 0, r, z, st, nb);
+void precond(bddc_handle_s* h, const double* r, double* z, cudaStream_t st, int nb = 1,
+             const FusedDot& dot = FusedDot()) {
+  interface_step(h, 0, r, z, st, nb, dot);
 }
 
 double dot_host(bddc_handle_s* h, const double* a, const double* b, int64_t n) {
@@ -1575,7 +1593,10 @@ void numeric_setup(bddc_handle_s* h) {
         L.d32.dinv = h->arena.alloc<float>(L.dinv_elems);
         L.d32.sgn = h->arena.alloc<float>(L.n_vec);
         L.v32 = h->arena.alloc<float>(L.n_vec * L.blk);
-        L.v32b = h->arena.alloc<float>(L.n_vec * L.blk);
+        ck(cudaMemsetAsync(L.v32, 0, sizeof(float) * (size_t)(L.n_vec * L.blk), st), "memset");   // padding positions
+        std::vector<int32_t> pos(L.mesh.n_dof);
+        for (int64_t q = 0; q < (int64_t)L.maps.sub_dofs.size(); ++q) pos[L.maps.sub_dofs[q]] = (int32_t)pad_pos(L.meta[0], q);
+        L.v32_pos = h->arena.upload(pos, st);
         if (L.n_vec <= kMaxCoarseInverse) L.winv = h->arena.alloc<float>(L.n_vec * L.n_vec);
         L.solve32 = true;
       }
@@ -1869,7 +1890,9 @@ void device_setup(bddc_handle_s* h) {
     h->d_lift = A.alloc<double>(h->n_free);
   }
   h->scal = A.alloc<double>(16);
-  h->partial = A.alloc<double>(kDotBlocks);
+  h->partial = A.alloc<double>(partial_size(h->lv[0].d.n_iface, 1));
+  h->dot_cnt = A.alloc<int>(kMaxBlock);
+  ck(cudaMemsetAsync(h->dot_cnt, 0, sizeof(int) * kMaxBlock, st), "memset");
   ck(cudaMallocHost(&h->h_scal, sizeof(double) * 16), "cudaMallocHost");
   const int64_t ni = std::max<int64_t>(h->lv[0].d.n_iface, 1);
   h->vx = A.alloc<double>(ni);
@@ -1913,21 +1936,26 @@ struct PcgResult {
 
 // One full PCG iteration (Sec. 4) on the level-1 interface for a block of nb right-hand sides,
 // all on the device: q = S p, alpha = r.z / p.q, x += alpha p, r -= alpha q, ||r||^2,
-// z = M^{-1} r (Algorithm 2), beta (Fletcher-Reeves or flexible), p = z + beta p.  Column k keeps
+// z = M^{-1} r (Algorithm 2), beta (Fletcher-Reeves or flexible), p = z + beta p.  The dot products and
+// scalar steps run inside the kernels that make q, r and z (FusedDot): a 48^3 iteration has 16 launches
+// instead of 33.  Column k keeps
 // its scalars at scal[16 k ..]; a column whose flag scal[16 k + 8] is set stays frozen.
 void pcg_body(bddc_handle_s* h, double* x, int flexible, cudaStream_t st, int nb) {
   const int64_t n = h->lv[0].d.n_iface;
   double* S = h->scal;
-  schur_apply(h, h->vp, h->vq, st, nb);
-  launch_dot(h->vp, h->vq, n, h->partial, kDotBlocks, S + 1, st, nb);
-  launch_pcg_scalars(S, 0, flexible, st, nb);
-  if (flexible) ck(cudaMemcpyAsync(h->vrold, h->vr, sizeof(double) * n * nb, cudaMemcpyDeviceToDevice, st), "copy");
-  launch_pcg_update_x_r(x, h->vr, h->vp, h->vq, S, n, st, nb);
-  launch_dot(h->vr, h->vr, n, h->partial, kDotBlocks, S + 5, st, nb);
-  precond(h, h->vr, h->vz, st, nb);
-  launch_dot(h->vr, h->vz, n, h->partial, kDotBlocks, S + 4, st, nb);
-  if (flexible) launch_dot(h->vz, h->vrold, n, h->partial, kDotBlocks, S + 7, st, nb);
-  launch_pcg_scalars(S, 1, flexible, st, nb);
+  FusedDot dot;
+  dot.flexible = flexible;
+  dot.scal = S;
+  dot.partial = h->partial;
+  dot.cnt = h->dot_cnt;
+  dot.mode = 1;
+  dot.a = h->vp;
+  schur_apply(h, h->vp, h->vq, st, nb, dot);                                 // q = S p, p . q, alpha
+  launch_pcg_update_x_r(x, h->vr, h->vp, h->vq, S, n, h->partial, h->dot_cnt, h->kstore, st, nb);   // x, r, r . r
+  dot.mode = 2;
+  dot.a = h->vr;
+  dot.b = h->vq;
+  precond(h, h->vr, h->vz, st, nb, dot);                                     // z = M^{-1} r, r . z, q . z, beta
   launch_pcg_update_p(h->vp, h->vz, S, n, st, nb);
 }
 
@@ -2034,7 +2062,7 @@ void ensure_block(bddc_handle_s* h, int nb) {
   h->vsh = A.alloc<double>(ni);
   h->vt = A.alloc<double>(ni);
   h->scal = A.alloc<double>(16 * blk);
-  h->partial = A.alloc<double>((int64_t)kDotBlocks * blk);
+  h->partial = A.alloc<double>(partial_size(h->lv[0].d.n_iface, blk));
   if (h->h_scal) cudaFreeHost(h->h_scal);
   h->h_scal = nullptr;
   ck(cudaMallocHost(&h->h_scal, sizeof(double) * 16 * blk), "cudaMallocHost");
@@ -2044,12 +2072,16 @@ void ensure_block(bddc_handle_s* h, int nb) {
 }
 
 // r = g - S x, z = M^{-1} r, p = z, rz = r.z  (start, or restart after a failed true-residual
-// check) for every column of the block
-void pcg_start(bddc_handle_s* h, const double* g, double* x, bool x_zero, cudaStream_t st, int nb) {
+// check) for every column of the block; project: x and r from the projection of g on the stored directions
+void pcg_start(bddc_handle_s* h, const double* g, double* x, bool x_zero, cudaStream_t st, int nb,
+               bool project = false) {
   const int64_t n = h->lv[0].d.n_iface;
   double* S = h->scal;
-  ck(cudaMemcpyAsync(h->vr, g, sizeof(double) * n * nb, cudaMemcpyDeviceToDevice, st), "copy");
-  if (!x_zero) {
+  if (project)
+    launch_project(h->kstore, g, x, h->vr, n, h->proj_coef, st, nb);
+  else
+    ck(cudaMemcpyAsync(h->vr, g, sizeof(double) * n * nb, cudaMemcpyDeviceToDevice, st), "copy");
+  if (!x_zero && !project) {
     schur_apply(h, x, h->vq, st, nb);
     launch_axpy_loc(h->vr, h->vq, -1.0, n * nb, st);
   }
@@ -2071,8 +2103,10 @@ void freeze_column(bddc_handle_s* h, int k) {
 // residual confirms it (after one failed confirmation every column restarts from its iterate with
 // the true residual; after a second the column stops as not converged); stopped columns stay
 // frozen while the others continue.  x: nb columns.
+// inner: a solve inside the outer refinement, whose FP64 residual judges the result, so the recursive
+// residual stops a column; project: start from the directions that this refinement's earlier solves stored.
 std::vector<PcgResult> pcg(bddc_handle_s* h, const double* g, double* x, const std::vector<double>& tol, int maxit,
-                           int nb) {
+                           int nb, bool inner = false, bool project = false) {
   cudaStream_t st = h->st;
   const int64_t n = h->lv[0].d.n_iface;
   std::vector<PcgResult> res(nb);
@@ -2102,7 +2136,7 @@ std::vector<PcgResult> pcg(bddc_handle_s* h, const double* g, double* x, const s
     }
   }
   if (active == 0) return res;
-  pcg_start(h, g, x, true, st, nb);
+  pcg_start(h, g, x, true, st, nb, project);
   const bool graphs = h->opts.use_graph && x == h->vx;
   drop_graph_if_kind_differs(h, flexible, nb);
   for (int it = 1; it <= maxit; ++it) {
@@ -2131,6 +2165,16 @@ std::vector<PcgResult> pcg(bddc_handle_s* h, const double* g, double* x, const s
       if (rel <= tol[k]) check.push_back(k);
     }
     if (check.empty()) continue;
+    if (inner) {
+      for (int k : check) {
+        res[k].converged = true;
+        frozen[k] = 1;
+        --active;
+        freeze_column(h, k);
+      }
+      if (active == 0) return res;
+      continue;
+    }
     schur_apply(h, x, h->vq, st, nb);                                 // true residuals g - S x
     ck(cudaMemcpyAsync(h->vrold, g, sizeof(double) * n * nb, cudaMemcpyDeviceToDevice, st), "copy");
     launch_axpy_loc(h->vrold, h->vq, -1.0, n * nb, st);
@@ -2386,6 +2430,30 @@ PcgResult fgmres(bddc_handle_s* h, const double* g, double* x, double tol, int m
   return res;
 }
 
+// Storage for the directions of a refined solve: up to 128 per column and 4 GB per handle, allocated by the
+// first refined solve (and again by the first block of right-hand sides); iterations past the capacity are
+// not stored.
+void prepare_kstore(bddc_handle_s* h, int nb) {
+  if (h->kstore.cap > 0 && h->kstore_blk >= nb) return;
+  ck(cudaStreamSynchronize(h->st), "sync");
+  drop_graph(h);   // a cached iteration refers to the old storage
+  DevArena& A = h->arena;
+  if (h->kstore.cap > 0) {
+    A.free_one(h->kstore.p);
+    A.free_one(h->kstore.q);
+  }
+  const int blk = h->blk;
+  const int64_t n = std::max<int64_t>(h->lv[0].d.n_iface, 1);
+  const int cap = (int)std::max<int64_t>(1, std::min<int64_t>(128, ((int64_t)4 << 30) / (8 * n * blk)));
+  h->kstore.p = A.alloc<float>(n * cap * blk);
+  h->kstore.q = A.alloc<float>(n * cap * blk);
+  h->kstore.d = A.alloc<double>((int64_t)cap * blk);
+  h->kstore.cnt = A.alloc<int>(kMaxBlock);
+  h->kstore.cap = cap;
+  h->kstore_blk = blk;
+  h->proj_coef = A.alloc<double>((int64_t)blk * cap * (kProjBlocks + 1));
+}
+
 // Mixed-precision iterative refinement around PCG (the outer iteration that restores FP64
 // accuracy), for a block of nb right-hand sides: x += S~^{-1} r with r = g - S x, where S is the
 // FP64 Schur operator (interior solves refined to FP64 accuracy) and S~ the same operator with
@@ -2394,7 +2462,10 @@ PcgResult fgmres(bddc_handle_s* h, const double* g, double* x, double tol, int m
 // below what the outer tolerance needs), starting from opts.inner_tol and adapted per column to its
 // observed outer reduction within the solve (so repeated solves are bitwise identical); an outer
 // step that fails to halve some column's residual switches the inner operator to the FP64 one.
-// Columns that meet the tolerance get a zero outer residual, so the inner PCG leaves them alone.
+// Columns that meet the tolerance get a zero outer residual, so the inner PCG leaves them alone.  Restarting
+// CG at every outer step lost its Krylov space (48^3, tol 1e-10: 96 iterations where one CG needs about 60);
+// each inner solve after the first starts from the Galerkin projection of its residual on the directions of
+// the earlier ones (S~ p is at hand as q), which takes the slow modes out (76 iterations).
 // The solution is left in h->vs; h->vt holds the outer residual.
 std::vector<PcgResult> pcg_refined(bddc_handle_s* h, const double* g, double tol, int maxit, int nb) {
   constexpr int kMaxOuter = 40;
@@ -2433,6 +2504,9 @@ std::vector<PcgResult> pcg_refined(bddc_handle_s* h, const double* g, double tol
                       tin(nb, 1.0);
   int inner = h->inner_steps;
   int its = 0;
+  prepare_kstore(h, nb);
+  ck(cudaMemsetAsync(h->kstore.cnt, 0, sizeof(int) * kMaxBlock, st), "memset");
+  bool stored = false;   // directions of the present inner operator
   for (int outer = 0; outer < kMaxOuter && its < maxit && left > 0; ++outer) {
     for (int k = 0; k < nb; ++k) {
       if (done[k]) {
@@ -2443,7 +2517,8 @@ std::vector<PcgResult> pcg_refined(bddc_handle_s* h, const double* g, double tol
       }
     }
     h->cur_steps = inner;
-    std::vector<PcgResult> in = pcg(h, ro, h->vx, tin, maxit - its, nb);
+    std::vector<PcgResult> in = pcg(h, ro, h->vx, tin, maxit - its, nb, true, stored);
+    stored = true;
     h->cur_steps = h->refine_steps;
     h->ext_of = nullptr;
     int most = 0;
@@ -2487,7 +2562,11 @@ std::vector<PcgResult> pcg_refined(bddc_handle_s* h, const double* g, double tol
         eta[k] = std::max(1e-4, 0.5 * eta[k]);
       rnorm[k] = rn[k];
     }
-    if (stagnated) inner = h->refine_steps;
+    if (stagnated && inner != h->refine_steps) {   // another operator: its own directions from here on
+      inner = h->refine_steps;
+      ck(cudaMemsetAsync(h->kstore.cnt, 0, sizeof(int) * kMaxBlock, st), "memset");
+      stored = false;
+    }
   }
   return res;
 }

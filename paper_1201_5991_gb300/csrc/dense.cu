@@ -1101,11 +1101,12 @@ __global__ void __launch_bounds__(256) k_coarse_inverse(LevelDev L, float* __res
   }
 }
 
-// y = W x for nr columns (x, y: columns of n_vec, padded local positions 0 .. npad-1); one warp
+// z = W x for nr columns (x: columns of n_vec, padded local positions 0 .. npad-1; z: level DOFs); one warp
 // per output row, lanes along the row (coalesced), FP32 sums in a fixed order.
 template <int NR>
 __global__ void k_coarse_apply(const float* __restrict__ W, int64_t npad, const float* __restrict__ x,
-                               float* __restrict__ y, int64_t n_vec) {
+                               double* __restrict__ z, const int32_t* __restrict__ loc2glob, int64_t n_vec,
+                               int64_t n_dof) {
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= npad) return;
@@ -1123,7 +1124,8 @@ __global__ void k_coarse_apply(const float* __restrict__ W, int64_t npad, const 
     }
   }
   lane_sums<NR>(acc, lane);
-  if (lane_sum_writer<NR>(lane)) y[(c0 + lane_sum_index<NR>(lane)) * n_vec + row] = acc[0];
+  const int32_t g = loc2glob[row];
+  if (lane_sum_writer<NR>(lane) && g >= 0) z[(c0 + lane_sum_index<NR>(lane)) * n_dof + g] = (double)acc[0];
 }
 
 }  // namespace
@@ -1137,8 +1139,8 @@ void launch_coarse_inverse(const LevelDev& L, int64_t npad, float* W, cudaStream
     k_coarse_inverse<64><<<(unsigned)((npad + 63) / 64), 256, 0, st>>>(L, W);
 }
 
-void launch_coarse_apply(const float* W, int64_t npad, const float* x, float* y, int64_t n_vec, int nr,
-                         cudaStream_t st) {
+void launch_coarse_apply(const float* W, int64_t npad, const float* x, double* z, const int32_t* loc2glob,
+                         int64_t n_vec, int64_t n_dof, int nr, cudaStream_t st) {
   if (npad <= 0 || nr <= 0) return;
   const unsigned gx = (unsigned)((npad + 7) / 8);
   for (int r0 = 0; r0 < nr;) {
@@ -1146,16 +1148,16 @@ void launch_coarse_apply(const float* W, int64_t npad, const float* x, float* y,
     const int g = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
     const int ng = left / g;
     const float* xs = x + (int64_t)r0 * n_vec;
-    float* ys = y + (int64_t)r0 * n_vec;
+    double* zs = z + (int64_t)r0 * n_dof;
     note_launch();
     if (g == 8)
-      k_coarse_apply<8><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, ys, n_vec);
+      k_coarse_apply<8><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, zs, loc2glob, n_vec, n_dof);
     else if (g == 4)
-      k_coarse_apply<4><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, ys, n_vec);
+      k_coarse_apply<4><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, zs, loc2glob, n_vec, n_dof);
     else if (g == 2)
-      k_coarse_apply<2><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, ys, n_vec);
+      k_coarse_apply<2><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, zs, loc2glob, n_vec, n_dof);
     else
-      k_coarse_apply<1><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, ys, n_vec);
+      k_coarse_apply<1><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, zs, loc2glob, n_vec, n_dof);
     r0 += ng * g;
   }
 }
@@ -1281,13 +1283,10 @@ void launch_constraint_corr(const LevelDev& L, T* vec, const int32_t* crow_sub, 
 }
 
 template <typename T>
-void launch_psi_t_apply(const LevelDev& L, const T* vec, double* part, int64_t sum_nc, double* rc_sub, int max_nGb,
-                        int max_ncb, cudaStream_t st, int nr) {
+void launch_psi_t_apply(const LevelDev& L, const T* vec, double* part, int64_t sum_nc, int max_nGb, int max_ncb,
+                        cudaStream_t st, int nr) {
   if (sum_nc <= 0 || max_nGb <= 0) return;
   rows_matvec<T, 1>(L, vec, part, sum_nc, max_nGb, max_ncb, st, nr);
-  const int zmax = rows_zmax(max_nGb);
-  note_launch();
-  k_sum_parts<<<dim3((unsigned)((sum_nc + 255) / 256), (unsigned)nr), 256, 0, st>>>(part, zmax, sum_nc, rc_sub);
 }
 
 template <typename T>
@@ -1323,8 +1322,7 @@ void launch_psi_transpose(const LevelDev& L, int max_nGb, int max_ncb, cudaStrea
   template void launch_psi<T>(const LevelDev&, int, int, cudaStream_t);                          \
   template void launch_constraint_corr<T>(const LevelDev&, T*, const int32_t*, int64_t, double*, double*, double*, \
                                          int, int, cudaStream_t, int);                                     \
-  template void launch_psi_t_apply<T>(const LevelDev&, const T*, double*, int64_t, double*, int, int, cudaStream_t, \
-                                      int);                                                              \
+  template void launch_psi_t_apply<T>(const LevelDev&, const T*, double*, int64_t, int, int, cudaStream_t, int);   \
   template void launch_psi_apply_add<T>(const LevelDev&, const double*, int64_t, T*, int, int, cudaStream_t, int); \
   template void launch_psi_transpose<T>(const LevelDev&, int, int, cudaStream_t);
 INST(float)

@@ -110,6 +110,8 @@ struct LevelDev {
   void* psiT;                     // Psi_G^T in tiles: tile (rb, j) of a subdomain at psiT_off + (rb nGb + j) NB2
   float* schur;                   // explicit augmented Schur complement of the interface (mixed inner operator), or null
   void* sgn;                      // [n_vec] pivot signs of the signed Cholesky (T; +1 for SPD levels)
+  int32_t* crow;                  // [n_vec] constraint row of a position (flat over the level) or -1 (level 1, FP32), or null
+  double* cval;                   // [n_vec] its entry
   const double* c_rho;            // [sum nc] 1 where a constraint row is augmented by rho, else 0
   int indefinite;                 // 1: negative pivots allowed (Stokes), 0: SPD
   int wait_probe;                 // test only: sweeps poll status[3] (never set) instead of the published solution blocks
@@ -220,8 +222,9 @@ void launch_psi(const LevelDev& L, int max_nGb, int max_nc, cudaStream_t st);
 // level's FP32 copy), npad x npad stored column after column; and y = W x for nr columns of n_vec
 // (padded local positions).
 void launch_coarse_inverse(const LevelDev& L, int64_t npad, float* W, cudaStream_t st);
-void launch_coarse_apply(const float* W, int64_t npad, const float* x, float* y, int64_t n_vec, int nr,
-                         cudaStream_t st);
+// the product writes z[loc2glob[row]] (columns of n_dof)
+void launch_coarse_apply(const float* W, int64_t npad, const float* x, double* z, const int32_t* loc2glob,
+                         int64_t n_vec, int64_t n_dof, int nr, cudaStream_t st);
 // sweep.cu: forward (backward = 0) or backward triangular sweep over part 0 (interior
 // block rows) or part 1 (interface block rows) of every subdomain; ctrl is the task counter and
 // pub a publication buffer of n_vec x min(nr, 8) words of T (both reset by the launch).
@@ -240,9 +243,10 @@ void launch_constraint_corr(const LevelDev& L, T* vec, const int32_t* crow_sub, 
 // those tiles once per group of up to 8 right-hand sides: row products t = M v over chunks of 4
 // tile columns (partial sums part[(c_off + p) * zmax + z], zmax = ceil(max_nGb / 4), summed in a
 // fixed order), column products v += M^T z one CTA per interface tile column.
+// parts only: launch_coarse_gather adds them
 template <typename T>
-void launch_psi_t_apply(const LevelDev& L, const T* vec, double* part, int64_t sum_nc, double* rc_sub,
-                        int max_nGb, int max_ncb, cudaStream_t st, int nr = 1);
+void launch_psi_t_apply(const LevelDev& L, const T* vec, double* part, int64_t sum_nc, int max_nGb, int max_ncb,
+                        cudaStream_t st, int nr = 1);
 template <typename T>
 void launch_psi_apply_add(const LevelDev& L, const double* zc_sub, int64_t sum_nc, T* vec, int max_nGb,
                           int max_ncb, cudaStream_t st, int nr = 1);
@@ -256,10 +260,44 @@ void launch_psi_transpose(const LevelDev& L, int max_nGb, int max_ncb, cudaStrea
 inline int rows_zmax(int max_nGb) { return (max_nGb + 3) / 4; }
 
 // ---------------------------------------------------------------- vectors (vector.cu)
+// Sums over the interface fused into the kernel that makes their factors (PCG, one pass instead of three
+// launches): per block, then by the last block of every column in block order, which also takes the
+// recurrence's scalar step.  partial: 2 nr iface_blocks doubles; cnt: nr counters, zero before and after.
+struct FusedDot {
+  int mode = 0;              // 0: none; 1: p . y and alpha; 2: r . y and q . y and beta
+  int flexible = 0;          // mode 2: Polak-Ribiere beta, z . (r - r_old) = -alpha z . q
+  const double* a = nullptr; // p, or r
+  const double* b = nullptr; // q (mode 2)
+  double* scal = nullptr;    // [16 nr]
+  double* partial = nullptr;
+  int* cnt = nullptr;
+};
+// Directions p and their images q of the inner PCG, FP32, kept over the outer steps of one solve: column k's
+// vector v at p + (k cap + v) n, its p . q in d, their number in cnt[k] (device; appended by the update of x and
+// r, none past cap).  The next inner solve of the same operator starts from the Galerkin projection of its
+// residual on them.
+struct KrylovStore {
+  float* p = nullptr;
+  float* q = nullptr;
+  double* d = nullptr;
+  int* cnt = nullptr;
+  int cap = 0;
+};
+inline int64_t iface_blocks(int64_t n_iface) { return (n_iface + 255) / 256; }
+
 template <typename T>
 void launch_gather_iface(const LevelDev& L, const double* x, int weighted, T* loc, cudaStream_t st, int nr = 1);
 template <typename T>
-void launch_scatter_iface(const LevelDev& L, const T* loc, int weighted, double* y, cudaStream_t st, int nr = 1);
+void launch_scatter_iface(const LevelDev& L, const T* loc, int weighted, double* y, cudaStream_t st, int nr = 1,
+                          const FusedDot& dot = FusedDot());
+// inner operator around its FP32 product: loc = R_i x (FP32) and t = R C_i R_i x per constraint row; then
+// y = sum R_i^T (loc - C_i^T t) with the constraint row and entry of every position (crow, cval)
+void launch_inner_gather(const LevelDev& L, const double* x, float* loc, const int32_t* crow_sub, int64_t total_rows,
+                         double* t, cudaStream_t st, int nr = 1);
+void launch_inner_scatter(const LevelDev& L, const float* loc, const double* t, int64_t total_rows, double* y,
+                          cudaStream_t st, int nr, const FusedDot& dot);
+// crow / cval of every padded position from the constraint rows (set-up)
+void launch_constraint_positions(const LevelDev& L, const int32_t* crow_sub, int64_t total_rows, cudaStream_t st);
 template <typename T>
 void launch_gather_glob(const LevelDev& L, const double* x, int part, T* loc, cudaStream_t st, int nr = 1);
 template <typename T>
@@ -275,18 +313,26 @@ void launch_convert(const Tin* in, Tout* out, int64_t n, cudaStream_t st);
 void launch_axpy_loc(double* y, const double* x, double a, int64_t n, cudaStream_t st);
 template <typename T>
 void launch_add_to_double(double* y, const T* x, int64_t n, cudaStream_t st);
-void launch_coarse_gather(const LevelDev& L, const double* rc_sub, int64_t sum_nc, double* rC, cudaStream_t st,
-                          int nr = 1);
+// r_C = sum R_Ci^T t_i with t_i = Psi_i^T r_i summed from its parts (part[(.) zmax + z], see launch_psi_t_apply)
+// and kept at rc_sub; v32 (or null): also as the FP32 input of the explicit coarsest inverse, position
+// v32_pos[g] of columns of n_v32
+void launch_coarse_gather(const LevelDev& L, const double* part, int zmax, double* rc_sub, int64_t sum_nc, double* rC,
+                          float* v32, const int32_t* v32_pos, int64_t n_v32, cudaStream_t st, int nr = 1);
 void launch_coarse_scatter_n(const int32_t* sub_coarse, int64_t total, const double* zC, int64_t n_coarse,
                              double* zc_sub, cudaStream_t st, int nr = 1);
 // nr dot products of the columns of a and b (length n each): out[k * ostride], partial [nr][nblk]
 void launch_dot(const double* a, const double* b, int64_t n, double* partial, int nblk, double* out,
                 cudaStream_t st, int nr = 1, int ostride = 16);
-// PCG of a block of right-hand sides: column k keeps its scalars at scal[16 k ..]
-void launch_pcg_update_x_r(double* x, double* r, const double* p, const double* q, const double* scal,
-                           int64_t n, cudaStream_t st, int nr = 1);
+// PCG of a block of right-hand sides: column k keeps its scalars at scal[16 k ..].  The update of x and r
+// also makes r . r (scal[16 k + 5]); partial, cnt as in FusedDot.
+void launch_pcg_update_x_r(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
+                           double* partial, int* cnt, const KrylovStore& ks, cudaStream_t st, int nr = 1);
+// x = sum_v c_v p_v, r = g - sum_v c_v q_v with c_v = (p_v . g) / d_v over the stored directions (coef: scratch,
+// [nr][cap][kProjBlocks + 1])
+constexpr int kProjBlocks = 32;
+void launch_project(const KrylovStore& ks, const double* g, double* x, double* r, int64_t n, double* coef,
+                    cudaStream_t st, int nr);
 void launch_pcg_update_p(double* p, const double* z, const double* scal, int64_t n, cudaStream_t st, int nr = 1);
-void launch_pcg_scalars(double* scal, int stage, int flexible, cudaStream_t st, int nr = 1);
 // conn: element -> nodes (ne / ndof per element); the full DOF of element slot a is
 // conn[a / ndof] * ndof + a % ndof
 void launch_grad_contract_slots(int64_t n_elems, int ne, const double* ke, const int32_t* slot_elem,
@@ -317,8 +363,6 @@ void launch_schur_symv(const LevelDev& L, int inverse, int max_nGb, const int64_
                        const float* x, float* part, float* y, cudaStream_t st, int nr = 1);
 void launch_trmv_schur(const LevelDev& L, int max_nGb, const float* x, float* y1, float* y, cudaStream_t st,
                        int nr = 1);
-void launch_sub_ctrc(const LevelDev& L, const int32_t* crow_sub, int64_t total_rows, const double* x, double* y,
-                     cudaStream_t st, int nr = 1);
 // flexible GMRES (vector.cu): out[i] = V_i . w (i < nv, partial holds nv * nblk doubles);
 // w += alpha sum_i c_i V_i; dst = src / sqrt(*nrm2)
 void launch_multidot(const double* V, int64_t ldv, int nv, const double* w, int64_t n, double* partial, int nblk,

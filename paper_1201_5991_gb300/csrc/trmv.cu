@@ -119,28 +119,6 @@ __global__ void __launch_bounds__(256) k_trmv_n(LevelDev L, const float* __restr
     }
 }
 
-// y -= C^T R C x over the padded local interface vectors (FP64); one warp per constraint row.
-// Distinct rows touch disjoint positions (each local DOF lies in one glob and has one
-// component), so the update needs no atomics.
-__global__ void k_sub_ctrc(LevelDev L, const int32_t* __restrict__ crow_sub, int64_t total_rows,
-                           const double* __restrict__ x, double* __restrict__ y) {
-  const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (g >= total_rows) return;
-  x += (int64_t)blockIdx.y * L.n_vec;   // column blockIdx.y of a block of right-hand sides
-  y += (int64_t)blockIdx.y * L.n_vec;
-  const int s = crow_sub[g];
-  const SubMeta m = L.meta[s];
-  const double rq = L.rho[s] * L.c_rho[g];
-  if (rq == 0.0) return;
-  const int64_t a = L.c_ptr[g], b = L.c_ptr[g + 1];
-  double t = 0.0;
-  for (int64_t e = a + lane; e < b; e += 32) t += L.c_val[e] * x[m.vec_off + L.c_pos[e]];
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-  for (int64_t e = a + lane; e < b; e += 32) y[m.vec_off + L.c_pos[e]] -= rq * t * L.c_val[e];
-}
-
 // ---- explicit augmented Schur complement (snapshot of the trailing interface block) ----------
 
 // tile (i, j), 0 <= j <= i < nGb, of a subdomain's explicit Schur complement
@@ -440,13 +418,6 @@ void launch_trmv_schur(const LevelDev& L, int max_nGb, const float* x, float* y1
       launch_trmv_nr<1>(L, grid, x + off, y1 + off, y + off, st);
     r0 += ng * g;
   }
-}
-
-void launch_sub_ctrc(const LevelDev& L, const int32_t* crow_sub, int64_t total_rows, const double* x, double* y,
-                     cudaStream_t st, int nr) {
-  if (total_rows <= 0) return;
-  note_launch();
-  k_sub_ctrc<<<dim3((unsigned)((total_rows + 7) / 8), nr), 256, 0, st>>>(L, crow_sub, total_rows, x, y);
 }
 
 }  // namespace bddc

@@ -26,18 +26,154 @@ __global__ void k_gather_iface(LevelDev L, const double* __restrict__ x, int wei
   loc[p] = (T)v;
 }
 
-template <typename T>
-__global__ void k_scatter_iface(LevelDev L, const T* __restrict__ loc, int weighted, double* __restrict__ y) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= L.n_iface) return;
-  loc += (int64_t)blockIdx.y * L.n_vec;
-  y += (int64_t)blockIdx.y * L.n_iface;
-  double s = 0.0;
-  for (int64_t o = L.iface_ptr[g]; o < L.iface_ptr[g + 1]; ++o) {
-    const int64_t p = L.iface_occ[o];
-    s += weighted ? L.w[p] * (double)loc[p] : (double)loc[p];
+// Sum v0 (and v1) over the block, then over the blocks of column blockIdx.y: every block writes its partial
+// sums, the last one to finish adds them in block order.  True in that block (all threads), totals in s0, s1.
+__device__ bool sum_over_grid(double v0, double v1, bool two, double* __restrict__ partial, int* cnt, double& s0,
+                              double& s1) {
+  __shared__ double red[2][8];
+  __shared__ int last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto block_sum = [&](double a, double b) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (two) b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (lane == 0) {
+      red[0][warp] = a;
+      red[1][warp] = b;
+    }
+    __syncthreads();
+    s0 = s1 = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      s0 += red[0][w];
+      if (two) s1 += red[1][w];
+    }
+    __syncthreads();
+  };
+  block_sum(v0, v1);
+  const int nb = gridDim.x;
+  double* p0 = partial + (int64_t)blockIdx.y * 2 * nb;
+  if (threadIdx.x == 0) {
+    p0[blockIdx.x] = s0;
+    if (two) p0[nb + blockIdx.x] = s1;
+    __threadfence();
+    last = atomicAdd(cnt + blockIdx.y, 1) == nb - 1;
   }
-  y[g] = s;
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  double a = 0.0, b = 0.0;
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) {
+    a += __ldcg(p0 + i);
+    if (two) b += __ldcg(p0 + nb + i);
+  }
+  block_sum(a, b);
+  if (threadIdx.x == 0) cnt[blockIdx.y] = 0;
+  return true;
+}
+
+// scal layout (see capi.cpp): 0 rz, 1 pq, 2 alpha, 3 beta, 4 rz_new, 5 rr, 6 gg, 8 frozen.  The scalar step of
+// the recurrence that follows the sums (one thread); frozen columns keep alpha = beta = 0.
+__device__ void pcg_step(const FusedDot& dot, double s0, double s1) {
+  double* S = dot.scal + 16 * blockIdx.y;
+  const bool frozen = S[8] != 0.0;
+  if (dot.mode == 1) {
+    S[1] = s0;
+    S[2] = !frozen && s0 != 0.0 ? S[0] / s0 : 0.0;
+  } else {
+    S[4] = s0;
+    const double num = dot.flexible ? -S[2] * s1 : s0;   // z . (r - r_old) = -alpha z . q
+    S[3] = !frozen && S[0] != 0.0 ? num / S[0] : 0.0;
+    if (!frozen) S[0] = s0;
+  }
+}
+
+// the sums of a fused scatter over its outputs y[g] and the scalar step
+__device__ void fused_dot(const FusedDot& dot, int64_t g, int64_t n, double y) {
+  double v0 = 0.0, v1 = 0.0, s0, s1;
+  if (g < n) {
+    const int64_t o = (int64_t)blockIdx.y * n + g;
+    v0 = dot.a[o] * y;
+    if (dot.mode == 2) v1 = dot.b[o] * y;
+  }
+  if (sum_over_grid(v0, v1, dot.mode == 2, dot.partial, dot.cnt, s0, s1) && threadIdx.x == 0) pcg_step(dot, s0, s1);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_scatter_iface(LevelDev L, const T* __restrict__ loc, int weighted,
+                                                       double* __restrict__ y, FusedDot dot) {
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  double s = 0.0;
+  if (g < L.n_iface) {
+    loc += (int64_t)blockIdx.y * L.n_vec;
+    for (int64_t o = L.iface_ptr[g]; o < L.iface_ptr[g + 1]; ++o) {
+      const int64_t p = L.iface_occ[o];
+      s += weighted ? L.w[p] * (double)loc[p] : (double)loc[p];
+    }
+    y[(int64_t)blockIdx.y * L.n_iface + g] = s;
+  }
+  if (dot.mode) fused_dot(dot, g, L.n_iface, s);
+}
+
+// inner operator, before its FP32 product: blocks below nv gather loc = R_i x, the others take one
+// constraint row per warp: t = rho c_rho (C_i R_i x)
+__global__ void __launch_bounds__(256) k_inner_gather(LevelDev L, const double* __restrict__ x, float* __restrict__ loc,
+                                                      int nv, const int32_t* __restrict__ crow_sub, int64_t total_rows,
+                                                      double* __restrict__ t) {
+  x += (int64_t)blockIdx.y * L.n_iface;
+  if ((int)blockIdx.x < nv) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= L.n_vec) return;
+    const int32_t g = L.loc2iface[p];
+    loc[(int64_t)blockIdx.y * L.n_vec + p] = g >= 0 ? (float)x[g] : 0.f;
+    return;
+  }
+  const int64_t r = (int64_t)(blockIdx.x - nv) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (r >= total_rows) return;
+  const int s = crow_sub[r];
+  const double rq = L.rho[s] * L.c_rho[r];
+  const int32_t* l2i = L.loc2iface + L.meta[s].vec_off;
+  double acc = 0.0;
+  if (rq != 0.0)
+    for (int64_t e = L.c_ptr[r] + lane; e < L.c_ptr[r + 1]; e += 32) acc += L.c_val[e] * x[l2i[L.c_pos[e]]];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) t[(int64_t)blockIdx.y * total_rows + r] = rq * acc;
+}
+
+// y = sum R_i^T (loc - C_i^T t): distinct constraint rows touch disjoint positions (each local DOF lies in
+// one glob and has one component)
+__global__ void __launch_bounds__(256) k_inner_scatter(LevelDev L, const float* __restrict__ loc,
+                                                       const double* __restrict__ t, int64_t total_rows,
+                                                       double* __restrict__ y, FusedDot dot) {
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  double s = 0.0;
+  if (g < L.n_iface) {
+    loc += (int64_t)blockIdx.y * L.n_vec;
+    t += (int64_t)blockIdx.y * total_rows;
+    for (int64_t o = L.iface_ptr[g]; o < L.iface_ptr[g + 1]; ++o) {
+      const int64_t p = L.iface_occ[o];
+      double v = (double)loc[p];
+      const int32_t r = L.crow[p];
+      if (r >= 0) v -= t[r] * L.cval[p];
+      s += v;
+    }
+    y[(int64_t)blockIdx.y * L.n_iface + g] = s;
+  }
+  if (dot.mode) fused_dot(dot, g, L.n_iface, s);
+}
+
+__global__ void k_constraint_positions(LevelDev L, const int32_t* __restrict__ crow_sub, int64_t total_rows) {
+  const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (r >= total_rows) return;
+  const int64_t off = L.meta[crow_sub[r]].vec_off;
+  for (int64_t e = L.c_ptr[r] + lane; e < L.c_ptr[r + 1]; e += 32) {
+    L.crow[off + L.c_pos[e]] = (int32_t)r;
+    L.cval[off + L.c_pos[e]] = L.c_val[e];
+  }
 }
 
 // part: 0 interior positions only, 1 interface only, 2 all
@@ -120,13 +256,35 @@ __global__ void k_axpy(double* __restrict__ y, const double* __restrict__ x, dou
   if (i < n) y[i] += a * x[i];
 }
 
-__global__ void k_coarse_gather(LevelDev L, const double* __restrict__ rc_sub, int64_t sum_nc, double* __restrict__ rC) {
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per coarse DOF, which owns its per-subdomain rows: 4 rows at a time, 8 lanes along each row's parts
+// (a thread per DOF summed up to 120 parts in a chain of loads).
+__global__ void k_coarse_gather(LevelDev L, const double* __restrict__ part, int zmax, double* __restrict__ rc_sub,
+                                int64_t sum_nc, double* __restrict__ rC, float* __restrict__ v32,
+                                const int32_t* __restrict__ v32_pos, int64_t n_v32) {
+  const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
   if (g >= L.n_coarse) return;
+  part += (int64_t)blockIdx.y * sum_nc * zmax;
   rc_sub += (int64_t)blockIdx.y * sum_nc;
+  const int64_t o1 = L.cinv_ptr[g + 1];
   double s = 0.0;
-  for (int64_t o = L.cinv_ptr[g]; o < L.cinv_ptr[g + 1]; ++o) s += rc_sub[L.cinv_occ[o]];
-  rC[(int64_t)blockIdx.y * L.n_coarse + g] = s;
+  for (int64_t o0 = L.cinv_ptr[g]; o0 < o1; o0 += 4) {
+    const int64_t o = o0 + (lane >> 3);
+    const int64_t r = o < o1 ? L.cinv_occ[o] : -1;
+    double t = 0.0;
+    if (r >= 0)
+      for (int z = lane & 7; z < zmax; z += 8) t += part[r * zmax + z];
+#pragma unroll
+    for (int h = 4; h > 0; h >>= 1) t += __shfl_xor_sync(0xffffffffu, t, h);
+    if (r >= 0 && (lane & 7) == 0) rc_sub[r] = t;
+    t += __shfl_xor_sync(0xffffffffu, t, 8);
+    t += __shfl_xor_sync(0xffffffffu, t, 16);
+    s += t;
+  }
+  if (lane == 0) {
+    rC[(int64_t)blockIdx.y * L.n_coarse + g] = s;
+    if (v32) v32[(int64_t)blockIdx.y * n_v32 + v32_pos[g]] = (float)s;
+  }
 }
 
 __global__ void k_coarse_scatter(const int32_t* __restrict__ sub_coarse, int64_t total, const double* __restrict__ zC,
@@ -169,34 +327,86 @@ __global__ void k_dot_final(const double* __restrict__ partial, int nblk, double
   if (threadIdx.x == 0) *out = red[0];
 }
 
-// scal layout (see capi.cpp): 0 rz, 1 pq, 2 alpha, 3 beta, 4 rz_new, 5 rr, 6 gg, 7 z.r_old, 8 frozen
-__global__ void k_pcg_scalars(double* scal, int stage, int flexible, int nr) {
-  if ((int)threadIdx.x >= nr) return;
-  scal += 16 * threadIdx.x;   // column threadIdx.x of a block of right-hand sides
-  if (scal[8] != 0.0) {   // converged column: freeze the iterate
-    scal[2] = 0.0;
-    scal[3] = 0.0;
-    return;
+__global__ void __launch_bounds__(256) k_pcg_xr(double* __restrict__ x, double* __restrict__ r,
+                                                const double* __restrict__ p, const double* __restrict__ q,
+                                                double* __restrict__ scal, int64_t n, double* __restrict__ partial,
+                                                int* cnt, KrylovStore ks) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  double rr = 0.0, s0, s1;
+  const double a = scal[16 * blockIdx.y + 2];
+  const int slot = ks.cap > 0 && a != 0.0 ? ks.cnt[blockIdx.y] : ks.cap;
+  if (i < n) {
+    const int64_t o = (int64_t)blockIdx.y * n + i;
+    const double pv = p[o], qv = q[o];
+    x[o] += a * pv;
+    const double v = r[o] - a * qv;
+    r[o] = v;
+    rr = v * v;
+    if (slot < ks.cap) {
+      const int64_t k = ((int64_t)blockIdx.y * ks.cap + slot) * n + i;
+      ks.p[k] = (float)pv;
+      ks.q[k] = (float)qv;
+    }
   }
-  if (stage == 0) {
-    const double pq = scal[1];
-    scal[2] = pq != 0.0 ? scal[0] / pq : 0.0;
-  } else {
-    const double rz_old = scal[0];
-    const double num = flexible ? (scal[4] - scal[7]) : scal[4];
-    scal[3] = rz_old != 0.0 ? num / rz_old : 0.0;
-    scal[0] = scal[4];
+  if (sum_over_grid(rr, 0.0, false, partial, cnt, s0, s1) && threadIdx.x == 0) {
+    scal[16 * blockIdx.y + 5] = s0;
+    if (slot < ks.cap) {   // every block has read its count (this one is the last)
+      ks.d[(int64_t)blockIdx.y * ks.cap + slot] = scal[16 * blockIdx.y + 1];
+      ks.cnt[blockIdx.y] = slot + 1;
+    }
   }
 }
 
-__global__ void k_pcg_xr(double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
-                         const double* __restrict__ q, const double* __restrict__ scal, int64_t n) {
+// coef[(k cap + v)(kProjBlocks + 1) + b] = slice b of p_v . g of column k
+__global__ void __launch_bounds__(256) k_project_dot(KrylovStore ks, const double* __restrict__ g, int64_t n,
+                                                     double* __restrict__ coef) {
+  const int v = blockIdx.y, k = blockIdx.z;
+  if (v >= ks.cnt[k]) return;
+  __shared__ double red[8];
+  const float* p = ks.p + ((int64_t)k * ks.cap + v) * n;
+  g += (int64_t)k * n;
+  double s = 0.0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    s += (double)p[i] * g[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) s += red[w];
+    coef[((int64_t)k * ks.cap + v) * (kProjBlocks + 1) + blockIdx.x] = s;
+  }
+}
+
+// c_v into slot kProjBlocks of its row; one thread per (v, column)
+__global__ void k_project_coef(KrylovStore ks, double* __restrict__ coef) {
+  const int v = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y;
+  if (v >= ks.cnt[k]) return;
+  double* c = coef + ((int64_t)k * ks.cap + v) * (kProjBlocks + 1);
+  double s = 0.0;
+  for (int b = 0; b < kProjBlocks; ++b) s += c[b];
+  const double d = ks.d[(int64_t)k * ks.cap + v];
+  c[kProjBlocks] = d > 0.0 ? s / d : 0.0;
+}
+
+__global__ void __launch_bounds__(256) k_project_apply(KrylovStore ks, const double* __restrict__ g,
+                                                       double* __restrict__ x, double* __restrict__ r, int64_t n,
+                                                       const double* __restrict__ coef) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int k = blockIdx.y, m = ks.cnt[k];
   if (i >= n) return;
-  const int64_t o = (int64_t)blockIdx.y * n;
-  const double a = scal[16 * blockIdx.y + 2];
-  x[o + i] += a * p[o + i];
-  r[o + i] -= a * q[o + i];
+  const float* p = ks.p + (int64_t)k * ks.cap * n + i;
+  const float* q = ks.q + (int64_t)k * ks.cap * n + i;
+  const double* c = coef + (int64_t)k * ks.cap * (kProjBlocks + 1) + kProjBlocks;
+  double xs = 0.0, rs = g[(int64_t)k * n + i];
+#pragma unroll 4
+  for (int v = 0; v < m; ++v) {
+    const double cv = c[(int64_t)v * (kProjBlocks + 1)];
+    xs += cv * (double)p[(int64_t)v * n];
+    rs -= cv * (double)q[(int64_t)v * n];
+  }
+  x[(int64_t)k * n + i] = xs;
+  r[(int64_t)k * n + i] = rs;
 }
 
 __global__ void k_pcg_p(double* __restrict__ p, const double* __restrict__ z, const double* __restrict__ scal,
@@ -368,8 +578,25 @@ void launch_gather_iface(const LevelDev& L, const double* x, int weighted, T* lo
   if (L.n_vec > 0) { note_launch(); k_gather_iface<T><<<dim3(nblocks(L.n_vec, 256), nr), 256, 0, st>>>(L, x, weighted, loc); }
 }
 template <typename T>
-void launch_scatter_iface(const LevelDev& L, const T* loc, int weighted, double* y, cudaStream_t st, int nr) {
-  if (L.n_iface > 0) { note_launch(); k_scatter_iface<T><<<dim3(nblocks(L.n_iface, 256), nr), 256, 0, st>>>(L, loc, weighted, y); }
+void launch_scatter_iface(const LevelDev& L, const T* loc, int weighted, double* y, cudaStream_t st, int nr,
+                          const FusedDot& dot) {
+  if (L.n_iface > 0) { note_launch(); k_scatter_iface<T><<<dim3(nblocks(L.n_iface, 256), nr), 256, 0, st>>>(L, loc, weighted, y, dot); }
+}
+void launch_inner_gather(const LevelDev& L, const double* x, float* loc, const int32_t* crow_sub, int64_t total_rows,
+                         double* t, cudaStream_t st, int nr) {
+  if (L.n_vec <= 0) return;
+  const unsigned nv = nblocks(L.n_vec, 256);
+  note_launch();
+  k_inner_gather<<<dim3(nv + nblocks(total_rows, 8), nr), 256, 0, st>>>(L, x, loc, (int)nv, crow_sub, total_rows, t);
+}
+void launch_inner_scatter(const LevelDev& L, const float* loc, const double* t, int64_t total_rows, double* y,
+                          cudaStream_t st, int nr, const FusedDot& dot) {
+  if (L.n_iface <= 0) return;
+  note_launch();
+  k_inner_scatter<<<dim3(nblocks(L.n_iface, 256), nr), 256, 0, st>>>(L, loc, t, total_rows, y, dot);
+}
+void launch_constraint_positions(const LevelDev& L, const int32_t* crow_sub, int64_t total_rows, cudaStream_t st) {
+  if (total_rows > 0) { note_launch(); k_constraint_positions<<<nblocks(total_rows, 8), 256, 0, st>>>(L, crow_sub, total_rows); }
 }
 template <typename T>
 void launch_gather_glob(const LevelDev& L, const double* x, int part, T* loc, cudaStream_t st, int nr) {
@@ -398,8 +625,11 @@ void launch_add_to_double(double* y, const T* x, int64_t n, cudaStream_t st) {
 void launch_axpy_loc(double* y, const double* x, double a, int64_t n, cudaStream_t st) {
   if (n > 0) { note_launch(); k_axpy<<<nblocks(n, 256), 256, 0, st>>>(y, x, a, n); }
 }
-void launch_coarse_gather(const LevelDev& L, const double* rc_sub, int64_t sum_nc, double* rC, cudaStream_t st, int nr) {
-  if (L.n_coarse > 0) { note_launch(); k_coarse_gather<<<dim3(nblocks(L.n_coarse, 256), nr), 256, 0, st>>>(L, rc_sub, sum_nc, rC); }
+void launch_coarse_gather(const LevelDev& L, const double* part, int zmax, double* rc_sub, int64_t sum_nc, double* rC,
+                          float* v32, const int32_t* v32_pos, int64_t n_v32, cudaStream_t st, int nr) {
+  if (L.n_coarse <= 0) return;
+  note_launch();
+  k_coarse_gather<<<dim3(nblocks(L.n_coarse, 8), nr), 256, 0, st>>>(L, part, zmax, rc_sub, sum_nc, rC, v32, v32_pos, n_v32);
 }
 void launch_coarse_scatter_n(const int32_t* sub_coarse, int64_t total, const double* zC, int64_t n_coarse,
                              double* zc_sub, cudaStream_t st, int nr) {
@@ -410,15 +640,22 @@ void launch_dot(const double* a, const double* b, int64_t n, double* partial, in
   { note_launch(); k_dot_partial<<<dim3(nblk, nr), 256, 0, st>>>(a, b, n, partial); }
   { note_launch(); k_dot_final<<<nr, 256, 0, st>>>(partial, nblk, out, ostride); }
 }
-void launch_pcg_update_x_r(double* x, double* r, const double* p, const double* q, const double* scal, int64_t n,
-                           cudaStream_t st, int nr) {
-  if (n > 0) { note_launch(); k_pcg_xr<<<dim3(nblocks(n, 256), nr), 256, 0, st>>>(x, r, p, q, scal, n); }
+void launch_pcg_update_x_r(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
+                           double* partial, int* cnt, const KrylovStore& ks, cudaStream_t st, int nr) {
+  if (n > 0) { note_launch(); k_pcg_xr<<<dim3(nblocks(n, 256), nr), 256, 0, st>>>(x, r, p, q, scal, n, partial, cnt, ks); }
+}
+void launch_project(const KrylovStore& ks, const double* g, double* x, double* r, int64_t n, double* coef,
+                    cudaStream_t st, int nr) {
+  if (n <= 0 || ks.cap <= 0) return;
+  note_launch();
+  k_project_dot<<<dim3(kProjBlocks, ks.cap, nr), 256, 0, st>>>(ks, g, n, coef);
+  note_launch();
+  k_project_coef<<<dim3(nblocks(ks.cap, 128), nr), 128, 0, st>>>(ks, coef);
+  note_launch();
+  k_project_apply<<<dim3(nblocks(n, 256), nr), 256, 0, st>>>(ks, g, x, r, n, coef);
 }
 void launch_pcg_update_p(double* p, const double* z, const double* scal, int64_t n, cudaStream_t st, int nr) {
   if (n > 0) { note_launch(); k_pcg_p<<<dim3(nblocks(n, 256), nr), 256, 0, st>>>(p, z, scal, n); }
-}
-void launch_pcg_scalars(double* scal, int stage, int flexible, cudaStream_t st, int nr) {
-  { note_launch(); k_pcg_scalars<<<1, 32, 0, st>>>(scal, stage, flexible, nr); }
 }
 void launch_grad_contract_slots(int64_t n_elems, int ne, const double* ke, const int32_t* slot_elem, const double* coef,
                                 const int32_t* conn, int ndof, const double* lam, const double* u, int nrhs,
@@ -479,7 +716,7 @@ void launch_bicg_xr(double* x, double* r, const double* ph, const double* sh, co
 
 #define INST(T)                                                                             \
   template void launch_gather_iface<T>(const LevelDev&, const double*, int, T*, cudaStream_t, int); \
-  template void launch_scatter_iface<T>(const LevelDev&, const T*, int, double*, cudaStream_t, int); \
+  template void launch_scatter_iface<T>(const LevelDev&, const T*, int, double*, cudaStream_t, int, const FusedDot&); \
   template void launch_gather_glob<T>(const LevelDev&, const double*, int, T*, cudaStream_t, int);  \
   template void launch_scatter_interior<T>(const LevelDev&, const T*, double*, cudaStream_t, int);  \
   template void launch_add_to_double<T>(double*, const T*, int64_t, cudaStream_t);
