@@ -790,23 +790,31 @@ __global__ void k_cc_mu(LevelDev L, const int32_t* __restrict__ crow_sub, int64_
   if (lane == 0) mu[g] = acc;
 }
 
-// out_p = z_C[R_Ci p] - sum_q G_pq t_q: one warp per constraint row
+// out_p = z_C[R_Ci p] - sum_q G_pq t_q: one warp per constraint row, its row of G read once for NR columns
+template <int NR>
 __global__ void k_coarse_coef(LevelDev L, const int32_t* __restrict__ crow_sub, int64_t total_rows,
                               const double* __restrict__ zC, const double* __restrict__ t, double* __restrict__ out) {
   const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (g >= total_rows) return;
-  zC += (int64_t)blockIdx.y * L.n_coarse;
-  t += (int64_t)blockIdx.y * total_rows;
   const int s = crow_sub[g];
   const SubMeta& m = L.meta[s];
   const int nc = m.nc;
   const int64_t c_off = m.c_off;
   const double* G = L.G + m.g_off + (g - c_off) * nc;
-  double acc = 0.0;
-  for (int q = lane; q < nc; q += 32) acc += G[q] * t[c_off + q];
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) out[(int64_t)blockIdx.y * total_rows + g] = zC[L.sub_coarse[g]] - acc;
+  double acc[NR];
+#pragma unroll
+  for (int k = 0; k < NR; ++k) acc[k] = 0.0;
+  for (int q = lane; q < nc; q += 32) {
+    const double a = G[q];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) acc[k] += a * t[(int64_t)k * total_rows + c_off + q];
+  }
+  lane_sums<NR>(acc, lane);
+  if (lane_sum_writer<NR>(lane)) {
+    const int k = lane_sum_index<NR>(lane);
+    out[(int64_t)k * total_rows + g] = zC[(int64_t)k * L.n_coarse + L.sub_coarse[g]] - acc[0];
+  }
 }
 
 // identity tiles of the inverse rows
@@ -1300,8 +1308,22 @@ void launch_psi_apply_add(const LevelDev& L, const double* zc_sub, int64_t sum_n
 void launch_coarse_coef(const LevelDev& L, const int32_t* crow_sub, int64_t sum_nc, const double* zC, const double* t,
                         double* out, cudaStream_t st, int nr) {
   if (sum_nc <= 0) return;
-  note_launch();
-  k_coarse_coef<<<dim3((unsigned)((sum_nc + 7) / 8), nr), 256, 0, st>>>(L, crow_sub, sum_nc, zC, t, out);
+  const unsigned gx = (unsigned)((sum_nc + 7) / 8);
+  for (int r0 = 0; r0 < nr;) {
+    const int left = nr - r0, g = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
+    const double *z = zC + (int64_t)r0 * L.n_coarse, *tt = t + (int64_t)r0 * sum_nc;
+    double* o = out + (int64_t)r0 * sum_nc;
+    note_launch();
+    if (g == 8)
+      k_coarse_coef<8><<<gx, 256, 0, st>>>(L, crow_sub, sum_nc, z, tt, o);
+    else if (g == 4)
+      k_coarse_coef<4><<<gx, 256, 0, st>>>(L, crow_sub, sum_nc, z, tt, o);
+    else if (g == 2)
+      k_coarse_coef<2><<<gx, 256, 0, st>>>(L, crow_sub, sum_nc, z, tt, o);
+    else
+      k_coarse_coef<1><<<gx, 256, 0, st>>>(L, crow_sub, sum_nc, z, tt, o);
+    r0 += g;
+  }
 }
 
 void launch_unit_rows(const LevelDev& L, int max_nGb, cudaStream_t st) {

@@ -207,36 +207,61 @@ __global__ void k_scatter_interior_diff(LevelDev L, const double* __restrict__ a
   if (g >= 0 && L.loc2iface[p] < 0) y[(int64_t)blockIdx.y * L.n_dof + g] = a[o] - b[o];
 }
 
-// y[row] = beta*y[row] + alpha * (K_i x)[row] for the rows of a list (interior rows, interface
-// rows or all rows of every subdomain); 16 lanes per row, two rows per warp.
-__global__ void k_spmv(LevelDev L, const int64_t* __restrict__ rows, int64_t nrows, const double* __restrict__ x,
-                       double* __restrict__ y, double alpha, double beta, const int32_t* __restrict__ row_sub) {
-  const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 4) + (threadIdx.x >> 4);
-  const int l = threadIdx.x & 15;
+// y[row] = beta*y[row] + alpha * (K_i x)[row] for the rows of a list (interior rows, interface rows or all rows
+// of every subdomain) and NR right-hand sides.  A group of LR lanes takes a row: its entries are read once
+// for all columns, and the FP64 units, which bound the product (2 operations per cycle and SM: 27 M entries
+// take 47 us, as long as their 12 bytes each from HBM), spend few additions on the sums over the lanes.
+// Sixteen lanes and one column at a time spent as many on those sums as on the products and read the matrix
+// once per column: 48^3, 8 columns 700 us.
+template <int NR, int LR>
+__global__ void __launch_bounds__(256) k_spmv(LevelDev L, const int64_t* __restrict__ rows, int64_t nrows,
+                                              const double* __restrict__ x, double* __restrict__ y, double alpha,
+                                              double beta, const int32_t* __restrict__ row_sub) {
+  const int64_t g = ((int64_t)blockIdx.x * 256 + threadIdx.x) / LR;
+  const int l = threadIdx.x % LR;
   const bool valid = g < nrows;
   const int64_t row = rows[valid ? g : 0];
-  const int s = row_sub[row];
-  x += (int64_t)blockIdx.y * L.n_vec;
-  y += (int64_t)blockIdx.y * L.n_vec;
-  const double* xs = x + L.meta[s].vec_off;
-  double acc = 0.0, acc2 = 0.0;
+  const double* xs = x + L.meta[row_sub[row]].vec_off;
+  double acc[NR];
+#pragma unroll
+  for (int k = 0; k < NR; ++k) acc[k] = 0.0;
   if (valid) {
-    // two entries per lane and iteration: both loads are issued before either product (the
-    // rows hold up to 81 entries, so a single chain of dependent loads left the kernel
-    // latency-bound); the two partial sums are added at the end, in a fixed order
     const int64_t q1 = L.row_ptr[row + 1];
+    constexpr int U = NR == 1 ? 4 : 2;   // entries in flight per lane
     int64_t q = L.row_ptr[row] + l;
-    for (; q + 16 < q1; q += 32) {
-      const double v0 = L.val[q], v1 = L.val[q + 16];
-      const int c0 = L.col[q], c1 = L.col[q + 16];
-      acc += v0 * xs[c0];
-      acc2 += v1 * xs[c1];
+    for (; q + (U - 1) * LR < q1; q += U * LR) {
+      double v[U];
+      int c[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        v[u] = __ldg(L.val + q + u * LR);
+        c[u] = __ldg(L.col + q + u * LR);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int k = 0; k < NR; ++k) acc[k] += v[u] * xs[(int64_t)k * L.n_vec + c[u]];
     }
-    if (q < q1) acc += L.val[q] * xs[L.col[q]];
+    for (; q < q1; q += LR) {
+      const double v = __ldg(L.val + q);
+      const int c = __ldg(L.col + q);
+#pragma unroll
+      for (int k = 0; k < NR; ++k) acc[k] += v * xs[(int64_t)k * L.n_vec + c];
+    }
   }
-  acc += acc2;
-  for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (valid && l == 0) y[row] = (beta == 0.0 ? 0.0 : beta * y[row]) + alpha * acc;
+#pragma unroll
+  for (int k = 0; k < NR; ++k) {
+#pragma unroll
+    for (int o = LR / 2; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+  }
+  if (valid) {
+#pragma unroll
+    for (int k = 0; k < NR; ++k)
+      if (l == k % LR) {
+        double* yr = y + (int64_t)k * L.n_vec + row;
+        *yr = (beta == 0.0 ? 0.0 : beta * *yr) + alpha * acc[k];
+      }
+  }
 }
 
 template <typename Tin, typename Tout>
@@ -610,9 +635,30 @@ void launch_scatter_interior_diff(const LevelDev& L, const double* a, const doub
                                   int nr) {
   if (L.n_vec > 0) { note_launch(); k_scatter_interior_diff<<<dim3(nblocks(L.n_vec, 256), nr), 256, 0, st>>>(L, a, b, y); }
 }
+template <int NR>
+void launch_spmv_nr(const LevelDev& L, const int64_t* rows, int64_t nrows, const double* x, double* y, double alpha,
+                    double beta, const int32_t* row_sub, cudaStream_t st) {
+  constexpr int LR = 4;
+  note_launch();
+  k_spmv<NR, LR><<<nblocks(nrows * LR, 256), 256, 0, st>>>(L, rows, nrows, x, y, alpha, beta, row_sub);
+}
 void launch_spmv_rows(const LevelDev& L, const int64_t* rows, int64_t nrows, const double* x, double* y, double alpha,
                       double beta, const int32_t* row_sub, cudaStream_t st, int nr) {
-  if (nrows > 0) { note_launch(); k_spmv<<<dim3(nblocks(nrows, 16), nr), 256, 0, st>>>(L, rows, nrows, x, y, alpha, beta, row_sub); }
+  if (nrows <= 0) return;
+  for (int r0 = 0; r0 < nr;) {   // columns in groups of 8, 4, 2, 1: one pass over the matrix each
+    const int left = nr - r0, g = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
+    const double* xs = x + (int64_t)r0 * L.n_vec;
+    double* ys = y + (int64_t)r0 * L.n_vec;
+    if (g == 8)
+      launch_spmv_nr<8>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st);
+    else if (g == 4)
+      launch_spmv_nr<4>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st);
+    else if (g == 2)
+      launch_spmv_nr<2>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st);
+    else
+      launch_spmv_nr<1>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st);
+    r0 += g;
+  }
 }
 template <typename Tin, typename Tout>
 void launch_convert(const Tin* in, Tout* out, int64_t n, cudaStream_t st) {
