@@ -651,17 +651,19 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
   for (int64_t s = 0; s < ns; ++s) {
     const SubMeta& m = L.meta[s];
     for (int k = 0; k < m.Bc; ++k) {
+      const int rows = k < m.nIb ? m.Bc : m.R;   // constraint rows are zero in interior columns
       int64_t cnt = 0;
-      for (int j = k + 1; j < m.Bc; ++j) cnt += m.R - j;
+      for (int j = k + 1; j < m.Bc; ++j) cnt += rows - j;
       L.max_tiles[k] = std::max(L.max_tiles[k], (int)cnt);
-      L.step_flops[k] += nb3 / 3.0 + nb3 * (double)(m.R - k - 1) + 2.0 * nb3 * (double)cnt;
+      L.step_flops[k] += nb3 / 3.0 + nb3 * (double)(rows - k - 1) + 2.0 * nb3 * (double)cnt;
     }
     for (int k = 0; k < m.Bc; ++k) {
       const int kb1 = (k / kSub + 1) * kSub;
+      const int rows = k < m.nIb ? m.Bc : m.R;
       int64_t cnt = 0;
-      for (int j = k + 1; j < std::min(kb1, (int)m.Bc); ++j) cnt += m.R - j;
+      for (int j = k + 1; j < std::min(kb1, (int)m.Bc); ++j) cnt += rows - j;
       L.narrow_tiles[k] = std::max(L.narrow_tiles[k], (int)cnt);
-      L.panel_flops[k] += nb3 / 3.0 + nb3 * (double)(m.R - k - 1) + 2.0 * nb3 * (double)cnt;
+      L.panel_flops[k] += nb3 / 3.0 + nb3 * (double)(rows - k - 1) + 2.0 * nb3 * (double)cnt;
       const int ilim = std::min(kb1, (int)m.Bc);   // the diagonal block's rows
       int64_t bcnt = 0;
       for (int j = k + 1; j < ilim; ++j) bcnt += ilim - j;
@@ -670,8 +672,9 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     }
     for (int kb0 = 0; kb0 < m.Bc; kb0 += kPanel) {
       int64_t tiles[2] = {0, 0};
-      for (int j = kb0 + kSub; j < std::min(kb0 + kPanel, (int)m.Bc); ++j) tiles[0] += m.R - j;
-      for (int j = kb0 + kPanel; j < m.Bc; ++j) tiles[1] += m.R - j;
+      const int rows0 = kb0 + kSub <= m.nIb ? m.Bc : m.R, rows1 = kb0 + kPanel <= m.nIb ? m.Bc : m.R;
+      for (int j = kb0 + kSub; j < std::min(kb0 + kPanel, (int)m.Bc); ++j) tiles[0] += rows0 - j;
+      for (int j = kb0 + kPanel; j < m.Bc; ++j) tiles[1] += rows1 - j;
       const int p = kb0 / kPanel;
       const int e0 = inverse_rows(m, kb0 + kSub), e1 = inverse_rows(m, kb0 + kPanel);   // inverse rows and columns
       tiles[0] += (int64_t)e0 * std::max(0, std::min(kb0 + kPanel, (int)m.Bc) - (kb0 + kSub));
@@ -688,7 +691,8 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
         const int k0 = kb0 + half * kSub;
         const int nd = std::min(kSub, (int)m.Bc - k0);
         if (nd <= 0) continue;
-        const double rows = (double)NB * (m.R - std::min(k0 + kSub, (int)m.Bc) + inverse_rows(m, k0 + kSub));
+        const double rows = (double)NB * ((k0 + kSub <= m.nIb ? m.Bc : m.R + inverse_rows(m, k0 + kSub)) -
+                                          std::min(k0 + kSub, (int)m.Bc));
         L.tc_flops[kTcLaunches * p + 3 + half] += rows * (double)(NB * nd) * (NB * nd);
       }
     }

@@ -261,7 +261,7 @@ __global__ void k_trsm_panel(LevelDev L, int k, int rlim) {
   const int s = blockIdx.y;
   const SubMeta m = L.meta[s];
   const int i = k + 1 + blockIdx.x;
-  const int ilim = rlim > 0 ? (rlim < m.Bc ? rlim : m.Bc) : m.R;
+  const int ilim = rlim > 0 ? (rlim < m.Bc ? rlim : m.Bc) : (k < m.nIb ? (int)m.Bc : (int)m.R);   // see k_syrk_update
   if (k >= m.Bc || i >= ilim) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* As = (T*)smem_raw;
@@ -282,6 +282,39 @@ __global__ void k_trsm_panel(LevelDev L, int k, int rlim) {
     for (int b = 0; b < 4; ++b) v[b] = acc[a][b] * sk[4 * tx + b];
     store4(g + (4 * ty + a) * NB + 4 * tx, v);
   }
+}
+
+// The same panel by blocks of 16 rows, for launches with fewer 64 x 64 tiles than SMs: an FP64 tile takes
+// one SM 131,000 cycles of FP64 products, so the coarsest level's panels (one subdomain, 3,345 DOFs: 52
+// tiles at most) ran on a third of the chip, 72 us per step.
+template <typename T>
+__global__ void __launch_bounds__(256) k_trsm_panel16(LevelDev L, int k, int rlim) {
+  const int s = blockIdx.y;
+  const SubMeta m = L.meta[s];
+  const int i = k + 1 + (int)(blockIdx.x >> 2), r0 = 16 * (blockIdx.x & 3);
+  const int ilim = rlim > 0 ? (rlim < m.Bc ? rlim : m.Bc) : (k < m.nIb ? (int)m.Bc : (int)m.R);
+  if (k >= m.Bc || i >= ilim) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* Xs = (T*)smem_raw;             // k-major inverse of the diagonal tile
+  T* As = Xs + NB * LDS;            // 16 rows of the panel tile
+  T* g = tile_ptr<T>(m, L.tiles, i, k) + r0 * NB;
+  load_kmajor(Xs, (const T*)L.dinv + m.dinv_off + (int64_t)k * NB2);
+  for (int t = threadIdx.x; t < 16 * NB; t += 256) As[t] = g[t];
+  __syncthreads();
+  const int tx = threadIdx.x % 16, r = threadIdx.x / 16;
+  T acc[4] = {};
+#pragma unroll 8
+  for (int q = 0; q < NB; ++q) {
+    const T a = As[r * NB + q];
+    T x[4];
+    load4(x, Xs + q * LDS + 4 * tx);
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[b] += a * x[b];
+  }
+  const T* sk = (const T*)L.sgn + m.vec_off + (int64_t)k * NB;
+#pragma unroll
+  for (int b = 0; b < 4; ++b) acc[b] *= sk[4 * tx + b];
+  store4(g + r * NB + 4 * tx, acc);
 }
 
 // ---- inverse of a sub-panel's 256 x 256 diagonal block (FP32, the tensor-core panel solve) ----
@@ -355,7 +388,9 @@ __global__ void k_syrk_update(LevelDev L, int k, int jmax, int fuse_next, int rl
   }
   if (k >= m.Bc) return;
   const int jend = jmax < m.Bc ? jmax : m.Bc;
-  const int ilim = rlim > 0 ? (rlim < m.Bc ? rlim : m.Bc) : m.R;
+  // constraints touch interface DOFs only, so the constraint rows are zero in interior columns k < nIb
+  // (a fifth of the trailing tiles of 64 subdomains of 6^3 elements)
+  const int ilim = rlim > 0 ? (rlim < m.Bc ? rlim : m.Bc) : (k < m.nIb ? (int)m.Bc : (int)m.R);
   int t = blockIdx.x, j = k + 1, i = -1;
   for (; j < jend; ++j) {
     const int cnt = ilim - j;
@@ -1180,13 +1215,20 @@ void launch_potrf_step(const LevelDev& L, int k, int max_R, int max_tiles, int j
   if (!attr) {
     cudaFuncSetAttribute(k_potrf_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_diag);
     cudaFuncSetAttribute(k_trsm_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_trsm_panel16<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     cudaFuncSetAttribute(k_syrk_update<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     attr = true;
   }
   static_assert(2 * NB * LDS >= 2 * NB * (NB + 1), "the update's shared memory holds the diagonal factorisation");
   if (!skip_diag) { note_launch(); k_potrf_diag<T><<<ns, 256, sm_diag, st>>>(L, k); }
   const int panel = (rlim > 0 && rlim < max_R ? rlim : max_R) - k - 1;
-  if (panel > 0) { note_launch(); k_trsm_panel<T><<<dim3((unsigned)panel, ns), 256, sm, st>>>(L, k, rlim); }
+  if (panel > 0) {
+    note_launch();
+    if (sizeof(T) == 8 && (int64_t)panel * ns < 152)
+      k_trsm_panel16<T><<<dim3((unsigned)panel * 4, ns), 256, sm, st>>>(L, k, rlim);
+    else
+      k_trsm_panel<T><<<dim3((unsigned)panel, ns), 256, sm, st>>>(L, k, rlim);
+  }
   static_assert(sizeof(float) * NB * (NB + 1 + 32) <= 2 * NB * LDS * sizeof(float), "block inverse shared memory");
   const int xq = xinv && sizeof(T) == 4 ? k - k0 : 0;   // block row of the diagonal block's inverse
   if (max_tiles > 0 || xq > 0) {

@@ -187,7 +187,8 @@ void launch_potrf_step(const LevelDev& L, int k, int max_R, int max_tiles, int j
 inline int split_rows_of(const SubMeta& m, int ib, int act, int panel_operand) {
   if (act >= m.Bc || (!panel_operand && !m.nV && ib >= m.Bc)) return 0;
   const int e = ib - m.nIb;
-  return m.R - (ib < m.Bc ? ib : m.Bc) + (e <= 0 ? 0 : (e < m.nV ? e : m.nV));
+  if (e <= 0) return m.Bc - (ib < m.Bc ? ib : m.Bc);   // the constraint rows are zero in interior columns
+  return m.R - (ib < m.Bc ? ib : m.Bc) + (e < m.nV ? e : m.nV);
 }
 void launch_split_panel(const LevelDev& L, int kb0, int nt, int ib, int act, int rows, uint8_t* split,
                         uint8_t* split_signed, float* rscale, const int64_t* prow_off, cudaStream_t st,

@@ -35,7 +35,8 @@ __host__ __device__ inline TcItems tc_items_of(const SubMeta& m, int jbeg, int j
   t.jlim = m.Bc < jend ? m.Bc : jend;
   t.ib = ibeg < m.Bc ? ibeg : m.Bc;
   t.R = m.R;
-  t.rend = m.R + e;
+  // constraints touch interface DOFs only: their rows are zero until the first interface column
+  t.rend = (panel ? jend : jbeg) <= m.nIb ? m.Bc : m.R + e;
   t.j0 = jbeg;
   t.n = on && t.jlim > jbeg ? (t.jlim - jbeg + 1) / 2 : 0;
   const int first = panel ? t.ib : jbeg;

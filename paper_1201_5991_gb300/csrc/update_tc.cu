@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(64 * NT) k_split_panel(LevelDev L, int kb0, in
   const SubMeta m = L.meta[s];
   if (act >= m.Bc || (!panel_operand && !m.nV && ib >= m.Bc)) return;
   const int i = (ib < m.Bc ? ib : m.Bc) + (int)blockIdx.x;
-  if (i >= m.R + inverse_rows(m, ib)) return;
+  if (i >= (ib <= m.nIb ? (int)m.Bc : m.R + inverse_rows(m, ib))) return;
   split_row_tile<NT>(L, s, m, i, kb0, split, split_signed, rscale, prow_off);
 }
 
