@@ -366,6 +366,14 @@ struct bddc_handle_s {
   int grid_max = 304;                  // persistent sweep grid: 2 CTAs per SM
   int blk = 1;                         // right-hand sides the Krylov work vectors hold
   cudaStream_t cap_st = nullptr;       // private stream for graph capture
+  // per BDDC level: a stream for the coarse part of its preconditioner step beside the local solves, and the
+  // events that fork it from and join it to the caller's stream (the join is always reached, so work on the
+  // caller's stream that follows the step also follows the coarse part)
+  struct Fork {
+    cudaStream_t st = nullptr;
+    cudaEvent_t out = nullptr, in = nullptr;
+  };
+  std::vector<Fork> forks;
   cudaGraphExec_t iter_graph = nullptr;  // one captured Krylov iteration
   int iter_graph_key = -1;               // graph_key() of the captured iteration
   int64_t graph_kernels = 0;           // kernel nodes in iter_graph
@@ -384,6 +392,11 @@ struct bddc_handle_s {
   ~bddc_handle_s() {
     if (iter_graph) cudaGraphExecDestroy(iter_graph);
     if (cap_st) cudaStreamDestroy(cap_st);
+    for (auto& f : forks) {
+      if (f.st) cudaStreamDestroy(f.st);
+      if (f.out) cudaEventDestroy(f.out);
+      if (f.in) cudaEventDestroy(f.in);
+    }
     for (auto& r : prof_pending) {
       cudaEventDestroy(r.a);
       cudaEventDestroy(r.b);
@@ -827,6 +840,12 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     for (int64_t p = 0; p < L.n_vec; ++p)
       if (loc2iface[p] >= 0) iface_occ[fill[loc2iface[p]]++] = p;
   }
+  std::vector<int4> occ4(mp.n_iface);
+  for (int64_t g = 0; g < mp.n_iface; ++g) {
+    const int64_t o = iface_ptr[g], c = iface_ptr[g + 1] - o;
+    auto at = [&](int64_t k) { return k < c ? (int)iface_occ[o + k] : -1; };
+    occ4[g] = make_int4(at(0), at(1), at(2), c > 4 ? -2 : at(3));
+  }
   std::vector<int32_t> sub_coarse(mp.sub_coarse.size());
   for (size_t t = 0; t < mp.sub_coarse.size(); ++t) {
     sub_coarse[t] = (int32_t)mp.sub_coarse[t];
@@ -884,6 +903,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
   d.loc2glob = A.upload(loc2glob, st);
   d.iface_ptr = A.upload(iface_ptr, st);
   d.iface_occ = A.upload(iface_occ, st);
+  d.iface_occ4 = A.upload(occ4, st);
   d.glob_occ_ptr = nullptr;
   d.glob_occ = nullptr;
   d.sub_coarse = A.upload(sub_coarse, st);
@@ -1348,9 +1368,17 @@ void interface_step_t(bddc_handle_s* h, int l, const double* rhat, double* zhat,
   launch_gather_iface<T>(L.d, rhat, 1, v, st, nb);          // r_i = E_i^T r_hat
   const bool last = l + 2 == (int)h->lv.size();
   const Level& C = h->lv.back();
-  launch_psi_t_apply<T>(L.d, v, L.psi_part, L.sum_nc, L.max_nGb, L.max_ncb, st, nb);   // Psi_i^T r_i
-  launch_coarse_gather(L.d, L.psi_part, rows_zmax(L.max_nGb), L.rc_sub, L.sum_nc, L.rC,
-                       last && C.winv ? C.v32 : nullptr, C.v32_pos, C.n_vec, st, nb);   // r_C = sum R_Ci^T Psi_i^T r_i
+  auto coarse_residual = [&](cudaStream_t cs) {   // r_C = sum R_Ci^T Psi_i^T r_i
+    launch_psi_t_apply<T>(L.d, v, L.psi_part, L.sum_nc, L.max_nGb, L.max_ncb, cs, nb);
+    launch_coarse_gather(L.d, L.psi_part, rows_zmax(L.max_nGb), L.rc_sub, L.sum_nc, L.rC,
+                         last && C.winv ? C.v32 : nullptr, C.v32_pos, C.n_vec, cs, nb);
+  };
+  auto coarse_correction = [&](cudaStream_t cs) {
+    if (last)
+      coarsest_solve(h, L.rC, L.zC, cs, nb);
+    else
+      full_step(h, l + 1, L.rC, L.zC, cs, nb);
+  };
   if (L.inverse) {
     // Eq. sub_cor with the explicit inverse of the augmented interface matrix: z_i = A_GG^{-1} r_i -
     // Psi_i G_i Psi_i^T r_i, one symmetric product over the stored lower triangle instead of a sweep pair
@@ -1358,29 +1386,31 @@ void interface_step_t(bddc_handle_s* h, int l, const double* rhat, double* zhat,
     // residual's, and both multiples of Psi_i are added in one product.  48^3 workload: a sweep pair of
     // 220 us and 33 us of products per application become 97 us at 0.8 of HBM; on 8 subdomains, whose
     // chains the sweeps could not hide, 150 us become 19.  The inverse rows add 21 % to the tiles and
-    // about 3 ms to the set-up.
+    // about 3 ms to the set-up.  The symmetric product and the coarse part (whose launches fill a
+    // fraction of the chip, 30 us on the 48^3 workload) only share r_i, so they run beside each other.
     float* z = (float*)L.locB;
+    const bddc_handle_s::Fork& f = h->forks[l];
+    ck(cudaEventRecord(f.out, st), "fork");
+    ck(cudaStreamWaitEvent(f.st, f.out, 0), "fork");
+    coarse_residual(f.st);
+    coarse_correction(f.st);
+    launch_coarse_coef(L.d, L.crow_sub, L.sum_nc, L.zC, L.rc_sub, L.zc_sub, f.st, nb);
+    ck(cudaEventRecord(f.in, f.st), "join");
     {
       ProfScope ps(h, BDDC_PROF_TRSV_IFACE, column_groups(nb, 4) * L.trsv_bytes[1], 0.0, st, 2);   // rows, columns
       launch_schur_symv(L.d, 1, L.max_nGb, L.symv_part_off, L.symv_stride, (const float*)v, L.symv_part, z, st, nb);
     }
-    if (last)
-      coarsest_solve(h, L.rC, L.zC, st, nb);
-    else
-      full_step(h, l + 1, L.rC, L.zC, st, nb);
-    launch_coarse_coef(L.d, L.crow_sub, L.sum_nc, L.zC, L.rc_sub, L.zc_sub, st, nb);
+    ck(cudaStreamWaitEvent(st, f.in, 0), "join");
     launch_psi_apply_add<float>(L.d, L.zc_sub, L.sum_nc, z, L.max_nGb, L.max_ncb, st, nb);
     launch_scatter_iface<float>(L.d, z, 1, zhat, st, nb, dot); // z_hat = sum E_i (...)
     return;
   }
+  coarse_residual(st);
   trsv_one<T>(h, L, v, 1, 0, st, nb);                       // Eq. sub_cor via the trailing factor
   launch_constraint_corr<T>(L.d, v, L.crow_sub, L.sum_nc, L.cc_t, L.cc_mu, L.psi_part, L.max_nGb, L.max_ncb, st,
                             nb);
   trsv_one<T>(h, L, v, 1, 1, st, nb);
-  if (last)
-    coarsest_solve(h, L.rC, L.zC, st, nb);
-  else
-    full_step(h, l + 1, L.rC, L.zC, st, nb);
+  coarse_correction(st);
   launch_coarse_scatter_n(L.d.sub_coarse, L.sum_nc, L.zC, L.d.n_coarse, L.zc_sub, st, nb);
   launch_psi_apply_add<T>(L.d, L.zc_sub, L.sum_nc, v, L.max_nGb, L.max_ncb, st, nb);   // Psi_i R_Ci z_C + z_i
   launch_scatter_iface<T>(L.d, v, 1, zhat, st, nb, dot);       // z_hat = sum E_i (...)
@@ -1843,6 +1873,14 @@ void device_setup(bddc_handle_s* h) {
       fprintf(stderr, "bddc prepare: level %d %8.2f ms (uploads %.2f ms, %.1f MB)\n", (int)l + 1, now_ms() - tl,
               A.upload_ms - u0, (double)(A.upload_bytes - b0) / 1e6);
   }
+  h->forks.resize(h->lv.size());
+  for (size_t l = 0; l < h->lv.size(); ++l)
+    if (h->lv[l].inverse) {
+      auto& f = h->forks[l];
+      ck(cudaStreamCreateWithFlags(&f.st, cudaStreamNonBlocking), "cudaStreamCreate");
+      ck(cudaEventCreateWithFlags(&f.out, cudaEventDisableTiming), "cudaEventCreate");
+      ck(cudaEventCreateWithFlags(&f.in, cudaEventDisableTiming), "cudaEventCreate");
+    }
   if (h->has_lift) {
     // occurrences (slot, element row) of every free DOF in elements that touch a non-zero
     // prescribed value, in slot order; u_d of every slot
@@ -3121,6 +3159,8 @@ int bddc_sizes(bddc_handle h, int64_t* n_free, int64_t* n_iface) {
 void bddc_free(bddc_handle h) {
   if (!h) return;
   if (h->st) cudaStreamSynchronize(h->st);
+  for (auto& f : h->forks)   // idle unless a call failed between a fork and its join
+    if (f.st) cudaStreamSynchronize(f.st);
   h->arena.release();
   if (h->h_scal) cudaFreeHost(h->h_scal);
   delete h;

@@ -93,6 +93,8 @@ struct LevelDev {
   const int32_t* loc2glob;        // [n_vec] level DOF id or -1
   const int64_t* iface_ptr;       // [n_iface + 1] occurrences of an interface DOF
   const int64_t* iface_occ;       //   flat padded positions, ascending subdomain
+  const int4* iface_occ4;         // [n_iface] its first four positions (-1: none); w = -2: more than four, the
+                                  //   list's entries from the fourth on follow x, y, z
   const int64_t* glob_occ_ptr;    // [n_dof + 1] occurrences of every level DOF
   const int64_t* glob_occ;
   const int32_t* sub_coarse;      // [sum nc] global coarse ids (R_Ci)

@@ -6,6 +6,7 @@
 // All sums run in a fixed order (ascending subdomain for the interface / coarse sums, a
 // fixed grid and tree for the dot products), so results are bit-reproducible.
 #include "internal.h"
+#include "reduce.cuh"
 
 namespace bddc {
 
@@ -100,6 +101,22 @@ __device__ void fused_dot(const FusedDot& dot, int64_t g, int64_t n, double y) {
   if (sum_over_grid(v0, v1, dot.mode == 2, dot.partial, dot.cnt, s0, s1) && threadIdx.x == 0) pcg_step(dot, s0, s1);
 }
 
+// sum of term(p) over the occurrences of interface DOF g, ascending subdomain: one 16-byte load instead of
+// the list's bounds and entries, so that the terms' loads are one step away (most DOFs have two occurrences)
+template <typename F>
+__device__ __forceinline__ double sum_occurrences(const LevelDev& L, int64_t g, F&& term) {
+  const int4 o = __ldg(L.iface_occ4 + g);
+  const double a = o.x >= 0 ? term((int64_t)o.x) : 0.0, b = o.y >= 0 ? term((int64_t)o.y) : 0.0;
+  const double c = o.z >= 0 ? term((int64_t)o.z) : 0.0, d = o.w >= 0 ? term((int64_t)o.w) : 0.0;
+  double s = a;
+  if (o.y >= 0) s += b;
+  if (o.z >= 0) s += c;
+  if (o.w >= 0) s += d;
+  if (o.w == -2)
+    for (int64_t q = L.iface_ptr[g] + 3; q < L.iface_ptr[g + 1]; ++q) s += term(L.iface_occ[q]);
+  return s;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_scatter_iface(LevelDev L, const T* __restrict__ loc, int weighted,
                                                        double* __restrict__ y, FusedDot dot) {
@@ -107,26 +124,24 @@ __global__ void __launch_bounds__(256) k_scatter_iface(LevelDev L, const T* __re
   double s = 0.0;
   if (g < L.n_iface) {
     loc += (int64_t)blockIdx.y * L.n_vec;
-    for (int64_t o = L.iface_ptr[g]; o < L.iface_ptr[g + 1]; ++o) {
-      const int64_t p = L.iface_occ[o];
-      s += weighted ? L.w[p] * (double)loc[p] : (double)loc[p];
-    }
+    s = sum_occurrences(L, g, [&](int64_t p) { return weighted ? L.w[p] * (double)loc[p] : (double)loc[p]; });
     y[(int64_t)blockIdx.y * L.n_iface + g] = s;
   }
   if (dot.mode) fused_dot(dot, g, L.n_iface, s);
 }
 
 // inner operator, before its FP32 product: blocks below nv gather loc = R_i x, the others take one
-// constraint row per warp: t = rho c_rho (C_i R_i x)
+// constraint row per warp: t = rho c_rho (C_i R_i x); NR columns per pass over the index lists
+template <int NR>
 __global__ void __launch_bounds__(256) k_inner_gather(LevelDev L, const double* __restrict__ x, float* __restrict__ loc,
                                                       int nv, const int32_t* __restrict__ crow_sub, int64_t total_rows,
                                                       double* __restrict__ t) {
-  x += (int64_t)blockIdx.y * L.n_iface;
   if ((int)blockIdx.x < nv) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= L.n_vec) return;
     const int32_t g = L.loc2iface[p];
-    loc[(int64_t)blockIdx.y * L.n_vec + p] = g >= 0 ? (float)x[g] : 0.f;
+#pragma unroll
+    for (int k = 0; k < NR; ++k) loc[k * L.n_vec + p] = g >= 0 ? (float)x[k * L.n_iface + g] : 0.f;
     return;
   }
   const int64_t r = (int64_t)(blockIdx.x - nv) * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -135,12 +150,18 @@ __global__ void __launch_bounds__(256) k_inner_gather(LevelDev L, const double* 
   const int s = crow_sub[r];
   const double rq = L.rho[s] * L.c_rho[r];
   const int32_t* l2i = L.loc2iface + L.meta[s].vec_off;
-  double acc = 0.0;
-  if (rq != 0.0)
-    for (int64_t e = L.c_ptr[r] + lane; e < L.c_ptr[r + 1]; e += 32) acc += L.c_val[e] * x[l2i[L.c_pos[e]]];
+  double acc[NR];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) t[(int64_t)blockIdx.y * total_rows + r] = rq * acc;
+  for (int k = 0; k < NR; ++k) acc[k] = 0.0;
+  if (rq != 0.0)
+    for (int64_t e = L.c_ptr[r] + lane; e < L.c_ptr[r + 1]; e += 32) {
+      const double c = L.c_val[e];
+      const int32_t g = l2i[L.c_pos[e]];
+#pragma unroll
+      for (int k = 0; k < NR; ++k) acc[k] += c * x[k * L.n_iface + g];
+    }
+  lane_sums<NR>(acc, lane);
+  if (lane_sum_writer<NR>(lane)) t[lane_sum_index<NR>(lane) * total_rows + r] = rq * acc[0];
 }
 
 // y = sum R_i^T (loc - C_i^T t): distinct constraint rows touch disjoint positions (each local DOF lies in
@@ -153,13 +174,11 @@ __global__ void __launch_bounds__(256) k_inner_scatter(LevelDev L, const float* 
   if (g < L.n_iface) {
     loc += (int64_t)blockIdx.y * L.n_vec;
     t += (int64_t)blockIdx.y * total_rows;
-    for (int64_t o = L.iface_ptr[g]; o < L.iface_ptr[g + 1]; ++o) {
-      const int64_t p = L.iface_occ[o];
-      double v = (double)loc[p];
+    s = sum_occurrences(L, g, [&](int64_t p) {
       const int32_t r = L.crow[p];
-      if (r >= 0) v -= t[r] * L.cval[p];
-      s += v;
-    }
+      const double v = (double)loc[p], c = L.cval[p];
+      return r >= 0 ? v - t[r] * c : v;
+    });
     y[(int64_t)blockIdx.y * L.n_iface + g] = s;
   }
   if (dot.mode) fused_dot(dot, g, L.n_iface, s);
@@ -610,9 +629,23 @@ void launch_scatter_iface(const LevelDev& L, const T* loc, int weighted, double*
 void launch_inner_gather(const LevelDev& L, const double* x, float* loc, const int32_t* crow_sub, int64_t total_rows,
                          double* t, cudaStream_t st, int nr) {
   if (L.n_vec <= 0) return;
-  const unsigned nv = nblocks(L.n_vec, 256);
-  note_launch();
-  k_inner_gather<<<dim3(nv + nblocks(total_rows, 8), nr), 256, 0, st>>>(L, x, loc, (int)nv, crow_sub, total_rows, t);
+  const unsigned nv = nblocks(L.n_vec, 256), nb = nv + nblocks(total_rows, 8);
+  for (int r0 = 0; r0 < nr;) {
+    const int left = nr - r0, g = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
+    const double* xs = x + (int64_t)r0 * L.n_iface;
+    float* ls = loc + (int64_t)r0 * L.n_vec;
+    double* ts = t + (int64_t)r0 * total_rows;
+    note_launch();
+    if (g == 8)
+      k_inner_gather<8><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+    else if (g == 4)
+      k_inner_gather<4><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+    else if (g == 2)
+      k_inner_gather<2><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+    else
+      k_inner_gather<1><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+    r0 += g;
+  }
 }
 void launch_inner_scatter(const LevelDev& L, const float* loc, const double* t, int64_t total_rows, double* y,
                           cudaStream_t st, int nr, const FusedDot& dot) {
