@@ -220,8 +220,7 @@ struct Level {
   int sweep_ctas[2] = {2, 2};
   int sweep_deep[2] = {1, 1};
   int sweep_order[2] = {0, 0};
-  int* ctrl = nullptr;         // task counter of the sweeps
-  void* pub = nullptr;         // sweep publication buffer: n_vec x min(blk, 8) words of the factor's type
+  void* sweep_scratch = nullptr;   // task counters and publication buffers of the sweeps
   int64_t* rows[3] = {nullptr, nullptr, nullptr};   // interior rows, interface rows, all rows
   int64_t nrows[3] = {0, 0, 0};
   int32_t* crow_sub = nullptr;                      // subdomain of every constraint row
@@ -271,7 +270,7 @@ void alloc_level_work(Level& L, DevArena& A, int blk) {
     L.locA = A.alloc<double>(nv);
     L.locB = A.alloc<double>(nv);
   }
-  L.pub = A.alloc<double>(L.n_vec * std::min(blk, 8));
+  L.sweep_scratch = A.alloc<char>(sweep_scratch_bytes(L.n_vec, blk));
   if (L.explicit_schur || L.inverse) L.symv_part = A.alloc<float>(std::max<int64_t>(L.symv_stride, 1) * blk);
   L.dl0 = A.alloc<double>(nv);
   L.dl1 = A.alloc<double>(nv);
@@ -1038,7 +1037,6 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
       }
   }
   ph("sweep tasks");
-  L.ctrl = A.alloc<int>(1);   // task counter of the sweeps
   {
     std::vector<int64_t> rl[3];
     std::vector<int32_t> cs;
@@ -1236,20 +1234,27 @@ int column_groups(int nb, int max_nr) {
   return n;
 }
 
+// which: 0 forward sweep, 1 backward, 2 the pair
+template <typename T>
+void trsv(bddc_handle_s* h, Level& L, T* v, int part, int which, cudaStream_t st, int nb) {
+  const bool copy32 = sizeof(T) == 4 && L.solve32;   // FP32 copy of an FP64 factor
+  const int sweeps = which == 2 ? 2 : 1;
+  const double groups = sweeps * column_groups(nb, sizeof(T) == 4 ? 8 : 4);
+  ProfScope ps(h, L.coarsest ? BDDC_PROF_COARSE : part == 0 ? BDDC_PROF_TRSV : BDDC_PROF_TRSV_IFACE,
+               groups * (copy32 ? 0.5 * L.trsv_bytes[part] : L.trsv_bytes[part]), 0.0, st, sweeps);
+  const auto& t = L.sweep_order[part] ? L.tasks_big : L.tasks;
+  launch_sweep<T>(copy32 ? L.d32 : L.d, v, t[part], L.ntasks[part], part, which, L.sweep_scratch,
+                  h->grid_max / 2 * L.sweep_ctas[part], L.sweep_deep[part], st, nb);
+}
+
 template <typename T>
 void trsv_one(bddc_handle_s* h, Level& L, T* v, int part, int backward, cudaStream_t st, int nb = 1) {
-  const bool copy32 = sizeof(T) == 4 && L.solve32;   // FP32 copy of an FP64 factor
-  const double groups = column_groups(nb, sizeof(T) == 4 ? 8 : 4);
-  ProfScope ps(h, L.coarsest ? BDDC_PROF_COARSE : part == 0 ? BDDC_PROF_TRSV : BDDC_PROF_TRSV_IFACE,
-               groups * (copy32 ? 0.5 * L.trsv_bytes[part] : L.trsv_bytes[part]), 0.0, st);
-  launch_sweep<T>(copy32 ? L.d32 : L.d, v, (L.sweep_order[part] ? L.tasks_big : L.tasks)[part][backward], L.ntasks[part][backward],
-                  part, backward, L.ctrl, L.pub, h->grid_max / 2 * L.sweep_ctas[part], L.sweep_deep[part], st, nb);
+  trsv<T>(h, L, v, part, backward, st, nb);
 }
 
 template <typename T>
 void trsv_pair(bddc_handle_s* h, Level& L, T* v, int part, cudaStream_t st, int nb = 1) {
-  trsv_one<T>(h, L, v, part, 0, st, nb);
-  trsv_one<T>(h, L, v, part, 1, st, nb);
+  trsv<T>(h, L, v, part, 2, st, nb);
 }
 
 // w = K_II^{-1} v on level 1 (interior positions), FP64 accuracy.
@@ -3086,8 +3091,9 @@ int bddc_batching_ablation(bddc_handle h, double* ms) {
     for (int dir = 0; dir < 2; ++dir)
       for (int64_t s = 0; s < (int64_t)L.meta.size(); ++s) {
         const int o0 = L.task_sub_off[dir][s], o1 = L.task_sub_off[dir][s + 1];
-        launch_sweep<float>(L.d, v, L.tasks_by_sub[dir] + o0, o1 - o0, 0, dir, L.ctrl, L.pub, grid,
-                            L.sweep_deep[0], st);
+        const int2* one[2] = {L.tasks_by_sub[dir] + o0, L.tasks_by_sub[dir] + o0};
+        const int cnt[2] = {o1 - o0, o1 - o0};
+        launch_sweep<float>(L.d, v, one, cnt, 0, dir, L.sweep_scratch, grid, L.sweep_deep[0], st);
       }
     ck(cudaEventRecord(b, st), "cudaEventRecord");
     ms[1] = elapsed();

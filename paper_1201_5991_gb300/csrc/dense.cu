@@ -10,6 +10,7 @@
 //    Lambda_i = R - G_i^{-1}), K_Ci = Psi_i^T K_i Psi_i = -Lambda_i = G_i^{-1} - R, where
 //    R = diag(rho c_rho) (rho on the rows that augment A_i, 0 on Stokes pressure rows).
 #include "internal.h"
+#include "pdl.cuh"
 #include "reduce.cuh"
 
 namespace bddc {
@@ -829,6 +830,8 @@ __global__ void k_cc_mu(LevelDev L, const int32_t* __restrict__ crow_sub, int64_
 template <int NR>
 __global__ void k_coarse_coef(LevelDev L, const int32_t* __restrict__ crow_sub, int64_t total_rows,
                               const double* __restrict__ zC, const double* __restrict__ t, double* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (g >= total_rows) return;
@@ -890,6 +893,8 @@ __device__ __forceinline__ const T* m_tile(const LevelDev& L, const SubMeta& m, 
 template <typename T, int NR, int MODE>
 __global__ void __launch_bounds__(256) k_rows_matvec(LevelDev L, const T* __restrict__ vec, double* __restrict__ part,
                                                      int zmax, int64_t sum_nc) {
+  pdl_wait();
+  pdl_trigger();
   using V2 = typename Pair<T>::type;
   const int z = blockIdx.x, rb = blockIdx.y, s = blockIdx.z;
   const SubMeta m = L.meta[s];
@@ -958,6 +963,8 @@ __global__ void k_sum_parts(const double* __restrict__ part, int zmax, int64_t t
 template <typename T, int NR, int MODE>
 __global__ void __launch_bounds__(256) k_cols_matvec(LevelDev L, T* __restrict__ vec, const double* __restrict__ zsub,
                                                      int64_t sum_nc, T sign) {
+  pdl_wait();
+  pdl_trigger();
   using V2 = typename Pair<T>::type;
   const int j = blockIdx.x, s = blockIdx.y;
   const SubMeta m = L.meta[s];
@@ -1150,6 +1157,8 @@ template <int NR>
 __global__ void k_coarse_apply(const float* __restrict__ W, int64_t npad, const float* __restrict__ x,
                                double* __restrict__ z, const int32_t* __restrict__ loc2glob, int64_t n_vec,
                                int64_t n_dof) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= npad) return;
@@ -1194,13 +1203,13 @@ void launch_coarse_apply(const float* W, int64_t npad, const float* x, double* z
     double* zs = z + (int64_t)r0 * n_dof;
     note_launch();
     if (g == 8)
-      k_coarse_apply<8><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, zs, loc2glob, n_vec, n_dof);
+      launch_pdl(k_coarse_apply<8>, dim3(gx, ng), 256, 0, st, W, npad, xs, zs, loc2glob, n_vec, n_dof);
     else if (g == 4)
-      k_coarse_apply<4><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, zs, loc2glob, n_vec, n_dof);
+      launch_pdl(k_coarse_apply<4>, dim3(gx, ng), 256, 0, st, W, npad, xs, zs, loc2glob, n_vec, n_dof);
     else if (g == 2)
-      k_coarse_apply<2><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, zs, loc2glob, n_vec, n_dof);
+      launch_pdl(k_coarse_apply<2>, dim3(gx, ng), 256, 0, st, W, npad, xs, zs, loc2glob, n_vec, n_dof);
     else
-      k_coarse_apply<1><<<dim3(gx, ng), 256, 0, st>>>(W, npad, xs, zs, loc2glob, n_vec, n_dof);
+      launch_pdl(k_coarse_apply<1>, dim3(gx, ng), 256, 0, st, W, npad, xs, zs, loc2glob, n_vec, n_dof);
     r0 += ng * g;
   }
 }
@@ -1357,13 +1366,13 @@ void launch_coarse_coef(const LevelDev& L, const int32_t* crow_sub, int64_t sum_
     double* o = out + (int64_t)r0 * sum_nc;
     note_launch();
     if (g == 8)
-      k_coarse_coef<8><<<gx, 256, 0, st>>>(L, crow_sub, sum_nc, z, tt, o);
+      launch_pdl(k_coarse_coef<8>, gx, 256, 0, st, L, crow_sub, sum_nc, z, tt, o);
     else if (g == 4)
-      k_coarse_coef<4><<<gx, 256, 0, st>>>(L, crow_sub, sum_nc, z, tt, o);
+      launch_pdl(k_coarse_coef<4>, gx, 256, 0, st, L, crow_sub, sum_nc, z, tt, o);
     else if (g == 2)
-      k_coarse_coef<2><<<gx, 256, 0, st>>>(L, crow_sub, sum_nc, z, tt, o);
+      launch_pdl(k_coarse_coef<2>, gx, 256, 0, st, L, crow_sub, sum_nc, z, tt, o);
     else
-      k_coarse_coef<1><<<gx, 256, 0, st>>>(L, crow_sub, sum_nc, z, tt, o);
+      launch_pdl(k_coarse_coef<1>, gx, 256, 0, st, L, crow_sub, sum_nc, z, tt, o);
     r0 += g;
   }
 }

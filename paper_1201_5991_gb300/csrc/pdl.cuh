@@ -1,0 +1,31 @@
+// Programmatic dependent launch for the solve phase's short kernels: a kernel launched with launch_pdl may be
+// set up, and its blocks may become resident, while the kernel before it in the stream still runs; pdl_wait,
+// its first instruction that touches global memory depends on, returns when that kernel has completed with
+// its stores visible.  Every such kernel waits, so completion is transitive along the stream.  pdl_trigger lets
+// the next kernel be set up once every block of this one has started (it would otherwise be at its end).
+// Use only where the launch before it in the same stream is a kernel (not a copy, a memset or an event wait).
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace bddc {
+
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+}  // namespace bddc

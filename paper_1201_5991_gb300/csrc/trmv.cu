@@ -10,6 +10,7 @@
 // the outer iteration applies the FP64 operator.  Several right-hand sides share each pass over
 // the triangle (up to eight per launch).
 #include "internal.h"
+#include "pdl.cuh"
 #include "reduce.cuh"
 
 namespace bddc {
@@ -27,6 +28,8 @@ __device__ __forceinline__ int64_t tile_index_t(int i, int j, int Bc) {
 // order (no barrier inside the tile loop).
 template <int NR>
 __global__ void __launch_bounds__(256) k_trmv_t(LevelDev L, const float* __restrict__ x, float* __restrict__ y1) {
+  pdl_wait();
+  pdl_trigger();
   const int s = blockIdx.y;
   const SubMeta m = L.meta[s];
   const int o = blockIdx.x;
@@ -77,6 +80,8 @@ __global__ void __launch_bounds__(256) k_trmv_t(LevelDev L, const float* __restr
 // the tail of the launch).  Warp w takes rows w, w+8, ..., lane l the columns 2l, 2l+1.
 template <int NR>
 __global__ void __launch_bounds__(256) k_trmv_n(LevelDev L, const float* __restrict__ y1, float* __restrict__ y) {
+  pdl_wait();
+  pdl_trigger();
   const int s = blockIdx.y;
   const SubMeta m = L.meta[s];
   if ((int)blockIdx.x >= m.nGb) return;
@@ -216,6 +221,8 @@ __global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, int inverse
     for (int k = 0; k < pre; ++k) tile_g2s(ring + k * NB2, Mrow + (int64_t)k * NB2, &full[k]);
     issued = (uint32_t)pre;
   }
+  pdl_wait();   // the matrix is not written during a solve: its first tiles are requested before x is ready
+  pdl_trigger();
   float xi[NR][8];   // x_i at this thread's rows
 #pragma unroll
   for (int q = 0; q < NR; ++q)
@@ -321,6 +328,8 @@ template <int NR>
 __global__ void __launch_bounds__(256) k_schur_symv_cols(LevelDev L, float sign, const int64_t* __restrict__ part_off,
                                                          int64_t part_stride, const float* __restrict__ part,
                                                          float* __restrict__ y) {
+  pdl_wait();
+  pdl_trigger();
   constexpr int G = 4;   // row segments
   const int s = blockIdx.y;
   const SubMeta m = L.meta[s];
@@ -365,9 +374,9 @@ void launch_symv_nr(const LevelDev& L, int inverse, const dim3& grid, const int6
     attr = true;
   }
   note_launch();
-  k_schur_symv_rows<NR><<<grid, 256, dyn, st>>>(L, inverse, x, part_off, part_stride, part, y);
+  launch_pdl(k_schur_symv_rows<NR>, grid, 256, dyn, st, L, inverse, x, part_off, part_stride, part, y);
   note_launch();
-  k_schur_symv_cols<NR><<<grid, 256, 0, st>>>(L, inverse ? -1.f : 1.f, part_off, part_stride, part, y);
+  launch_pdl(k_schur_symv_cols<NR>, grid, 256, 0, st, L, inverse ? -1.f : 1.f, part_off, part_stride, part, y);
 }
 
 void launch_schur_symv(const LevelDev& L, int inverse, int max_nGb, const int64_t* part_off, int64_t part_stride,
@@ -394,9 +403,9 @@ void launch_schur_symv(const LevelDev& L, int inverse, int max_nGb, const int64_
 template <int NR>
 void launch_trmv_nr(const LevelDev& L, const dim3& grid, const float* x, float* y1, float* y, cudaStream_t st) {
   note_launch();
-  k_trmv_t<NR><<<grid, 256, 0, st>>>(L, x, y1);
+  launch_pdl(k_trmv_t<NR>, grid, 256, 0, st, L, x, y1);
   note_launch();
-  k_trmv_n<NR><<<grid, 256, 0, st>>>(L, y1, y);
+  launch_pdl(k_trmv_n<NR>, grid, 256, 0, st, L, y1, y);
 }
 
 void launch_trmv_schur(const LevelDev& L, int max_nGb, const float* x, float* y1, float* y, cudaStream_t st, int nr) {

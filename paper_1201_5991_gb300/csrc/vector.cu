@@ -6,6 +6,7 @@
 // All sums run in a fixed order (ascending subdomain for the interface / coarse sums, a
 // fixed grid and tree for the dot products), so results are bit-reproducible.
 #include "internal.h"
+#include "pdl.cuh"
 #include "reduce.cuh"
 
 namespace bddc {
@@ -17,6 +18,8 @@ namespace {
 // vectors n_iface, level vectors n_dof, coarse vectors n_coarse, per-subdomain coarse vectors sum nc).
 template <typename T>
 __global__ void k_gather_iface(LevelDev L, const double* __restrict__ x, int weighted, T* __restrict__ loc) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= L.n_vec) return;
   x += (int64_t)blockIdx.y * L.n_iface;
@@ -120,6 +123,8 @@ __device__ __forceinline__ double sum_occurrences(const LevelDev& L, int64_t g, 
 template <typename T>
 __global__ void __launch_bounds__(256) k_scatter_iface(LevelDev L, const T* __restrict__ loc, int weighted,
                                                        double* __restrict__ y, FusedDot dot) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double s = 0.0;
   if (g < L.n_iface) {
@@ -136,6 +141,8 @@ template <int NR>
 __global__ void __launch_bounds__(256) k_inner_gather(LevelDev L, const double* __restrict__ x, float* __restrict__ loc,
                                                       int nv, const int32_t* __restrict__ crow_sub, int64_t total_rows,
                                                       double* __restrict__ t) {
+  pdl_wait();
+  pdl_trigger();
   if ((int)blockIdx.x < nv) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= L.n_vec) return;
@@ -169,6 +176,8 @@ __global__ void __launch_bounds__(256) k_inner_gather(LevelDev L, const double* 
 __global__ void __launch_bounds__(256) k_inner_scatter(LevelDev L, const float* __restrict__ loc,
                                                        const double* __restrict__ t, int64_t total_rows,
                                                        double* __restrict__ y, FusedDot dot) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double s = 0.0;
   if (g < L.n_iface) {
@@ -236,6 +245,8 @@ template <int NR, int LR>
 __global__ void __launch_bounds__(256) k_spmv(LevelDev L, const int64_t* __restrict__ rows, int64_t nrows,
                                               const double* __restrict__ x, double* __restrict__ y, double alpha,
                                               double beta, const int32_t* __restrict__ row_sub) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t g = ((int64_t)blockIdx.x * 256 + threadIdx.x) / LR;
   const int l = threadIdx.x % LR;
   const bool valid = g < nrows;
@@ -285,17 +296,23 @@ __global__ void __launch_bounds__(256) k_spmv(LevelDev L, const int64_t* __restr
 
 template <typename Tin, typename Tout>
 __global__ void k_convert(const Tin* __restrict__ in, Tout* __restrict__ out, int64_t n) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = (Tout)in[i];
 }
 
 template <typename T>
 __global__ void k_add_to_double(double* __restrict__ y, const T* __restrict__ x, int64_t n) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] += (double)x[i];
 }
 
 __global__ void k_axpy(double* __restrict__ y, const double* __restrict__ x, double a, int64_t n) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] += a * x[i];
 }
@@ -305,6 +322,8 @@ __global__ void k_axpy(double* __restrict__ y, const double* __restrict__ x, dou
 __global__ void k_coarse_gather(LevelDev L, const double* __restrict__ part, int zmax, double* __restrict__ rc_sub,
                                 int64_t sum_nc, double* __restrict__ rC, float* __restrict__ v32,
                                 const int32_t* __restrict__ v32_pos, int64_t n_v32) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (g >= L.n_coarse) return;
@@ -375,6 +394,8 @@ __global__ void __launch_bounds__(256) k_pcg_xr(double* __restrict__ x, double* 
                                                 const double* __restrict__ p, const double* __restrict__ q,
                                                 double* __restrict__ scal, int64_t n, double* __restrict__ partial,
                                                 int* cnt, KrylovStore ks) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double rr = 0.0, s0, s1;
   const double a = scal[16 * blockIdx.y + 2];
@@ -455,6 +476,8 @@ __global__ void __launch_bounds__(256) k_project_apply(KrylovStore ks, const dou
 
 __global__ void k_pcg_p(double* __restrict__ p, const double* __restrict__ z, const double* __restrict__ scal,
                         int64_t n) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t o = (int64_t)blockIdx.y * n;
@@ -619,12 +642,12 @@ inline unsigned nblocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); 
 
 template <typename T>
 void launch_gather_iface(const LevelDev& L, const double* x, int weighted, T* loc, cudaStream_t st, int nr) {
-  if (L.n_vec > 0) { note_launch(); k_gather_iface<T><<<dim3(nblocks(L.n_vec, 256), nr), 256, 0, st>>>(L, x, weighted, loc); }
+  if (L.n_vec > 0) { note_launch(); launch_pdl(k_gather_iface<T>, dim3(nblocks(L.n_vec, 256), nr), 256, 0, st, L, x, weighted, loc); }
 }
 template <typename T>
 void launch_scatter_iface(const LevelDev& L, const T* loc, int weighted, double* y, cudaStream_t st, int nr,
                           const FusedDot& dot) {
-  if (L.n_iface > 0) { note_launch(); k_scatter_iface<T><<<dim3(nblocks(L.n_iface, 256), nr), 256, 0, st>>>(L, loc, weighted, y, dot); }
+  if (L.n_iface > 0) { note_launch(); launch_pdl(k_scatter_iface<T>, dim3(nblocks(L.n_iface, 256), nr), 256, 0, st, L, loc, weighted, y, dot); }
 }
 void launch_inner_gather(const LevelDev& L, const double* x, float* loc, const int32_t* crow_sub, int64_t total_rows,
                          double* t, cudaStream_t st, int nr) {
@@ -637,13 +660,13 @@ void launch_inner_gather(const LevelDev& L, const double* x, float* loc, const i
     double* ts = t + (int64_t)r0 * total_rows;
     note_launch();
     if (g == 8)
-      k_inner_gather<8><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+      launch_pdl(k_inner_gather<8>, nb, 256, 0, st, L, xs, ls, (int)nv, crow_sub, total_rows, ts);
     else if (g == 4)
-      k_inner_gather<4><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+      launch_pdl(k_inner_gather<4>, nb, 256, 0, st, L, xs, ls, (int)nv, crow_sub, total_rows, ts);
     else if (g == 2)
-      k_inner_gather<2><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+      launch_pdl(k_inner_gather<2>, nb, 256, 0, st, L, xs, ls, (int)nv, crow_sub, total_rows, ts);
     else
-      k_inner_gather<1><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+      launch_pdl(k_inner_gather<1>, nb, 256, 0, st, L, xs, ls, (int)nv, crow_sub, total_rows, ts);
     r0 += g;
   }
 }
@@ -651,7 +674,7 @@ void launch_inner_scatter(const LevelDev& L, const float* loc, const double* t, 
                           cudaStream_t st, int nr, const FusedDot& dot) {
   if (L.n_iface <= 0) return;
   note_launch();
-  k_inner_scatter<<<dim3(nblocks(L.n_iface, 256), nr), 256, 0, st>>>(L, loc, t, total_rows, y, dot);
+  launch_pdl(k_inner_scatter, dim3(nblocks(L.n_iface, 256), nr), 256, 0, st, L, loc, t, total_rows, y, dot);
 }
 void launch_constraint_positions(const LevelDev& L, const int32_t* crow_sub, int64_t total_rows, cudaStream_t st) {
   if (total_rows > 0) { note_launch(); k_constraint_positions<<<nblocks(total_rows, 8), 256, 0, st>>>(L, crow_sub, total_rows); }
@@ -673,7 +696,7 @@ void launch_spmv_nr(const LevelDev& L, const int64_t* rows, int64_t nrows, const
                     double beta, const int32_t* row_sub, cudaStream_t st) {
   constexpr int LR = 4;
   note_launch();
-  k_spmv<NR, LR><<<nblocks(nrows * LR, 256), 256, 0, st>>>(L, rows, nrows, x, y, alpha, beta, row_sub);
+  launch_pdl(k_spmv<NR, LR>, nblocks(nrows * LR, 256), 256, 0, st, L, rows, nrows, x, y, alpha, beta, row_sub);
 }
 void launch_spmv_rows(const LevelDev& L, const int64_t* rows, int64_t nrows, const double* x, double* y, double alpha,
                       double beta, const int32_t* row_sub, cudaStream_t st, int nr) {
@@ -695,20 +718,20 @@ void launch_spmv_rows(const LevelDev& L, const int64_t* rows, int64_t nrows, con
 }
 template <typename Tin, typename Tout>
 void launch_convert(const Tin* in, Tout* out, int64_t n, cudaStream_t st) {
-  if (n > 0) { note_launch(); k_convert<Tin, Tout><<<nblocks(n, 256), 256, 0, st>>>(in, out, n); }
+  if (n > 0) { note_launch(); launch_pdl(k_convert<Tin, Tout>, nblocks(n, 256), 256, 0, st, in, out, n); }
 }
 template <typename T>
 void launch_add_to_double(double* y, const T* x, int64_t n, cudaStream_t st) {
-  if (n > 0) { note_launch(); k_add_to_double<T><<<nblocks(n, 256), 256, 0, st>>>(y, x, n); }
+  if (n > 0) { note_launch(); launch_pdl(k_add_to_double<T>, nblocks(n, 256), 256, 0, st, y, x, n); }
 }
 void launch_axpy_loc(double* y, const double* x, double a, int64_t n, cudaStream_t st) {
-  if (n > 0) { note_launch(); k_axpy<<<nblocks(n, 256), 256, 0, st>>>(y, x, a, n); }
+  if (n > 0) { note_launch(); launch_pdl(k_axpy, nblocks(n, 256), 256, 0, st, y, x, a, n); }
 }
 void launch_coarse_gather(const LevelDev& L, const double* part, int zmax, double* rc_sub, int64_t sum_nc, double* rC,
                           float* v32, const int32_t* v32_pos, int64_t n_v32, cudaStream_t st, int nr) {
   if (L.n_coarse <= 0) return;
   note_launch();
-  k_coarse_gather<<<dim3(nblocks(L.n_coarse, 8), nr), 256, 0, st>>>(L, part, zmax, rc_sub, sum_nc, rC, v32, v32_pos, n_v32);
+  launch_pdl(k_coarse_gather, dim3(nblocks(L.n_coarse, 8), nr), 256, 0, st, L, part, zmax, rc_sub, sum_nc, rC, v32, v32_pos, n_v32);
 }
 void launch_coarse_scatter_n(const int32_t* sub_coarse, int64_t total, const double* zC, int64_t n_coarse,
                              double* zc_sub, cudaStream_t st, int nr) {
@@ -721,7 +744,7 @@ void launch_dot(const double* a, const double* b, int64_t n, double* partial, in
 }
 void launch_pcg_update_x_r(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
                            double* partial, int* cnt, const KrylovStore& ks, cudaStream_t st, int nr) {
-  if (n > 0) { note_launch(); k_pcg_xr<<<dim3(nblocks(n, 256), nr), 256, 0, st>>>(x, r, p, q, scal, n, partial, cnt, ks); }
+  if (n > 0) { note_launch(); launch_pdl(k_pcg_xr, dim3(nblocks(n, 256), nr), 256, 0, st, x, r, p, q, scal, n, partial, cnt, ks); }
 }
 void launch_project(const KrylovStore& ks, const double* g, double* x, double* r, int64_t n, double* coef,
                     cudaStream_t st, int nr) {
@@ -734,7 +757,7 @@ void launch_project(const KrylovStore& ks, const double* g, double* x, double* r
   k_project_apply<<<dim3(nblocks(n, 256), nr), 256, 0, st>>>(ks, g, x, r, n, coef);
 }
 void launch_pcg_update_p(double* p, const double* z, const double* scal, int64_t n, cudaStream_t st, int nr) {
-  if (n > 0) { note_launch(); k_pcg_p<<<dim3(nblocks(n, 256), nr), 256, 0, st>>>(p, z, scal, n); }
+  if (n > 0) { note_launch(); launch_pdl(k_pcg_p, dim3(nblocks(n, 256), nr), 256, 0, st, p, z, scal, n); }
 }
 void launch_grad_contract_slots(int64_t n_elems, int ne, const double* ke, const int32_t* slot_elem, const double* coef,
                                 const int32_t* conn, int ndof, const double* lam, const double* u, int nrhs,
