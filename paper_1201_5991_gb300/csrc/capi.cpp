@@ -189,7 +189,6 @@ struct Level {
   std::vector<int> block_tiles;    // per step k: update tiles inside the sub-panel's diagonal block
   std::vector<double> block_flops; // per step k: flops of the diagonal block's CUDA-core steps
   bool tc_panels = false;          // panel solves below the diagonal blocks on the tensor cores
-  float* xinv = nullptr;           // [n_sub][4 x 4 tiles] inverse of the current diagonal block
   // per 512-wide super-panel p and launch u of the tensor cores (0: rank-256 update of the second
   // half's columns, 1: rank-512 update of the trailing columns, 2: rank-256 update of all trailing
   // columns, 3 / 4: panel solve of the first / second half): 128 x 128 work items and
@@ -577,7 +576,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
   };
   L.level1 = &L == &h->lv[0];
   L.meta.resize(ns);
-  int64_t tile = 0, dinv = 0, vec = 0, coff = 0, goff = 0, psi = 0, psiT = 0, schur = 0, symv = 0;
+  int64_t tile = 0, dinv = 0, vec = 0, coff = 0, goff = 0, psi = 0, psiT = 0, schur = 0, symv = 0, xoff = 0;
   L.max_R = L.max_Bc = L.max_nc = L.max_nG = L.max_nGb = L.max_ncb = 0;
   // the explicit inner operator snapshots the trailing interface block when the interior is
   // eliminated; the batched factorisation reaches that point for every subdomain at a sub-panel
@@ -612,6 +611,8 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     tile += ((int64_t)m.Bc * (m.Bc + 1) / 2 + (int64_t)m.ncb * m.Bc) * NB2;
     m.inv_off = tile + (int64_t)m.nV * (m.nV + 1) / 2 * NB2;
     tile += (int64_t)m.nV * (m.nV + 1) * NB2;
+    m.x_off = xoff;
+    xoff += ceil_div(m.Bc, kSub) * 6 * NB2;
     m.dinv_off = dinv;
     dinv += (int64_t)m.Bc * NB2;
     m.vec_off = vec;
@@ -916,6 +917,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
       c_rho[t] = ((ms.rigid_mask >> mp.coarse_comp[mp.sub_coarse[t]]) & 1u) ? 1.0 : 0.0;
     d.c_rho = A.upload(c_rho, st);
   }
+  d.xinv = nullptr;
   d.indefinite = h->physics == BDDC_STOKES ? 1 : 0;
   d.wait_probe = h->opts.wait_probe ? 1 : 0;
   d.sgn = L.fp32 ? (void*)A.alloc<float>(L.n_vec) : (void*)A.alloc<double>(L.n_vec);
@@ -939,7 +941,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     if (h->physics == BDDC_STOKES) L.split_signed = A.alloc<uint8_t>(rows * kPanel * 2 * NB2 * 2);
     L.rscale = A.alloc<float>(rows * NB);
     L.tc_panels = h->opts.tensor_cores != 2;
-    if (L.tc_panels) L.xinv = A.alloc<float>(ns * 16 * NB2);
+    if (L.tc_panels) d.xinv = A.alloc<float>(xoff);
     // work items (128 x 128 output blocks) of the updates of every super-panel, flattened over the
     // subdomains; update 0 covers the columns [kb0 + kSub, kb0 + kPanel), update 1 the columns
     // >= kb0 + kPanel, update 2 (a super-panel where some interior ends in the middle, explicit
@@ -1134,10 +1136,10 @@ void factor_level(bddc_handle_s* h, Level& L, cudaStream_t st) {
             bool fused = false;
             for (int k = k0; k < std::min(k1, L.max_Bc); ++k) {
               const bool fuse = k + 1 < k1 && L.block_tiles[k] > 0;
-              launch_potrf_step<T>(d, k, L.max_R, L.block_tiles[k], k1, st, fused, fuse, k1, L.xinv, k0);
+              launch_potrf_step<T>(d, k, L.max_R, L.block_tiles[k], k1, st, fused, fuse, k1, 1, k0);
               fused = fuse;
             }
-            launch_split_inverse(d, k0, L.xinv, L.split, L.rscale, L.prow_off, st);
+            launch_split_inverse(d, k0, L.split, L.rscale, L.prow_off, st);
             launch_split_panel(d, k0, kSub, k1, k0, L.split_rows[kTcLaunches * p + 3 + half], L.split, nullptr,
                                L.rscale, L.prow_off, st, 1);
           }

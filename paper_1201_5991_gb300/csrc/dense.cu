@@ -325,9 +325,9 @@ __global__ void __launch_bounds__(256) k_trsm_panel16(LevelDev L, int k, int rli
 // the block's factorisation, by blocks of that step's in-block update launch (next to the one that
 // factors tile Q + 1).  One CTA of 256 threads takes 16 columns c0 .. c0 + 15 of X_QP (thread:
 // row r, columns cg .. cg + 3), the sums in ascending K and t; X_QP is stored as a row-major tile
-// at xinv + (s * 16 + 4 Q + P) * 4096 (the diagonal tiles X_QQ are read from the inverses).
-__device__ void xinv_row_part(const LevelDev& L, const SubMeta& m, int s, int k0, int Q, int P, int c0,
-                              float* __restrict__ xinv, unsigned char* smem_raw) {
+// at x_tile(k0, Q, P) (the diagonal tiles X_QQ are read from the inverses).
+__device__ void xinv_row_part(const LevelDev& L, const SubMeta& m, int k0, int Q, int P, int c0,
+                              unsigned char* smem_raw) {
   float(*Ls)[NB + 1] = (float(*)[NB + 1])smem_raw;                               // L_QK, then L_QQ^{-1}
   float(*Xk)[16] = (float(*)[16])(smem_raw + sizeof(float) * NB * (NB + 1));     // X_KP(:, c0 ..)
   float(*Ts)[16] = (float(*)[16])(smem_raw + sizeof(float) * NB * (NB + 1 + 16));
@@ -336,7 +336,7 @@ __device__ void xinv_row_part(const LevelDev& L, const SubMeta& m, int s, int k0
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
   for (int K = P; K < Q; ++K) {   // T = sum_K L_QK X_KP
     const float* lq = tile_ptr<float>(m, L.tiles, k0 + Q, k0 + K);
-    const float* xk = K == P ? dinv + (int64_t)(k0 + P) * NB2 : xinv + ((int64_t)s * 16 + 4 * K + P) * NB2;
+    const float* xk = K == P ? dinv + (int64_t)(k0 + P) * NB2 : L.xinv + x_tile(m, k0, K, P);
     for (int e = tid; e < NB2; e += blockDim.x) Ls[e >> 6][e & 63] = lq[e];
     for (int e = tid; e < NB * 16; e += blockDim.x) Xk[e >> 4][e & 15] = xk[(e >> 4) * NB + c0 + (e & 15)];
     __syncthreads();
@@ -364,7 +364,7 @@ __device__ void xinv_row_part(const LevelDev& L, const SubMeta& m, int s, int k0
     y[2] += a * x.z;
     y[3] += a * x.w;
   }
-  float* dst = xinv + ((int64_t)s * 16 + 4 * Q + P) * NB2 + r * NB + c0 + cg;
+  float* dst = L.xinv + x_tile(m, k0, Q, P) + r * NB + c0 + cg;
   *(float4*)dst = make_float4(-y[0], -y[1], -y[2], -y[3]);
 }
 
@@ -375,7 +375,7 @@ __device__ void xinv_row_part(const LevelDev& L, const SubMeta& m, int s, int k0
 // solves): the blocks n_upd .. n_upd + 4 xq - 1 of the grid form block row xq = k - k0 of the
 // inverse of the diagonal block [k0, k0 + 4) (block column P = e / 4, columns 16 (e % 4) ..).
 template <typename T>
-__global__ void k_syrk_update(LevelDev L, int k, int jmax, int fuse_next, int rlim, int n_upd, float* xinv,
+__global__ void k_syrk_update(LevelDev L, int k, int jmax, int fuse_next, int rlim, int n_upd, int xinv,
                               int k0) {
   const int s = blockIdx.y;
   const SubMeta m = L.meta[s];
@@ -383,7 +383,7 @@ __global__ void k_syrk_update(LevelDev L, int k, int jmax, int fuse_next, int rl
     if constexpr (sizeof(T) == 4) {
       const int e = (int)blockIdx.x - n_upd, Q = k - k0;
       extern __shared__ __align__(16) unsigned char smem_raw[];
-      if (xinv && Q < m.Bc - k0) xinv_row_part(L, m, s, k0, Q, e >> 2, 16 * (e & 3), xinv, smem_raw);
+      if (xinv && Q < m.Bc - k0) xinv_row_part(L, m, k0, Q, e >> 2, 16 * (e & 3), smem_raw);
     }
     return;
   }
@@ -1216,7 +1216,7 @@ void launch_coarse_apply(const float* W, int64_t npad, const float* x, double* z
 
 template <typename T>
 void launch_potrf_step(const LevelDev& L, int k, int max_R, int max_tiles, int jmax, cudaStream_t st, int skip_diag,
-                       int fuse_next, int rlim, float* xinv, int k0) {
+                       int fuse_next, int rlim, int xinv, int k0) {
   const unsigned ns = (unsigned)L.n_sub;
   const size_t sm = 2 * NB * LDS * sizeof(T);
   const size_t sm_diag = 2 * NB * (NB + 1) * sizeof(T);
@@ -1391,7 +1391,7 @@ void launch_psi_transpose(const LevelDev& L, int max_nGb, int max_ncb, cudaStrea
 }
 
 #define INST(T)                                                                                 \
-  template void launch_potrf_step<T>(const LevelDev&, int, int, int, int, cudaStream_t, int, int, int, float*, int); \
+  template void launch_potrf_step<T>(const LevelDev&, int, int, int, int, cudaStream_t, int, int, int, int, int); \
   template void launch_psi<T>(const LevelDev&, int, int, cudaStream_t);                          \
   template void launch_constraint_corr<T>(const LevelDev&, T*, const int32_t*, int64_t, double*, double*, double*, \
                                          int, int, cudaStream_t, int);                                     \

@@ -46,6 +46,7 @@ struct SubMeta {
   int64_t psi_off;                // offset of Psi_G (nGb*NB rows x nc, row-major)
   int64_t psiT_off;               // offset of Psi_G^T as ncb x nGb tiles (set-up copy for the solve phase)
   int64_t inv_off;                // offset of the tiles of -A_GG^{-1} (row-major lower triangle) in the tile buffer
+  int64_t x_off;                  // offset of the off-diagonal tiles of the 256-wide diagonal blocks' inverses
   int64_t schur_off;              // offset of the explicit augmented Schur complement (nGb (nGb+1)/2 tiles)
 };
 
@@ -62,6 +63,11 @@ __host__ __device__ inline int64_t tile_of(const SubMeta& m, int i, int j) {
 
 __host__ __device__ inline bool tile_exists(const SubMeta& m, int i, int j) {
   return j <= i && (i < m.R || j >= m.R || j - m.nIb >= i - m.R);
+}
+
+// tile (Q, P), P < Q < 4, of the inverse of the diagonal block that starts at block column k0 (a multiple of 4)
+__host__ __device__ inline int64_t x_tile(const SubMeta& m, int k0, int Q, int P) {
+  return m.x_off + ((int64_t)(k0 / 4) * 6 + Q * (Q - 1) / 2 + P) * NB2;
 }
 
 // Raw device pointers of one level, passed by value to kernels.
@@ -110,6 +116,8 @@ struct LevelDev {
   void* dinv;                     // diagonal inverses
   void* psi;                      // Psi_G
   void* psiT;                     // Psi_G^T in tiles: tile (rb, j) of a subdomain at psiT_off + (rb nGb + j) NB2
+  float* xinv;                    // FP32 levels with tensor-core panels, or null: of every 256-wide diagonal block
+                                  // D = [4 d, 4 d + 4) the tiles (Q, P), P < Q, of X = L_D^{-1} (x_tile)
   float* schur;                   // explicit augmented Schur complement of the interface (mixed inner operator), or null
   void* sgn;                      // [n_vec] pivot signs of the signed Cholesky (T; +1 for SPD levels)
   int32_t* crow;                  // [n_vec] constraint row of a position (flat over the level) or -1 (level 1, FP32), or null
@@ -167,13 +175,13 @@ void launch_weights(const LevelDev& L, int multiplicity, const double* unused, c
 // fuse_next: the update's block for tile (k+1, k+1) factors it (only when max_tiles > 0 and
 // k + 1 < jmax, i.e. that tile receives its last update in this step).
 // rlim > 0: the rows of the diagonal block only (i < min(rlim, Bc) in the panel and the update).
-// xinv (FP32, rlim = k0 + 4): the step also forms block row k - k0 of X = L_D^{-1}, the inverse of
+// xinv = 1 (FP32, rlim = k0 + 4): the step also forms block row k - k0 of X = L_D^{-1}, the inverse of
 // the diagonal block D = [k0, k0 + nd) (nd = min(4, Bc - k0)), X_QP = -X_QQ sum_{P <= K < Q} L_QK X_KP
-// for P < Q, as row-major 64 x 64 tiles at xinv + (s * 16 + 4 Q + P) * 4096 (X_QQ = L_QQ^{-1} stays
-// in the stored inverses); a step with no in-block update tiles then launches for X alone.
+// for P < Q, as row-major 64 x 64 tiles at L.xinv + x_tile(k0, Q, P) (X_QQ = L_QQ^{-1} stays in the
+// stored inverses); a step with no in-block update tiles then launches for X alone.
 template <typename T>
 void launch_potrf_step(const LevelDev& L, int k, int max_R, int max_tiles, int jmax, cudaStream_t st,
-                       int skip_diag = 0, int fuse_next = 0, int rlim = 0, float* xinv = nullptr, int k0 = 0);
+                       int skip_diag = 0, int fuse_next = 0, int rlim = 0, int xinv = 0, int k0 = 0);
 // update_tc.cu, FP32 levels with tensor cores: rank-(64 nt) update of the output columns
 // ib <= j < jend from the nt panel tile columns kb0 .. kb0+nt-1 (nt = 4 or 8).  k_split_panel
 // writes the two scaled FP16 parts of the panel tiles L(i, kb0 + q), i >= ib, at
@@ -198,7 +206,7 @@ void launch_split_panel(const LevelDev& L, int kb0, int nt, int ib, int act, int
 // The B operand of a sub-panel's panel solve L(i, D) = A(i, D) X^T S_D: the rows of -S_D X (block
 // row Q of xinv and L_QQ^{-1}, pivot signs of the block's columns) split like the panel rows into
 // the split rows prow_off[s] + k0 + Q, tile columns 0 .. 3, with their unscaling factors in rscale.
-void launch_split_inverse(const LevelDev& L, int k0, const float* xinv, uint8_t* split, float* rscale,
+void launch_split_inverse(const LevelDev& L, int k0, uint8_t* split, float* rscale,
                           const int64_t* prow_off, cudaStream_t st);
 // The update adds its output into the tiles with TMA reduce-adds through this tensor map: the
 // FP32 tile buffer viewed as [tile_elems / 64 rows][64 columns], 32 x 32 boxes, 128-byte
@@ -238,7 +246,7 @@ void launch_coarse_apply(const float* W, int64_t npad, const float* x, double* z
 template <typename T>
 void launch_sweep(const LevelDev& L, T* vec, const int2* const* tasks, const int* ntasks, int part, int which,
                   void* scratch, int grid_max, int deep, cudaStream_t st, int nr = 1);
-inline int64_t sweep_scratch_bytes(int64_t n_vec, int blk) { return 64 + 2 * 8 * n_vec * (blk < 8 ? blk : 8); }
+inline int64_t sweep_scratch_bytes(int64_t n_vec, int blk) { return 64 + 4 * 8 * n_vec * (blk < 8 ? blk : 8); }
 // crow_sub: subdomain of every constraint row (flat over the level); t, mu: scratch [nr][total_rows]
 template <typename T>
 void launch_constraint_corr(const LevelDev& L, T* vec, const int32_t* crow_sub, int64_t total_rows, double* t,

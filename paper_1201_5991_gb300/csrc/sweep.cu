@@ -110,13 +110,19 @@ struct Vec2<double> {
 };
 
 // One task: (subdomain, block row).  Forward consumes tiles (i, B0..i-1) then D_i^{-1};
-// backward consumes tiles (B1-1..i+1, i) then D_i^{-1}.  NR right-hand sides are solved together
+// backward consumes tiles (B1-1..i+1, i) then D_i^{-1}.
+// GRP (interior sweeps of levels that keep the inverses X_D of their 256-wide diagonal blocks
+// D = [g0, g0 + 4)): row g0 + Q consumes the tiles left of its block, publishes its remaining right-hand side
+// r'_Q (p2), and then y_Q = sum_{P <= Q} X_QP r'_P (backward: X_PQ^T, P >= Q) with the other rows' r'.  The rows of
+// a block no longer wait for one another's solutions: two dependent L2 round trips per four block rows
+// instead of four.  It matters where the chain bounds the sweep: 8 subdomains of 81 interior block rows
+// took 1.3 us per row, 100 us for bytes of 47.  NR right-hand sides are solved together
 // (column r at vec + r * vstride): every factor tile is streamed from HBM once per task and
 // applied to all of them from shared memory.
-template <typename T, int S, bool BWD, int NR>
+template <typename T, int S, bool BWD, int NR, bool GRP>
 __global__ void __launch_bounds__(kThreads, 2)
     k_sweep(LevelDev L, T* __restrict__ vec, int64_t vstride, const int2* __restrict__ tasks, int ntasks, int part,
-            int* __restrict__ ctrl, T* pub) {
+            int* __restrict__ ctrl, T* pub, T* pub2) {
   using V2 = typename Vec2<T>::type;
   constexpr int YS = NR == 1 ? kYSlots : (NR == 2 ? 8 : 4);   // solution blocks staged at a time
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -138,6 +144,9 @@ __global__ void __launch_bounds__(kThreads, 2)
   __syncthreads();
   pdl_wait();
   pdl_trigger();
+  constexpr int NV = 8 * NR, NC = NV < 32 ? 1 : NV / 32;   // row sums (lane_sums)
+  const int f0 = lane_sum_index<NV>(lane);
+  const bool writer = lane_sum_writer<NV>(lane);
   uint32_t cons = 0;     // tiles consumed by this CTA (ring position and phase)
   uint32_t issued = 0;   // tiles issued (thread 0)
   bool lost = false;     // a tile wait gave up: drain before exit
@@ -152,15 +161,18 @@ __global__ void __launch_bounds__(kThreads, 2)
     // interior part: the block rows that hold interior DOFs (padding identity block rows, whose
     // rows and columns of L are unit vectors and whose right-hand sides are zero, are skipped)
     const int B0 = part == 0 ? 0 : m.nIb, B1 = part == 0 ? (m.nI + NB - 1) / NB : m.Bc;
-    const int nL = BWD ? (B1 - 1 - i) : (i - B0);   // factor tiles before D_i^{-1}
-    const int ntile = nL + 1;
+    const int g0 = GRP ? (i & ~3) : i, g1 = GRP ? (g0 + 4 < B1 ? g0 + 4 : B1) : i + 1;   // the row's diagonal block
+    const int nL = BWD ? (B1 - g1) : (g0 - B0);           // factor tiles beside the diagonal block
+    const int ntile = BWD ? (B1 - i) : (i - B0 + 1);      // and its inverse's tiles, D_i^{-1} last
     const T* tiles = (const T*)L.tiles + m.tile_off;
     const T* dinv = (const T*)L.dinv + m.dinv_off + (int64_t)i * NB2;
     T* v = vec + m.vec_off;
     T* pv = pub + m.vec_off;   // this subdomain's published blocks (same layout as v)
+    T* p2 = GRP ? pub2 + m.vec_off : nullptr;   // and remaining right-hand sides
     auto tile_src = [&](int k) -> const T* {
-      if (k == nL) return dinv;
+      if (k == ntile - 1) return dinv;
       const int j = BWD ? (B1 - 1 - k) : (B0 + k);
+      if (GRP && k >= nL) return (const T*)L.xinv + (BWD ? x_tile(m, g0, j - g0, i - g0) : x_tile(m, g0, i - g0, j - g0));
       return BWD ? tiles + tile_index(j, i, m.Bc) * NB2 : tiles + tile_index(i, j, m.Bc) * NB2;
     };
     // the task's own right-hand side block depends on no other task: read it into rhs now, off
@@ -187,11 +199,46 @@ __global__ void __launch_bounds__(kThreads, 2)
     for (int q = 0; q < NR; ++q) accc[q][0] = accc[q][1] = (T)0;
     int staged_end = 0;   // tiles [staged_begin, staged_end) have their solution block in ybuf
     for (int k = 0; k < ntile; ++k) {
-      if (k < nL && k >= staged_end) {
+      if (k == nL) {
+        // the factor's part is complete: the remaining right-hand side of the row
+        if (!BWD) {
+          lane_sums<NV>(&acc[0][0], lane);   // N = 8 NR values per lane: value 8 q + r is row warp + 8 r of column q
+          if (writer)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) rhs[(f0 + c) / 8][warp + 8 * ((f0 + c) % 8)] -= (&acc[0][0])[c];
+#pragma unroll
+          for (int q = 0; q < NR; ++q)
+#pragma unroll
+            for (int r = 0; r < 8; ++r) acc[q][r] = (T)0;
+          __syncthreads();
+        } else {
+#pragma unroll
+          for (int q = 0; q < NR; ++q) {
+            red[warp][q][2 * lane] = accc[q][0];
+            red[warp][q][2 * lane + 1] = accc[q][1];
+            accc[q][0] = accc[q][1] = (T)0;
+          }
+          __syncthreads();
+          for (int e = tid; e < NR * NB; e += kThreads) {
+            const int q = e / NB, c = e % NB;
+            T a = (T)0;
+#pragma unroll
+            for (int w = 0; w < kThreads / 32; ++w) a += red[w][q][c];
+            rhs[q][c] -= a;
+          }
+          __syncthreads();
+        }
+        if (GRP && g1 - g0 > 1 && i != (BWD ? g0 : g1 - 1))
+          for (int e = tid; e < NR * NB; e += kThreads)
+            pub_st(p2 + (e / NB) * vstride + i * NB + e % NB, rhs[e / NB][e % NB]);
+      }
+      if (k < ntile - 1 && k >= staged_end) {
         // wait until the next solution blocks are published, then stage up to YS of them: warp w
         // polls blocks k + w and k + w + 8 (all their words at once), writes the ready ones into
         // ybuf, and the consecutive ready blocks from k are staged
-        const int want = nL - k < YS ? nL - k : YS;
+        const int upto = k < nL ? nL : ntile - 1;   // factor tiles, then the inverse's
+        const int want = upto - k < YS ? upto - k : YS;
+        const T* pb = k < nL ? pv : p2;
         int cnt = 0;
         long long spins = 0;
         for (;;) {
@@ -201,13 +248,13 @@ __global__ void __launch_bounds__(kThreads, 2)
             V2 y[NR];
             bool ok = true;
 #pragma unroll
-            for (int q = 0; q < NR; ++q) ok &= pub_ld2(pv + q * vstride + j * NB + 2 * lane, y[q]);
+            for (int q = 0; q < NR; ++q) ok &= pub_ld2(pb + q * vstride + j * NB + 2 * lane, y[q]);
             // the timeout probe waits for a word that nothing sets (status[3]) instead
             if (L.wait_probe) ok = ld_acquire(status + 3) != 0;
             ok = __all_sync(0xffffffffu, ok);
             if (ok) {
               V2 sg = {(T)1, (T)1};
-              if (!BWD && L.indefinite)   // solved rows hold S_j y_j: the update needs y_j
+              if (!BWD && L.indefinite && k < nL)   // solved rows hold S_j y_j: the update needs y_j
                 sg = *(const V2*)((const T*)L.sgn + m.vec_off + (int64_t)j * NB + 2 * lane);
 #pragma unroll
               for (int q = 0; q < NR; ++q) {
@@ -244,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
       }
       const T* tl = stage + slot * NB2;
-      if (k < nL) {
+      if (k < ntile - 1) {
         const int ys = k % YS;
         if (!BWD) {
           V2 a[8];
@@ -270,22 +317,13 @@ __global__ void __launch_bounds__(kThreads, 2)
           }
         }
       } else {
-        // diagonal block: right-hand side, then D_i^{-1} (forward) or D_i^{-T} (backward)
+        // the diagonal tile's inverse on the row's own right-hand side: D_i^{-1} (forward), D_i^{-T} (backward).
+        // The sums over the lanes end a link of the dependency chain; as one butterfly per value
+        // they bound the forward sweep where the factor is small or FP64 (64 subdomains of 6^3
+        // elements, FP64 interior: 166 us against 54 us for the backward sweep).  Whole calls with
+        // lane_sums instead: FP64 24^3 elasticity 84.6 -> 73.9 ms, FP32 solve of 24^3 (8 subdomains)
+        // 18.3 -> 15.5 ms, FP64 operator on 8 columns (48^3) 9.61 -> 7.94 ms, same bits
         if (!BWD) {
-          // the row sums over the lanes (N = 8 NR values per lane): value 8 q + r is row warp + 8 r of
-          // right-hand side q.  They end a link of the dependency chain; as one butterfly per value
-          // they bound the forward sweep where the factor is small or FP64 (64 subdomains of 6^3
-          // elements, FP64 interior: 166 us against 54 us for the backward sweep).  Whole calls with
-          // lane_sums instead: FP64 24^3 elasticity 84.6 -> 73.9 ms, FP32 solve of 24^3 (8 subdomains)
-          // 18.3 -> 15.5 ms, FP64 operator on 8 columns (48^3) 9.61 -> 7.94 ms, same bits
-          constexpr int NV = 8 * NR, NC = NV < 32 ? 1 : NV / 32;
-          const int f0 = lane_sum_index<NV>(lane);
-          const bool writer = lane_sum_writer<NV>(lane);
-          lane_sums<NV>(&acc[0][0], lane);
-          if (writer)
-#pragma unroll
-            for (int k = 0; k < NC; ++k) rhs[(f0 + k) / 8][warp + 8 * ((f0 + k) % 8)] -= (&acc[0][0])[k];
-          __syncthreads();
           const bool signed_rows = L.indefinite != 0;   // forward output is S L^{-1} b
           V2 a[8];
 #pragma unroll
@@ -294,51 +332,33 @@ __global__ void __launch_bounds__(kThreads, 2)
           for (int q = 0; q < NR; ++q) {
             const V2 rv = *(const V2*)(&rhs[q][2 * lane]);
 #pragma unroll
-            for (int r = 0; r < 8; ++r) acc[q][r] = a[r].x * rv.x + a[r].y * rv.y;
+            for (int r = 0; r < 8; ++r) acc[q][r] += a[r].x * rv.x + a[r].y * rv.y;
           }
           lane_sums<NV>(&acc[0][0], lane);
           if (writer)
 #pragma unroll
-            for (int k = 0; k < NC; ++k) {
-              const int q = (f0 + k) / 8, row = warp + 8 * ((f0 + k) % 8);
-              const T yv = (&acc[0][0])[k];
+            for (int c = 0; c < NC; ++c) {
+              const int q = (f0 + c) / 8, row = warp + 8 * ((f0 + c) % 8);
+              const T yv = (&acc[0][0])[c];
               const T out = signed_rows ? yv * s_sg[row] : yv;
               v[q * vstride + i * NB + row] = out;
               pub_st(pv + q * vstride + i * NB + row, out);
             }
         } else {
 #pragma unroll
-          for (int q = 0; q < NR; ++q) {
-            red[warp][q][2 * lane] = accc[q][0];
-            red[warp][q][2 * lane + 1] = accc[q][1];
-          }
-          __syncthreads();
-          for (int e = tid; e < NR * NB; e += kThreads) {
-            const int q = e / NB, c = e % NB;
-            T a = (T)0;
-#pragma unroll
-            for (int w = 0; w < kThreads / 32; ++w) a += red[w][q][c];
-            rhs[q][c] -= a;
-          }
-          __syncthreads();
-          T p[NR][2];
-#pragma unroll
-          for (int q = 0; q < NR; ++q) p[q][0] = p[q][1] = (T)0;
-#pragma unroll
           for (int r = 0; r < 8; ++r) {
             const int row = warp + 8 * r;
             const V2 a = *(const V2*)(tl + row * NB + 2 * lane);
 #pragma unroll
             for (int q = 0; q < NR; ++q) {
-              p[q][0] += a.x * rhs[q][row];
-              p[q][1] += a.y * rhs[q][row];
+              accc[q][0] += a.x * rhs[q][row];
+              accc[q][1] += a.y * rhs[q][row];
             }
           }
-          __syncthreads();
 #pragma unroll
           for (int q = 0; q < NR; ++q) {
-            red[warp][q][2 * lane] = p[q][0];
-            red[warp][q][2 * lane + 1] = p[q][1];
+            red[warp][q][2 * lane] = accc[q][0];
+            red[warp][q][2 * lane + 1] = accc[q][1];
           }
           __syncthreads();
           for (int e = tid; e < NR * NB; e += kThreads) {
@@ -375,38 +395,54 @@ __global__ void __launch_bounds__(kThreads, 2)
 }  // namespace
 
 // Task lists and the scratch buffer live in the level (see capi.cpp).  scratch: two task counters (forward,
-// backward) in its first 64 bytes, then a publication buffer for either direction, n_vec NR words of T each; one
+// backward) in its first 64 bytes, then the publication buffers of either direction (solutions, with GRP also the
+// remaining right-hand sides), n_vec NR words of T each; one
 // memset to all ones resets what a launch uses (counters start at -1).  A pair resets both directions at
 // once and its backward sweep is launched over the forward sweep's end (pdl.cuh): per pair one memset
 // instead of four, each 1.5 to 2 us between short sweeps.
-template <typename T, int S, int NR>
+template <typename T, int S, int NR, bool GRP>
 void launch_sweep_s(const LevelDev& L, T* vec, const int2* const* tasks, const int* ntasks, int part, int which,
                     void* scratch, int grid_max, cudaStream_t st) {
   const size_t dyn = (size_t)S * NB2 * sizeof(T);
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_sweep<T, S, false, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    cudaFuncSetAttribute(k_sweep<T, S, true, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    cudaFuncSetAttribute(k_sweep<T, S, false, NR, GRP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    cudaFuncSetAttribute(k_sweep<T, S, true, NR, GRP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     attr = true;
   }
-  const size_t words = (size_t)L.n_vec * NR;
+  const size_t words = (size_t)L.n_vec * NR, dir = words * (GRP ? 2 : 1);   // published words per direction
   int* ctrl = (int*)scratch;
   T* pub = (T*)((char*)scratch + 64);
-  cudaMemsetAsync(scratch, 0xFF, 64 + sizeof(T) * words * (which == 2 ? 2 : 1), st);
+  cudaMemsetAsync(scratch, 0xFF, 64 + sizeof(T) * dir * (which == 2 ? 2 : 1), st);
   if (which != 1) {
     note_launch();
-    k_sweep<T, S, false, NR><<<ntasks[0] < grid_max ? ntasks[0] : grid_max, kThreads, dyn, st>>>(
-        L, vec, L.n_vec, tasks[0], ntasks[0], part, ctrl, pub);
+    k_sweep<T, S, false, NR, GRP><<<ntasks[0] < grid_max ? ntasks[0] : grid_max, kThreads, dyn, st>>>(
+        L, vec, L.n_vec, tasks[0], ntasks[0], part, ctrl, pub, pub + words);
   }
   if (which == 2) {
     note_launch();
-    launch_pdl(k_sweep<T, S, true, NR>, ntasks[1] < grid_max ? ntasks[1] : grid_max, kThreads, dyn, st, L, vec,
-               (int64_t)L.n_vec, tasks[1], ntasks[1], part, ctrl + 1, pub + words);
+    launch_pdl(k_sweep<T, S, true, NR, GRP>, ntasks[1] < grid_max ? ntasks[1] : grid_max, kThreads, dyn, st, L, vec,
+               (int64_t)L.n_vec, tasks[1], ntasks[1], part, ctrl + 1, pub + dir, pub + dir + words);
   } else if (which == 1) {
     note_launch();
-    k_sweep<T, S, true, NR><<<ntasks[1] < grid_max ? ntasks[1] : grid_max, kThreads, dyn, st>>>(
-        L, vec, L.n_vec, tasks[1], ntasks[1], part, ctrl, pub);
+    k_sweep<T, S, true, NR, GRP><<<ntasks[1] < grid_max ? ntasks[1] : grid_max, kThreads, dyn, st>>>(
+        L, vec, L.n_vec, tasks[1], ntasks[1], part, ctrl, pub, pub + words);
   }
+}
+
+template <typename T, int S, int NR>
+void launch_sweep_g(const LevelDev& L, T* vec, const int2* const* tasks, const int* ntasks, int part, int which,
+                    void* scratch, int grid_max, cudaStream_t st) {
+  // Up to two columns, where the chain of block rows counts: 24^3 solve (8 subdomains) 8.41 -> 7.50 ms, tetrahedra
+  // 11.4 -> 10.9, 48^3 (bound by HBM) as before.  With eight columns the tiles' products bound the sweep and
+  // the extra exchange costs: FP64 operator on 8 columns (48^3) 5.97 -> 6.19 ms, so those keep single rows.
+  if constexpr (sizeof(T) == 4 && NR <= 2) {
+    if (part == 0 && L.xinv) {   // the inverses of the 256-wide diagonal blocks are at hand
+      launch_sweep_s<T, S, NR, true>(L, vec, tasks, ntasks, part, which, scratch, grid_max, st);
+      return;
+    }
+  }
+  launch_sweep_s<T, S, NR, false>(L, vec, tasks, ntasks, part, which, scratch, grid_max, st);
 }
 
 template <typename T, int S>
@@ -419,13 +455,13 @@ void launch_sweep_nr(const LevelDev& L, T* vec, const int2* const* tasks, const 
     const int g = left >= kMaxNR ? kMaxNR : left >= 4 ? 4 : left >= 2 ? 2 : 1;
     T* v = vec + (int64_t)r0 * L.n_vec;
     if (g == 8)
-      launch_sweep_s<T, S, (sizeof(T) == 4 ? 8 : 4)>(L, v, tasks, ntasks, part, which, scratch, grid_max, st);
+      launch_sweep_g<T, S, (sizeof(T) == 4 ? 8 : 4)>(L, v, tasks, ntasks, part, which, scratch, grid_max, st);
     else if (g == 4)
-      launch_sweep_s<T, S, 4>(L, v, tasks, ntasks, part, which, scratch, grid_max, st);
+      launch_sweep_g<T, S, 4>(L, v, tasks, ntasks, part, which, scratch, grid_max, st);
     else if (g == 2)
-      launch_sweep_s<T, S, 2>(L, v, tasks, ntasks, part, which, scratch, grid_max, st);
+      launch_sweep_g<T, S, 2>(L, v, tasks, ntasks, part, which, scratch, grid_max, st);
     else
-      launch_sweep_s<T, S, 1>(L, v, tasks, ntasks, part, which, scratch, grid_max, st);
+      launch_sweep_g<T, S, 1>(L, v, tasks, ntasks, part, which, scratch, grid_max, st);
     r0 += g;
   }
 }

@@ -152,8 +152,7 @@ __global__ void __launch_bounds__(64 * NT) k_split_panel(LevelDev L, int kb0, in
 
 // one block per block row Q of the inverse X of every subdomain's diagonal block (Q < nd): the
 // rows of -S_D X, the B operand of the panel solve (its update kernel subtracts A B^T)
-__global__ void __launch_bounds__(256) k_split_inverse(LevelDev L, int k0, const float* __restrict__ xinv,
-                                                       uint8_t* __restrict__ split, float* __restrict__ rscale,
+__global__ void __launch_bounds__(256) k_split_inverse(LevelDev L, int k0, uint8_t* __restrict__ split, float* __restrict__ rscale,
                                                        const int64_t* __restrict__ prow_off) {
   const int s = blockIdx.y, Q = blockIdx.x;
   const SubMeta m = L.meta[s];
@@ -164,7 +163,7 @@ __global__ void __launch_bounds__(256) k_split_inverse(LevelDev L, int k0, const
   if (threadIdx.x < NB) rm[threadIdx.x] = sg[threadIdx.x] < 0.f ? 1.f : -1.f;   // -s_r
   __syncthreads();
   const int c = threadIdx.x >> 6;   // block column of X; zero above the diagonal blocks
-  const float* src = c < Q    ? xinv + ((int64_t)s * 16 + Q * 4 + c) * NB2
+  const float* src = c < Q    ? L.xinv + x_tile(m, k0, Q, c)
                      : c == Q ? (const float*)L.dinv + m.dinv_off + (int64_t)(k0 + Q) * NB2
                               : nullptr;
   split_rows<4>(src, rm, prow_off[s] + k0 + Q, split, nullptr, rscale, nullptr);
@@ -511,11 +510,11 @@ void launch_split_panel(const LevelDev& L, int kb0, int nt, int ib, int act, int
     k_split_panel<4><<<grid, 256, 0, st>>>(L, kb0, ib, act, panel_operand, split, split_signed, rscale, prow_off);
 }
 
-void launch_split_inverse(const LevelDev& L, int k0, const float* xinv, uint8_t* split, float* rscale,
+void launch_split_inverse(const LevelDev& L, int k0, uint8_t* split, float* rscale,
                           const int64_t* prow_off, cudaStream_t st) {
   if (L.n_sub <= 0) return;
   note_launch();
-  k_split_inverse<<<dim3(4, (unsigned)L.n_sub), 256, 0, st>>>(L, k0, xinv, split, rscale, prow_off);
+  k_split_inverse<<<dim3(4, (unsigned)L.n_sub), 256, 0, st>>>(L, k0, split, rscale, prow_off);
 }
 
 void launch_update_tc2(const LevelDev& L, int nq, int jbeg, int jend, int ibeg, int panel, int act, int grid,
