@@ -137,7 +137,7 @@ typedef struct {
                                results of such a call are meaningless; the CUDA context stays usable).
                                Tile-copy waits are not affected. */
   int inner_operator;       /* mixed PCG, inner operator S~ of the outer refinement: 0 = automatic
-                               (the explicit form when the interior padding it needs adds at most 8 %
+                               (the explicit form when the interior padding it needs adds at most 40 %
                                to the interior factor, else the factor products), 1 = products with
                                the stored interface factor, S~ x = L_GG S L_GG^T x - C^T R C x,
                                2 = the explicit augmented Schur complement S_i + C_i^T R C_i, copied

@@ -581,6 +581,11 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
   // the explicit inner operator snapshots the trailing interface block when the interior is
   // eliminated; the batched factorisation reaches that point for every subdomain at a sub-panel
   // boundary only if the interior block count is a multiple of kSub (identity tiles pad it)
+  // automatic: where the padding adds at most 40 % to the interior triangle.  The padded tiles cost tensor-core
+  // time of the set-up only (the sweeps skip them; 216 subdomains of 8^3 elements: 0.3 ms), while the factor
+  // products read the interface triangle twice per inner iteration, in two dependent launches: one pass
+  // took the 24^3 tetrahedra's solve from 10.9 to 7.8 ms, 64^3 with 16 loads from 495 to 449, a design step
+  // with 8 loads from 251 to 228 ms.  Interiors of a few tiles (6 -> 8: 71 %) keep the factor products.
   L.explicit_schur = false;
   if (&L == &h->lv[0] && L.fp32 && h->opts.tensor_cores && h->physics != BDDC_STOKES &&
       krylov_kind(h) == BDDC_KRYLOV_PCG && h->opts.inner_operator != 1) {
@@ -590,7 +595,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
       base += b * (b + 1) / 2;
       padded += bp * (bp + 1) / 2;
     }
-    L.explicit_schur = h->opts.inner_operator == 2 || padded <= 1.08 * base;
+    L.explicit_schur = h->opts.inner_operator == 2 || padded <= 1.4 * base;
   }
   // the interface inverse comes with the tensor-core factorisation (its panel solves carry the inverse rows)
   L.inverse = L.fp32 && !L.coarsest && h->opts.tensor_cores && h->opts.tensor_cores != 2;

@@ -206,10 +206,11 @@ __global__ void __launch_bounds__(kThreads, 2)
           if (writer)
 #pragma unroll
             for (int c = 0; c < NC; ++c) rhs[(f0 + c) / 8][warp + 8 * ((f0 + c) % 8)] -= (&acc[0][0])[c];
+          if constexpr (GRP)
 #pragma unroll
-          for (int q = 0; q < NR; ++q)
+            for (int q = 0; q < NR; ++q)
 #pragma unroll
-            for (int r = 0; r < 8; ++r) acc[q][r] = (T)0;
+              for (int r = 0; r < 8; ++r) acc[q][r] = (T)0;
           __syncthreads();
         } else {
 #pragma unroll
@@ -332,7 +333,10 @@ __global__ void __launch_bounds__(kThreads, 2)
           for (int q = 0; q < NR; ++q) {
             const V2 rv = *(const V2*)(&rhs[q][2 * lane]);
 #pragma unroll
-            for (int r = 0; r < 8; ++r) acc[q][r] += a[r].x * rv.x + a[r].y * rv.y;
+            for (int r = 0; r < 8; ++r) {
+              const T d = a[r].x * rv.x + a[r].y * rv.y;
+              acc[q][r] = GRP ? acc[q][r] + d : d;
+            }
           }
           lane_sums<NV>(&acc[0][0], lane);
           if (writer)
