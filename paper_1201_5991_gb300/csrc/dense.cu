@@ -720,6 +720,133 @@ __global__ void k_small_chol_inv(LevelDev L) {
   }
 }
 
+// ---- G^{-1} and K_C of SPD levels with many constraints per subdomain (max n_c > 96) ----------
+// k_small_chol_inv works on one SM per subdomain, whose FP64 units give two products per cycle: n_c = 258
+// took 10 ms, with one thread per column of L^{-1}.  Here only the Cholesky factorisation (n_c^3 / 6
+// products) stays on one SM, by panels of 16 columns in shared memory; the inverse of the factor takes a
+// warp per column and the product W^T W a thread per entry, over the whole chip.
+
+// G = L L^T in place; the strictly upper part receives L^T (its rows are the columns of L)
+__global__ void __launch_bounds__(1024) k_gram_potrf(LevelDev L) {
+  constexpr int PW = 16;
+  const int s = blockIdx.x;
+  const SubMeta m = L.meta[s];
+  const int n = m.nc, tid = threadIdx.x;
+  if (n == 0) return;
+  double* G = L.Ginv + m.g_off;
+  extern __shared__ __align__(16) double panel[];   // [n][PW + 1]: rows p0 .. of the panel
+  __shared__ double diag[PW][PW + 1];
+  __shared__ int bad;
+  if (tid == 0) bad = 0;
+  for (int p0 = 0; p0 < n; p0 += PW) {
+    const int w = min(PW, n - p0), rows = n - p0 - w;
+    __syncthreads();
+    for (int e = tid; e < w * w; e += blockDim.x) diag[e / w][e % w] = G[(int64_t)(p0 + e / w) * n + p0 + e % w];
+    __syncthreads();
+    if (tid < 32) {   // the diagonal block, one lane per row
+      for (int j = 0; j < w; ++j) {
+        double d = diag[j][j];
+        if (!(d > 0.0)) {
+          if (tid == 0) bad = 1;
+          d = 1.0;
+        }
+        const double piv = sqrt(d);
+        __syncwarp();
+        if (tid == j) diag[j][j] = piv;
+        if (tid > j && tid < w) diag[tid][j] /= piv;
+        __syncwarp();
+        if (tid > j && tid < w)
+          for (int c = j + 1; c <= tid; ++c) diag[tid][c] -= diag[tid][j] * diag[c][j];
+        __syncwarp();
+      }
+    }
+    __syncthreads();
+    for (int e = tid; e < w * w; e += blockDim.x) {
+      const int r = e / w, c = e % w;
+      if (c <= r) {
+        G[(int64_t)(p0 + r) * n + p0 + c] = diag[r][c];
+        if (c < r) G[(int64_t)(p0 + c) * n + p0 + r] = diag[r][c];
+      }
+    }
+    for (int r = tid; r < rows; r += blockDim.x) {   // L(i, panel) = A(i, panel) L_D^{-T}
+      const int i = p0 + w + r;
+      double* row = panel + r * (PW + 1);
+      for (int j = 0; j < w; ++j) {
+        double a = G[(int64_t)i * n + p0 + j];
+        for (int c = 0; c < j; ++c) a -= row[c] * diag[j][c];
+        row[j] = a / diag[j][j];
+      }
+      for (int j = 0; j < w; ++j) {
+        G[(int64_t)i * n + p0 + j] = row[j];
+        G[(int64_t)(p0 + j) * n + i] = row[j];
+      }
+    }
+    __syncthreads();
+    for (int64_t e = tid; e < (int64_t)rows * rows; e += blockDim.x) {
+      const int r = (int)(e / rows), c = (int)(e % rows);
+      if (c > r) continue;
+      double* g = G + (int64_t)(p0 + w + r) * n + p0 + w + c;
+      double a = *g;
+      for (int j = 0; j < w; ++j) a -= panel[r * (PW + 1) + j] * panel[c * (PW + 1) + j];
+      *g = a;
+    }
+  }
+  __syncthreads();
+  if (tid == 0 && bad) flag_breakdown(L.status, s);
+}
+
+// W = L^{-1} into the K_C buffer, column c per warp: w_q = b_q / l_qq, b_i -= l_iq w_q for i > q (row q of the
+// upper part of G holds column q of L); b in shared memory
+__global__ void __launch_bounds__(128) k_gram_linv(LevelDev L, int max_nc) {
+  const int s = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const SubMeta m = L.meta[s];
+  const int n = m.nc, c = blockIdx.x * 4 + warp;
+  if (c >= n) return;
+  extern __shared__ __align__(16) double bs[];
+  double* b = bs + (int64_t)warp * max_nc;
+  const double* G = L.Ginv + m.g_off;
+  double* W = L.KC + m.g_off;
+  for (int i = lane; i < n; i += 32) b[i] = i == c ? 1.0 : 0.0;
+  __syncwarp();
+  for (int q = c; q < n; ++q) {
+    const double w = b[q] / G[(int64_t)q * n + q];
+    const double* lq = G + (int64_t)q * n;
+    for (int i = q + 1 + lane; i < n; i += 32) b[i] -= lq[i] * w;
+    __syncwarp();
+    if (lane == 0) b[q] = w;
+    __syncwarp();
+  }
+  for (int i = lane; i < n; i += 32) W[(int64_t)i * n + c] = b[i];
+}
+
+// G^{-1} = W^T W: one thread per entry (a, b), b <= a
+__global__ void __launch_bounds__(256) k_gram_inverse(LevelDev L) {
+  const int s = blockIdx.y;
+  const SubMeta m = L.meta[s];
+  const int n = m.nc;
+  const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (t >= (int64_t)n * n) return;
+  const int a = (int)(t / n), b = (int)(t % n);
+  if (b > a) return;
+  const double* W = L.KC + m.g_off;
+  double acc = 0.0;
+  for (int q = a; q < n; ++q) acc += W[(int64_t)q * n + a] * W[(int64_t)q * n + b];
+  double* G = L.Ginv + m.g_off;
+  G[(int64_t)a * n + b] = acc;
+  G[(int64_t)b * n + a] = acc;
+}
+
+// K_C = G^{-1} - R
+__global__ void __launch_bounds__(256) k_gram_kc(LevelDev L) {
+  const int s = blockIdx.y;
+  const SubMeta m = L.meta[s];
+  const int n = m.nc;
+  const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (t >= (int64_t)n * n) return;
+  const int a = (int)(t / n), b = (int)(t % n);
+  L.KC[m.g_off + t] = L.Ginv[m.g_off + t] - (a == b ? L.rho[s] * L.c_rho[m.c_off + a] : 0.0);
+}
+
 // FP64 levels: Z = Y_G^T G^{-1}, written into the Psi buffer (rows: interface padded positions)
 __global__ void k_psi_rhs(LevelDev L) {
   const int s = blockIdx.y;
@@ -1257,7 +1384,25 @@ void launch_gram_chol(const LevelDev& L, int precision_fp32, int max_nc, cudaStr
     const unsigned gx = (unsigned)(((int64_t)max_nc * max_nc + 7) / 8);
     k_gram<<<dim3(gx, ns), 256, 0, st>>>(L);
   }
-  { note_launch(); k_small_chol_inv<<<ns, 256, 0, st>>>(L); }
+  // one pass per subdomain where n_c is small (its four launches would be longer) or G indefinite, and where the
+  // panel of 16 columns does not fit
+  if (L.indefinite || max_nc <= 96 || max_nc > 1600) {
+    note_launch();
+    k_small_chol_inv<<<ns, 256, 0, st>>>(L);
+    return;
+  }
+  const size_t sm = sizeof(double) * 17 * (size_t)max_nc, smw = sizeof(double) * 4 * (size_t)max_nc;
+  static size_t attr = 48 * 1024;
+  if (sm > attr) {
+    cudaFuncSetAttribute(k_gram_potrf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaFuncSetAttribute(k_gram_linv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smw > 49152 ? smw : 49152));
+    attr = sm;
+  }
+  const unsigned ge = (unsigned)(((int64_t)max_nc * max_nc + 255) / 256);
+  { note_launch(); k_gram_potrf<<<ns, 1024, sm, st>>>(L); }
+  { note_launch(); k_gram_linv<<<dim3((unsigned)((max_nc + 3) / 4), ns), 128, smw, st>>>(L, max_nc); }
+  { note_launch(); k_gram_inverse<<<dim3(ge, ns), 256, 0, st>>>(L); }
+  { note_launch(); k_gram_kc<<<dim3(ge, ns), 256, 0, st>>>(L); }
 }
 
 template <typename T>
