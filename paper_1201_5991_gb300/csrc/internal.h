@@ -295,6 +295,8 @@ struct KrylovStore {
   int* cnt = nullptr;
   int cap = 0;
 };
+// Mail of column k (pinned host memory): r . r, alpha and the iteration before's beta at mail[4 k ..], then the
+// iteration's number (as int64) at mail[4 k + 3]; written by the update of x and r, half an iteration before its end.
 inline int64_t iface_blocks(int64_t n_iface) { return (n_iface + 255) / 256; }
 
 template <typename T>
@@ -338,7 +340,7 @@ void launch_dot(const double* a, const double* b, int64_t n, double* partial, in
 // PCG of a block of right-hand sides: column k keeps its scalars at scal[16 k ..].  The update of x and r
 // also makes r . r (scal[16 k + 5]); partial, cnt as in FusedDot.
 void launch_pcg_update_x_r(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
-                           double* partial, int* cnt, const KrylovStore& ks, cudaStream_t st, int nr = 1);
+                           double* partial, int* cnt, const KrylovStore& ks, double* mail, cudaStream_t st, int nr = 1);
 // x = sum_v c_v p_v, r = g - sum_v c_v q_v with c_v = (p_v . g) / d_v over the stored directions (coef: scratch,
 // [nr][cap][kProjBlocks + 1])
 constexpr int kProjBlocks = 32;

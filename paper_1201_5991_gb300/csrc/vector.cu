@@ -77,7 +77,7 @@ __device__ bool sum_over_grid(double v0, double v1, bool two, double* __restrict
   return true;
 }
 
-// scal layout (see capi.cpp): 0 rz, 1 pq, 2 alpha, 3 beta, 4 rz_new, 5 rr, 6 gg, 8 frozen.  The scalar step of
+// scal layout (see capi.cpp): 0 rz, 1 pq, 2 alpha, 3 beta, 4 rz_new, 5 rr, 6 gg, 7 iteration, 8 frozen.  The scalar step of
 // the recurrence that follows the sums (one thread); frozen columns keep alpha = beta = 0.
 __device__ void pcg_step(const FusedDot& dot, double s0, double s1) {
   double* S = dot.scal + 16 * blockIdx.y;
@@ -393,7 +393,7 @@ __global__ void k_dot_final(const double* __restrict__ partial, int nblk, double
 __global__ void __launch_bounds__(256) k_pcg_xr(double* __restrict__ x, double* __restrict__ r,
                                                 const double* __restrict__ p, const double* __restrict__ q,
                                                 double* __restrict__ scal, int64_t n, double* __restrict__ partial,
-                                                int* cnt, KrylovStore ks) {
+                                                int* cnt, KrylovStore ks, double* mail) {
   pdl_wait();
   pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -414,7 +414,15 @@ __global__ void __launch_bounds__(256) k_pcg_xr(double* __restrict__ x, double* 
     }
   }
   if (sum_over_grid(rr, 0.0, false, partial, cnt, s0, s1) && threadIdx.x == 0) {
-    scal[16 * blockIdx.y + 5] = s0;
+    double* S = scal + 16 * blockIdx.y;
+    S[5] = s0;
+    S[7] += 1.0;   // iteration number
+    double* box = mail + 4 * blockIdx.y;
+    box[0] = s0;
+    box[1] = a;
+    box[2] = S[3];
+    __threadfence_system();
+    *(volatile long long*)(box + 3) = (long long)S[7];
     if (slot < ks.cap) {   // every block has read its count (this one is the last)
       ks.d[(int64_t)blockIdx.y * ks.cap + slot] = scal[16 * blockIdx.y + 1];
       ks.cnt[blockIdx.y] = slot + 1;
@@ -743,8 +751,8 @@ void launch_dot(const double* a, const double* b, int64_t n, double* partial, in
   { note_launch(); k_dot_final<<<nr, 256, 0, st>>>(partial, nblk, out, ostride); }
 }
 void launch_pcg_update_x_r(double* x, double* r, const double* p, const double* q, double* scal, int64_t n,
-                           double* partial, int* cnt, const KrylovStore& ks, cudaStream_t st, int nr) {
-  if (n > 0) { note_launch(); launch_pdl(k_pcg_xr, dim3(nblocks(n, 256), nr), 256, 0, st, x, r, p, q, scal, n, partial, cnt, ks); }
+                           double* partial, int* cnt, const KrylovStore& ks, double* mail, cudaStream_t st, int nr) {
+  if (n > 0) { note_launch(); launch_pdl(k_pcg_xr, dim3(nblocks(n, 256), nr), 256, 0, st, x, r, p, q, scal, n, partial, cnt, ks, mail); }
 }
 void launch_project(const KrylovStore& ks, const double* g, double* x, double* r, int64_t n, double* coef,
                     cudaStream_t st, int nr) {
