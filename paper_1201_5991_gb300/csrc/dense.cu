@@ -1165,79 +1165,102 @@ __global__ void k_psi_transpose(LevelDev L) {
 // c CW .. c CW + CW - 1 through the tiled factor: forward y_i = D_i (e_i - sum_{j<i} L_ij y_j),
 // t = S y, backward x_i = D_i^T (t_i - sum_{j>i} L_ji^T x_j), with D_i the stored inverses of the
 // diagonal tiles (the same steps as the sweeps, in the same precision).  Column q of the result is
-// kept at W + (c CW + q) n_pad, so W is stored column after column; A_C is symmetric, so row q of
-// the stored matrix is row q of A_C^{-1} up to rounding.  Each product of a tile with a 64 x CW
-// block runs from shared memory, the tile k-major, every thread a block of CW/16 rows x 4 columns.
-template <int CW>
+// kept at W + (c CW + q) npad, so W is stored column after column.  The forward solution is zero above the
+// column's own block b0, and A_C^{-1} is symmetric, so only the blocks i >= b0 are computed (a third of
+// the products) and k_coarse_mirror fills in the rest.  Each product of a tile with a 64 x CW block runs from
+// shared memory, the tile k-major, one row x 4 columns per thread; the next tile is in registers meanwhile.
+// Bound by the chain of tiles of the first column block (nb^2 of them, about 1 us each), hence narrow blocks
+// of columns: 3,345 coarse DOFs took 14.5 ms with 53 blocks of 64 columns.
+constexpr int CW = 16;
+
 __global__ void __launch_bounds__(256) k_coarse_inverse(LevelDev L, float* __restrict__ W) {
-  constexpr int RR = CW / 16;                 // rows per thread
-  constexpr int CG = CW / 4;                  // column groups of four
   const SubMeta m = L.meta[0];
   const int nb = m.Bc;
   const int64_t npad = (int64_t)nb * NB;
   const int c0 = blockIdx.x * CW;
   if (c0 >= npad) return;
+  const int b0 = c0 / NB;
   __shared__ __align__(16) float As[NB][NB + 4];   // tile, k-major: As[k][r]
   __shared__ __align__(16) float Bs[NB][CW + 4];   // 64 x CW block: Bs[k][c]
   const int tid = threadIdx.x;
-  const int cg = tid % CG, rg = tid / CG;          // columns 4 cg .. +3, rows RR rg .. +RR-1
+  const int cg = tid % (CW / 4), r = tid / (CW / 4);   // columns 4 cg .. +3 of row r
   float* Wc = W + (int64_t)c0 * npad;              // this CTA's columns, each of npad entries
   const float* tiles = (const float*)L.tiles + m.tile_off;
   const float* dinv = (const float*)L.dinv + m.dinv_off;
   const float* sgn = (const float*)L.sgn + m.vec_off;
-  auto load_tile = [&](const float* t, bool transpose) {   // As[k][r] = t[r][k] (or t[k][r])
-    for (int e = tid; e < NB2; e += 256) {
-      const int a = e / NB, b = e % NB;
-      if (transpose) As[b][a] = t[e]; else As[a][b] = t[e];
-    }
+  float4 ta[4], tb;   // the next tile and block
+  auto fetch_tile = [&](const float* t) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) ta[u] = __ldg((const float4*)t + tid + 256 * u);
   };
-  auto load_block = [&](int blk) {                  // Bs[k][c] = W column c, rows of block blk
-    for (int e = tid; e < NB * CW; e += 256) {
-      const int c = e / NB, k = e % NB;
-      Bs[k][c] = Wc[(int64_t)c * npad + (int64_t)blk * NB + k];
-    }
+  auto fetch_block = [&](int blk) {   // 16 columns x 64 rows: column tid / 16, rows 4 (tid % 16) ..
+    tb = *(const float4*)(Wc + (int64_t)(tid >> 4) * npad + (int64_t)blk * NB + 4 * (tid & 15));
   };
-  auto mma = [&](float (&acc)[RR][4]) {
-#pragma unroll 8
-    for (int k = 0; k < NB; ++k) {
-      float a[RR], b[4];
+  auto put_tile = [&](bool transpose) {   // As[k][r] = t[r][k] (transpose) or t[k][r]
 #pragma unroll
-      for (int r = 0; r < RR; ++r) a[r] = As[k][RR * rg + r];
-      const float4 bv = *(const float4*)&Bs[k][4 * cg];
-      b[0] = bv.x; b[1] = bv.y; b[2] = bv.z; b[3] = bv.w;
-#pragma unroll
-      for (int r = 0; r < RR; ++r)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[r][q] += a[r] * b[q];
-    }
-  };
-  auto store_block = [&](int blk, const float (&v)[RR][4]) {
-#pragma unroll
-    for (int r = 0; r < RR; ++r)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) Wc[(int64_t)(4 * cg + q) * npad + (int64_t)blk * NB + RR * rg + r] = v[r][q];
-  };
-  // forward: y_i = D_i (e_i - sum_{j<i} L_ij y_j)
-  for (int i = 0; i < nb; ++i) {
-    float acc[RR][4] = {};
-    for (int j = 0; j < i; ++j) {
-      __syncthreads();
-      load_tile(tiles + ((int64_t)i * (i + 1) / 2 + j) * NB2, true);
-      load_block(j);
-      __syncthreads();
-      mma(acc);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < RR; ++r)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int64_t row = (int64_t)i * NB + RR * rg + r;
-        Bs[RR * rg + r][4 * cg + q] = (row == c0 + 4 * cg + q ? 1.f : 0.f) - acc[r][q];
+    for (int u = 0; u < 4; ++u) {
+      const int q = tid + 256 * u, a = q >> 4, b = 4 * (q & 15);
+      if (transpose) {
+        As[b][a] = ta[u].x;
+        As[b + 1][a] = ta[u].y;
+        As[b + 2][a] = ta[u].z;
+        As[b + 3][a] = ta[u].w;
+      } else {
+        *(float4*)&As[a][b] = ta[u];
       }
-    load_tile(dinv + (int64_t)i * NB2, true);
+    }
+  };
+  auto put_block = [&]() {
+    const int c = tid >> 4, k = 4 * (tid & 15);
+    Bs[k][c] = tb.x;
+    Bs[k + 1][c] = tb.y;
+    Bs[k + 2][c] = tb.z;
+    Bs[k + 3][c] = tb.w;
+  };
+  auto mma = [&](float (&acc)[4]) {
+#pragma unroll 16
+    for (int k = 0; k < NB; ++k) {
+      const float a = As[k][r];
+      const float4 b = *(const float4*)&Bs[k][4 * cg];
+      acc[0] += a * b.x;
+      acc[1] += a * b.y;
+      acc[2] += a * b.z;
+      acc[3] += a * b.w;
+    }
+  };
+  auto store_block = [&](int blk, const float (&v)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) Wc[(int64_t)(4 * cg + q) * npad + (int64_t)blk * NB + r] = v[q];
+  };
+  // forward: y_i = D_i (e_i - sum_{b0 <= j < i} L_ij y_j)
+  for (int i = b0; i < nb; ++i) {
+    float acc[4] = {};
+    const float* row = tiles + (int64_t)i * (i + 1) / 2 * NB2;
+    __syncthreads();   // the blocks stored so far are visible to the whole CTA
+    if (b0 < i) {
+      fetch_tile(row + (int64_t)b0 * NB2);
+      fetch_block(b0);
+    }
+    for (int j = b0; j < i; ++j) {
+      put_tile(true);
+      put_block();
+      __syncthreads();
+      if (j + 1 < i) {
+        fetch_tile(row + (int64_t)(j + 1) * NB2);
+        fetch_block(j + 1);
+      } else {
+        fetch_tile(dinv + (int64_t)i * NB2);
+      }
+      mma(acc);
+      __syncthreads();
+    }
+    if (b0 == i) fetch_tile(dinv + (int64_t)i * NB2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      Bs[r][4 * cg + q] = ((int64_t)i * NB + r == c0 + 4 * cg + q ? 1.f : 0.f) - acc[q];
+    put_tile(true);
     __syncthreads();
-    float y[RR][4] = {};
+    float y[4] = {};
     mma(y);
     store_block(i, y);
   }
@@ -1245,37 +1268,56 @@ __global__ void __launch_bounds__(256) k_coarse_inverse(LevelDev L, float* __res
   // t = S y (pivot signs of the signed factor; all +1 on SPD levels)
   for (int e = tid; e < NB * CW; e += 256) {
     const int c = e / NB;
-    for (int64_t row = e % NB; row < npad; row += NB) Wc[(int64_t)c * npad + row] *= sgn[row];
+    for (int64_t row = (int64_t)b0 * NB + e % NB; row < npad; row += NB) Wc[(int64_t)c * npad + row] *= sgn[row];
   }
-  // backward: x_i = D_i^T (t_i - sum_{j>i} L_ji^T x_j)
-  for (int i = nb - 1; i >= 0; --i) {
-    float acc[RR][4] = {};
-    for (int j = i + 1; j < nb; ++j) {
-      __syncthreads();
-      load_tile(tiles + ((int64_t)j * (j + 1) / 2 + i) * NB2, false);
-      load_block(j);
-      __syncthreads();
-      mma(acc);
+  // backward: x_i = D_i^T (t_i - sum_{j>i} L_ji^T x_j), i >= b0
+  for (int i = nb - 1; i >= b0; --i) {
+    float acc[4] = {};
+    __syncthreads();
+    if (i + 1 < nb) {
+      fetch_tile(tiles + ((int64_t)(i + 1) * (i + 2) / 2 + i) * NB2);
+      fetch_block(i + 1);
     }
+    for (int j = i + 1; j < nb; ++j) {
+      put_tile(false);
+      put_block();
+      __syncthreads();
+      if (j + 1 < nb) {
+        fetch_tile(tiles + ((int64_t)(j + 1) * (j + 2) / 2 + i) * NB2);
+        fetch_block(j + 1);
+      } else {
+        fetch_tile(dinv + (int64_t)i * NB2);
+        fetch_block(i);
+      }
+      mma(acc);
+      __syncthreads();
+    }
+    if (i + 1 == nb) {
+      fetch_tile(dinv + (int64_t)i * NB2);
+      fetch_block(i);
+    }
+    put_tile(false);
+    put_block();
     __syncthreads();
-    load_block(i);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) Bs[r][4 * cg + q] -= acc[q];   // this thread's own entries
     __syncthreads();
-    float rhs[RR][4];
-#pragma unroll
-    for (int r = 0; r < RR; ++r)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) rhs[r][q] = Bs[RR * rg + r][4 * cg + q] - acc[r][q];
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < RR; ++r)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) Bs[RR * rg + r][4 * cg + q] = rhs[r][q];
-    load_tile(dinv + (int64_t)i * NB2, false);
-    __syncthreads();
-    float x[RR][4] = {};
+    float x[4] = {};
     mma(x);
     store_block(i, x);
   }
+}
+
+// the blocks above every column's own: W(i, j) = W(j, i), one 64 x 64 block (j > i) per CTA
+__global__ void __launch_bounds__(256) k_coarse_mirror(float* __restrict__ W, int64_t npad) {
+  const int i = blockIdx.x, j = blockIdx.y;
+  if (i >= j) return;
+  __shared__ float t[NB][NB + 1];
+  for (int e = threadIdx.x; e < NB2; e += 256)   // columns of block i, rows of block j
+    t[e / NB][e % NB] = W[((int64_t)i * NB + e / NB) * npad + (int64_t)j * NB + e % NB];
+  __syncthreads();
+  for (int e = threadIdx.x; e < NB2; e += 256)
+    W[((int64_t)j * NB + e / NB) * npad + (int64_t)i * NB + e % NB] = t[e % NB][e / NB];
 }
 
 // z = W x for nr columns (x: columns of n_vec, padded local positions 0 .. npad-1; z: level DOFs); one warp
@@ -1312,10 +1354,12 @@ __global__ void k_coarse_apply(const float* __restrict__ W, int64_t npad, const 
 void launch_coarse_inverse(const LevelDev& L, int64_t npad, float* W, cudaStream_t st) {
   if (npad <= 0) return;
   note_launch();
-  if (npad <= 2048)
-    k_coarse_inverse<16><<<(unsigned)((npad + 15) / 16), 256, 0, st>>>(L, W);
-  else
-    k_coarse_inverse<64><<<(unsigned)((npad + 63) / 64), 256, 0, st>>>(L, W);
+  k_coarse_inverse<<<(unsigned)((npad + CW - 1) / CW), 256, 0, st>>>(L, W);
+  const unsigned nb = (unsigned)(npad / NB);
+  if (nb > 1) {
+    note_launch();
+    k_coarse_mirror<<<dim3(nb, nb), 256, 0, st>>>(W, npad);
+  }
 }
 
 void launch_coarse_apply(const float* W, int64_t npad, const float* x, double* z, const int32_t* loc2glob,
