@@ -111,30 +111,42 @@ __device__ void factor_diag_tile(const LevelDev& L, const SubMeta& m, int s, int
   // is updated as a_ic -= (a_ij / d_j) a_cj (d_j = a_jj after the updates of the columns before
   // j), which equals l_ij s_j l_cj with l_ij = a_ij / (s_j sqrt|d_j|), s_j = sign d_j; the columns
   // are scaled to L afterwards.  Blocked by panels of 16 columns, with three barriers per panel:
-  //   (a1) warp 0 eliminates inside the 16 x 16 diagonal block (warp-synchronous steps);
+  //   (a1) warp 0 eliminates inside the 16 x 16 diagonal block from registers: lane i + 16 h holds row i's
+  //        columns of parity h, column j and its pivot come by shuffle (from shared memory, each
+  //        step was a chain of up to eight dependent reads and writes);
   //   (a2) one thread per row below it applies the panel's 16 eliminations to its 16 panel
   //        entries and keeps the multipliers a_ij / d_j (in X, unused until the inverse);
-  //   (b)  the trailing block takes a_rc -= sum_j (a_rj / d_j) a_cj over the panel columns.
+  //   (b)  the trailing block takes a_rc -= sum_j (a_rj / d_j) a_cj over the panel columns, 2 x 2 entries per
+  //        thread, the blocks on and below the diagonal only.
   // Every entry receives the same updates in the same order (j ascending) as column by column.
+  // The chain of diagonal tiles is the critical path of the factorisation (one CTA per subdomain).
   {
     constexpr int PW = 16;
     T(*F)[PW + 1] = (T(*)[PW + 1])(&X[0][0]);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int p0 = 0; p0 < NB; p0 += PW) {
       if (warp == 0) {
-        const int i = p0 + (lane & 15), half = lane >> 4;
-        for (int jj = 0; jj < PW; ++jj) {
-          const int j = p0 + jj;
-          T d = A[j][j];
+        const int i = lane & 15, half = lane >> 4;
+        T a[PW / 2];   // row i, columns 2 q + half (above the diagonal: never read by another row)
+#pragma unroll
+        for (int q = 0; q < PW / 2; ++q) a[q] = A[p0 + i][p0 + 2 * q + half];
+#pragma unroll
+        for (int j = 0; j < PW; ++j) {
+          const T v = __shfl_sync(0xffffffffu, a[j >> 1], ((j & 1) << 4) | i);   // a_ij
+          T d = __shfl_sync(0xffffffffu, v, j);
           // a failed pivot (flagged below from the same value) continues as 1, as in the scaling
           if (L.indefinite ? !(fabs(d) > (T)1e-30) : !(d > (T)0)) d = (T)1;
-          if (lane == 0) dd[j] = d;
-          if (i > j) {
-            const T f = A[i][j] / d;
-            for (int c = j + 1 + half; c <= i; c += 2) A[i][c] -= f * A[c][j];
+          if (lane == 0) dd[p0 + j] = d;
+          const T f = v / d;
+#pragma unroll
+          for (int q = j >> 1; q < PW / 2; ++q) {
+            const T vc = __shfl_sync(0xffffffffu, v, 2 * q + half);   // a_cj, c = 2 q + half
+            if (2 * q + half > j) a[q] -= f * vc;
           }
-          __syncwarp();
         }
+#pragma unroll
+        for (int q = 0; q < PW / 2; ++q)
+          if (2 * q + half <= i) A[p0 + i][p0 + 2 * q + half] = a[q];
       }
       __syncthreads();
       const int nb = NB - p0 - PW;   // rows below the diagonal block
@@ -146,21 +158,34 @@ __device__ void factor_diag_tile(const LevelDev& L, const SubMeta& m, int s, int
 #pragma unroll
         for (int jj = 0; jj < PW; ++jj) {
           const T f = a[jj] / dd[p0 + jj];
-          F[tid][jj] = f;
 #pragma unroll
           for (int c = jj + 1; c < PW; ++c) a[c] -= f * A[p0 + c][p0 + jj];
+          F[tid][jj] = f;   // last, so that the next column's reads run beside its division
         }
 #pragma unroll
         for (int jj = 0; jj < PW; ++jj) A[i][p0 + jj] = a[jj];
       }
       __syncthreads();
-      for (int e = tid; e < nb * nb; e += blockDim.x) {
-        const int r = e / nb, c = e % nb;
-        if (c > r) continue;
-        T acc = A[p0 + PW + r][p0 + PW + c];
+      const int nt = nb / 2;   // block rows nt - 1 - u and u together hold nt + 1 blocks
+      for (int e = tid; e < nt / 2 * (nt + 1); e += blockDim.x) {
+        const int u = e / (nt + 1), q = e % (nt + 1);
+        const int r = 2 * (q < nt - u ? nt - 1 - u : u), c = 2 * (q < nt - u ? q : q - (nt - u));
+        T* A0 = &A[p0 + PW + r][p0 + PW + c];
+        T* A1 = A0 + NB + 1;
+        T s00 = A0[0], s01 = A0[1], s10 = A1[0], s11 = A1[1];
 #pragma unroll
-        for (int jj = 0; jj < PW; ++jj) acc -= F[r][jj] * A[p0 + PW + c][p0 + jj];
-        A[p0 + PW + r][p0 + PW + c] = acc;
+        for (int jj = 0; jj < PW; ++jj) {
+          const T f0 = F[r][jj], f1 = F[r + 1][jj];
+          const T v0 = A[p0 + PW + c][p0 + jj], v1 = A[p0 + PW + c + 1][p0 + jj];
+          s00 -= f0 * v0;
+          s01 -= f0 * v1;
+          s10 -= f1 * v0;
+          s11 -= f1 * v1;
+        }
+        A0[0] = s00;
+        if (c < r) A0[1] = s01;
+        A1[0] = s10;
+        A1[1] = s11;
       }
       __syncthreads();
     }
@@ -188,9 +213,10 @@ __device__ void factor_diag_tile(const LevelDev& L, const SubMeta& m, int s, int
     X[0][j] = sqrt(d);   // pivots, kept in the first row of X until the inverse is formed
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < NB * NB; t += blockDim.x) {
-    const int r = t / NB, c = t % NB;
-    if (r > c) A[r][c] /= X[0][c] * sg[c];
+  for (int t = threadIdx.x; t < NB / 2 * (NB - 1); t += blockDim.x) {   // rows NB - 1 - u and u: NB - 1 entries
+    const int u = t / (NB - 1), q = t % (NB - 1);
+    const int r = q < NB - 1 - u ? NB - 1 - u : u, c = q < NB - 1 - u ? q : q - (NB - 1 - u);
+    A[r][c] /= X[0][c] * sg[c];
   }
   __syncthreads();
   if (threadIdx.x < NB) A[threadIdx.x][threadIdx.x] = X[0][threadIdx.x];
@@ -198,22 +224,25 @@ __device__ void factor_diag_tile(const LevelDev& L, const SubMeta& m, int s, int
   if (threadIdx.x < NB) ((T*)L.sgn)[m.vec_off + (int64_t)k * NB + threadIdx.x] = sg[threadIdx.x];
   if (threadIdx.x == 0 && bad) flag_breakdown(L.status, s);
   // X = L^{-1} by 16 x 16 blocks: the four diagonal blocks X_PP = L_PP^{-1} by forward
-  // substitution (one warp each, one lane per column), then the blocks below the diagonal by
+  // substitution (half a warp each, one lane per column, in registers), then the blocks below the diagonal by
   // their distance d = Q - P: X_QP = -X_QQ (sum_{P <= K < Q} L_QK X_KP), the inner sum into a
   // scratch block first (3 - d + 1 blocks per distance, one entry per thread and block).
   {
     constexpr int PW = 16;
     __shared__ T Tq[3][PW][PW + 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (warp < 4 && lane < PW) {
-      const int p0 = PW * warp, c = p0 + lane;
-      for (int r = p0; r < c; ++r) X[r][c] = (T)0;
-      X[c][c] = (T)1 / A[c][c];
-      for (int i = c + 1; i < p0 + PW; ++i) {
-        T part = (T)0;
-        for (int q = c; q < i; ++q) part += A[i][q] * X[q][c];
-        X[i][c] = -part / A[i][i];
+    if (warp < 2) {
+      const int p0 = PW * (2 * warp + (lane >> 4)), c = lane & 15;
+      T x[PW];
+#pragma unroll
+      for (int i = 0; i < PW; ++i) {
+        T part = (T)0;   // x[q] = 0 above the column's own row
+#pragma unroll
+        for (int q = 0; q < i; ++q) part += A[p0 + i][p0 + q] * x[q];
+        x[i] = i < c ? (T)0 : (i == c ? (T)1 : -part) / A[p0 + i][p0 + i];
       }
+#pragma unroll
+      for (int i = 0; i < PW; ++i) X[p0 + i][p0 + c] = x[i];
     }
     __syncthreads();
     for (int dist = 1; dist < 4; ++dist) {
@@ -223,6 +252,7 @@ __device__ void factor_diag_tile(const LevelDev& L, const SubMeta& m, int s, int
         const int P = bq, Q = bq + dist;
         T acc = (T)0;
         for (int K = P; K < Q; ++K)
+#pragma unroll
           for (int q = 0; q < PW; ++q) acc += A[PW * Q + r][PW * K + q] * X[PW * K + q][PW * P + c];
         Tq[bq][r][c] = acc;
       }
@@ -231,7 +261,9 @@ __device__ void factor_diag_tile(const LevelDev& L, const SubMeta& m, int s, int
         const int bq = e / (PW * PW), r = (e / PW) % PW, c = e % PW;
         const int P = bq, Q = bq + dist;
         T acc = (T)0;
-        for (int q = 0; q <= r; ++q) acc += X[PW * Q + r][PW * Q + q] * Tq[bq][q][c];
+        for (int q0 = 0; q0 <= r; q0 += 4)   // X_QQ is zero above its diagonal
+#pragma unroll
+          for (int q = q0; q < q0 + 4; ++q) acc += X[PW * Q + r][PW * Q + q] * Tq[bq][q][c];
         X[PW * Q + r][PW * P + c] = -acc;
       }
       __syncthreads();
