@@ -156,15 +156,13 @@ class ClockSampler:
 
 def traffic_ratio(cls):
     """DRAM bytes per algorithmic unit of the roofline kernel class from the committed ncu summary:
-    per algorithmic byte for the sweeps (profiles/trsv_sweep_traffic.json) and the factor products
-    (profiles/trmv_schur_traffic.json), per FP32-equivalent flop for the tensor-core update
+    per algorithmic byte for the sweeps (profiles/trsv_sweep_traffic.json) and the symmetric products of
+    the inner operator and the interface inverse (profiles/trmv_schur_traffic.json), per FP32-equivalent flop for the tensor-core update
     (profiles/update_tc2_traffic.json); None when the kernel source changed since the counters
     were taken."""
     from paper_1201_5991_gb300 import capi
     if cls == capi.PROF_TRSV:
         fname, src_name, key = "trsv_sweep_traffic.json", "sweep.cu", "traffic_over_algorithmic"
-    elif cls == capi.PROF_TRSV_IFACE:
-        fname, src_name, key = "trsv_sweep_traffic.json", "sweep.cu", "traffic_over_algorithmic_interface"
     elif cls == capi.PROF_TC_UPDATE:
         fname, src_name, key = "update_tc2_traffic.json", "update_tc.cu", "traffic_over_fp32_flop"
     else:
@@ -497,7 +495,8 @@ def run_gpu(args, rank, world, local_rank):
     traffic = ratio * units / max(prof[1], 1) if ratio is not None else None
     names = {capi.PROF_TRSV: "k_sweep<float> forward/backward over interior block rows (Schur operator; "
                              "streaming triangular sweeps, TMA-staged tiles)",
-             capi.PROF_TRSV_IFACE: "k_sweep<float> forward/backward over interface block rows (subdomain corrections)",
+             capi.PROF_TRSV_IFACE: "subdomain corrections: k_schur_symv_rows + _cols with the explicit interface inverse "
+                                   "of tensor-core factors, else k_sweep<float> over interface block rows",
              capi.PROF_COARSE: "coarsest-level solves (k_coarse_apply with the explicit FP32 inverse of the "
                                "FP64 coarse factor, else sweeps over it)",
              capi.PROF_TRMV: "inner Schur operator: k_schur_symv_rows + _cols over the explicit augmented Schur "

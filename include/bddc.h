@@ -160,9 +160,11 @@ typedef struct {
 #define BDDC_PROF_TRSV 0    /* streaming triangular sweeps over interior block rows (Schur operator) */
 #define BDDC_PROF_FACTOR 1  /* batched blocked Cholesky steps on CUDA cores (diagonal, panel, in-panel update) */
 #define BDDC_PROF_SPMV 2    /* FP64 sparse products with K_i */
-#define BDDC_PROF_TRMV 3    /* inner Schur operator: products with the stored interface factor */
-#define BDDC_PROF_TRSV_IFACE 4   /* sweeps over interface block rows (subdomain corrections) */
-#define BDDC_PROF_COARSE 5  /* sweeps of the coarsest level's FP64 factor */
+#define BDDC_PROF_TRMV 3    /* inner Schur operator: the explicit augmented Schur complement, else products with
+                               the stored interface factor */
+#define BDDC_PROF_TRSV_IFACE 4   /* subdomain corrections: product with the interface inverse of a tensor-core
+                                    factor (its two kernels counted), else sweeps over interface block rows */
+#define BDDC_PROF_COARSE 5  /* coarsest level: product with the explicit inverse, else sweeps of its factor */
 #define BDDC_PROF_TC_UPDATE 6   /* tensor-core trailing updates of the factorisation (FP32-equivalent flops) */
 #define BDDC_PROF_TC_PANEL 7    /* tensor-core panel solves below the diagonal blocks (flops of the
                                    triangular solves they replace) */

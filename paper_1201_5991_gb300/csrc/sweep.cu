@@ -1,7 +1,8 @@
 // Streaming triangular sweeps with the tiled factors, batched over all subdomains of a level:
 // forward y = S L^{-1} b and backward L^T x = y over the interior block rows (the discrete
 // Dirichlet problems of the Schur operator, Sec. 2) or over the interface block rows (the
-// constrained Neumann problem of Eq. sub_cor, restricted to the interface).  S holds the pivot
+// constrained Neumann problem of Eq. sub_cor, restricted to the interface; factors that hold the
+// interface inverse apply that instead, trmv.cu).  S holds the pivot
 // signs of the signed Cholesky (identity for SPD levels), so the pair solves L S L^T x = b.
 //
 // Design (GB300): the sweep is bound by reading the factor from HBM once.  A persistent grid

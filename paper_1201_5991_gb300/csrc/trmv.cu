@@ -1,4 +1,8 @@
-// Inner Schur operator from the stored factor (mixed precision only).
+// Products with the interface blocks (mixed precision only): the inner Schur operator, and the
+// preconditioner's local solve by the explicit inverse of the interface block.  The inverse, and the
+// augmented Schur complement where every interior ends at a sub-panel boundary, are explicit lower
+// triangles: one symmetric product each (k_schur_symv_rows, k_schur_symv_cols).  Elsewhere the inner
+// operator multiplies by the stored factor:
 //
 // The trailing block of the partial factorisation of A_i = K_i + C_i^T R C_i is the factor of
 // the augmented local Schur complement: L_GG S L_GG^T = S_i + C_i^T R C_i, S_i = K_GG -

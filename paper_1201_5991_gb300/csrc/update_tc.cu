@@ -8,7 +8,7 @@
 // after the second half, one rank-512 update (nq = 8) serves every trailing column.  Each
 // trailing element is read and written once per 512 columns instead of once per 256 (without its
 // output write-back the rank-256 kernel ran 27 % faster): on the 48^3 factorisation the update
-// went from 254 to 300 TFLOP/s FP32-equivalent.
+// went from 254 to 300 TFLOP/s FP32-equivalent (before the two MMA issuers).
 //
 // FP32 accuracy from FP16 tensor cores: for the 64 x 256 slab of panel row tile i, every row r
 // is scaled by 2^e_r so that its largest entry lies in [2^14, 2^15), and each scaled entry a is
@@ -20,16 +20,19 @@
 // that both operands of every MMA stay FP16.  Measured against FP64 on factor-like data (rows
 // spanning four decades): 2-4e-7 of sum |a||b| (three-part BF16 splitting with six products:
 // 1.3e-7, FP32 dot: 8e-7).  Accumulating all products in one TMEM accumulator over K = 256
-// loses an order of magnitude, so the dominant hi hi product has its own accumulator and both
-// are promoted into FP32 registers after every 64-wide panel column.
+// loses an order of magnitude, so the dominant hi hi product has its own accumulator, which is
+// promoted into FP32 registers after every 64-wide panel column; the cross products (2^-11 of
+// it) are accumulated over the whole work item.
 //
 // k_split_panel writes the parts in the exact shared-memory operand image (K-major, 128-byte
 // swizzle), so the update moves bytes with cp.async.bulk only.  A work item is a 128 x 128
 // output block (row tiles i0, i0+1 by column tiles j, j+1); per panel column q the producer
-// warp copies the two parts of the four tiles (64 KB) into one of three shared-memory stages
-// and one thread issues 12 MMAs (3 products x 4 K-steps, M = N = 128) into one of two TMEM
-// accumulator pairs (hi hi; the two cross products); eight epilogue warps promote each pair
-// into FP32 registers after every column and finally update the output tiles.
+// warp copies the two parts of the four tiles (64 KB) into one of three shared-memory stages,
+// one thread issues the 4 hi hi MMAs (M = N = 128, K = 16) into one of two TMEM accumulators, a
+// second thread in another warp the 8 MMAs of the cross products into the item's own
+// accumulator (two of those), and eight epilogue warps promote and finally update the output
+// tiles.  The two issuers wait independently, so the tensor pipe holds the cross products while
+// a promotion is under way; one issuer for all twelve left it idle between commit and wait.
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
