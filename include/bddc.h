@@ -371,6 +371,10 @@ int bddc_batching_ablation(bddc_handle h, double* ms);
  * wait of the update kernel gave up). */
 int bddc_tc_update_check(int64_t n, int rank, float* a, double* ms);
 
+/* Test only: while bytes > 0, an allocation of device memory that a call on this host thread makes for a
+ * handle fails as out of memory if the handle would then hold more than `bytes`; 0 ends it. */
+int bddc_alloc_probe(int64_t bytes);
+
 /* Message of the last failure on the calling thread ("" if none). */
 const char* bddc_last_error(void);
 

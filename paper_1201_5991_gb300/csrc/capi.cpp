@@ -36,6 +36,7 @@ void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 namespace {
 
 thread_local std::string g_err;
+thread_local int64_t t_alloc_limit = 0;   // bddc_alloc_probe
 
 struct Fail {
   int code;
@@ -48,7 +49,10 @@ struct Fail {
 
 void ck(cudaError_t e, const char* what) {
   if (e == cudaSuccess) return;
-  if (e == cudaErrorMemoryAllocation) fail(BDDC_ERR_OOM, std::string(what) + ": out of device memory");
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();   // the context is intact: no later call may take this for its own error
+    fail(BDDC_ERR_OOM, std::string(what) + ": out of device memory");
+  }
   fail(BDDC_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
@@ -118,6 +122,8 @@ struct DevArena {
   T* alloc(int64_t n) {
     if (n <= 0) n = 1;
     void* p = nullptr;
+    if (t_alloc_limit > 0 && bytes + (int64_t)sizeof(T) * n > t_alloc_limit)
+      ck(cudaErrorMemoryAllocation, "allocation limit of the probe");
     ck(cudaMallocFromPoolAsync(&p, sizeof(T) * (size_t)n, library_pool(), st), "cudaMallocFromPoolAsync");
     ptrs.push_back(p);
     bytes += (int64_t)sizeof(T) * n;
@@ -345,6 +351,7 @@ struct bddc_handle_s {
   int* dot_cnt = nullptr;              // [blk] counters of the fused sums
   KrylovStore kstore;                  // directions of the running refined solve (allocated by the first one)
   double* proj_coef = nullptr;
+  void* kstore_mem = nullptr;          // the block of memory that both lie in
   int kstore_blk = 0;
   double* h_scal = nullptr;            // pinned [16 kMaxBlock]
   double* mail = nullptr;              // pinned [4 kMaxBlock], written by the device (see launch_pcg_update_x_r)
@@ -2512,20 +2519,26 @@ void prepare_kstore(bddc_handle_s* h, int nb) {
   ck(cudaStreamSynchronize(h->st), "sync");
   drop_graph(h);   // a cached iteration refers to the old storage
   DevArena& A = h->arena;
-  if (h->kstore.cap > 0) {
-    A.free_one(h->kstore.p);
-    A.free_one(h->kstore.q);
-  }
+  // one block of memory, and the handle holds none while it changes: an allocation that fails leaves no
+  // pointer to the old one behind
+  void* old = h->kstore_mem;
+  h->kstore = KrylovStore();
+  h->kstore_mem = nullptr;
+  h->kstore_blk = 0;
+  if (old) A.free_one(old);
   const int blk = h->blk;
   const int64_t n = std::max<int64_t>(h->lv[0].d.n_iface, 1);
   const int cap = (int)std::max<int64_t>(1, std::min<int64_t>(128, ((int64_t)4 << 30) / (8 * n * blk)));
-  h->kstore.p = A.alloc<float>(n * cap * blk);
-  h->kstore.q = A.alloc<float>(n * cap * blk);
-  h->kstore.d = A.alloc<double>((int64_t)cap * blk);
-  h->kstore.cnt = A.alloc<int>(kMaxBlock);
-  h->kstore.cap = cap;
+  const int64_t vec = n * cap * blk, coef = (int64_t)blk * cap * (kProjBlocks + 1);
+  double* mem = A.alloc<double>(vec + (int64_t)cap * blk + coef + kMaxBlock);   // p, q (FP32); d; coef; cnt
+  h->kstore_mem = mem;
   h->kstore_blk = blk;
-  h->proj_coef = A.alloc<double>((int64_t)blk * cap * (kProjBlocks + 1));
+  h->proj_coef = mem + vec + (int64_t)cap * blk;
+  h->kstore.p = (float*)mem;
+  h->kstore.q = (float*)mem + vec;
+  h->kstore.d = mem + vec;
+  h->kstore.cnt = (int*)(h->proj_coef + coef);
+  h->kstore.cap = cap;
 }
 
 // Mixed-precision iterative refinement around PCG (the outer iteration that restores FP64
@@ -3077,6 +3090,11 @@ int bddc_tc_update_check(int64_t n, int rank, float* a, double* ms) {
     A.release();
     return BDDC_OK;
   });
+}
+
+int bddc_alloc_probe(int64_t bytes) {
+  t_alloc_limit = bytes > 0 ? bytes : 0;
+  return BDDC_OK;
 }
 
 int bddc_get_stats(bddc_handle h, bddc_stats* out) {
