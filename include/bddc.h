@@ -187,7 +187,7 @@ typedef struct {
   int inner_steps;                    /* inner operator in use: -1 none, 0 factor products, k steps */
   int outer_iterations;               /* FP64 outer refinement steps of the last solve (max over rhs) */
   double analysis_ms, factor_ms, solve_ms;
-  int64_t factor_bytes;               /* device bytes held by factors */
+  int64_t factor_bytes;               /* device bytes the handle holds (factors, maps, work vectors) */
   double prof_ms[BDDC_PROF_CLASSES];          /* summed CUDA-event durations per class */
   int64_t prof_launches[BDDC_PROF_CLASSES];   /* launches per class */
   double prof_bytes[BDDC_PROF_CLASSES];       /* algorithmic bytes moved (TRSV, SPMV) */

@@ -113,7 +113,7 @@ template <typename T>
 using raw_vector = std::vector<T, NoInitAlloc<T>>;
 
 struct DevArena {
-  std::vector<void*> ptrs;
+  std::vector<std::pair<void*, int64_t>> ptrs;   // with their bytes
   int64_t bytes = 0;
   double upload_ms = 0.0;       // host time spent in upload (pageable copies stage synchronously)
   int64_t upload_bytes = 0;
@@ -125,7 +125,7 @@ struct DevArena {
     if (t_alloc_limit > 0 && bytes + (int64_t)sizeof(T) * n > t_alloc_limit)
       ck(cudaErrorMemoryAllocation, "allocation limit of the probe");
     ck(cudaMallocFromPoolAsync(&p, sizeof(T) * (size_t)n, library_pool(), st), "cudaMallocFromPoolAsync");
-    ptrs.push_back(p);
+    ptrs.emplace_back(p, (int64_t)sizeof(T) * n);
     bytes += (int64_t)sizeof(T) * n;
     return (T*)p;
   }
@@ -153,14 +153,15 @@ struct DevArena {
   }
   void free_one(void* p) {   // return one allocation to the pool early (stream-ordered)
     for (size_t k = 0; k < ptrs.size(); ++k)
-      if (ptrs[k] == p) {
+      if (ptrs[k].first == p) {
         cudaFreeAsync(p, st);
+        bytes -= ptrs[k].second;
         ptrs.erase(ptrs.begin() + (int64_t)k);
         return;
       }
   }
   void release() {
-    for (void* p : ptrs) cudaFreeAsync(p, st);
+    for (auto& p : ptrs) cudaFreeAsync(p.first, st);
     if (!ptrs.empty()) cudaStreamSynchronize(st);
     ptrs.clear();
     bytes = 0;

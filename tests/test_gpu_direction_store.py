@@ -49,3 +49,16 @@ def test_growth_that_fails_leaves_no_freed_memory_in_use(probe):
     for k in range(3):
         assert _rel(a.solve(F[k].contiguous(), tol=1e-10).cpu().numpy(), ref[:, k]) < 1e-7
     assert torch.equal(b.apply_precond(r), z)
+
+
+def test_held_bytes_count_the_store_once():
+    p = meshgen.elasticity3d(8, 4, seed=4, nrhs=8)
+    F = _dev(p.f.T)
+    held = []
+    for first in (True, False):   # the store grows from one column to eight, or starts with eight
+        s = BddcSolver(p, precision="mixed")
+        if first:
+            s.solve(F[0].contiguous(), tol=1e-10)
+        s.solve(F, tol=1e-10)
+        held.append(s.last_stats.factor_bytes)
+    assert held[0] == held[1]
