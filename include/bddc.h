@@ -247,6 +247,9 @@ int bddc_analyze(const bddc_mesh* mesh, const bddc_partition* part, unsigned con
  * K_i + rho C_i^T C_i with the constraint rows (yields the interior factor, Eq. psi_def's
  * coarse basis Psi_i and K_Ci = -Lambda_i), assembly of the next level, and the FP64
  * factorisation of the coarsest matrix K_C.  stream: a cudaStream_t (NULL = default).
+ * Mixed PCG handles with an outer refinement also keep the search directions of a solve: 1 KB per
+ * interface DOF, 8 KB from the first block of right-hand sides on, at most 4 GB; where that memory
+ * is not to be had they keep fewer or none, and solves take more iterations.
  * Errors: INVALID, BREAKDOWN (stats via bddc_get_stats), CUDA, OOM. */
 int bddc_setup(const bddc_mesh* mesh, const bddc_partition* part, unsigned constraints,
                const bddc_opts* opts, void* stream, bddc_handle* out);
@@ -307,10 +310,11 @@ int bddc_grad(bddc_handle h, const double* dJdu, const double* u, int nrhs, doub
  * by every GPU that loads the library until the process exits: meshes with
  * n_nodes * dofs_per_node > 1,048,576 are rejected with BDDC_ERR_INVALID.  The first call on a
  * device looks up that array's device address (cudaGetSymbolAddress).  The adjoint solve is the
- * handle's own: the first solve on a handle, and the first after the Krylov method changes,
- * builds the handle's cached CUDA graph of one iteration with its capture stream and events, so
- * warm a handle with one bddc_solve (or one call of this entry point) before relying on
- * allocation-free calls in a loop.  The call synchronises the handle's stream (it reads the
+ * handle's own, on the buffers of its set-up: the first solve on a handle, and the first after the
+ * Krylov method changes, builds the handle's cached CUDA graph of one iteration with its capture
+ * stream and events, and the handle's first block (nrhs > 1, PCG) allocates the work vectors of a
+ * block, so warm a handle with one bddc_solve (or one call of this entry point) of as many
+ * right-hand sides before relying on allocation-free calls in a loop.  The call synchronises the handle's stream (it reads the
  * Krylov scalars back every iteration), so it must not be made while that stream or the calling
  * thread is capturing a CUDA graph.  Every call on a device shares the array and overwrites the
  * part it reads, so calls whose work overlaps on the GPU (several streams, several host threads)

@@ -129,6 +129,17 @@ struct DevArena {
     bytes += (int64_t)sizeof(T) * n;
     return (T*)p;
   }
+  // as alloc, for memory that the caller can do without: null where there is none left
+  template <typename T>
+  T* try_alloc(int64_t n) {
+    try {
+      return alloc<T>(n);
+    } catch (const Fail& f) {
+      if (f.code != BDDC_ERR_OOM) throw;
+      g_err.clear();
+      return nullptr;
+    }
+  }
   template <typename T>
   T* upload(const raw_vector<T>& v, cudaStream_t st) {
     return upload_n(v.data(), (int64_t)v.size(), st);
@@ -350,10 +361,10 @@ struct bddc_handle_s {
   double* scal = nullptr;              // [16]
   double* partial = nullptr;           // [kDotBlocks], and the fused sums' 2 iface_blocks(n_iface) per column
   int* dot_cnt = nullptr;              // [blk] counters of the fused sums
-  KrylovStore kstore;                  // directions of the running refined solve (allocated by the first one)
+  KrylovStore kstore;                  // directions of the running refined solve (cap 0: none kept)
   double* proj_coef = nullptr;
   void* kstore_mem = nullptr;          // the block of memory that both lie in
-  int kstore_blk = 0;
+  int kstore_blk = 0;                  // the block size that it was asked for with
   double* h_scal = nullptr;            // pinned [16 kMaxBlock]
   double* mail = nullptr;              // pinned [4 kMaxBlock], written by the device (see launch_pcg_update_x_r)
   double *vx = nullptr, *vr = nullptr, *vz = nullptr, *vp = nullptr, *vq = nullptr, *vrold = nullptr, *vg = nullptr;
@@ -1608,6 +1619,8 @@ void tune_sweeps(bddc_handle_s* h, Level& L, cudaStream_t st) {
                        L.sweep_order[1]};
 }
 
+void prepare_kstore(bddc_handle_s* h);
+
 void numeric_setup(bddc_handle_s* h) {
   cudaStream_t st = h->st;
   const double t0 = now_ms();
@@ -1688,6 +1701,7 @@ void numeric_setup(bddc_handle_s* h) {
     h->use_outer = true;
     h->inner_steps = h->opts.inner_steps;
   }
+  prepare_kstore(h);
   h->stats.inner_steps = h->use_outer ? h->inner_steps : -1;
   h->stats.inner_operator = h->use_outer ? (h->lv[0].explicit_schur ? 2 : 1) : 0;
   h->factored = true;
@@ -2512,11 +2526,12 @@ PcgResult fgmres(bddc_handle_s* h, const double* g, double* x, double tol, int m
   return res;
 }
 
-// Storage for the directions of a refined solve: up to 128 per column and 4 GB per handle, allocated by the
-// first refined solve (and again by the first block of right-hand sides); iterations past the capacity are
-// not stored.
-void prepare_kstore(bddc_handle_s* h, int nb) {
-  if (h->kstore.cap > 0 && h->kstore_blk >= nb) return;
+// Storage for the directions of a refined solve: up to 128 per column and 4 GB per handle; iterations past the
+// capacity are not stored.  Made by the set-up for one column and by the first block of right-hand sides for
+// kMaxBlock.  It only saves iterations, so where device memory is short it gets a part of that capacity, or none
+// and every inner solve starts from zero.
+void prepare_kstore(bddc_handle_s* h) {
+  if (!h->use_outer || h->kstore_blk >= h->blk) return;
   ck(cudaStreamSynchronize(h->st), "sync");
   drop_graph(h);   // a cached iteration refers to the old storage
   DevArena& A = h->arena;
@@ -2525,21 +2540,23 @@ void prepare_kstore(bddc_handle_s* h, int nb) {
   void* old = h->kstore_mem;
   h->kstore = KrylovStore();
   h->kstore_mem = nullptr;
-  h->kstore_blk = 0;
   if (old) A.free_one(old);
-  const int blk = h->blk;
+  const int blk = h->kstore_blk = h->blk;
   const int64_t n = std::max<int64_t>(h->lv[0].d.n_iface, 1);
-  const int cap = (int)std::max<int64_t>(1, std::min<int64_t>(128, ((int64_t)4 << 30) / (8 * n * blk)));
-  const int64_t vec = n * cap * blk, coef = (int64_t)blk * cap * (kProjBlocks + 1);
-  double* mem = A.alloc<double>(vec + (int64_t)cap * blk + coef + kMaxBlock);   // p, q (FP32); d; coef; cnt
-  h->kstore_mem = mem;
-  h->kstore_blk = blk;
-  h->proj_coef = mem + vec + (int64_t)cap * blk;
-  h->kstore.p = (float*)mem;
-  h->kstore.q = (float*)mem + vec;
-  h->kstore.d = mem + vec;
-  h->kstore.cnt = (int*)(h->proj_coef + coef);
-  h->kstore.cap = cap;
+  int cap = (int)std::max<int64_t>(1, std::min<int64_t>(128, ((int64_t)4 << 30) / (8 * n * blk)));
+  for (; cap > 0; cap /= 2) {
+    const int64_t vec = n * cap * blk, coef = (int64_t)blk * cap * (kProjBlocks + 1);
+    double* mem = A.try_alloc<double>(vec + (int64_t)cap * blk + coef + kMaxBlock);   // p, q (FP32); d; coef; cnt
+    if (!mem) continue;
+    h->kstore_mem = mem;
+    h->proj_coef = mem + vec + (int64_t)cap * blk;
+    h->kstore.p = (float*)mem;
+    h->kstore.q = (float*)mem + vec;
+    h->kstore.d = mem + vec;
+    h->kstore.cnt = (int*)(h->proj_coef + coef);
+    h->kstore.cap = cap;
+    return;
+  }
 }
 
 // Mixed-precision iterative refinement around PCG (the outer iteration that restores FP64
@@ -2592,8 +2609,11 @@ std::vector<PcgResult> pcg_refined(bddc_handle_s* h, const double* g, double tol
                       tin(nb, 1.0);
   int inner = h->inner_steps;
   int its = 0;
-  prepare_kstore(h, nb);
-  ck(cudaMemsetAsync(h->kstore.cnt, 0, sizeof(int) * kMaxBlock, st), "memset");
+  if (nb > h->kstore_blk) prepare_kstore(h);   // the first block
+  auto forget_directions = [&]() {
+    if (h->kstore.cap > 0) ck(cudaMemsetAsync(h->kstore.cnt, 0, sizeof(int) * kMaxBlock, st), "memset");
+  };
+  forget_directions();
   bool stored = false;   // directions of the present inner operator
   for (int outer = 0; outer < kMaxOuter && its < maxit && left > 0; ++outer) {
     for (int k = 0; k < nb; ++k) {
@@ -2606,7 +2626,7 @@ std::vector<PcgResult> pcg_refined(bddc_handle_s* h, const double* g, double tol
     }
     h->cur_steps = inner;
     std::vector<PcgResult> in = pcg(h, ro, h->vx, tin, maxit - its, nb, true, stored);
-    stored = true;
+    stored = h->kstore.cap > 0;
     h->cur_steps = h->refine_steps;
     h->ext_of = nullptr;
     int most = 0;
@@ -2652,7 +2672,7 @@ std::vector<PcgResult> pcg_refined(bddc_handle_s* h, const double* g, double tol
     }
     if (stagnated && inner != h->refine_steps) {   // another operator: its own directions from here on
       inner = h->refine_steps;
-      ck(cudaMemsetAsync(h->kstore.cnt, 0, sizeof(int) * kMaxBlock, st), "memset");
+      forget_directions();
       stored = false;
     }
   }

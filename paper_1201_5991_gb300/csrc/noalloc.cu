@@ -10,8 +10,9 @@
 // one at a time, so the limit is 2 * n_full * 8 bytes <= 16 MiB, i.e. n_full <= 1,048,576
 // (n_full = nodes * DOFs per node, prescribed DOFs included); larger meshes are rejected with
 // BDDC_ERR_INVALID.  The adjoint solve itself uses only the buffers the handle allocated at
-// set-up, once the handle is warm: its first solve (and the first after a change of Krylov
-// method) captures the CUDA graph of one iteration and creates that graph's stream and events.
+// set-up (and, for several right-hand sides, at its first block of them), once the handle is warm:
+// its first solve (and the first after a change of Krylov method) captures the CUDA graph of one
+// iteration and creates that graph's stream and events.
 // The call synchronises the handle's stream, so it cannot run inside a stream capture.
 #include <cuda_runtime.h>
 

@@ -62,3 +62,37 @@ def test_held_bytes_count_the_store_once():
         s.solve(F, tol=1e-10)
         held.append(s.last_stats.factor_bytes)
     assert held[0] == held[1]
+
+
+def test_first_solve_allocates_nothing(probe):
+    p = meshgen.elasticity3d(8, 4, seed=4)
+    ref = fem.direct_solve(p)[:, 0]
+    for prec in ("mixed", "fp64"):
+        s = BddcSolver(p, precision=prec)
+        probe(1)                                           # no further allocation of a handle succeeds
+        assert _rel(s.solve(_dev(p.f[:, 0]), tol=1e-10).cpu().numpy(), ref) < 1e-7
+        probe(0)
+
+
+def test_solves_with_less_store_or_none(probe):
+    # a block's store takes 8 columns; the column's own 128 directions make room for 16 of each, one byte less for
+    # 8 (fewer than the iterations of one solve), and less than a sixteenth of them for none
+    p = meshgen.elasticity3d(8, 4, seed=4, nrhs=8)
+    ref = fem.direct_solve(p)
+    F = _dev(p.f.T)
+    its = {}
+    for room in ("all", "16", "8", "none"):
+        s = BddcSolver(p, precision="mixed")
+        s.apply_schur(torch.zeros(8, s.n_iface, dtype=torch.float64, device="cuda"))
+        s.solve(F[0].contiguous(), tol=1e-10)
+        held, store = s.last_stats.factor_bytes, 128 * 8 * s.n_iface
+        probe({"all": 0, "16": held, "8": held - 1, "none": held - store * 31 // 32}[room])
+        U = s.solve(F, tol=1e-10).cpu().numpy()
+        assert s.last_stats.converged == 1
+        its[room] = s.last_stats.iterations
+        assert all(_rel(U[k], ref[:, k]) < 1e-7 for k in range(8)), room
+        assert torch.equal(s.solve(F, tol=1e-10), s.solve(F, tol=1e-10)), room
+        grown = s.last_stats.factor_bytes - held
+        assert {"all": grown > 6 * store, "16": grown == 0, "8": -store < grown < 0, "none": grown <= -store}[room], room
+        probe(0)
+    assert its["all"] <= its["16"] <= its["none"] and its["8"] <= its["none"], its
