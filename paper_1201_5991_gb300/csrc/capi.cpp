@@ -337,6 +337,7 @@ struct bddc_handle_s {
   std::vector<int64_t> n_parts;
   int n_levels = 2;
   std::vector<Level> lv;               // BDDC levels 1..L-1, then the coarsest
+  bool compact = false;                // set-up without the memory that only saves time (bddc_setup)
   DevArena arena;
   // device copies of level-1 mesh data
   double* d_coords = nullptr;
@@ -615,10 +616,10 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
       base += b * (b + 1) / 2;
       padded += bp * (bp + 1) / 2;
     }
-    L.explicit_schur = h->opts.inner_operator == 2 || padded <= 1.4 * base;
+    L.explicit_schur = h->opts.inner_operator == 2 || padded <= (h->compact ? 1.08 : 1.4) * base;
   }
   // the interface inverse comes with the tensor-core factorisation (its panel solves carry the inverse rows)
-  L.inverse = L.fp32 && !L.coarsest && h->opts.tensor_cores && h->opts.tensor_cores != 2;
+  L.inverse = L.fp32 && !L.coarsest && h->opts.tensor_cores && h->opts.tensor_cores != 2 && !h->compact;
   for (int64_t s = 0; s < ns; ++s) {
     SubMeta& m = L.meta[s];
     m.n = (int32_t)(mp.sub_dof_ptr[s + 1] - mp.sub_dof_ptr[s]);
@@ -637,7 +638,8 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     m.inv_off = tile + (int64_t)m.nV * (m.nV + 1) / 2 * NB2;
     tile += (int64_t)m.nV * (m.nV + 1) * NB2;
     m.x_off = xoff;
-    xoff += ceil_div(m.Bc, kSub) * 6 * NB2;
+    m.x_step = h->compact ? 0 : 6;
+    xoff += (h->compact ? 1 : ceil_div(m.Bc, kSub)) * 6 * NB2;
     m.dinv_off = dinv;
     dinv += (int64_t)m.Bc * NB2;
     m.vec_off = vec;
@@ -943,6 +945,7 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     d.c_rho = A.upload(c_rho, st);
   }
   d.xinv = nullptr;
+  d.x_kept = 0;
   d.indefinite = h->physics == BDDC_STOKES ? 1 : 0;
   d.wait_probe = h->opts.wait_probe ? 1 : 0;
   d.sgn = L.fp32 ? (void*)A.alloc<float>(L.n_vec) : (void*)A.alloc<double>(L.n_vec);
@@ -966,7 +969,10 @@ void prepare_level(bddc_handle_s* h, Level& L, DevArena& A, cudaStream_t st) {
     if (h->physics == BDDC_STOKES) L.split_signed = A.alloc<uint8_t>(rows * kPanel * 2 * NB2 * 2);
     L.rscale = A.alloc<float>(rows * NB);
     L.tc_panels = h->opts.tensor_cores != 2;
-    if (L.tc_panels) d.xinv = A.alloc<float>(xoff);
+    if (L.tc_panels) {
+      d.xinv = A.alloc<float>(xoff);
+      d.x_kept = h->compact ? 0 : 1;
+    }
     // work items (128 x 128 output blocks) of the updates of every super-panel, flattened over the
     // subdomains; update 0 covers the columns [kb0 + kSub, kb0 + kPanel), update 1 the columns
     // >= kb0 + kPanel, update 2 (a super-panel where some interior ends in the middle, explicit
@@ -2842,24 +2848,42 @@ int bddc_setup(const bddc_mesh* mesh, const bddc_partition* part, unsigned const
   return guarded([&]() {
     if (!out) fail(BDDC_ERR_INVALID, "null output handle");
     *out = nullptr;
-    auto* h = new bddc_handle_s();
-    if (opts) h->opts = *opts; else bddc_default_opts(&h->opts);
-    if (h->opts.maxit <= 0) h->opts.maxit = 500;
-    h->constraints = constraints;
-    h->st = (cudaStream_t)stream;
-    h->arena.st = h->st;
-    try {
-      analysis(h, mesh, part, [h]() { early_device(h); });
-      device_setup(h);
-      numeric_setup(h);
-    } catch (...) {
-      h->arena.release();
-      if (h->h_scal) cudaFreeHost(h->h_scal);
-      delete h;
-      throw;
+    // Mixed handles keep more than their factors to save time: the interface inverses (by the tile counts 1.3x the
+    // memory of the tiles for subdomains of 12^3 elements, 1.5x for 8^3, 1.7x for 4^3), padded interiors for the
+    // explicit inner operator and the diagonal blocks' inverses.  Where that does not fit the device, the set-up is
+    // made again in the compact form: interface sweeps, plain interior sweeps, padding of at most 8 %.
+    for (bool compact = false;; compact = true) {
+      auto* h = new bddc_handle_s();
+      if (opts) h->opts = *opts; else bddc_default_opts(&h->opts);
+      if (h->opts.maxit <= 0) h->opts.maxit = 500;
+      h->compact = compact;
+      h->constraints = constraints;
+      h->st = (cudaStream_t)stream;
+      h->arena.st = h->st;
+      const bool may_compact = !compact && h->opts.precision == BDDC_PREC_MIXED && h->opts.tensor_cores;
+      auto discard = [h]() {
+        h->arena.release();
+        if (h->h_scal) cudaFreeHost(h->h_scal);
+        delete h;
+      };
+      try {
+        analysis(h, mesh, part, [h]() { early_device(h); });
+        device_setup(h);
+        numeric_setup(h);
+      } catch (const Fail& f) {
+        const bool again = f.code == BDDC_ERR_OOM && may_compact;
+        discard();
+        if (!again) throw;
+        g_err.clear();
+        cudaMemPoolTrimTo(library_pool(), 0);   // blocks of other sizes come next
+        continue;
+      } catch (...) {
+        discard();
+        throw;
+      }
+      *out = h;
+      return BDDC_OK;
     }
-    *out = h;
-    return BDDC_OK;
   });
 }
 

@@ -37,6 +37,7 @@ struct SubMeta {
   int32_t nIb, nGb, ncb, Bc;      // block counts; Bc = nIb + nGb
   int32_t R;                      // block rows = Bc + ncb
   int32_t nV;                     // inverse rows (nGb, or 0)
+  int32_t x_step;                 // tiles of the 256-wide diagonal blocks' inverses kept per block: 6, or 0 (one block's place)
   int64_t tile_off;               // element offset of the tiles in the level's tile buffer
   int64_t dinv_off;               // element offset of the Bc diagonal inverses
   int64_t vec_off;                // offset of the padded local vector
@@ -67,7 +68,7 @@ __host__ __device__ inline bool tile_exists(const SubMeta& m, int i, int j) {
 
 // tile (Q, P), P < Q < 4, of the inverse of the diagonal block that starts at block column k0 (a multiple of 4)
 __host__ __device__ inline int64_t x_tile(const SubMeta& m, int k0, int Q, int P) {
-  return m.x_off + ((int64_t)(k0 / 4) * 6 + Q * (Q - 1) / 2 + P) * NB2;
+  return m.x_off + ((int64_t)(k0 / 4) * m.x_step + Q * (Q - 1) / 2 + P) * NB2;
 }
 
 // Raw device pointers of one level, passed by value to kernels.
@@ -118,6 +119,7 @@ struct LevelDev {
   void* psiT;                     // Psi_G^T in tiles: tile (rb, j) of a subdomain at psiT_off + (rb nGb + j) NB2
   float* xinv;                    // FP32 levels with tensor-core panels, or null: of every 256-wide diagonal block
                                   // D = [4 d, 4 d + 4) the tiles (Q, P), P < Q, of X = L_D^{-1} (x_tile)
+  int x_kept;                     // 1: those of every block at once (x_step 6), 0: the block's that is being factored
   float* schur;                   // explicit augmented Schur complement of the interface (mixed inner operator), or null
   void* sgn;                      // [n_vec] pivot signs of the signed Cholesky (T; +1 for SPD levels)
   int32_t* crow;                  // [n_vec] constraint row of a position (flat over the level) or -1 (level 1, FP32), or null

@@ -442,7 +442,7 @@ void launch_sweep_g(const LevelDev& L, T* vec, const int2* const* tasks, const i
   // 11.4 -> 10.9, 48^3 (bound by HBM) as before.  With eight columns the tiles' products bound the sweep and
   // the extra exchange costs: FP64 operator on 8 columns (48^3) 5.97 -> 6.19 ms, so those keep single rows.
   if constexpr (sizeof(T) == 4 && NR <= 2) {
-    if (part == 0 && L.xinv) {   // the inverses of the 256-wide diagonal blocks are at hand
+    if (part == 0 && L.x_kept) {   // the inverses of the 256-wide diagonal blocks are at hand
       launch_sweep_s<T, S, NR, true>(L, vec, tasks, ntasks, part, which, scratch, grid_max, st);
       return;
     }
