@@ -1555,12 +1555,14 @@ void choose_refinement(bddc_handle_s* h) {
 // CTAs per SM of the persistent grid (1, 2), tile-ring depth (shallow, deep), task order (subdomain
 // order, longest chains first).  The sweeps compute the same result bit for bit in every variant
 // (each block row adds its tile contributions in a fixed order), so the choice only moves time.
-// Results are cached per level shape (precision, subdomain count, block-row histogram).
+// Results are cached per level shape (precision, subdomain count, block-row histogram) and form of its sweeps
+// (grouped interior sweeps; none over the interface with its inverse, so none is tuned there).
 std::mutex g_tune_mu;
 std::map<std::string, std::array<int, 6>> g_tune_cache;
 
 std::string level_shape_key(const Level& L) {
-  std::string k = (L.fp32 || L.solve32 ? "f" : "d") + std::to_string(L.meta.size()) + ":";
+  std::string k = std::string(L.fp32 || L.solve32 ? "f" : "d") + (L.inverse ? "i" : "s") + (L.d.x_kept ? "g" : "p") +
+                  std::to_string(L.meta.size()) + ":";
   for (const SubMeta& m : L.meta) k += std::to_string(m.nIb) + "," + std::to_string(m.nGb) + ";";
   return k;
 }

@@ -45,3 +45,11 @@ def test_setup_that_does_not_fit_is_made_compact(prob):
     finally:
         capi.lib().bddc_alloc_probe(0)
     assert smallest is not None and smallest < 0.9 * rest, (smallest, rest, held)
+
+
+def test_forms_of_one_shape_are_tuned_apart():
+    # a handle without the interface inverse has interface sweeps to tune, whatever was cached for one with it
+    p = meshgen.poisson2d(91, 7)   # 49 subdomains: a shape of this test alone
+    assert BddcSolver(p, precision="mixed").stats().tune_ms > 0
+    assert BddcSolver(p, precision="mixed").stats().tune_ms == 0
+    assert BddcSolver(p, precision="mixed", tensor_cores=2).stats().tune_ms > 0
