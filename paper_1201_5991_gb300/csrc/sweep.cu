@@ -438,10 +438,11 @@ void launch_sweep_s(const LevelDev& L, T* vec, const int2* const* tasks, const i
 template <typename T, int S, int NR>
 void launch_sweep_g(const LevelDev& L, T* vec, const int2* const* tasks, const int* ntasks, int part, int which,
                     void* scratch, int grid_max, cudaStream_t st) {
-  // Up to two columns, where the chain of block rows counts: 24^3 solve (8 subdomains) 8.41 -> 7.50 ms, tetrahedra
-  // 11.4 -> 10.9, 48^3 (bound by HBM) as before.  With eight columns the tiles' products bound the sweep and
-  // the extra exchange costs: FP64 operator on 8 columns (48^3) 5.97 -> 6.19 ms, so those keep single rows.
-  if constexpr (sizeof(T) == 4 && NR <= 2) {
+  // Any number of columns, so that a column of a block has the arithmetic of a single one.  It pays up to two columns,
+  // where the chain of block rows counts: 24^3 solve (8 subdomains) 8.41 -> 7.50 ms, tetrahedra 11.4 -> 10.9, 48^3
+  // (bound by HBM) as before.  With eight columns the tiles' products bound the sweep and the extra exchange
+  // costs up to 1 %: FP64 operator on 8 columns (48^3) 6.11 -> 6.16 ms, 64^3 with 16 loads 444.6 -> 448.3.
+  if constexpr (sizeof(T) == 4) {
     if (part == 0 && L.x_kept) {   // the inverses of the 256-wide diagonal blocks are at hand
       launch_sweep_s<T, S, NR, true>(L, vec, tasks, ntasks, part, which, scratch, grid_max, st);
       return;
