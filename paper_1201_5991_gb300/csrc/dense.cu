@@ -989,7 +989,7 @@ __global__ void k_cc_mu(LevelDev L, const int32_t* __restrict__ crow_sub, int64_
 // out_p = z_C[R_Ci p] - sum_q G_pq t_q: one warp per constraint row, its row of G read once for NR columns
 template <int NR>
 __global__ void k_coarse_coef(LevelDev L, const int32_t* __restrict__ crow_sub, int64_t total_rows,
-                              const double* __restrict__ zC, const double* __restrict__ t, double* __restrict__ out) {
+                              const double* zC, const double* t, double* __restrict__ out) {
   pdl_wait();
   pdl_trigger();
   const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -1051,7 +1051,7 @@ __device__ __forceinline__ const T* m_tile(const LevelDev& L, const SubMeta& m, 
 // no such tile columns).  Warp w takes the rows w, w+8, .., lane l the columns 2l, 2l+1 of every
 // tile, so each tile row is one coalesced 256-byte read; rows past nc are not read.
 template <typename T, int NR, int MODE>
-__global__ void __launch_bounds__(256) k_rows_matvec(LevelDev L, const T* __restrict__ vec, double* __restrict__ part,
+__global__ void __launch_bounds__(256) k_rows_matvec(LevelDev L, const T* vec, double* __restrict__ part,
                                                      int zmax, int64_t sum_nc) {
   pdl_wait();
   pdl_trigger();
@@ -1121,7 +1121,7 @@ __global__ void k_sum_parts(const double* __restrict__ part, int zmax, int64_t t
 // zsub + q sum_nc, per-subdomain coarse vectors); the eight warps' partial sums are added in a
 // fixed order.
 template <typename T, int NR, int MODE>
-__global__ void __launch_bounds__(256) k_cols_matvec(LevelDev L, T* __restrict__ vec, const double* __restrict__ zsub,
+__global__ void __launch_bounds__(256) k_cols_matvec(LevelDev L, T* __restrict__ vec, const double* zsub,
                                                      int64_t sum_nc, T sign) {
   pdl_wait();
   pdl_trigger();
@@ -1356,7 +1356,7 @@ __global__ void __launch_bounds__(256) k_coarse_mirror(float* __restrict__ W, in
 // z = W x for nr columns (x: columns of n_vec, padded local positions 0 .. npad-1; z: level DOFs); one warp
 // per output row, lanes along the row (coalesced), FP32 sums in a fixed order.
 template <int NR>
-__global__ void k_coarse_apply(const float* __restrict__ W, int64_t npad, const float* __restrict__ x,
+__global__ void k_coarse_apply(const float* __restrict__ W, int64_t npad, const float* x,
                                double* __restrict__ z, const int32_t* __restrict__ loc2glob, int64_t n_vec,
                                int64_t n_dof) {
   pdl_wait();

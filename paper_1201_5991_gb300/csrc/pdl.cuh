@@ -3,6 +3,9 @@
 // its first instruction that touches global memory depends on, returns when that kernel has completed with
 // its stores visible.  Every such kernel waits, so completion is transitive along the stream.  pdl_trigger lets
 // the next kernel be set up once every block of this one has started (it would otherwise be at its end).
+// Such a kernel is alive while the kernels before it still write, so what they write may not be read as data that
+// is constant for the kernel's life: no __ldg, and no const __restrict__ parameter (from which the compiler
+// makes the same loads), for vectors of the running solve.  Data of the set-up may be read so.
 // Use only where the launch before it in the same stream is a kernel (not a copy, a memset or an event wait).
 #pragma once
 

@@ -31,7 +31,7 @@ __device__ __forceinline__ int64_t tile_index_t(int i, int j, int Bc) {
 // read, applied to all NR columns; the eight warps' column sums are added at the end in a fixed
 // order (no barrier inside the tile loop).
 template <int NR>
-__global__ void __launch_bounds__(256) k_trmv_t(LevelDev L, const float* __restrict__ x, float* __restrict__ y1) {
+__global__ void __launch_bounds__(256) k_trmv_t(LevelDev L, const float* x, float* __restrict__ y1) {
   pdl_wait();
   pdl_trigger();
   const int s = blockIdx.y;
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256) k_trmv_t(LevelDev L, const float* __restr
       const float2 a = __ldg((const float2*)(t + row * NB));
 #pragma unroll
       for (int q = 0; q < NR; ++q) {
-        const float xr = grow < nGrow ? __ldg(xv + q * L.n_vec + grow) : 0.f;
+        const float xr = grow < nGrow ? xv[q * L.n_vec + grow] : 0.f;
         ax[q] += a.x * xr;
         ay[q] += a.y * xr;
       }
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(256) k_trmv_t(LevelDev L, const float* __restr
 // with o = nGb - 1 - o' (the longest block rows are scheduled first, so that the short ones fill
 // the tail of the launch).  Warp w takes rows w, w+8, ..., lane l the columns 2l, 2l+1.
 template <int NR>
-__global__ void __launch_bounds__(256) k_trmv_n(LevelDev L, const float* __restrict__ y1, float* __restrict__ y) {
+__global__ void __launch_bounds__(256) k_trmv_n(LevelDev L, const float* y1, float* __restrict__ y) {
   pdl_wait();
   pdl_trigger();
   const int s = blockIdx.y;
@@ -196,7 +196,7 @@ __device__ __forceinline__ void tile_g2s(float* dst, const float* src, uint64_t*
 }
 
 template <int NR>
-__global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, int inverse, const float* __restrict__ x,
+__global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, int inverse, const float* x,
                                                          const int64_t* __restrict__ part_off, int64_t part_stride,
                                                          float* __restrict__ part, float* __restrict__ y) {
   const int s = blockIdx.y;
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, int inverse
   for (int j = 0; j < ntile; ++j) {
     float2 xj[NR];
 #pragma unroll
-    for (int q = 0; q < NR; ++q) xj[q] = __ldg((const float2*)(xv + q * L.n_vec + (int64_t)j * NB + 2 * lane));
+    for (int q = 0; q < NR; ++q) xj[q] = *(const float2*)(xv + q * L.n_vec + (int64_t)j * NB + 2 * lane);
     const int slot = j % kSymvStages;
     {
       long long spins = 0;
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(256) k_schur_symv_rows(LevelDev L, int inverse
 // order: a fixed order, the same for any number of columns per launch.
 template <int NR>
 __global__ void __launch_bounds__(256) k_schur_symv_cols(LevelDev L, float sign, const int64_t* __restrict__ part_off,
-                                                         int64_t part_stride, const float* __restrict__ part,
+                                                         int64_t part_stride, const float* part,
                                                          float* __restrict__ y) {
   pdl_wait();
   pdl_trigger();

@@ -17,7 +17,7 @@ namespace {
 // columns one after another with its own length as the stride (local vectors n_vec, interface
 // vectors n_iface, level vectors n_dof, coarse vectors n_coarse, per-subdomain coarse vectors sum nc).
 template <typename T>
-__global__ void k_gather_iface(LevelDev L, const double* __restrict__ x, int weighted, T* __restrict__ loc) {
+__global__ void k_gather_iface(LevelDev L, const double* x, int weighted, T* __restrict__ loc) {
   pdl_wait();
   pdl_trigger();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -121,7 +121,7 @@ __device__ __forceinline__ double sum_occurrences(const LevelDev& L, int64_t g, 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_scatter_iface(LevelDev L, const T* __restrict__ loc, int weighted,
+__global__ void __launch_bounds__(256) k_scatter_iface(LevelDev L, const T* loc, int weighted,
                                                        double* __restrict__ y, FusedDot dot) {
   pdl_wait();
   pdl_trigger();
@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(256) k_scatter_iface(LevelDev L, const T* __re
 // inner operator, before its FP32 product: blocks below nv gather loc = R_i x, the others take one
 // constraint row per warp: t = rho c_rho (C_i R_i x); NR columns per pass over the index lists
 template <int NR>
-__global__ void __launch_bounds__(256) k_inner_gather(LevelDev L, const double* __restrict__ x, float* __restrict__ loc,
+__global__ void __launch_bounds__(256) k_inner_gather(LevelDev L, const double* x, float* __restrict__ loc,
                                                       int nv, const int32_t* __restrict__ crow_sub, int64_t total_rows,
                                                       double* __restrict__ t) {
   pdl_wait();
@@ -173,8 +173,8 @@ __global__ void __launch_bounds__(256) k_inner_gather(LevelDev L, const double* 
 
 // y = sum R_i^T (loc - C_i^T t): distinct constraint rows touch disjoint positions (each local DOF lies in
 // one glob and has one component)
-__global__ void __launch_bounds__(256) k_inner_scatter(LevelDev L, const float* __restrict__ loc,
-                                                       const double* __restrict__ t, int64_t total_rows,
+__global__ void __launch_bounds__(256) k_inner_scatter(LevelDev L, const float* loc,
+                                                       const double* t, int64_t total_rows,
                                                        double* __restrict__ y, FusedDot dot) {
   pdl_wait();
   pdl_trigger();
@@ -243,7 +243,7 @@ __global__ void k_scatter_interior_diff(LevelDev L, const double* __restrict__ a
 // once per column: 48^3, 8 columns 700 us.
 template <int NR, int LR>
 __global__ void __launch_bounds__(256) k_spmv(LevelDev L, const int64_t* __restrict__ rows, int64_t nrows,
-                                              const double* __restrict__ x, double* __restrict__ y, double alpha,
+                                              const double* x, double* __restrict__ y, double alpha,
                                               double beta, const int32_t* __restrict__ row_sub) {
   pdl_wait();
   pdl_trigger();
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(256) k_spmv(LevelDev L, const int64_t* __restr
 }
 
 template <typename Tin, typename Tout>
-__global__ void k_convert(const Tin* __restrict__ in, Tout* __restrict__ out, int64_t n) {
+__global__ void k_convert(const Tin* in, Tout* __restrict__ out, int64_t n) {
   pdl_wait();
   pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -303,14 +303,14 @@ __global__ void k_convert(const Tin* __restrict__ in, Tout* __restrict__ out, in
 }
 
 template <typename T>
-__global__ void k_add_to_double(double* __restrict__ y, const T* __restrict__ x, int64_t n) {
+__global__ void k_add_to_double(double* __restrict__ y, const T* x, int64_t n) {
   pdl_wait();
   pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) y[i] += (double)x[i];
 }
 
-__global__ void k_axpy(double* __restrict__ y, const double* __restrict__ x, double a, int64_t n) {
+__global__ void k_axpy(double* __restrict__ y, const double* x, double a, int64_t n) {
   pdl_wait();
   pdl_trigger();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -319,7 +319,7 @@ __global__ void k_axpy(double* __restrict__ y, const double* __restrict__ x, dou
 
 // One warp per coarse DOF, which owns its per-subdomain rows: 4 rows at a time, 8 lanes along each row's parts
 // (a thread per DOF summed up to 120 parts in a chain of loads).
-__global__ void k_coarse_gather(LevelDev L, const double* __restrict__ part, int zmax, double* __restrict__ rc_sub,
+__global__ void k_coarse_gather(LevelDev L, const double* part, int zmax, double* __restrict__ rc_sub,
                                 int64_t sum_nc, double* __restrict__ rC, float* __restrict__ v32,
                                 const int32_t* __restrict__ v32_pos, int64_t n_v32) {
   pdl_wait();
@@ -391,7 +391,7 @@ __global__ void k_dot_final(const double* __restrict__ partial, int nblk, double
 }
 
 __global__ void __launch_bounds__(256) k_pcg_xr(double* __restrict__ x, double* __restrict__ r,
-                                                const double* __restrict__ p, const double* __restrict__ q,
+                                                const double* p, const double* q,
                                                 double* __restrict__ scal, int64_t n, double* __restrict__ partial,
                                                 int* cnt, KrylovStore ks, double* mail) {
   pdl_wait();
@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(256) k_project_apply(KrylovStore ks, const dou
   r[(int64_t)k * n + i] = rs;
 }
 
-__global__ void k_pcg_p(double* __restrict__ p, const double* __restrict__ z, const double* __restrict__ scal,
+__global__ void k_pcg_p(double* __restrict__ p, const double* z, const double* scal,
                         int64_t n) {
   pdl_wait();
   pdl_trigger();
