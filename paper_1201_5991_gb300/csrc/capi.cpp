@@ -1290,7 +1290,10 @@ void trsv_pair(bddc_handle_s* h, Level& L, T* v, int part, cudaStream_t st, int 
   trsv<T>(h, L, v, part, 2, st, nb);
 }
 
-// w = K_II^{-1} v on level 1 (interior positions), FP64 accuracy.
+// w = K_II^{-1} v on level 1 (interior positions), FP64 accuracy; the operation before it is a kernel.  The launch
+// behind a sweep is a plain one, here and in full_step: with it launched over the sweep's end too, the short
+// kernels up to the next sweep are a chain of four such launches, and S x takes longer by 30 us of 628 (24^3, 8
+// subdomains; 64 subdomains 205 -> 188, 48^3 2,562 -> 2,553).
 // FP64 factors: two sweeps.  FP32 factors: iterative refinement with the FP64 K_II.
 void interior_solve_l1(bddc_handle_s* h, Level& L, const double* v, double* w, cudaStream_t st, int nb = 1) {
   const int64_t n = L.n_vec * nb;
@@ -1301,15 +1304,17 @@ void interior_solve_l1(bddc_handle_s* h, Level& L, const double* v, double* w, c
   }
   float* t = (float*)L.locB;
   double* r = L.dl3;
-  ck(cudaMemsetAsync(w, 0, sizeof(double) * n, st), "memset");
   const int steps = std::max(1, h->cur_steps);
   for (int it = 0; it < steps; ++it) {
-    launch_convert<double, float>(it == 0 ? v : r, t, n, st);
+    launch_convert<double, float>(it == 0 ? v : r, t, n, st, kAfterKernel);
     trsv_pair<float>(h, L, t, 0, st, nb);
-    launch_add_to_double<float>(w, t, n, st);
-    if (it + 1 < steps) {
-      ck(cudaMemcpyAsync(r, v, sizeof(double) * n, cudaMemcpyDeviceToDevice, st), "copy");
-      launch_spmv_rows(L.d, L.rows[0], L.nrows[0], w, r, -1.0, 1.0, L.row_sub, st, nb);
+    if (it == 0)
+      launch_convert<float, double>(t, w, n, st);
+    else
+      launch_add_to_double<float>(w, t, n, st);
+    if (it + 1 < steps) {   // r = v - K_II w
+      launch_convert<double, double>(v, r, n, st, kAfterKernel);
+      launch_spmv_rows(L.d, L.rows[0], L.nrows[0], w, r, -1.0, 1.0, L.row_sub, st, nb, kAfterKernel);
     }
   }
 }
@@ -1336,13 +1341,14 @@ void schur_apply(bddc_handle_s* h, const double* x, double* y, cudaStream_t st, 
     launch_inner_scatter(L.d, yf, L.cc_t, L.sum_nc, y, st, nb, dot);
     return;
   }
-  launch_gather_iface<double>(L.d, x, 0, L.dl0, st, nb);                 // x_i = R_i x
   ck(cudaMemsetAsync(L.dl1, 0, sizeof(double) * n, st), "memset");
-  launch_spmv_rows(L.d, L.rows[0], L.nrows[0], L.dl0, L.dl1, 1.0, 0.0, L.row_sub, st, nb);  // v = K_IG x_i
+  launch_gather_iface<double>(L.d, x, 0, L.dl0, st, nb);                 // x_i = R_i x
+  launch_spmv_rows(L.d, L.rows[0], L.nrows[0], L.dl0, L.dl1, 1.0, 0.0, L.row_sub, st, nb, kAfterKernel);  // v = K_IG x_i
   interior_solve_l1(h, L, L.dl1, L.dl2, st, nb);                        // w = K_II^{-1} v
-  launch_axpy_loc(L.dl0, L.dl2, -1.0, n, st);                           // t = [-w ; x_i]
-  launch_spmv_rows(L.d, L.rows[1], L.nrows[1], L.dl0, L.dl1, 1.0, 0.0, L.row_sub, st, nb);  // y_i = K_GG x_i - K_GI w
-  launch_scatter_iface<double>(L.d, L.dl1, 0, y, st, nb, dot);           // y = sum R_i^T y_i
+  launch_axpy_loc(L.dl0, L.dl2, -1.0, n, st, L.fp32 ? kAfterKernel : 0);   // t = [-w ; x_i]
+  launch_spmv_rows(L.d, L.rows[1], L.nrows[1], L.dl0, L.dl1, 1.0, 0.0, L.row_sub, st, nb,
+                   kAfterKernel);                                       // y_i = K_GG x_i - K_GI w
+  launch_scatter_iface<double>(L.d, L.dl1, 0, y, st, nb, dot, kAfterKernel);   // y = sum R_i^T y_i
 }
 
 // g = f_G - sum R_i^T K_GI K_II^{-1} f_I   (f: nb columns of n_free)
@@ -1350,8 +1356,8 @@ void condensed_rhs(bddc_handle_s* h, const double* f, double* g, cudaStream_t st
   Level& L = h->lv[0];
   launch_gather_glob<double>(L.d, f, 0, L.dl1, st, nb);
   interior_solve_l1(h, L, L.dl1, L.wf, st, nb);
-  launch_spmv_rows(L.d, L.rows[1], L.nrows[1], L.wf, L.dl0, 1.0, 0.0, L.row_sub, st, nb);
-  launch_scatter_iface<double>(L.d, L.dl0, 0, L.gi0, st, nb);
+  launch_spmv_rows(L.d, L.rows[1], L.nrows[1], L.wf, L.dl0, 1.0, 0.0, L.row_sub, st, nb, L.fp32 ? kAfterKernel : 0);
+  launch_scatter_iface<double>(L.d, L.dl0, 0, L.gi0, st, nb, FusedDot(), kAfterKernel);
   launch_iface_rhs(g, f, L.d.n_dof, L.iface_dofs, L.gi0, L.d.n_iface, st, nb);
 }
 
@@ -1368,7 +1374,7 @@ void recover(bddc_handle_s* h, const double* f, const double* uG, double* u, cud
   } else {
     launch_gather_iface<double>(L.d, uG, 0, L.dl0, st, nb);
     launch_gather_glob<double>(L.d, f, 0, L.dl1, st, nb);
-    launch_spmv_rows(L.d, L.rows[0], L.nrows[0], L.dl0, L.dl1, -1.0, 1.0, L.row_sub, st, nb);
+    launch_spmv_rows(L.d, L.rows[0], L.nrows[0], L.dl0, L.dl1, -1.0, 1.0, L.row_sub, st, nb, kAfterKernel);
     interior_solve_l1(h, L, L.dl1, L.dl2, st, nb);
     launch_scatter_interior<double>(L.d, L.dl2, u, st, nb);
   }
@@ -1400,10 +1406,10 @@ void full_step(bddc_handle_s* h, int l, const double* r, double* z, cudaStream_t
 // coarse residual, coarse correction (coarsest solve or the next level), combine.
 template <typename T>
 void interface_step_t(bddc_handle_s* h, int l, const double* rhat, double* zhat, cudaStream_t st, int nb,
-                      const FusedDot& dot) {
+                      const FusedDot& dot, int after_kernel) {
   Level& L = h->lv[l];
   T* v = (T*)L.locA;
-  launch_gather_iface<T>(L.d, rhat, 1, v, st, nb);          // r_i = E_i^T r_hat
+  launch_gather_iface<T>(L.d, rhat, 1, v, st, nb, after_kernel);   // r_i = E_i^T r_hat
   const bool last = l + 2 == (int)h->lv.size();
   const Level& C = h->lv.back();
   auto coarse_residual = [&](cudaStream_t cs) {   // r_C = sum R_Ci^T Psi_i^T r_i
@@ -1440,7 +1446,7 @@ void interface_step_t(bddc_handle_s* h, int l, const double* rhat, double* zhat,
     }
     ck(cudaStreamWaitEvent(st, f.in, 0), "join");
     launch_psi_apply_add<float>(L.d, L.zc_sub, L.sum_nc, z, L.max_nGb, L.max_ncb, st, nb);
-    launch_scatter_iface<float>(L.d, z, 1, zhat, st, nb, dot); // z_hat = sum E_i (...)
+    launch_scatter_iface<float>(L.d, z, 1, zhat, st, nb, dot, L.sum_nc > 0 ? kAfterKernel : 0);   // z_hat = sum E_i (...)
     return;
   }
   coarse_residual(st);
@@ -1451,15 +1457,15 @@ void interface_step_t(bddc_handle_s* h, int l, const double* rhat, double* zhat,
   coarse_correction(st);
   launch_coarse_scatter_n(L.d.sub_coarse, L.sum_nc, L.zC, L.d.n_coarse, L.zc_sub, st, nb);
   launch_psi_apply_add<T>(L.d, L.zc_sub, L.sum_nc, v, L.max_nGb, L.max_ncb, st, nb);   // Psi_i R_Ci z_C + z_i
-  launch_scatter_iface<T>(L.d, v, 1, zhat, st, nb, dot);       // z_hat = sum E_i (...)
+  launch_scatter_iface<T>(L.d, v, 1, zhat, st, nb, dot, kAfterKernel);   // z_hat = sum E_i (...)
 }
 
 void interface_step(bddc_handle_s* h, int l, const double* rhat, double* zhat, cudaStream_t st, int nb,
-                    const FusedDot& dot = FusedDot()) {
+                    const FusedDot& dot = FusedDot(), int after_kernel = 0) {
   if (h->lv[l].fp32)
-    interface_step_t<float>(h, l, rhat, zhat, st, nb, dot);
+    interface_step_t<float>(h, l, rhat, zhat, st, nb, dot, after_kernel);
   else
-    interface_step_t<double>(h, l, rhat, zhat, st, nb, dot);
+    interface_step_t<double>(h, l, rhat, zhat, st, nb, dot, after_kernel);
 }
 
 // Levels l > 1: interior pre-correction, interface step, interior post-correction
@@ -1471,14 +1477,15 @@ void full_step_t(bddc_handle_s* h, int l, const double* r, double* z, cudaStream
   launch_gather_glob<T>(L.d, r, 0, v, st, nb);                     // r_I
   trsv_pair<T>(h, L, v, 0, st, nb);                                // u1 = A_II^{-1} r_I
   launch_convert<T, double>(v, L.dl0, n, st);
-  launch_spmv_rows(L.d, L.rows[1], L.nrows[1], L.dl0, L.dl1, 1.0, 0.0, L.row_sub, st, nb);   // (A_GI u1)_i
-  launch_scatter_iface<double>(L.d, L.dl1, 0, L.gi0, st, nb);
+  launch_spmv_rows(L.d, L.rows[1], L.nrows[1], L.dl0, L.dl1, 1.0, 0.0, L.row_sub, st, nb, kAfterKernel);   // (A_GI u1)_i
+  launch_scatter_iface<double>(L.d, L.dl1, 0, L.gi0, st, nb, FusedDot(), kAfterKernel);
   launch_iface_rhs(L.gi1, r, L.d.n_dof, L.iface_dofs, L.gi0, L.d.n_iface, st, nb);   // r'_G = r_G - A_GI u1
-  interface_step(h, l, L.gi1, L.gi2, st, nb);                       // z_G
-  launch_gather_iface<double>(L.d, L.gi2, 0, L.dl0, st, nb);
+  interface_step(h, l, L.gi1, L.gi2, st, nb, FusedDot(), kAfterKernel);   // z_G
+  launch_gather_iface<double>(L.d, L.gi2, 0, L.dl0, st, nb, L.d.n_iface > 0 ? kAfterKernel : 0);
   launch_gather_glob<double>(L.d, r, 0, L.dl1, st, nb);
-  launch_spmv_rows(L.d, L.rows[0], L.nrows[0], L.dl0, L.dl1, -1.0, 1.0, L.row_sub, st, nb);  // r_I - A_IG z_G
-  launch_convert<double, T>(L.dl1, v, n, st);
+  launch_spmv_rows(L.d, L.rows[0], L.nrows[0], L.dl0, L.dl1, -1.0, 1.0, L.row_sub, st, nb,
+                   kAfterKernel);                                       // r_I - A_IG z_G
+  launch_convert<double, T>(L.dl1, v, n, st, kAfterKernel);
   trsv_pair<T>(h, L, v, 0, st, nb);                                 // z_I
   ck(cudaMemsetAsync(z, 0, sizeof(double) * L.d.n_dof * nb, st), "memset");
   launch_scatter_interior<T>(L.d, v, z, st, nb);
@@ -1493,8 +1500,8 @@ void full_step(bddc_handle_s* h, int l, const double* r, double* z, cudaStream_t
 }
 
 void precond(bddc_handle_s* h, const double* r, double* z, cudaStream_t st, int nb = 1,
-             const FusedDot& dot = FusedDot()) {
-  interface_step(h, 0, r, z, st, nb, dot);
+             const FusedDot& dot = FusedDot(), int after_kernel = 0) {
+  interface_step(h, 0, r, z, st, nb, dot, after_kernel);
 }
 
 double dot_host(bddc_handle_s* h, const double* a, const double* b, int64_t n) {
@@ -1533,14 +1540,16 @@ void choose_refinement(bddc_handle_s* h) {
   double prev = 1e300;
   float* t = (float*)L.locB;
   double* r = L.dl3;
-  ck(cudaMemsetAsync(w, 0, sizeof(double) * n, st), "memset");
   for (int steps = 1; steps <= 8; ++steps) {
     h->refine_steps = h->cur_steps = steps;
     launch_convert<double, float>(steps == 1 ? v : r, t, n, st);
     trsv_pair<float>(h, L, t, 0, st);
-    launch_add_to_double<float>(w, t, n, st);
-    ck(cudaMemcpyAsync(r, v, sizeof(double) * n, cudaMemcpyDeviceToDevice, st), "copy");
-    launch_spmv_rows(L.d, L.rows[0], L.nrows[0], w, r, -1.0, 1.0, L.row_sub, st);
+    if (steps == 1)
+      launch_convert<float, double>(t, w, n, st);
+    else
+      launch_add_to_double<float>(w, t, n, st);
+    launch_convert<double, double>(v, r, n, st, kAfterKernel);
+    launch_spmv_rows(L.d, L.rows[0], L.nrows[0], w, r, -1.0, 1.0, L.row_sub, st, 1, kAfterKernel);
     const double rel = nv > 0 ? std::sqrt(dot_host(h, r, r, n)) / nv : 0.0;
     if (rel > 0.5 * prev) break;          // stagnated at round-off: the previous count suffices
     best = steps;
@@ -2041,7 +2050,7 @@ void pcg_body(bddc_handle_s* h, double* x, int flexible, cudaStream_t st, int nb
   dot.mode = 2;
   dot.a = h->vr;
   dot.b = h->vq;
-  precond(h, h->vr, h->vz, st, nb, dot);                                     // z = M^{-1} r, r . z, q . z, beta
+  precond(h, h->vr, h->vz, st, nb, dot, kAfterKernel);                       // z = M^{-1} r, r . z, q . z, beta
   launch_pcg_update_p(h->vp, h->vz, S, n, st, nb);
 }
 
@@ -2055,12 +2064,12 @@ void bicg_body(bddc_handle_s* h, double* x, cudaStream_t st) {
   launch_dot(h->vrold, h->vr, n, h->partial, kDotBlocks, S + 3, st);
   launch_bicg_scalars(S, 0, st);
   launch_bicg_p(h->vp, h->vr, h->vq, S, n, st);
-  precond(h, h->vp, h->vz, st);
+  precond(h, h->vp, h->vz, st, 1, FusedDot(), kAfterKernel);
   schur_apply(h, h->vz, h->vq, st);
   launch_dot(h->vrold, h->vq, n, h->partial, kDotBlocks, S + 4, st);
   launch_bicg_scalars(S, 1, st);
   launch_bicg_s(h->vs, h->vr, h->vq, S, n, st);
-  precond(h, h->vs, h->vsh, st);
+  precond(h, h->vs, h->vsh, st, 1, FusedDot(), kAfterKernel);
   schur_apply(h, h->vsh, h->vt, st);
   launch_dot(h->vt, h->vs, n, h->partial, kDotBlocks, S + 5, st);
   launch_dot(h->vt, h->vt, n, h->partial, kDotBlocks, S + 6, st);

@@ -301,11 +301,15 @@ struct KrylovStore {
 // iteration's number (as int64) at mail[4 k + 3]; written by the update of x and r, half an iteration before its end.
 inline int64_t iface_blocks(int64_t n_iface) { return (n_iface + 255) / 256; }
 
+// after_kernel: kAfterKernel where the caller's last operation in the stream is a kernel launch (not a copy, a memset
+// or an event wait): the launch may then overlap that kernel's end (pdl.cuh)
+constexpr int kAfterKernel = 1;
 template <typename T>
-void launch_gather_iface(const LevelDev& L, const double* x, int weighted, T* loc, cudaStream_t st, int nr = 1);
+void launch_gather_iface(const LevelDev& L, const double* x, int weighted, T* loc, cudaStream_t st, int nr = 1,
+                         int after_kernel = 0);
 template <typename T>
 void launch_scatter_iface(const LevelDev& L, const T* loc, int weighted, double* y, cudaStream_t st, int nr = 1,
-                          const FusedDot& dot = FusedDot());
+                          const FusedDot& dot = FusedDot(), int after_kernel = 0);
 // inner operator around its FP32 product: loc = R_i x (FP32) and t = R C_i R_i x per constraint row; then
 // y = sum R_i^T (loc - C_i^T t) with the constraint row and entry of every position (crow, cval)
 void launch_inner_gather(const LevelDev& L, const double* x, float* loc, const int32_t* crow_sub, int64_t total_rows,
@@ -323,12 +327,12 @@ void launch_scatter_interior_diff(const LevelDev& L, const double* a, const doub
                                   int nr = 1);
 // rows: flat padded row indices (interior rows, interface rows or both, of every subdomain)
 void launch_spmv_rows(const LevelDev& L, const int64_t* rows, int64_t nrows, const double* x, double* y, double alpha,
-                      double beta, const int32_t* row_sub, cudaStream_t st, int nr = 1);
+                      double beta, const int32_t* row_sub, cudaStream_t st, int nr = 1, int after_kernel = 0);
 template <typename Tin, typename Tout>
-void launch_convert(const Tin* in, Tout* out, int64_t n, cudaStream_t st);
-void launch_axpy_loc(double* y, const double* x, double a, int64_t n, cudaStream_t st);
+void launch_convert(const Tin* in, Tout* out, int64_t n, cudaStream_t st, int after_kernel = 0);
+void launch_axpy_loc(double* y, const double* x, double a, int64_t n, cudaStream_t st, int after_kernel = 0);
 template <typename T>
-void launch_add_to_double(double* y, const T* x, int64_t n, cudaStream_t st);
+void launch_add_to_double(double* y, const T* x, int64_t n, cudaStream_t st, int after_kernel = 0);
 // r_C = sum R_Ci^T t_i with t_i = Psi_i^T r_i summed from its parts (part[(.) zmax + z], see launch_psi_t_apply)
 // and kept at rc_sub; v32 (or null): also as the FP32 input of the explicit coarsest inverse, position
 // v32_pos[g] of columns of n_v32

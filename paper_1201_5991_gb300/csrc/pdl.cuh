@@ -6,7 +6,8 @@
 // Such a kernel is alive while the kernels before it still write, so what they write may not be read as data that
 // is constant for the kernel's life: no __ldg, and no const __restrict__ parameter (from which the compiler
 // makes the same loads), for vectors of the running solve.  Data of the set-up may be read so.
-// Use only where the launch before it in the same stream is a kernel (not a copy, a memset or an event wait).
+// Use only where the launch before it in the same stream is a kernel (not a copy, a memset or an event wait):
+// the attribute speaks of the kernel before.  Helpers that are called in either place take after_kernel.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -17,7 +18,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
-inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+inline void launch_pdl_if(int after_kernel, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                          A... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -27,8 +29,13 @@ inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = after_kernel ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+template <typename... P, typename... A>
+inline void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  launch_pdl_if(1, kernel, grid, block, smem, st, args...);
 }
 
 }  // namespace bddc

@@ -649,13 +649,14 @@ inline unsigned nblocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); 
 }  // namespace
 
 template <typename T>
-void launch_gather_iface(const LevelDev& L, const double* x, int weighted, T* loc, cudaStream_t st, int nr) {
-  if (L.n_vec > 0) { note_launch(); launch_pdl(k_gather_iface<T>, dim3(nblocks(L.n_vec, 256), nr), 256, 0, st, L, x, weighted, loc); }
+void launch_gather_iface(const LevelDev& L, const double* x, int weighted, T* loc, cudaStream_t st, int nr,
+                         int after_kernel) {
+  if (L.n_vec > 0) { note_launch(); launch_pdl_if(after_kernel, k_gather_iface<T>, dim3(nblocks(L.n_vec, 256), nr), 256, 0, st, L, x, weighted, loc); }
 }
 template <typename T>
 void launch_scatter_iface(const LevelDev& L, const T* loc, int weighted, double* y, cudaStream_t st, int nr,
-                          const FusedDot& dot) {
-  if (L.n_iface > 0) { note_launch(); launch_pdl(k_scatter_iface<T>, dim3(nblocks(L.n_iface, 256), nr), 256, 0, st, L, loc, weighted, y, dot); }
+                          const FusedDot& dot, int after_kernel) {
+  if (L.n_iface > 0) { note_launch(); launch_pdl_if(after_kernel, k_scatter_iface<T>, dim3(nblocks(L.n_iface, 256), nr), 256, 0, st, L, loc, weighted, y, dot); }
 }
 void launch_inner_gather(const LevelDev& L, const double* x, float* loc, const int32_t* crow_sub, int64_t total_rows,
                          double* t, cudaStream_t st, int nr) {
@@ -668,13 +669,13 @@ void launch_inner_gather(const LevelDev& L, const double* x, float* loc, const i
     double* ts = t + (int64_t)r0 * total_rows;
     note_launch();
     if (g == 8)
-      launch_pdl(k_inner_gather<8>, nb, 256, 0, st, L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+      k_inner_gather<8><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
     else if (g == 4)
-      launch_pdl(k_inner_gather<4>, nb, 256, 0, st, L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+      k_inner_gather<4><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
     else if (g == 2)
-      launch_pdl(k_inner_gather<2>, nb, 256, 0, st, L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+      k_inner_gather<2><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
     else
-      launch_pdl(k_inner_gather<1>, nb, 256, 0, st, L, xs, ls, (int)nv, crow_sub, total_rows, ts);
+      k_inner_gather<1><<<nb, 256, 0, st>>>(L, xs, ls, (int)nv, crow_sub, total_rows, ts);
     r0 += g;
   }
 }
@@ -701,39 +702,40 @@ void launch_scatter_interior_diff(const LevelDev& L, const double* a, const doub
 }
 template <int NR>
 void launch_spmv_nr(const LevelDev& L, const int64_t* rows, int64_t nrows, const double* x, double* y, double alpha,
-                    double beta, const int32_t* row_sub, cudaStream_t st) {
+                    double beta, const int32_t* row_sub, cudaStream_t st, int after_kernel) {
   constexpr int LR = 4;
   note_launch();
-  launch_pdl(k_spmv<NR, LR>, nblocks(nrows * LR, 256), 256, 0, st, L, rows, nrows, x, y, alpha, beta, row_sub);
+  launch_pdl_if(after_kernel, k_spmv<NR, LR>, nblocks(nrows * LR, 256), 256, 0, st, L, rows, nrows, x, y, alpha, beta, row_sub);
 }
 void launch_spmv_rows(const LevelDev& L, const int64_t* rows, int64_t nrows, const double* x, double* y, double alpha,
-                      double beta, const int32_t* row_sub, cudaStream_t st, int nr) {
+                      double beta, const int32_t* row_sub, cudaStream_t st, int nr, int after_kernel) {
   if (nrows <= 0) return;
   for (int r0 = 0; r0 < nr;) {   // columns in groups of 8, 4, 2, 1: one pass over the matrix each
     const int left = nr - r0, g = left >= 8 ? 8 : left >= 4 ? 4 : left >= 2 ? 2 : 1;
     const double* xs = x + (int64_t)r0 * L.n_vec;
     double* ys = y + (int64_t)r0 * L.n_vec;
     if (g == 8)
-      launch_spmv_nr<8>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st);
+      launch_spmv_nr<8>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st, after_kernel);
     else if (g == 4)
-      launch_spmv_nr<4>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st);
+      launch_spmv_nr<4>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st, after_kernel);
     else if (g == 2)
-      launch_spmv_nr<2>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st);
+      launch_spmv_nr<2>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st, after_kernel);
     else
-      launch_spmv_nr<1>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st);
+      launch_spmv_nr<1>(L, rows, nrows, xs, ys, alpha, beta, row_sub, st, after_kernel);
     r0 += g;
+    after_kernel = kAfterKernel;
   }
 }
 template <typename Tin, typename Tout>
-void launch_convert(const Tin* in, Tout* out, int64_t n, cudaStream_t st) {
-  if (n > 0) { note_launch(); launch_pdl(k_convert<Tin, Tout>, nblocks(n, 256), 256, 0, st, in, out, n); }
+void launch_convert(const Tin* in, Tout* out, int64_t n, cudaStream_t st, int after_kernel) {
+  if (n > 0) { note_launch(); launch_pdl_if(after_kernel, k_convert<Tin, Tout>, nblocks(n, 256), 256, 0, st, in, out, n); }
 }
 template <typename T>
-void launch_add_to_double(double* y, const T* x, int64_t n, cudaStream_t st) {
-  if (n > 0) { note_launch(); launch_pdl(k_add_to_double<T>, nblocks(n, 256), 256, 0, st, y, x, n); }
+void launch_add_to_double(double* y, const T* x, int64_t n, cudaStream_t st, int after_kernel) {
+  if (n > 0) { note_launch(); launch_pdl_if(after_kernel, k_add_to_double<T>, nblocks(n, 256), 256, 0, st, y, x, n); }
 }
-void launch_axpy_loc(double* y, const double* x, double a, int64_t n, cudaStream_t st) {
-  if (n > 0) { note_launch(); launch_pdl(k_axpy, nblocks(n, 256), 256, 0, st, y, x, a, n); }
+void launch_axpy_loc(double* y, const double* x, double a, int64_t n, cudaStream_t st, int after_kernel) {
+  if (n > 0) { note_launch(); launch_pdl_if(after_kernel, k_axpy, nblocks(n, 256), 256, 0, st, y, x, a, n); }
 }
 void launch_coarse_gather(const LevelDev& L, const double* part, int zmax, double* rc_sub, int64_t sum_nc, double* rC,
                           float* v32, const int32_t* v32_pos, int64_t n_v32, cudaStream_t st, int nr) {
@@ -825,16 +827,16 @@ void launch_bicg_xr(double* x, double* r, const double* ph, const double* sh, co
 }
 
 #define INST(T)                                                                             \
-  template void launch_gather_iface<T>(const LevelDev&, const double*, int, T*, cudaStream_t, int); \
-  template void launch_scatter_iface<T>(const LevelDev&, const T*, int, double*, cudaStream_t, int, const FusedDot&); \
+  template void launch_gather_iface<T>(const LevelDev&, const double*, int, T*, cudaStream_t, int, int); \
+  template void launch_scatter_iface<T>(const LevelDev&, const T*, int, double*, cudaStream_t, int, const FusedDot&, int); \
   template void launch_gather_glob<T>(const LevelDev&, const double*, int, T*, cudaStream_t, int);  \
   template void launch_scatter_interior<T>(const LevelDev&, const T*, double*, cudaStream_t, int);  \
-  template void launch_add_to_double<T>(double*, const T*, int64_t, cudaStream_t);
+  template void launch_add_to_double<T>(double*, const T*, int64_t, cudaStream_t, int);
 INST(float)
 INST(double)
 #undef INST
-template void launch_convert<double, float>(const double*, float*, int64_t, cudaStream_t);
-template void launch_convert<float, double>(const float*, double*, int64_t, cudaStream_t);
-template void launch_convert<double, double>(const double*, double*, int64_t, cudaStream_t);
+template void launch_convert<double, float>(const double*, float*, int64_t, cudaStream_t, int);
+template void launch_convert<float, double>(const float*, double*, int64_t, cudaStream_t, int);
+template void launch_convert<double, double>(const double*, double*, int64_t, cudaStream_t, int);
 
 }  // namespace bddc

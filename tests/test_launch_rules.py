@@ -1,7 +1,8 @@
-"""The rule of pdl.cuh for kernels that may start before the kernel before them has ended, kept by the sources.
+"""The rules of pdl.cuh for kernels that may start before the kernel before them has ended, kept by the sources.
 
 Such a kernel (its body calls pdl_wait) is alive while others still write, so a vector of the running solve may
-not be read as constant data: not through __ldg and not through a const __restrict__ parameter."""
+not be read as constant data: not through __ldg and not through a const __restrict__ parameter.  And it may be
+launched so only directly behind a kernel, not behind a copy, a memset or an event wait."""
 import glob
 import os
 import re
@@ -36,3 +37,21 @@ def test_early_kernels_read_running_vectors_with_ordinary_loads():
         assert const <= SETUP_PARAMS, (name, const - SETUP_PARAMS)
         for load in re.findall(r"__ldg\(\s*(?:\(const \w+\*\))?\s*\(?\s*([\w.]+)", body):
             assert load in SETUP_LOADS, (name, load)
+
+
+def test_early_launches_follow_kernels():
+    s = _source("capi.cpp")
+    breaks = ("cudaMemcpyAsync", "cudaMemsetAsync", "cudaStreamWaitEvent")
+    stmts = [t for t in re.split(r"[;{}]", s)]
+    early = 0
+    for i, t in enumerate(stmts):
+        if "kAfterKernel" not in t or "launch_" not in t:
+            continue
+        early += 1
+        before = next(b for b in reversed(stmts[:i]) if re.search(r"\w+(<[^()]*>)?\s*\(", b) and "ProfScope" not in b)
+        assert not any(b in before for b in breaks), (before, t)
+    assert early > 8
+    # helpers that are called behind copies and memsets launch plainly unless their caller says otherwise
+    v = _source("vector.cu")
+    for helper in ("gather_iface", "spmv", "convert", "add_to_double", "axpy"):
+        assert not re.search(r"launch_pdl\(k_" + helper + r"\b", v), helper
