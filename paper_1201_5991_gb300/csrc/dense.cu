@@ -759,6 +759,8 @@ __global__ void k_small_chol_inv(LevelDev L) {
 // products) stays on one SM, by panels of 16 columns in shared memory; the inverse of the factor takes a
 // warp per column and the product W^T W a thread per entry, over the whole chip.
 
+constexpr int kPanelMaxNc = 1600;   // its panel of 16 columns takes 213 KB of shared memory
+
 // G = L L^T in place; the strictly upper part receives L^T (its rows are the columns of L)
 __global__ void __launch_bounds__(1024) k_gram_potrf(LevelDev L) {
   constexpr int PW = 16;
@@ -1463,18 +1465,16 @@ void launch_gram_chol(const LevelDev& L, int precision_fp32, int max_nc, cudaStr
   }
   // one pass per subdomain where n_c is small (its four launches would be longer) or G indefinite, and where the
   // panel of 16 columns does not fit
-  if (L.indefinite || max_nc <= 96 || max_nc > 1600) {
+  if (L.indefinite || max_nc <= 96 || max_nc > kPanelMaxNc) {
     note_launch();
     k_small_chol_inv<<<ns, 256, 0, st>>>(L);
     return;
   }
   const size_t sm = sizeof(double) * 17 * (size_t)max_nc, smw = sizeof(double) * 4 * (size_t)max_nc;
-  static size_t attr = 48 * 1024;
-  if (sm > attr) {
-    cudaFuncSetAttribute(k_gram_potrf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(k_gram_linv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smw > 49152 ? smw : 49152));
-    attr = sm;
-  }
+  // the limits of the largest n_c at every set-up: the attribute is one per device, other threads launch with it, and
+  // one set to this level's need could fall below theirs
+  cudaFuncSetAttribute(k_gram_potrf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double) * 17 * kPanelMaxNc));
+  cudaFuncSetAttribute(k_gram_linv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double) * 4 * kPanelMaxNc));
   const unsigned ge = (unsigned)(((int64_t)max_nc * max_nc + 255) / 256);
   { note_launch(); k_gram_potrf<<<ns, 1024, sm, st>>>(L); }
   { note_launch(); k_gram_linv<<<dim3((unsigned)((max_nc + 3) / 4), ns), 128, smw, st>>>(L, max_nc); }
