@@ -2190,17 +2190,23 @@ void freeze_column(bddc_handle_s* h, int k) {
 }
 
 // Wait until the device has mailed iteration `it` of every column.  The stream is asked now and then, so that a
-// failed launch or kernel ends the wait.
-void wait_mail(bddc_handle_s* h, int64_t it, int nb) {
+// failed launch or kernel ends the wait.  The host thread waits as the device's flags say: with blocking
+// synchronisation it sleeps until the whole iteration has ended (its preconditioner too), with yielding it offers the
+// core between polls, else it polls.
+void wait_mail(bddc_handle_s* h, int64_t it, int nb, unsigned schedule) {
+  if (schedule == cudaDeviceScheduleBlockingSync) ck(cudaStreamSynchronize(h->st), "sync");
+  const bool yield = schedule == cudaDeviceScheduleYield;
   for (int k = 0; k < nb; ++k) {
     const int64_t* seq = (const int64_t*)(h->mail + 4 * k + 3);
-    for (int64_t spins = 1; __atomic_load_n(seq, __ATOMIC_ACQUIRE) < it; ++spins)
-      if (spins % (1 << 16) == 0) {
+    for (int64_t spins = 1; __atomic_load_n(seq, __ATOMIC_ACQUIRE) < it; ++spins) {
+      if (yield) std::this_thread::yield();
+      if (spins % (yield ? 1 << 10 : 1 << 16) == 0) {
         const cudaError_t e = cudaStreamQuery(h->st);
         if (e == cudaErrorNotReady) continue;
         ck(e, "Krylov iteration");
         if (__atomic_load_n(seq, __ATOMIC_ACQUIRE) < it) fail(BDDC_ERR_CUDA, "a Krylov iteration did not report");
       }
+    }
   }
 }
 
@@ -2244,6 +2250,9 @@ std::vector<PcgResult> pcg(bddc_handle_s* h, const double* g, double* x, const s
   }
   if (active == 0) return res;
   std::memset(h->mail, 0, sizeof(double) * 4 * kMaxBlock);   // no iteration is in flight
+  unsigned schedule = 0;
+  ck(cudaGetDeviceFlags(&schedule), "cudaGetDeviceFlags");
+  schedule &= cudaDeviceScheduleMask;
   pcg_start(h, g, x, true, st, nb, project);
   const bool graphs = h->opts.use_graph && x == h->vx;
   drop_graph_if_kind_differs(h, flexible, nb);
@@ -2260,7 +2269,7 @@ std::vector<PcgResult> pcg(bddc_handle_s* h, const double* g, double* x, const s
     // the residual comes by mail when the iteration has updated it, while its preconditioner still runs: the
     // next iteration is enqueued behind it without a gap (a copy and a synchronisation at the end of every
     // iteration left the GPU idle for about 12 us)
-    wait_mail(h, it, nb);
+    wait_mail(h, it, nb, schedule);
     if (replayed && !h->graph_prof.empty()) {
       ck(cudaStreamSynchronize(st), "sync");
       accumulate_graph_profile(h);
