@@ -375,6 +375,14 @@ int bddc_batching_ablation(bddc_handle h, double* ms);
  * wait of the update kernel gave up). */
 int bddc_tc_update_check(int64_t n, int rank, float* a, double* ms);
 
+/* Test entry point for the products around G = Y S Y^T of mixed levels, through the kernels of the set-up (FP32
+ * entries, sums that hold FP64's digits): g = Y S Y^T (nc x nc, FP64) and z = Y^T Ginv (n x nc, rounded to FP32).
+ * y: host FP32 nc x n row-major; sgn: host FP32 [n], entries 1 or -1; ginv: host FP64 nc x nc, symmetric; rho > 0:
+ * the augmentation of the subdomain, whose square root the kernels scale Y by.  Device buffers are allocated and
+ * freed by the call, on the default stream.  Errors: INVALID, CUDA, OOM. */
+int bddc_gram_check(int64_t n, int64_t nc, double rho, const float* y, const float* sgn, const double* ginv, double* g,
+                    float* z);
+
 /* Test only: while bytes > 0, an allocation of device memory that a call on this host thread makes for a
  * handle fails as out of memory if the handle would then hold more than `bytes`; 0 ends it. */
 int bddc_alloc_probe(int64_t bytes);

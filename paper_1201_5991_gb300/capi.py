@@ -34,7 +34,7 @@ EXPORTED = [
     "bddc_solve_host", "bddc_apply_precond", "bddc_apply_schur", "bddc_grad", "bddc_get_maps",
     "bddc_get_stats", "bddc_sizes", "bddc_free", "bddc_last_error", "bddc_kernel_launches",
     "bddc_reset_profile", "bddc_grad_noalloc", "bddc_batching_ablation", "bddc_get_coarse",
-    "bddc_tc_update_check", "bddc_apply_inner_schur", "bddc_alloc_probe",
+    "bddc_tc_update_check", "bddc_apply_inner_schur", "bddc_alloc_probe", "bddc_gram_check",
 ]
 (PROF_TRSV, PROF_FACTOR, PROF_SPMV, PROF_TRMV, PROF_TRSV_IFACE, PROF_COARSE, PROF_TC_UPDATE, PROF_TC_PANEL,
  PROF_CLASSES) = (0, 1, 2, 3, 4, 5, 6, 7, 8)
@@ -129,6 +129,8 @@ def lib() -> C.CDLL:
     L.bddc_get_maps.argtypes = [H, C.c_int, C.POINTER(LevelMaps)]
     L.bddc_get_coarse.argtypes = [H, C.c_int, C.POINTER(C.c_double), C.c_int64]
     L.bddc_tc_update_check.argtypes = [C.c_int64, C.c_int, C.POINTER(C.c_float), C.POINTER(C.c_double)]
+    L.bddc_gram_check.argtypes = [C.c_int64, C.c_int64, C.c_double, C.POINTER(C.c_float), C.POINTER(C.c_float),
+                                  C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_float)]
     L.bddc_alloc_probe.argtypes = [C.c_int64]
     L.bddc_get_stats.argtypes = [H, C.POINTER(Stats)]
     L.bddc_sizes.argtypes = [H, C.POINTER(C.c_int64), C.POINTER(C.c_int64)]

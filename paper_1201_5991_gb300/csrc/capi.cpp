@@ -3081,6 +3081,57 @@ int bddc_get_coarse(bddc_handle h, int level, double* kc, int64_t n) {
   });
 }
 
+int bddc_gram_check(int64_t n, int64_t nc, double rho, const float* y, const float* sgn, const double* ginv, double* g,
+                    float* z) {
+  return guarded([&]() {
+    if (n < 1 || nc < 1 || n > 65536 || nc > 4096 || !y || !sgn || !ginv || !g || !z)
+      fail(BDDC_ERR_INVALID, "bddc_gram_check: needs 1 <= n <= 65536, 1 <= nc <= 4096 and buffers");
+    cudaStream_t st = nullptr;
+    DevArena A;
+    A.st = st;
+    try {
+      // one subdomain without interior: its constraint rows Y lie below the (unused) factor tiles
+      SubMeta m{};
+      m.n = m.nG = (int32_t)n;
+      m.nc = (int32_t)nc;
+      m.nGb = m.Bc = (int32_t)ceil_div(n, NB);
+      m.ncb = (int32_t)ceil_div(nc, NB);
+      m.R = m.Bc + m.ncb;
+      std::vector<float> yt((size_t)m.ncb * m.Bc * NB2, 0.f), s((size_t)m.Bc * NB, 1.f);
+      for (int64_t a = 0; a < nc; ++a)
+        for (int64_t c = 0; c < n; ++c)
+          yt[(size_t)(((a / NB) * m.Bc + c / NB) * NB2 + (a % NB) * NB + c % NB)] = y[a * n + c];
+      std::copy(sgn, sgn + n, s.begin());
+      const int64_t yo = tile_of(m, m.Bc, 0) * NB2;
+      LevelDev d{};
+      d.n_sub = 1;
+      d.n_vec = (int64_t)m.Bc * NB;
+      d.meta = A.upload(std::vector<SubMeta>{m}, st);
+      float* tiles = A.alloc<float>(yo + (int64_t)yt.size());
+      d.tiles = tiles;
+      ck(cudaMemcpyAsync(tiles + yo, yt.data(), sizeof(float) * yt.size(), cudaMemcpyHostToDevice, st), "upload");
+      d.sgn = A.upload(s, st);
+      d.rho = A.upload(std::vector<double>{rho}, st);
+      d.Ginv = A.alloc<double>(nc * nc);
+      float* psi = A.alloc<float>(d.n_vec * nc);
+      d.psi = psi;
+      launch_gram_f32(d, (int)nc, st);
+      ck(cudaGetLastError(), "launch");
+      ck(cudaMemcpyAsync(g, d.Ginv, sizeof(double) * (size_t)(nc * nc), cudaMemcpyDeviceToHost, st), "d2h");
+      ck(cudaMemcpyAsync(d.Ginv, ginv, sizeof(double) * (size_t)(nc * nc), cudaMemcpyHostToDevice, st), "h2d");
+      launch_psi_rhs_f32(d, m.nGb, (int)nc, st);
+      ck(cudaGetLastError(), "launch");
+      ck(cudaMemcpyAsync(z, psi, sizeof(float) * (size_t)(n * nc), cudaMemcpyDeviceToHost, st), "d2h");
+      ck(cudaStreamSynchronize(st), "sync");
+    } catch (...) {
+      A.release();
+      throw;
+    }
+    A.release();
+    return BDDC_OK;
+  });
+}
+
 int bddc_tc_update_check(int64_t n, int rank, float* a, double* ms) {
   return guarded([&]() {
     if (rank != 256 && rank != 512) fail(BDDC_ERR_INVALID, "bddc_tc_update_check: rank must be 256 or 512");

@@ -492,24 +492,45 @@ __global__ void k_gram(LevelDev L) {
   }
 }
 
-// ---- FP32 factors: G and Z = Y^T G^{-1} with double-float sums -------------------------------
+// ---- FP32 factors: G and Z = Y^T G^{-1} with sums in three FP32 parts -------------------------
 // The FP64 units give 2 products per cycle and SM, so these two products (n_G n_c^2 each) were bound by
 // them, with one warp or thread per entry and few blocks where n_c is large: 48^3 elasticity (n_c <= 78)
 // 1.5 + 1.4 ms per set-up, 64 k-means subdomains (n_c <= 258) 15 + 22 ms.  The factor's entries are FP32, so
-// a product a b is p + e exactly (e = fma(a, b, -p)), and a sum kept as an unevaluated FP32 pair (two-sum,
-// Knuth; Dekker) has 2^-46 relative error, far below the 2^-24 of the factor's entries: 10 FP32
-// operations per product at 128 lanes per cycle.  One block per 64 x 64 tile of the result, both
-// operands k-major in shared memory, 4 x 4 entries per thread.
-struct Pair2 {
-  float hi, lo;
+// a product a b is p + e exactly (e = fma(a, b, -p)), and a sum is kept as three unevaluated FP32 parts:
+// p goes into the first, what its addition rounds off and e into the second, what those additions round
+// off into the third, each by two-sum (Knuth; Dekker).  Only the additions into the third part round, at
+// 2^-72 of the sum: 22 FP32 operations per product at 128 lanes per cycle, and the sum comes out as exact as FP64
+// holds it.  With two parts (10 operations) the second rounds at every addition, and the error grows with the
+// length: root mean square relative to the sum for 64 / 1,024 / 6,016 squares 2^-46 / 2^-42 / 2^-40, where FP64 (32
+// lanes, then a tree) keeps 2^-53.6 / 2^-53 / 2^-50 and three parts 2^-54.2 at any of them.  The third part costs
+// 1 % of a 48^3 set-up and solve (96.0 -> 97.0 ms) and 2 % with 64 k-means subdomains (157.2 -> 160.4).
+// One block per 64 x 64 tile of the result, both operands k-major in shared memory, 4 x 4 entries per
+// thread.  Y is scaled by 2^k, G^{-1} by 2^-2k with 4^k about rho (G is at most 1 / rho), exactly, so that the small
+// parts stay above FP32's least numbers whatever the unit of the moduli.
+struct Sum3 {
+  float hi, mid, lo;
 };
 
-__device__ __forceinline__ void df_add(Pair2& s, float p, float e) {   // s += p + e, no contraction
-  const float t = __fadd_rn(s.hi, p);
-  const float b = __fsub_rn(t, s.hi);
-  const float err = __fadd_rn(__fsub_rn(s.hi, __fsub_rn(t, b)), __fsub_rn(p, b));
-  s.hi = t;
-  s.lo = __fadd_rn(s.lo, __fadd_rn(err, e));
+__device__ __forceinline__ float two_sum(float& s, float x) {   // s + x rounded into s; returns what was lost
+  const float t = __fadd_rn(s, x);
+  const float b = __fsub_rn(t, s);
+  const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b));
+  s = t;
+  return err;
+}
+
+__device__ __forceinline__ void add3(Sum3& s, float p, float e) {   // s += p + e
+  float r = two_sum(s.hi, p);
+  const float l = two_sum(r, e);
+  s.lo = __fadd_rn(s.lo, __fadd_rn(l, two_sum(s.mid, r)));
+}
+
+__device__ __forceinline__ double value3(const Sum3& s) { return (double)s.hi + ((double)s.mid + (double)s.lo); }
+
+__device__ __forceinline__ int gram_exponent(const LevelDev& L, int s) {
+  const double rho = L.rho[s];
+  const int k = rho > 0.0 && rho < 1e300 ? ilogb(rho) / 2 : 0;
+  return min(max(k, -60), 60);
 }
 
 // tile (a, b), b <= a, of G = Y_G S Y_G^T
@@ -522,19 +543,20 @@ __global__ void __launch_bounds__(256) k_gram_f32(LevelDev L) {
   if (ab >= m.ncb) return;
   __shared__ __align__(16) float As[NB][LDS], Bs[NB][LDS];
   const float* sG = (const float*)L.sgn + m.vec_off + (int64_t)m.nIb * NB;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  Pair2 acc[4][4];
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16, ex = gram_exponent(L, s);
+  const float sc = ldexpf(1.f, ex);
+  Sum3 acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = {0.f, 0.f};
+    for (int j = 0; j < 4; ++j) acc[i][j] = {0.f, 0.f, 0.f};
   for (int c = 0; c < m.nGb; ++c) {
     const float* ya = tile_ptr<float>(m, L.tiles, m.Bc + ab, m.nIb + c);
     const float* yb = tile_ptr<float>(m, L.tiles, m.Bc + bb, m.nIb + c);
     for (int e = threadIdx.x; e < NB2; e += 256) {
       const int r = e / NB, k = e % NB;
-      As[k][r] = ya[e];
-      Bs[k][r] = sG[c * NB + k] * yb[e];   // S = +-1: exact
+      As[k][r] = sc * ya[e];
+      Bs[k][r] = sG[c * NB + k] * (sc * yb[e]);   // S = +-1: exact
     }
     __syncthreads();
 #pragma unroll 4
@@ -547,7 +569,7 @@ __global__ void __launch_bounds__(256) k_gram_f32(LevelDev L) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const float p = __fmul_rn(a[i], b[j]);
-          df_add(acc[i][j], p, __fmaf_rn(a[i], b[j], -p));
+          add3(acc[i][j], p, __fmaf_rn(a[i], b[j], -p));
         }
     }
     __syncthreads();
@@ -561,7 +583,7 @@ __global__ void __launch_bounds__(256) k_gram_f32(LevelDev L) {
     for (int j = 0; j < 4; ++j) {
       const int r = ab * NB + 4 * ty + i, c = bb * NB + 4 * tx + j;
       if (r >= nc || c >= nc || c > r) continue;   // the diagonal tiles' upper halves mirror the lower
-      const double v = (double)acc[i][j].hi + (double)acc[i][j].lo;
+      const double v = ldexp(value3(acc[i][j]), -2 * ex);
       G[(int64_t)r * nc + c] = v;
       G[(int64_t)c * nc + r] = v;
       if (G0) {   // kept: Ginv is inverted in place
@@ -571,7 +593,7 @@ __global__ void __launch_bounds__(256) k_gram_f32(LevelDev L) {
     }
 }
 
-// rows 64 j .. of Z = Y_G^T G^{-1}, columns 64 qb ..: G^{-1} as an FP32 pair (gh + gl, 2^-48)
+// rows 64 j .. of Z = Y_G^T G^{-1}, columns 64 qb ..: G^{-1} as an FP32 pair (gh + gl, 2^-49); Z is rounded to FP32
 __global__ void __launch_bounds__(256) k_psi_rhs_f32(LevelDev L) {
   const int j = blockIdx.x, qb = blockIdx.y, s = blockIdx.z;
   const SubMeta m = L.meta[s];
@@ -580,19 +602,21 @@ __global__ void __launch_bounds__(256) k_psi_rhs_f32(LevelDev L) {
   float(*Ys)[NB] = (float(*)[NB])smem_raw;
   float(*Gh)[NB] = Ys + NB;
   float(*Gl)[NB] = Gh + NB;
-  const int nc = m.nc, tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const int nc = m.nc, tx = threadIdx.x % 16, ty = threadIdx.x / 16, ex = gram_exponent(L, s);
+  const float sc = ldexpf(1.f, ex);
+  const double scg = ldexp(1.0, -2 * ex);
   const double* Gi = L.Ginv + m.g_off;
-  Pair2 acc[4][4];
+  Sum3 acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = {0.f, 0.f};
+    for (int b = 0; b < 4; ++b) acc[a][b] = {0.f, 0.f, 0.f};
   for (int pb = 0; pb < m.ncb; ++pb) {
     const float* y = tile_ptr<float>(m, L.tiles, m.Bc + pb, m.nIb + j);
     for (int e = threadIdx.x; e < NB2; e += 256) {
       const int p = e / NB, c = e % NB, gp = pb * NB + p, gq = qb * NB + c;
-      Ys[p][c] = y[e];
-      const double g = gp < nc && gq < nc ? Gi[(int64_t)gp * nc + gq] : 0.0;
+      Ys[p][c] = sc * y[e];
+      const double g = gp < nc && gq < nc ? scg * Gi[(int64_t)gp * nc + gq] : 0.0;
       const float h = (float)g;
       Gh[p][c] = h;
       Gl[p][c] = (float)(g - (double)h);
@@ -610,7 +634,7 @@ __global__ void __launch_bounds__(256) k_psi_rhs_f32(LevelDev L) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const float v = __fmul_rn(a[i], h[k]);
-          df_add(acc[i][k], v, __fmaf_rn(a[i], l[k], __fmaf_rn(a[i], h[k], -v)));
+          add3(acc[i][k], v, __fmaf_rn(a[i], l[k], __fmaf_rn(a[i], h[k], -v)));
         }
     }
     __syncthreads();
@@ -621,7 +645,7 @@ __global__ void __launch_bounds__(256) k_psi_rhs_f32(LevelDev L) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int q = qb * NB + 4 * tx + k;
-      if (q < nc) Z[(int64_t)(j * NB + 4 * ty + i) * nc + q] = __fadd_rn(acc[i][k].hi, acc[i][k].lo);
+      if (q < nc) Z[(int64_t)(j * NB + 4 * ty + i) * nc + q] = (float)ldexp(value3(acc[i][k]), ex);
     }
 }
 
@@ -1453,13 +1477,24 @@ void launch_potrf_step(const LevelDev& L, int k, int max_R, int max_tiles, int j
   }
 }
 
+void launch_gram_f32(const LevelDev& L, int max_nc, cudaStream_t st) {
+  const unsigned nb = (unsigned)((max_nc + NB - 1) / NB);
+  note_launch();
+  k_gram_f32<<<dim3(nb * (nb + 1) / 2, (unsigned)L.n_sub), 256, 0, st>>>(L);
+}
+
+void launch_psi_rhs_f32(const LevelDev& L, int max_nGb, int max_nc, cudaStream_t st) {
+  note_launch();
+  k_psi_rhs_f32<<<dim3((unsigned)max_nGb, (unsigned)((max_nc + NB - 1) / NB), (unsigned)L.n_sub), 256,
+                  3 * NB2 * sizeof(float), st>>>(L);
+}
+
 void launch_gram_chol(const LevelDev& L, int precision_fp32, int max_nc, cudaStream_t st) {
   const unsigned ns = (unsigned)L.n_sub;
-  note_launch();
   if (precision_fp32) {
-    const unsigned nb = (unsigned)((max_nc + NB - 1) / NB);
-    k_gram_f32<<<dim3(nb * (nb + 1) / 2, ns), 256, 0, st>>>(L);
+    launch_gram_f32(L, max_nc, st);
   } else {
+    note_launch();
     const unsigned gx = (unsigned)(((int64_t)max_nc * max_nc + 7) / 8);
     k_gram<<<dim3(gx, ns), 256, 0, st>>>(L);
   }
@@ -1486,11 +1521,10 @@ template <typename T>
 void launch_psi(const LevelDev& L, int max_nGb, int max_nc, cudaStream_t st) {
   const unsigned ns = (unsigned)L.n_sub;
   if (max_nc <= 0 || max_nGb <= 0) return;
-  note_launch();
   if constexpr (sizeof(T) == 4) {
-    const size_t sm = 3 * NB2 * sizeof(float);
-    k_psi_rhs_f32<<<dim3((unsigned)max_nGb, (unsigned)((max_nc + NB - 1) / NB), ns), 256, sm, st>>>(L);
+    launch_psi_rhs_f32(L, max_nGb, max_nc, st);
   } else {
+    note_launch();
     k_psi_rhs<<<dim3(16, ns), 256, 0, st>>>(L);
   }
   const unsigned chunks = (unsigned)((max_nc + 15) / 16);

@@ -228,6 +228,9 @@ void launch_update_tc2(const LevelDev& L, int nq, int jbeg, int jend, int ibeg, 
                        const int64_t* item_pref, const TensorMap128& tmap, cudaStream_t st);
 // the identity tiles (R + r, nIb + r) of the inverse rows (the other tiles start as zero)
 void launch_unit_rows(const LevelDev& L, int max_nGb, cudaStream_t st);
+// FP32 levels: G = Y_G S Y_G^T (Ginv, and G where it is kept), and Z = Y_G^T G^{-1} into psi
+void launch_gram_f32(const LevelDev& L, int max_nc, cudaStream_t st);
+void launch_psi_rhs_f32(const LevelDev& L, int max_nGb, int max_nc, cudaStream_t st);
 void launch_gram_chol(const LevelDev& L, int precision_fp32, int max_nc, cudaStream_t st);
 template <typename T>
 void launch_psi(const LevelDev& L, int max_nGb, int max_nc, cudaStream_t st);

@@ -298,3 +298,16 @@ def tc_update_check(a: np.ndarray, rank: int = 512):
     ms = C.c_double()
     capi.check(capi.lib().bddc_tc_update_check(a.shape[0], int(rank), _ptr(a, C.c_float), C.byref(ms)))
     return a, ms.value
+
+
+def gram_check(y: np.ndarray, sgn: np.ndarray, ginv: np.ndarray, rho: float = 1.0):
+    """(Y S Y^T in FP64, Y^T Ginv in FP32) of FP32 rows y [nc, n], signs sgn [n] and ginv [nc, nc], through the kernels
+    that make G and Psi's right-hand side in a mixed set-up."""
+    y = np.ascontiguousarray(y, dtype=np.float32)
+    sgn = np.ascontiguousarray(sgn, dtype=np.float32)
+    ginv = np.ascontiguousarray(ginv, dtype=np.float64)
+    nc, n = y.shape
+    g, z = np.empty((nc, nc)), np.empty((n, nc), dtype=np.float32)
+    capi.check(capi.lib().bddc_gram_check(n, nc, float(rho), _ptr(y, C.c_float), _ptr(sgn, C.c_float), _ptr(ginv, C.c_double),
+                                          _ptr(g, C.c_double), _ptr(z, C.c_float)))
+    return g, z
