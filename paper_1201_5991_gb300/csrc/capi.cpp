@@ -2558,8 +2558,10 @@ PcgResult fgmres(bddc_handle_s* h, const double* g, double* x, double tol, int m
 // and every inner solve starts from zero.
 void prepare_kstore(bddc_handle_s* h) {
   if (!h->use_outer || h->kstore_blk >= h->blk) return;
-  ck(cudaStreamSynchronize(h->st), "sync");
-  drop_graph(h);   // a cached iteration refers to the old storage
+  if (h->iter_graph) {   // a cached iteration refers to the old storage
+    ck(cudaStreamSynchronize(h->st), "sync");
+    drop_graph(h);
+  }
   DevArena& A = h->arena;
   // one block of memory, and the handle holds none while it changes: an allocation that fails leaves no
   // pointer to the old one behind
