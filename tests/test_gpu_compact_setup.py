@@ -53,3 +53,28 @@ def test_forms_of_one_shape_are_tuned_apart():
     assert BddcSolver(p, precision="mixed").stats().tune_ms > 0
     assert BddcSolver(p, precision="mixed").stats().tune_ms == 0
     assert BddcSolver(p, precision="mixed", tensor_cores=2).stats().tune_ms > 0
+
+
+def test_compact_operators_match():
+    # interiors of 17 block rows: sweeps by 256-wide diagonal blocks against plain ones, and the interface inverse
+    # against interface sweeps; S x is refined to FP64 accuracy (1e-11: kappa(K_II) 2^-53 and some), the preconditioner
+    # has the tensor-core factor's accuracy (1e-2, as in test_gpu_tc_panels.py)
+    p = meshgen.elasticity3d(16, 2, seed=4)
+    full = BddcSolver(p, precision="mixed")
+    full.solve(_dev(p.f[:, 0]), tol=1e-10)
+    held, small = full.last_stats.factor_bytes, None
+    try:
+        for step in range(40):
+            capi.lib().bddc_alloc_probe(int(held * (1.2 - 0.025 * step)))
+            s = BddcSolver(p, precision="mixed")
+            s.solve(_dev(p.f[:, 0]), tol=1e-10)
+            if s.last_stats.factor_bytes < 0.9 * (held - 1024 * s.n_iface):
+                small = s
+                break
+    finally:
+        capi.lib().bddc_alloc_probe(0)
+    assert small is not None
+    R = _dev(np.random.default_rng(2).standard_normal((3, full.n_iface)))
+    for op, tol in (("apply_schur", 1e-11), ("apply_precond", 1e-2)):
+        a, b = getattr(full, op)(R), getattr(small, op)(R)
+        assert float((a - b).norm() / a.norm()) < tol, op

@@ -96,3 +96,19 @@ def test_solves_with_less_store_or_none(probe):
         assert {"all": grown > 6 * store, "16": grown == 0, "8": -store < grown < 0, "none": grown <= -store}[room], room
         probe(0)
     assert its["all"] <= its["16"] <= its["none"] and its["8"] <= its["none"], its
+
+
+def test_directions_are_forgotten_when_the_inner_operator_changes():
+    # a tolerance below what FP64 reaches: the outer steps stagnate, the inner operator becomes the FP64 one, whose
+    # solves start from its own directions; neither that solve nor the next, with the first operator again, is wrong
+    p = meshgen.elasticity3d(8, 4, seed=4, nrhs=2)
+    ref = fem.direct_solve(p)
+    s = BddcSolver(p, precision="mixed")
+    f = _dev(p.f[:, 0])
+    before = s.solve(f, tol=1e-10)
+    u = s.solve(f, tol=1e-18, allow_not_converged=True)
+    assert s.last_stats.outer_iterations > 6 and s.last_stats.rel_residual < 1e-12
+    assert _rel(u.cpu().numpy(), ref[:, 0]) < 1e-9
+    assert torch.equal(s.solve(f, tol=1e-10), before)
+    U = s.solve(_dev(p.f.T), tol=1e-18, allow_not_converged=True).cpu().numpy()
+    assert all(_rel(U[k], ref[:, k]) < 1e-9 for k in range(2))
