@@ -1293,7 +1293,8 @@ void trsv_pair(bddc_handle_s* h, Level& L, T* v, int part, cudaStream_t st, int 
 // w = K_II^{-1} v on level 1 (interior positions), FP64 accuracy; the operation before it is a kernel.  The launch
 // behind a sweep is a plain one, here and in full_step: with it launched over the sweep's end too, the short
 // kernels up to the next sweep are a chain of four such launches, and S x takes longer by 30 us of 628 (24^3, 8
-// subdomains; 64 subdomains 205 -> 188, 48^3 2,562 -> 2,553).
+// subdomains; 64 subdomains 205 -> 188, 48^3 2,562 -> 2,553).  The plain FP64 form has one sweep pair and fewer
+// kernels behind it; there the early launch stays (32^2 Poisson solve 1.40 -> 1.38 ms).
 // FP64 factors: two sweeps.  FP32 factors: iterative refinement with the FP64 K_II.
 void interior_solve_l1(bddc_handle_s* h, Level& L, const double* v, double* w, cudaStream_t st, int nb = 1) {
   const int64_t n = L.n_vec * nb;
@@ -1318,6 +1319,9 @@ void interior_solve_l1(bddc_handle_s* h, Level& L, const double* v, double* w, c
     }
   }
 }
+
+// whether an interior solve's last operation is a kernel (without interiors an FP64 one is a copy)
+int interior_solve_kernel(const Level& L) { return L.fp32 || L.ntasks[0][0] > 0 ? kAfterKernel : 0; }
 
 // y = S x on the level-1 interface (Sec. 2, discrete Dirichlet problems).  With cur_steps = 0
 // on an FP32 level: the inner operator S~ = sum R_i^T (L_GG S L_GG^T - C_i^T R C_i) R_i from the
@@ -1345,7 +1349,7 @@ void schur_apply(bddc_handle_s* h, const double* x, double* y, cudaStream_t st, 
   launch_gather_iface<double>(L.d, x, 0, L.dl0, st, nb);                 // x_i = R_i x
   launch_spmv_rows(L.d, L.rows[0], L.nrows[0], L.dl0, L.dl1, 1.0, 0.0, L.row_sub, st, nb, kAfterKernel);  // v = K_IG x_i
   interior_solve_l1(h, L, L.dl1, L.dl2, st, nb);                        // w = K_II^{-1} v
-  launch_axpy_loc(L.dl0, L.dl2, -1.0, n, st, L.fp32 ? kAfterKernel : 0);   // t = [-w ; x_i]
+  launch_axpy_loc(L.dl0, L.dl2, -1.0, n, st, interior_solve_kernel(L));   // t = [-w ; x_i]
   launch_spmv_rows(L.d, L.rows[1], L.nrows[1], L.dl0, L.dl1, 1.0, 0.0, L.row_sub, st, nb,
                    kAfterKernel);                                       // y_i = K_GG x_i - K_GI w
   launch_scatter_iface<double>(L.d, L.dl1, 0, y, st, nb, dot, kAfterKernel);   // y = sum R_i^T y_i
@@ -1356,7 +1360,7 @@ void condensed_rhs(bddc_handle_s* h, const double* f, double* g, cudaStream_t st
   Level& L = h->lv[0];
   launch_gather_glob<double>(L.d, f, 0, L.dl1, st, nb);
   interior_solve_l1(h, L, L.dl1, L.wf, st, nb);
-  launch_spmv_rows(L.d, L.rows[1], L.nrows[1], L.wf, L.dl0, 1.0, 0.0, L.row_sub, st, nb, L.fp32 ? kAfterKernel : 0);
+  launch_spmv_rows(L.d, L.rows[1], L.nrows[1], L.wf, L.dl0, 1.0, 0.0, L.row_sub, st, nb, interior_solve_kernel(L));
   launch_scatter_iface<double>(L.d, L.dl0, 0, L.gi0, st, nb, FusedDot(), kAfterKernel);
   launch_iface_rhs(g, f, L.d.n_dof, L.iface_dofs, L.gi0, L.d.n_iface, st, nb);
 }
