@@ -502,10 +502,11 @@ __global__ void k_gram(LevelDev L) {
 // 2^-72 of the sum: 22 FP32 operations per product at 128 lanes per cycle, and the sum comes out as exact as FP64
 // holds it.  With two parts (10 operations) the second rounds at every addition, and the error grows with the
 // length: root mean square relative to the sum for 64 / 1,024 / 6,016 squares 2^-46 / 2^-42 / 2^-40, where FP64 (32
-// lanes, then a tree) keeps 2^-53.6 / 2^-53 / 2^-50 and three parts 2^-54.2 at any of them.  The third part costs
-// 1 % of a 48^3 set-up and solve (96.0 -> 97.0 ms) and 2 % with 64 k-means subdomains (157.2 -> 160.4).
-// One block per 64 x 64 tile of the result, both operands k-major in shared memory, 4 x 4 entries per
-// thread.  Y is scaled by 2^k, G^{-1} by 2^-2k with 4^k about rho (G is at most 1 / rho), exactly, so that the small
+// lanes, then a tree) keeps 2^-53.6 / 2^-53 / 2^-50 and three parts 2^-54.2 at any of them.
+// One block per 32 x 32 part of the result, both operands k-major in shared memory, 2 x 2 entries per thread: bound
+// by the FP32 operations, with 64 x 64 parts there were too few blocks (48^3: 192 of them for 152 SMs) and more
+// padding (n_c = 78 took 128 columns, now 96).  48^3 set-up and solve: pairs 96.2 ms, three parts by 64 x 64 97.7,
+// by 32 x 32 96.4; 64 k-means subdomains 157.4 / 159.6 / 159.2.  Y is scaled by 2^k, G^{-1} by 2^-2k with 4^k about rho (G is at most 1 / rho), exactly, so that the small
 // parts stay above FP32's least numbers whatever the unit of the moduli.
 struct Sum3 {
   float hi, mid, lo;
@@ -533,56 +534,58 @@ __device__ __forceinline__ int gram_exponent(const LevelDev& L, int s) {
   return min(max(k, -60), 60);
 }
 
-// tile (a, b), b <= a, of G = Y_G S Y_G^T
+constexpr int GB = 32;       // edge of a block's part of the result
+constexpr int LDG = GB + 2;   // k-major stride: two-way bank conflicts in the transposing stores
+
+// block (a, b), b <= a, of G = Y_G S Y_G^T
 __global__ void __launch_bounds__(256) k_gram_f32(LevelDev L) {
   const int s = blockIdx.y;
   const SubMeta m = L.meta[s];
   int ab = 0, t = blockIdx.x;
   while (t > ab) t -= ++ab;   // row block ab, column block t
-  const int bb = t;
-  if (ab >= m.ncb) return;
-  __shared__ __align__(16) float As[NB][LDS], Bs[NB][LDS];
+  const int r0 = GB * ab, c0 = GB * t, nc = m.nc;
+  if (r0 >= nc) return;
+  __shared__ __align__(16) float As[NB][LDG], Bs[NB][LDG];
   const float* sG = (const float*)L.sgn + m.vec_off + (int64_t)m.nIb * NB;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16, ex = gram_exponent(L, s);
   const float sc = ldexpf(1.f, ex);
-  Sum3 acc[4][4];
+  Sum3 acc[2][2];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = {0.f, 0.f, 0.f};
+    for (int j = 0; j < 2; ++j) acc[i][j] = {0.f, 0.f, 0.f};
   for (int c = 0; c < m.nGb; ++c) {
-    const float* ya = tile_ptr<float>(m, L.tiles, m.Bc + ab, m.nIb + c);
-    const float* yb = tile_ptr<float>(m, L.tiles, m.Bc + bb, m.nIb + c);
-    for (int e = threadIdx.x; e < NB2; e += 256) {
-      const int r = e / NB, k = e % NB;
+    const float* ya = tile_ptr<float>(m, L.tiles, m.Bc + r0 / NB, m.nIb + c) + (r0 % NB) * NB;
+    const float* yb = tile_ptr<float>(m, L.tiles, m.Bc + c0 / NB, m.nIb + c) + (c0 % NB) * NB;
+#pragma unroll
+    for (int u = 0; u < GB * NB / 256; ++u) {
+      const int e = threadIdx.x + 256 * u, r = e / NB, k = e % NB;
       As[k][r] = sc * ya[e];
       Bs[k][r] = sG[c * NB + k] * (sc * yb[e]);   // S = +-1: exact
     }
     __syncthreads();
-#pragma unroll 4
+#pragma unroll 8
     for (int k = 0; k < NB; ++k) {
-      float a[4], b[4];
-      load4(a, &As[k][4 * ty]);
-      load4(b, &Bs[k][4 * tx]);
+      const float2 av = *(const float2*)&As[k][2 * ty], bv = *(const float2*)&Bs[k][2 * tx];
+      const float a[2] = {av.x, av.y}, b[2] = {bv.x, bv.y};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < 2; ++j) {
           const float p = __fmul_rn(a[i], b[j]);
           add3(acc[i][j], p, __fmaf_rn(a[i], b[j], -p));
         }
     }
     __syncthreads();
   }
-  const int nc = m.nc;
   double* G = L.Ginv + m.g_off;
   double* G0 = L.G ? L.G + m.g_off : nullptr;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int r = ab * NB + 4 * ty + i, c = bb * NB + 4 * tx + j;
-      if (r >= nc || c >= nc || c > r) continue;   // the diagonal tiles' upper halves mirror the lower
+    for (int j = 0; j < 2; ++j) {
+      const int r = r0 + 2 * ty + i, c = c0 + 2 * tx + j;
+      if (r >= nc || c >= nc || c > r) continue;   // the diagonal blocks' upper halves mirror the lower
       const double v = ldexp(value3(acc[i][j]), -2 * ex);
       G[(int64_t)r * nc + c] = v;
       G[(int64_t)c * nc + r] = v;
@@ -593,46 +596,43 @@ __global__ void __launch_bounds__(256) k_gram_f32(LevelDev L) {
     }
 }
 
-// rows 64 j .. of Z = Y_G^T G^{-1}, columns 64 qb ..: G^{-1} as an FP32 pair (gh + gl, 2^-49); Z is rounded to FP32
+// rows 32 jb .. of Z = Y_G^T G^{-1}, columns 32 qb ..: G^{-1} as an FP32 pair (gh + gl, 2^-49); Z is rounded to FP32
 __global__ void __launch_bounds__(256) k_psi_rhs_f32(LevelDev L) {
-  const int j = blockIdx.x, qb = blockIdx.y, s = blockIdx.z;
+  const int j = blockIdx.x / (NB / GB), h0 = GB * (blockIdx.x % (NB / GB)), q0 = GB * blockIdx.y, s = blockIdx.z;
   const SubMeta m = L.meta[s];
-  if (j >= m.nGb || qb >= m.ncb) return;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float(*Ys)[NB] = (float(*)[NB])smem_raw;
-  float(*Gh)[NB] = Ys + NB;
-  float(*Gl)[NB] = Gh + NB;
-  const int nc = m.nc, tx = threadIdx.x % 16, ty = threadIdx.x / 16, ex = gram_exponent(L, s);
+  const int nc = m.nc;
+  if (j >= m.nGb || q0 >= nc) return;
+  __shared__ __align__(16) float Ys[NB][GB], Gh[NB][GB], Gl[NB][GB];
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16, ex = gram_exponent(L, s);
   const float sc = ldexpf(1.f, ex);
   const double scg = ldexp(1.0, -2 * ex);
   const double* Gi = L.Ginv + m.g_off;
-  Sum3 acc[4][4];
+  Sum3 acc[2][2];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = {0.f, 0.f, 0.f};
-  for (int pb = 0; pb < m.ncb; ++pb) {
-    const float* y = tile_ptr<float>(m, L.tiles, m.Bc + pb, m.nIb + j);
-    for (int e = threadIdx.x; e < NB2; e += 256) {
-      const int p = e / NB, c = e % NB, gp = pb * NB + p, gq = qb * NB + c;
-      Ys[p][c] = sc * y[e];
-      const double g = gp < nc && gq < nc ? scg * Gi[(int64_t)gp * nc + gq] : 0.0;
+    for (int b = 0; b < 2; ++b) acc[a][b] = {0.f, 0.f, 0.f};
+  for (int p0 = 0; p0 < nc; p0 += NB) {
+    const float* y = tile_ptr<float>(m, L.tiles, m.Bc + p0 / NB, m.nIb + j) + h0;
+    const int pn = min(NB, nc - p0);
+#pragma unroll
+    for (int u = 0; u < GB * NB / 256; ++u) {
+      const int e = threadIdx.x + 256 * u, p = e / GB, c = e % GB, gq = q0 + c;
+      Ys[p][c] = sc * y[p * NB + c];
+      const double g = p < pn && gq < nc ? scg * Gi[(int64_t)(p0 + p) * nc + gq] : 0.0;
       const float h = (float)g;
       Gh[p][c] = h;
       Gl[p][c] = (float)(g - (double)h);
     }
     __syncthreads();
-    const int pn = min(NB, nc - pb * NB);
-#pragma unroll 2
+#pragma unroll 4
     for (int p = 0; p < pn; ++p) {
-      float a[4], h[4], l[4];
-      load4(a, &Ys[p][4 * ty]);
-      load4(h, &Gh[p][4 * tx]);
-      load4(l, &Gl[p][4 * tx]);
+      const float2 av = *(const float2*)&Ys[p][2 * ty], hv = *(const float2*)&Gh[p][2 * tx], lv = *(const float2*)&Gl[p][2 * tx];
+      const float a[2] = {av.x, av.y}, h[2] = {hv.x, hv.y}, l[2] = {lv.x, lv.y};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 2; ++k) {
           const float v = __fmul_rn(a[i], h[k]);
           add3(acc[i][k], v, __fmaf_rn(a[i], l[k], __fmaf_rn(a[i], h[k], -v)));
         }
@@ -641,11 +641,11 @@ __global__ void __launch_bounds__(256) k_psi_rhs_f32(LevelDev L) {
   }
   float* Z = (float*)L.psi + m.psi_off;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int q = qb * NB + 4 * tx + k;
-      if (q < nc) Z[(int64_t)(j * NB + 4 * ty + i) * nc + q] = (float)ldexp(value3(acc[i][k]), ex);
+    for (int k = 0; k < 2; ++k) {
+      const int q = q0 + 2 * tx + k;
+      if (q < nc) Z[(int64_t)(j * NB + h0 + 2 * ty + i) * nc + q] = (float)ldexp(value3(acc[i][k]), ex);
     }
 }
 
@@ -1478,15 +1478,15 @@ void launch_potrf_step(const LevelDev& L, int k, int max_R, int max_tiles, int j
 }
 
 void launch_gram_f32(const LevelDev& L, int max_nc, cudaStream_t st) {
-  const unsigned nb = (unsigned)((max_nc + NB - 1) / NB);
+  const unsigned nb = (unsigned)((max_nc + GB - 1) / GB);
   note_launch();
   k_gram_f32<<<dim3(nb * (nb + 1) / 2, (unsigned)L.n_sub), 256, 0, st>>>(L);
 }
 
 void launch_psi_rhs_f32(const LevelDev& L, int max_nGb, int max_nc, cudaStream_t st) {
   note_launch();
-  k_psi_rhs_f32<<<dim3((unsigned)max_nGb, (unsigned)((max_nc + NB - 1) / NB), (unsigned)L.n_sub), 256,
-                  3 * NB2 * sizeof(float), st>>>(L);
+  k_psi_rhs_f32<<<dim3((unsigned)max_nGb * (NB / GB), (unsigned)((max_nc + GB - 1) / GB), (unsigned)L.n_sub), 256, 0,
+                  st>>>(L);
 }
 
 void launch_gram_chol(const LevelDev& L, int precision_fp32, int max_nc, cudaStream_t st) {
