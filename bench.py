@@ -503,7 +503,7 @@ def run_gpu(args, rank, world, local_rank):
                              "complement, else k_trmv_t + k_trmv_n with the stored interface factor",
              capi.PROF_SPMV: "k_spmv (FP64 CSR products with K_i)",
              capi.PROF_FACTOR: "factorisation steps on CUDA cores (diagonal blocks: k_potrf_diag, k_trsm_panel, "
-                               "k_syrk_update; k_block_inverse, k_split_inverse, k_split_panel)",
+                               "k_syrk_update with the inverse rows of the blocks, k_split_inverse, k_split_panel)",
              capi.PROF_TC_PANEL: "k_update_tc2 as the panel solve A(i, D) X^T S_D below each 256 x 256 diagonal "
                                  "block (FP32-equivalent flops of the triangular solves it replaces)",
              capi.PROF_TC_UPDATE: "k_update_tc2 (rank-256 and rank-512 trailing updates of 512-wide super-panels "

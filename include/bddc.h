@@ -138,7 +138,7 @@ typedef struct {
                                Tile-copy waits are not affected. */
   int inner_operator;       /* mixed PCG, inner operator S~ of the outer refinement: 0 = automatic
                                (the explicit form when the interior padding it needs adds at most 40 %
-                               to the interior factor, else the factor products), 1 = products with
+                               to the interior factor, 8 % in a compact set-up, else the factor products), 1 = products with
                                the stored interface factor, S~ x = L_GG S L_GG^T x - C^T R C x,
                                2 = the explicit augmented Schur complement S_i + C_i^T R C_i, copied
                                from the tiles when the interior is eliminated (the interior block
@@ -250,6 +250,8 @@ int bddc_analyze(const bddc_mesh* mesh, const bddc_partition* part, unsigned con
  * Mixed PCG handles with an outer refinement also keep the search directions of a solve: 1 KB per
  * interface DOF, 8 KB from the first block of right-hand sides on, at most 4 GB; where that memory
  * is not to be had they keep fewer or none, and solves take more iterations.
+ * Mixed handles hold interface inverses and other data that only saves time; a set-up that runs
+ * out of device memory with them is made again in a compact form without (interface sweeps).
  * Errors: INVALID, BREAKDOWN (stats via bddc_get_stats), CUDA, OOM. */
 int bddc_setup(const bddc_mesh* mesh, const bddc_partition* part, unsigned constraints,
                const bddc_opts* opts, void* stream, bddc_handle* out);

@@ -2602,7 +2602,7 @@ void prepare_kstore(bddc_handle_s* h) {
 // Columns that meet the tolerance get a zero outer residual, so the inner PCG leaves them alone.  Restarting
 // CG at every outer step lost its Krylov space (48^3, tol 1e-10: 96 iterations where one CG needs about 60);
 // each inner solve after the first starts from the Galerkin projection of its residual on the directions of
-// the earlier ones (S~ p is at hand as q), which takes the slow modes out (76 iterations).
+// the earlier ones (S~ p is at hand as q), which takes the slow modes out (79 iterations).
 // The solution is left in h->vs; h->vt holds the outer residual.
 std::vector<PcgResult> pcg_refined(bddc_handle_s* h, const double* g, double tol, int maxit, int nb) {
   constexpr int kMaxOuter = 40;
